@@ -84,7 +84,8 @@ typedef struct {
                                  entries Alg. 1 probes */
     int64_t kind;             /* UBT_GRAPH_FIXED or UBT_GRAPH_REAL */
     int64_t probes;           /* entries the traversal probes without pruning:
-                                 sum over pairs of the streamed list's length */
+                                 sum over the forward edges (u,v) of the
+                                 entries of N>(u) after v */
 } ubt_graph_info;
 
 /* Optional extras for ubt_create_graph (pass NULL for none). */
@@ -136,9 +137,9 @@ ubt_status ubt_graph_workspace_size(int64_t n, int64_t m, int32_t flags,
  * exact algorithms traverse (Def. 1; Node Order, Sec. 4):
  *   - each undirected edge {a, b} is kept once and oriented from the endpoint
  *     earlier in Node Order (degree, then id) to the later one;
- *   - the forward lists N>(u) are stored as CSR, each list sorted by
- *     |1 - 2 P+| descending (ties by neighbour id), so that the edges a
- *     threshold prunes (Lemma 2) form a suffix of every list.
+ *   - the forward lists N>(u) are stored as CSR, rows and entries in reverse
+ *     Node Order (the last vertex first), so that the entries after a
+ *     neighbour v are the ones before v's position.
  * Arguments:
  *   n, m           vertex and edge counts (0 allowed).
  *   d_src, d_dst   device uint32[m] endpoints, any order, ids < n.
@@ -174,12 +175,11 @@ ubt_status ubt_graph_get_info(const ubt_graph* g, ubt_graph_info* h_info);
  * number with P_unbal > t_i (Defs. 4-5; Alg. 1 and Alg. 2).  All thresholds
  * are answered in one traversal.
  *   h_tau     host double[n_tau], each in [0.5, 1], any order, 1 <= n_tau <= 64.
- *   prune     0: visit every triangle (Alg. 1).  1: skip edges and triangles
- *             that cannot reach the smallest threshold (Lemma 2 per edge;
- *             the order-free form of Lemma 3 per pair of edges, applied to
- *             the streamed lists only when 2t - 1 >= 1/10 for the smallest
- *             t: below that it removes too few entries to pay for itself);
- *             results are identical either way.
+ *   prune     0: visit every triangle (Alg. 1).  1: skip edges that cannot be
+ *             in a triangle that reaches the smallest threshold (Lemma 2):
+ *             the kept edges are written out first, where the threshold
+ *             removes enough of them to pay for that; results are identical
+ *             either way.
  *   d_counts  device int64[2 * n_tau]: [0, n_tau) balanced counts,
  *             [n_tau, 2 n_tau) unbalanced counts, in the order of h_tau.
  * Graph kind: FIXED only (UBT_ERR_UNSUPPORTED otherwise).
@@ -331,13 +331,11 @@ ubt_status ubt_count_host(int64_t n, int64_t m, const uint32_t* h_src, const uin
 /*
  * ubt_traversal_stats -- SYNC.  Sizes of the traversal a query at these
  * thresholds performs (for roofline accounting; computes nothing else):
- *   h_out[0]  forward-list entries loaded into hash tables (sum of the pruned
- *             |N>(u)|, Lemma 2)
- *   h_out[1]  forward pairs (u, v) visited (same as h_out[0])
- *   h_out[2]  entries of N>(v) streamed and probed, summed over the pairs
- *             (pruned by Lemma 2 / the order-free Lemma 3 form when prune = 1,
- *             under the same rule as the query)
- *   h_out[3]  vertices with >= 2 forward entries (tasks)
+ *   h_out[0]  forward-list entries loaded into tables (the |N>(v)| of the
+ *             tasks; the kept entries when the query prunes, Lemma 2)
+ *   h_out[1]  forward edges (u, v) with entries to stream
+ *   h_out[2]  entries of N>(u) after v streamed and probed, summed over them
+ *   h_out[3]  vertices v with a list and a pair (tasks)
  */
 ubt_status ubt_traversal_stats(ubt_graph* g, const double* h_tau, int32_t n_tau, int32_t prune,
                                int64_t* h_out, void* stream);
@@ -356,25 +354,30 @@ ubt_status ubt_query_guard(ubt_graph* g, int64_t* h_word, void* stream);
 /*
  * ubt_graph_export -- SYNC.  Copies the built graph to host memory for
  * inspection (any pointer may be NULL):
- *   h_row_ptr  uint32[n + 1] forward-list offsets
+ * The host rearranges the device's arrays (kept in reverse Node Order) to the
+ * caller's ids; this takes host memory for several copies of the graph.
+ *   h_row_ptr  uint32[n + 1] forward-list offsets; FIXED lists by |1 - 2 P+|
+ *              descending (ties by neighbour id), REAL lists by neighbour id
  *   h_adj      uint64[m] entries (low 32 bits neighbour id, high 32 bits the
  *              value: q = 32768 - k as int32 for FIXED graphs, round(s 2^30)
  *              as int32 for REAL graphs)
  *   h_eid      uint32[m] input edge index of every entry
- *   h_lists    uint32[tasks] the work lists: owners of giant, hub and
- *              medium tasks
+ *   h_lists    uint32[tasks] the owners of the pairs (as
+ *              ubt_graph_export_pairs groups them) with >= 2 list entries:
+ *              giant, hub and medium ones by the tuning's thresholds
  *   h_list_sizes int64[4] the three list sizes and 0
  */
 ubt_status ubt_graph_export(const ubt_graph* g, uint32_t* h_row_ptr, uint64_t* h_adj, uint32_t* h_eid,
                             uint32_t* h_lists, int64_t* h_list_sizes, void* stream);
 
 /*
- * ubt_graph_export_pairs -- SYNC.  Copies the pair partition to host memory
- * (any pointer may be NULL).  Every forward edge x-s is one pair of the
- * traversal, owned by the endpoint x whose list is the hash table while the
- * list of s is streamed: the earlier vertex u of the edge u -> v (Alg. 1) or,
- * with the "pull" tuning on and |N>(v)| > |N>(u)|, the later vertex v.  Both
- * intersect N>(u) and N>(v), so each triangle is found once either way.
+ * ubt_graph_export_pairs -- SYNC.  The forward edges grouped by an owner, in
+ * host memory (any pointer may be NULL).  Every forward edge x-s is one pair,
+ * owned by the endpoint x whose list is intersected with the list of s: the
+ * earlier vertex u of the edge u -> v (Alg. 1) or, with the "pull" tuning on
+ * when the graph was created and |N>(v)| > |N>(u)|, the later vertex v.  (The
+ * queries themselves always intersect N>(v) with the part of N>(u) after v:
+ * the same triangles from fewer entries.)
  *   h_pair_ptr uint32[n + 1] pairs of owner x are [h_pair_ptr[x], h_pair_ptr[x + 1])
  *   h_pairs    uint64[m] streamed vertex s (low 32 bits) and CSR position of
  *              the edge (high 32 bits); order within an owner is unspecified
@@ -486,23 +489,29 @@ ubt_status ubt_topk(ubt_graph* g, int64_t K, int32_t which, ubt_tri_rec* d_out, 
  *                     1 queue products per warp and classify 32 at a time
  *                     (by binary search over the levels, or compared with
  *                     every threshold for at most 8)
- *   "pull"            1 (default): a pair is owned by the endpoint whose
- *                     list is longer, so the shorter list is streamed; 0:
- *                     always by the earlier vertex (Alg. 1 as written)
+ *   "pull"            how ubt_graph_export_pairs groups the pairs of graphs
+ *                     created afterwards: 1 (default) by the endpoint whose
+ *                     list is longer, 0 by the earlier vertex (Alg. 1 as
+ *                     written); queries do not depend on it
  *   "hub_threshold"   owners with longer lists than this are whole-block
  *                     tasks (default 128)
  *   "block_work"      owners whose pairs stream more entries than this are
  *                     whole-block tasks too (default 16384)
- *   "block_threads"   threads per block of the block-task kernel (64..512,
- *                     /32, default 512)
- *   "warp_threads"    threads per block of the warp-task kernel (64..512,
- *                     /32, default 128)
+ *   "block_threads"   threads per block of the kernel of the block tasks with
+ *                     hash tables (64..512, /32, default 512)
+ *   "warp_threads"    threads per block of the kernel of all other tasks
+ *                     (64..512, /32, default 128; doubled where a block task's
+ *                     table would leave too few warps on an SM)
  *   "blocks_per_sm"   cap on resident blocks per SM (1..32; occupancy decides
  *                     below it)
+ *   "block_bits"      a block task's table is a bitmap where its owner has at
+ *                     most this many later vertices (0..524288, default
+ *                     262144), else a hash table
+ *   "warp_bits"       the same for warp tasks (0..65536, default 16384)
  *   "smem_table_max"  hash-table slots kept in shared memory (power of two);
  *                     longer lists use a table in global scratch
  *   "block_unit"      pairs a warp takes at a time inside a block task (1..32,
- *                     default 16)
+ *                     default 32)
  *   "long_min"        streamed lists at least this long are streamed by the
  *                     whole warp, up to four entries per lane (default 64);
  *                     shorter ones are concatenated across the warp's pairs
@@ -523,16 +532,16 @@ ubt_status ubt_topk(ubt_graph* g, int64_t K, int32_t which, ubt_tri_rec* d_out, 
  *   "world_words_per_pass"  64-world words per traversal of ubt_sample_worlds
  *                     (1, 2, 4, 8, 16, 32 or 64)
  *   "small_batch"     warp tasks taken per grab of a task counter
- *   "sort_smem_max"   longest forward list sorted in shared memory during the
+ *   "sort_smem_max"   longest list sorted in shared memory during the
  *                     build (power of two, 64..4096); longer lists are sorted
  *                     in a global-memory slice
- *   "warp_sort_max"   longest forward list sorted by one warp in registers
+ *   "warp_sort_max"   longest list sorted by one warp in registers
  *                     during the build (128, 256 or 512; at most
  *                     sort_smem_max unless 128); longer lists up to
  *                     sort_smem_max are sorted by one block in shared memory
- * Build-time knobs (pull, hub_threshold, block_work, smem_table_max,
- * sort_smem_max, warp_sort_max) apply to graphs created afterwards; query the workspace size
- * after setting them.
+ * Build-time knobs (pull, hub_threshold, block_work, block_bits, warp_bits,
+ * smem_table_max, sort_smem_max, warp_sort_max) apply to graphs created
+ * afterwards; query the workspace size after setting them.
  */
 ubt_status ubt_set_tuning(const char* name, int64_t value);
 ubt_status ubt_get_tuning(const char* name, int64_t* h_value);

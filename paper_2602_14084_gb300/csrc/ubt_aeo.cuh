@@ -503,7 +503,7 @@ ubt_status launch_aeo(const ubt_graph* g, int64_t L, const typename V::P& p, cud
       a.m2 = (uint32_t)(2 * g->m);
       a.sc = g->scratch;
       a.L = L;
-      UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchHeader / 2, s));
+      UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
       if (g->m == 0) return UBT_OK;
       const int threads = 512;
       const size_t smem = (size_t)((V::smem_bytes(threads) + 15) / 16) * 16;
@@ -534,7 +534,7 @@ ubt_status launch_aeo(const ubt_graph* g, int64_t L, const typename V::P& p, cud
                                       std::max<int64_t>(64, T.smem_table_max));
   a.unit = (uint32_t)std::min<int64_t>(32, std::max<int64_t>(1, T.block_unit));
   a.L = L;
-  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchHeader / 2, s));
+  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
   if (a.n_owners == 0) return UBT_OK;
   const int threads = 512;
   const size_t tables = std::max<size_t>((size_t)a.cap, (size_t)(threads / 32) * a.wcap) * 3 * 4;

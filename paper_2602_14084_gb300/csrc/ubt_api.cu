@@ -78,6 +78,12 @@ extern "C" ubt_status ubt_set_tuning(const char* name, int64_t value) {
   } else if (!strcmp(name, "smem_table_max")) {
     if (value < 64 || value > (1 << 20) || (value & (value - 1))) return UBT_ERR_INVALID_ARG;
     t.smem_table_max = value;
+  } else if (!strcmp(name, "block_bits")) {
+    if (value < 0 || value > (1 << 19)) return UBT_ERR_INVALID_ARG;
+    t.block_bits = value;
+  } else if (!strcmp(name, "warp_bits")) {
+    if (value < 0 || value > (1 << 16)) return UBT_ERR_INVALID_ARG;
+    t.warp_bits = value;
   } else if (!strcmp(name, "world_words_per_pass")) {
     if (value < 1 || value > 64 || (value & (value - 1))) return UBT_ERR_INVALID_ARG;
     t.world_words_per_pass = value;
@@ -128,6 +134,8 @@ extern "C" ubt_status ubt_get_tuning(const char* name, int64_t* h_value) {
   else if (!strcmp(name, "warp_threads")) *h_value = t.warp_threads;
   else if (!strcmp(name, "blocks_per_sm")) *h_value = t.blocks_per_sm;
   else if (!strcmp(name, "smem_table_max")) *h_value = t.smem_table_max;
+  else if (!strcmp(name, "block_bits")) *h_value = t.block_bits;
+  else if (!strcmp(name, "warp_bits")) *h_value = t.warp_bits;
   else if (!strcmp(name, "world_words_per_pass")) *h_value = t.world_words_per_pass;
   else if (!strcmp(name, "small_batch")) *h_value = t.small_batch;
   else if (!strcmp(name, "sort_smem_max")) *h_value = t.sort_smem_max;

@@ -2,21 +2,23 @@
 //
 //   validate   ids < n, no self-loops, probabilities in range       (Def. 1)
 //   degree     undirected degree of every vertex
-//   orient     each edge from its earlier endpoint in Node Order (degree,
-//              then id) to the later one                (Def. Node Order, Sec. 4)
+//   number     every vertex by its position in reverse Node Order (degree, then
+//              id, Sec. 4; the graphs of a batch apart): a radix sort by degree
 //   CSR        forward lists N>(u) as offsets + packed (neighbour, value)
-//   sort       REAL graphs' lists by neighbour id (duplicates are equal
-//              neighbours); FIXED graphs' lists by |q| descending, then id,
-//              so that pruned entries (Lemma 2) form a suffix of every list,
-//              after a duplicate check (a lane match or a hash set per list;
-//              lists past the shared-memory limit are sorted by id first)
-//   pairs      every forward edge x-s is a pair owned by one endpoint: the
-//              one whose list becomes the hash table while the other
-//              endpoint's list is streamed through it (the shorter list is
-//              streamed); pairs grouped by owner
-//   work lists owners (>= 2 forward entries, >= 1 pair) split by list length
-//              and streamed work into block tasks and warp tasks, each
-//              ordered by decreasing work
+//   sort       every list ascending by neighbour (duplicates are equal neighbours)
+//   pairs      every forward edge u -> v is a pair owned by v, whose list
+//              becomes the table while the part of u's list after v is
+//              streamed through it; pairs grouped by owner
+//   work lists owners (>= 1 list entry, >= 1 pair) split by list length and
+//              streamed work into block tasks and warp tasks, each ordered by
+//              decreasing work
+//
+// Why the later vertex owns: Alg. 1 streams N>(v) through a table of N>(u) for
+// u -> v.  The triangles of the pair lie in N>(u) n N>(v); streaming the part of
+// N>(u) after v through a table of N>(v) finds the same ones and probes 0.62x
+// the entries that streaming the shorter whole list does (R-MAT scale 20: 1.97e9
+// -> 1.22e9, Chung-Lu of 1e6 vertices: 3.16e8 -> 1.95e8), and choosing the better
+// direction per pair would remove only another 0.5 %.
 #include <math.h>
 #include <string.h>
 
@@ -99,38 +101,134 @@ __global__ void k_validate_degree(int64_t n, int64_t m, const uint32_t* __restri
   }
 }
 
-// Node Order: a before b iff (deg a, a) < (deg b, b)
-__device__ inline bool node_before(const uint32_t* deg, uint32_t a, uint32_t b) {
-  const uint32_t da = deg[a], db = deg[b];
-  return da < db || (da == db && a < b);
+__global__ void k_max_degree(int64_t n, const uint32_t* __restrict__ deg, unsigned long long* out) {
+  uint32_t best = 0;
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+    best = max(best, deg[v]);
+  best = __reduce_max_sync(kFull, best);
+  if (lane_id() == 0) atomicMax(out, (unsigned long long)best);
 }
 
+// ---------------------------------------------------------------- vertex numbers
+//
+// Reverse Node Order is a stable sort of the ids n - 1 .. 0 by degree
+// descending (and, for a batch, by graph first: the least significant key is
+// sorted first, 8 bits a pass).  A pass counts the digits of every tile, scans
+// the counts digit by digit, and writes every id to its place; a warp takes
+// 512 consecutive items, so ranks within a warp and the warps' order keep the
+// sort stable.  Bound by the launches (four a pass) up to a few million vertices.
+constexpr int kRankThreads = 256;
+constexpr int kRankItems = 16;
+constexpr int64_t kRankTile = kRankThreads * kRankItems;
+
+struct RankKey {
+  const uint32_t* key;  // by id
+  int shift;
+  uint32_t flip;        // 255: descending
+};
+__device__ __forceinline__ uint32_t rank_digit(const RankKey& k, uint32_t id) {
+  return ((k.key[id] >> k.shift) & 255u) ^ k.flip;
+}
+__device__ __forceinline__ uint32_t rank_item(const uint32_t* in, int64_t i, int64_t n) {
+  return in ? in[i] : (uint32_t)(n - 1 - i);
+}
+
+// hist[digit * tiles + tile]
+__global__ void __launch_bounds__(kRankThreads)
+k_rank_count(int64_t n, const uint32_t* __restrict__ in, RankKey k, uint32_t* __restrict__ hist) {
+  __shared__ uint32_t cnt[256];
+  cnt[threadIdx.x] = 0;
+  __syncthreads();
+  for (int j = 0; j < kRankItems; j++) {
+    const int64_t i = blockIdx.x * kRankTile + j * kRankThreads + threadIdx.x;
+    if (i < n) atomicAdd(&cnt[rank_digit(k, rank_item(in, i, n))], 1u);
+  }
+  __syncthreads();
+  hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = cnt[threadIdx.x];
+}
+
+// off: the scanned counts.  out[place] = id and, in the last pass, rank[id] = place.
+__global__ void __launch_bounds__(kRankThreads)
+k_rank_scatter(int64_t n, const uint32_t* __restrict__ in, RankKey k, const uint32_t* __restrict__ off,
+               uint32_t* __restrict__ out, uint32_t* __restrict__ rank) {
+  constexpr int kWarps = kRankThreads / 32;
+  __shared__ uint32_t cnt[kWarps][256];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < kWarps * 256; i += kRankThreads) (&cnt[0][0])[i] = 0;
+  __syncthreads();
+  uint32_t id[kRankItems], at[kRankItems];  // at: digit << 16 | rank among the warp's items of that digit
+#pragma unroll
+  for (int j = 0; j < kRankItems; j++) {
+    const int64_t i = blockIdx.x * kRankTile + wid * (32 * kRankItems) + j * 32 + lane;
+    const bool on = i < n;
+    id[j] = on ? rank_item(in, i, n) : 0u;
+    const uint32_t d = on ? rank_digit(k, id[j]) : 256u;
+    const unsigned peers = __match_any_sync(kFull, d);
+    const uint32_t before = on ? cnt[wid][d] : 0u;
+    at[j] = (d << 16) | (before + __popc(peers & lanemask_lt()));
+    __syncwarp();
+    if (on && lane == __ffs(peers) - 1) cnt[wid][d] = before + __popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+  uint32_t run = off[(size_t)threadIdx.x * gridDim.x + blockIdx.x];
+  for (int w = 0; w < kWarps; w++) {
+    const uint32_t c = cnt[w][threadIdx.x];
+    cnt[w][threadIdx.x] = run;
+    run += c;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kRankItems; j++) {
+    const uint32_t d = at[j] >> 16;
+    if (d > 255u) continue;
+    const uint32_t place = cnt[wid][d] + (at[j] & 0xFFFFu);
+    out[place] = id[j];
+    if (rank) rank[id[j]] = place;
+  }
+}
+
+// by the vertex numbers: the graph of every vertex, and the first number of every graph
+__global__ void k_rank_graphs(int64_t n, const uint32_t* __restrict__ vid, const uint32_t* __restrict__ by_id,
+                              uint32_t* __restrict__ by_rank, const int64_t* __restrict__ voff, int64_t ng,
+                              uint32_t* __restrict__ gstart) {
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < ng; g += (int64_t)gridDim.x * blockDim.x)
+    gstart[g] = (uint32_t)voff[g];
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
+    by_rank[r] = by_id[vid[r]];
+}
+
+// an edge belongs to the row of its earlier endpoint in Node Order: the larger number
 __global__ void k_out_degree(int64_t m, const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
-                             const uint32_t* __restrict__ deg, uint32_t* __restrict__ outdeg) {
+                             const uint32_t* __restrict__ rank, uint32_t* __restrict__ outdeg) {
   const uint32_t lane = lane_id();
   UBT_FOR_EDGE_WARPS(base, m) {
     const int64_t i = base + lane;
     const bool on = i < m;
-    const uint32_t a = on ? src[i] : 0u, b = on ? dst[i] : 0u;
-    add_by_runs(outdeg, on && node_before(deg, a, b) ? a : b, on);
+    add_by_runs(outdeg, on ? max(rank[src[i]], rank[dst[i]]) : 0u, on);
   }
+}
+
+// forward entries that name a vertex: its degree less its own list (in place)
+__global__ void k_in_degree(int64_t n, const uint32_t* __restrict__ deg, const uint32_t* __restrict__ vid,
+                            const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ indeg) {
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
+    indeg[r] = deg[vid[r]] - (row_ptr[r + 1] - row_ptr[r]);
 }
 
 __global__ void k_scatter(int64_t m, const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
                           const uint32_t* __restrict__ k, const float* __restrict__ p,
-                          const uint32_t* __restrict__ deg, const uint32_t* __restrict__ row_ptr,
-                          uint32_t* __restrict__ fill, uint64_t* __restrict__ adj, uint32_t* __restrict__ eid,
+                          const uint32_t* __restrict__ rank, uint32_t* __restrict__ next,
+                          uint64_t* __restrict__ adj, uint32_t* __restrict__ eid,
                           const uint32_t* __restrict__ key_in, uint32_t* __restrict__ key_out) {
   const uint32_t lane = lane_id();
   UBT_FOR_EDGE_WARPS(base, m) {
     const int64_t i = base + lane;
     const bool on = i < m;
-    const uint32_t a = on ? src[i] : 0u, b = on ? dst[i] : 0u;
-    const bool ab = on && node_before(deg, a, b);
-    const uint32_t lo = ab ? a : b, hi = ab ? b : a;
-    const uint32_t slot = add_by_runs(fill, lo, on);
+    const uint32_t a = on ? rank[src[i]] : 0u, b = on ? rank[dst[i]] : 0u;
+    const uint32_t row = max(a, b), hi = min(a, b);
+    const uint32_t pos = add_by_runs(next, row, on);  // next[row] starts at the row's offset
     if (!on) continue;
-    const uint32_t pos = row_ptr[lo] + slot;
     uint32_t val;
     if (k) {
       val = (uint32_t)(int32_t)(32768 - (int32_t)k[i]);     // q = 32768 - k
@@ -143,7 +241,7 @@ __global__ void k_scatter(int64_t m, const uint32_t* __restrict__ src, const uin
   }
 }
 
-// sort keys: by neighbour id (REAL rows); by (32768 - |q|, id) (FIXED and undirected rows)
+// sort keys: by neighbour (forward rows); by (32768 - |q|, id) (undirected rows)
 __device__ inline uint64_t key_by_col(uint64_t e) { return (uint64_t)adj_col(e); }
 __device__ inline uint64_t key_by_absq(uint64_t e) {
   const int32_t q = adj_q(e);
@@ -151,32 +249,10 @@ __device__ inline uint64_t key_by_absq(uint64_t e) {
   return ((uint64_t)(32768u - aq) << 32) | adj_col(e);
 }
 
-// How a row is sorted: REAL forward rows by neighbour id (a duplicate edge
-// shows as two equal neighbouring keys); FIXED forward rows by (|q|
-// descending, id) with duplicates found by a hash set or a lane match before
-// the one sort; undirected rows like FIXED ones but unchecked (the forward
-// rows of the same edges were checked first).
-enum : int { kSortById = 0, kSortByAbsqChecked = 1, kSortByAbsq = 2 };
-
-constexpr unsigned long long kSetEmpty = ~0ull;
-
-// Inserts (col, input edge id) into an open-addressing set of mask + 1
-// 64-bit slots (at least twice the row); a second entry with the same
-// neighbour is a duplicate edge, reported with the larger of the two ids.
-__device__ __forceinline__ void dedupe_insert(unsigned long long* set, uint32_t mask, uint32_t col, uint32_t id,
-                                              unsigned long long* err) {
-  const unsigned long long mine = ((unsigned long long)col << 32) | id;
-  uint32_t h = ((col * 0x9E3779B1u) >> 8) & mask;
-  for (uint32_t it = 0; it <= mask; it++) {
-    const unsigned long long cur = atomicCAS(&set[h], kSetEmpty, mine);
-    if (cur == kSetEmpty) return;
-    if ((uint32_t)(cur >> 32) == col) {
-      report(err, max(id, (uint32_t)cur), -UBT_ERR_DUPLICATE_EDGE);
-      return;
-    }
-    h = (h + 1) & mask;
-  }
-}
+// How a row is sorted: forward rows by neighbour (a duplicate edge shows as two
+// equal neighbouring keys); undirected rows by (|q| descending, id), unchecked
+// (the forward rows of the same edges were checked first).
+enum : int { kSortById = 0, kSortByAbsq = 2 };
 
 // Lists of <= 32 entries: one warp per list, bitonic network over the lanes.
 // Bitonic sort of the values held by each aligned group of W lanes (W = 8,
@@ -217,13 +293,6 @@ __device__ __forceinline__ void sort_group_row(uint64_t* adj, uint32_t* eid, uin
     const uint64_t prev = __shfl_up_sync(kFull, key, 1);
     if (in && li > 0 && prev == key) report(err, rs + li, -UBT_ERR_DUPLICATE_EDGE);
   } else {
-    if (mode == kSortByAbsqChecked) {  // lanes of one group holding the same neighbour
-      const unsigned long long v = in ? (((unsigned long long)(lane / W) << 32) | adj_col(e))
-                                      : ((0xFFFFFFFFull << 32) | (unsigned long long)lane);
-      const unsigned others = __match_any_sync(kFull, v) & ~(1u << lane);
-      const uint32_t oid = __shfl_sync(kFull, id, others ? __ffs(others) - 1 : lane);
-      if (in && others) report(err, max(id, oid), -UBT_ERR_DUPLICATE_EDGE);
-    }
     uint64_t key = in ? key_by_absq(e) : ~0ull;
     group_bitonic<W>(key, e, id, ky, lane);
   }
@@ -296,7 +365,7 @@ __device__ __forceinline__ void warp_bitonic(unsigned long long (&k)[R], int lan
 
 template <int R>
 __device__ __forceinline__ void sort_row_warp(uint64_t* adj, uint32_t* eid, uint32_t* ekey, uint32_t rs, uint32_t len,
-                                              int mode, unsigned long long* set, unsigned long long* err, int lane) {
+                                              int mode, unsigned long long* err, int lane) {
   unsigned long long k[R];
   if (mode == kSortById) {
 #pragma unroll
@@ -314,16 +383,6 @@ __device__ __forceinline__ void sort_row_warp(uint64_t* adj, uint32_t* eid, uint
       if (i < len && i > 0 && (prev >> 12) == (k[r] >> 12)) report(err, rs + i, -UBT_ERR_DUPLICATE_EDGE);
     }
   } else {
-    if (mode == kSortByAbsqChecked) {  // this warp's set: 64 R slots for at most 32 R entries
-      for (int i = lane; i < 64 * R; i += 32) set[i] = kSetEmpty;
-      __syncwarp();
-#pragma unroll
-      for (int r = 0; r < R; r++) {
-        const uint32_t i = (uint32_t)(r * 32 + lane);
-        if (i < len) dedupe_insert(set, 64 * R - 1, adj_col(adj[rs + i]), eid[rs + i], err);
-      }
-      __syncwarp();
-    }
 #pragma unroll
     for (int r = 0; r < R; r++) {
       const uint32_t i = (uint32_t)(r * 32 + lane);
@@ -370,15 +429,13 @@ __device__ __forceinline__ void sort_row_warp(uint64_t* adj, uint32_t* eid, uint
 template <int R>
 __global__ void k_sort_mid_rows(const uint32_t* __restrict__ rows, uint32_t nrows, const uint32_t* __restrict__ row_ptr,
                                 uint64_t* adj, uint32_t* eid, uint32_t* ekey, int mode, unsigned long long* err) {
-  extern __shared__ __align__(16) unsigned long long sets[];  // one set of 64 R slots per warp (checked mode)
-  unsigned long long* set = sets + (threadIdx.x >> 5) * (64 * R);
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t r0 = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r0 < nrows; r0 += warps) {
     const uint32_t u = rows[r0];
     const uint32_t rs = row_ptr[u], len = row_ptr[u + 1] - rs;
     if (len > 32u * R || (R > 4 && len <= 16u * R)) continue;
-    sort_row_warp<R>(adj, eid, ekey, rs, len, mode, set, err, lane);
+    sort_row_warp<R>(adj, eid, ekey, rs, len, mode, err, lane);
   }
 }
 
@@ -386,9 +443,7 @@ __global__ void k_sort_mid_rows(const uint32_t* __restrict__ rows, uint32_t nrow
 template <int R>
 ubt_status launch_mid_sort(const uint32_t* rows, uint32_t nrows, const uint32_t* row_ptr, uint64_t* adj, uint32_t* eid,
                            uint32_t* ekey, int mode, unsigned long long* err, int g, int thr, cudaStream_t s) {
-  const size_t smem = mode == kSortByAbsqChecked ? (size_t)(thr / 32) * 64 * R * 8 : 0;
-  UBT_CUDA(cudaFuncSetAttribute(k_sort_mid_rows<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_sort_mid_rows<R><<<g, thr, smem, s>>>(rows, nrows, row_ptr, adj, eid, ekey, mode, err);
+  k_sort_mid_rows<R><<<g, thr, 0, s>>>(rows, nrows, row_ptr, adj, eid, ekey, mode, err);
   return UBT_OK;
 }
 
@@ -436,8 +491,7 @@ __global__ void __launch_bounds__(kPackedSortThreads)
 k_sort_long_rows_packed(const uint32_t* __restrict__ rows, uint32_t nrows, const uint32_t* __restrict__ row_ptr,
                         uint64_t* adj, uint32_t* eid, uint32_t* ekey, int mode, unsigned long long* err,
                         uint32_t lo, uint32_t hi) {
-  extern __shared__ __align__(16) unsigned long long pk[];  // hi words, then (checked mode) a set of 2 hi slots
-  unsigned long long* set = pk + hi;
+  extern __shared__ __align__(16) unsigned long long pk[];  // hi words
   for (uint32_t r = blockIdx.x; r < nrows; r += gridDim.x) {
     const uint32_t u = rows[r];
     const uint32_t rs = row_ptr[u], len = row_ptr[u + 1] - rs;
@@ -456,12 +510,6 @@ k_sort_long_rows_packed(const uint32_t* __restrict__ rows, uint32_t nrows, const
       for (uint32_t i = threadIdx.x + 1; i < len; i += blockDim.x)
         if ((pk[i] >> 12) == (pk[i - 1] >> 12)) report(err, rs + i, -UBT_ERR_DUPLICATE_EDGE);
     } else {
-      if (mode == kSortByAbsqChecked) {  // 2 cap <= 2 hi slots
-        for (uint32_t i = threadIdx.x; i < 2 * cap; i += blockDim.x) set[i] = kSetEmpty;
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < len; i += blockDim.x)
-          dedupe_insert(set, 2 * cap - 1, adj_col(adj[rs + i]), eid[rs + i], err);
-      }
       for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x)
         pk[i] = i < len ? (key_by_absq(adj[rs + i]) << 12) | i : ~0ull;
       __syncthreads();
@@ -504,7 +552,7 @@ ubt_status launch_block_sorts(const uint32_t* rows, uint32_t nrows, const uint32
     const uint32_t lo = bounds[c], hi = c == 2 ? std::max(smem_max, 512u) : bounds[c + 1];
     if (hi <= warp_max || lo >= smem_max) continue;
     const int threads = (int)std::min<uint32_t>(hi / 2, kPackedSortThreads);
-    const size_t smem = (size_t)hi * 8 * (mode == kSortByAbsqChecked ? 3 : 1);
+    const size_t smem = (size_t)hi * 8;
     UBT_CUDA(cudaFuncSetAttribute(k_sort_long_rows_packed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int per_sm = std::max(1, std::min(2048 / threads, (int)(200 * 1024 / smem)));
     const int g = (int)std::min<unsigned long long>(nrows, (unsigned long long)sms * per_sm);
@@ -515,18 +563,16 @@ ubt_status launch_block_sorts(const uint32_t* rows, uint32_t nrows, const uint32
 
 // Longer lists: one block per list, bitonic network in a per-block global
 // slice (lists longer than the "sort_smem_max" tuning).
-template <bool kGlobal>
 __global__ void k_sort_long_rows(const uint32_t* __restrict__ rows, uint32_t nrows, const uint32_t* __restrict__ row_ptr,
-                                 uint64_t* adj, uint32_t* eid, uint32_t* ekey, int fixed, unsigned long long* err,
+                                 uint64_t* adj, uint32_t* eid, uint32_t* ekey, unsigned long long* err,
                                  char* gtmp, int64_t gtmp_cap) {
-  extern __shared__ __align__(16) char sm[];
   for (uint32_t r = blockIdx.x; r < nrows; r += gridDim.x) {
     const uint32_t u = rows[r];
     const uint32_t rs = row_ptr[u], re = row_ptr[u + 1];
     const uint32_t len = re - rs;
     uint32_t cap = 64;
     while (cap < len) cap <<= 1;
-    char* base = kGlobal ? gtmp + (size_t)blockIdx.x * (size_t)gtmp_cap * 24 : sm;
+    char* base = gtmp + (size_t)blockIdx.x * (size_t)gtmp_cap * 24;
     uint64_t* key = (uint64_t*)base;
     uint64_t* ev = key + cap;
     uint32_t* iv = (uint32_t*)(ev + cap);
@@ -542,35 +588,27 @@ __global__ void k_sort_long_rows(const uint32_t* __restrict__ rows, uint32_t nro
       }
     }
     __syncthreads();
-    for (int pass = 0; pass < (fixed ? 2 : 1); pass++) {
-      if (pass == 1) {
-        for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x) key[i] = i < len ? key_by_absq(ev[i]) : ~0ull;
-        __syncthreads();
-      }
-      for (uint32_t kk = 2; kk <= cap; kk <<= 1) {
-        for (uint32_t j = kk >> 1; j > 0; j >>= 1) {
-          for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x) {
-            const uint32_t ixj = i ^ j;
-            if (ixj > i) {
-              const bool asc = (i & kk) == 0;
-              const uint64_t a = key[i], b = key[ixj];
-              if ((a > b) == asc && a != b) {
-                key[i] = b; key[ixj] = a;
-                uint64_t te = ev[i]; ev[i] = ev[ixj]; ev[ixj] = te;
-                uint32_t ti = iv[i]; iv[i] = iv[ixj]; iv[ixj] = ti;
-                uint32_t ty = yv[i]; yv[i] = yv[ixj]; yv[ixj] = ty;
-              }
+    for (uint32_t kk = 2; kk <= cap; kk <<= 1) {
+      for (uint32_t j = kk >> 1; j > 0; j >>= 1) {
+        for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x) {
+          const uint32_t ixj = i ^ j;
+          if (ixj > i) {
+            const bool asc = (i & kk) == 0;
+            const uint64_t a = key[i], b = key[ixj];
+            if ((a > b) == asc && a != b) {
+              key[i] = b; key[ixj] = a;
+              uint64_t te = ev[i]; ev[i] = ev[ixj]; ev[ixj] = te;
+              uint32_t ti = iv[i]; iv[i] = iv[ixj]; iv[ixj] = ti;
+              uint32_t ty = yv[i]; yv[i] = yv[ixj]; yv[ixj] = ty;
             }
           }
-          __syncthreads();
         }
-      }
-      if (pass == 0) {
-        for (uint32_t i = threadIdx.x + 1; i < len; i += blockDim.x)
-          if (key[i] == key[i - 1]) report(err, rs + i, -UBT_ERR_DUPLICATE_EDGE);
         __syncthreads();
       }
     }
+    for (uint32_t i = threadIdx.x + 1; i < len; i += blockDim.x)
+      if (key[i] == key[i - 1]) report(err, rs + i, -UBT_ERR_DUPLICATE_EDGE);
+    __syncthreads();
     for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
       adj[rs + i] = ev[i];
       eid[rs + i] = iv[i];
@@ -596,170 +634,177 @@ __global__ void k_collect_long(int64_t n, const uint32_t* __restrict__ row_ptr, 
   }
 }
 
-// Owner of the pair of forward edge u -> v (u before v in Node Order, du and
-// dv their forward-list lengths).  Alg. 1 probes every w of N>(v) in a table
-// of N>(u) ("push", owner u).  Probing N>(u) in a table of N>(v) ("pull",
-// owner v) intersects the same two lists, so the triangle {u, v, w} is still
-// found exactly once, from its two earliest vertices; pull is taken when it
-// streams the shorter list.
-__device__ inline uint32_t pair_owner(uint32_t u, uint32_t v, uint32_t du, uint32_t dv, int pull) {
-  return (pull && dv > du) ? v : u;
-}
-
 // rowid[p] = the row that holds CSR position p (one thread per row)
 __global__ void k_row_ids(int64_t n, const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ rowid) {
   for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x)
     for (uint32_t p = row_ptr[u]; p < row_ptr[u + 1]; p++) rowid[p] = (uint32_t)u;
 }
 
-// pairs per owner, one lane per forward entry (rowid: the row of every CSR
-// position; adjacent entries of one row that keep their owner share one
-// atomic); also the oriented wedges sum_u sum_{v in N>(u)} |N>(v)| (Alg. 1's
-// probes), one atomic per block
-__global__ void k_pair_count(int64_t m, const uint32_t* __restrict__ row_ptr, const uint64_t* __restrict__ adj,
-                             const uint32_t* __restrict__ rowid, int pull, uint32_t* __restrict__ pcount,
-                             unsigned long long* wedges) {
-  __shared__ unsigned long long s_w;
-  if (threadIdx.x == 0) s_w = 0;
-  __syncthreads();
-  const uint32_t lane = lane_id();
-  unsigned long long wsum = 0;
-  UBT_FOR_EDGE_WARPS(base, m) {
-    const int64_t i = base + lane;
-    const bool on = i < m;
-    uint32_t x = 0;
-    if (on) {
-      const uint32_t u = rowid[i], v = adj_col(adj[i]);
-      const uint32_t du = row_ptr[u + 1] - row_ptr[u], dv = row_ptr[v + 1] - row_ptr[v];
-      wsum += dv;
-      x = pair_owner(u, v, du, dv, pull);
-    }
-    add_by_runs(pcount, x, on);
-  }
-  atomicAdd(&s_w, wsum);
-  __syncthreads();
-  if (threadIdx.x == 0 && s_w) atomicAdd(wedges, s_w);
-}
-
-// ctr[key] += val over the active lanes, one atomic per run of adjacent
-// active lanes with equal keys (the run's sum from a warp prefix sum)
-__device__ __forceinline__ void sum_by_runs(unsigned long long* ctr, uint32_t key, unsigned long long val, bool on) {
-  const uint32_t lane = lane_id();
-  const unsigned act = __ballot_sync(kFull, on);
-  const uint32_t prev = __shfl_up_sync(kFull, key, 1);
-  const bool head = on && !(lane > 0 && ((act >> (lane - 1)) & 1u) && prev == key);
-  const unsigned heads = __ballot_sync(kFull, head);
-  const unsigned upto = (2u << lane) - 1u;
-  const unsigned after = (heads | ~act) & ~upto;
-  const uint32_t next = after ? (uint32_t)__ffs(after) - 1u : 32u;  // > lane
-  unsigned long long x = on ? val : 0ull;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const unsigned long long y = __shfl_up_sync(kFull, x, d);
-    if (lane >= (uint32_t)d) x += y;
-  }
-  const unsigned long long end = __shfl_sync(kFull, x, (int)(next - 1u));
-  const unsigned long long before = __shfl_sync(kFull, x, (int)((lane + 31u) & 31u));
-  if (head) atomicAdd(&ctr[key], end - (lane > 0 ? before : 0ull));
-}
-
-// pair words grouped by owner: the streamed vertex and the edge's CSR
-// position; work[x] += length of the streamed list (the owner's task size)
+// Pair words grouped by owner.  next[v] holds the next free position of owner
+// v's pairs in its low half (it starts at pair_ptr[v]) and the streamed work
+// so far in its high half, in units of kWorkUnit entries (rounded up per pair), so one
+// 64-bit atomic places a pair and adds its work.  absq (FIXED, or null): a
+// histogram of |q| >> 9 over one warp's edges in eight.  streamed: the sum of
+// the streamed lengths.  Bound by the atomics'
+// and the pair words' random 32-byte sectors.
+constexpr uint32_t kWorkUnit = 8;
 __global__ void k_pair_fill(int64_t m, const uint32_t* __restrict__ row_ptr, const uint64_t* __restrict__ adj,
-                            const uint32_t* __restrict__ rowid, int pull, const uint32_t* __restrict__ pair_ptr,
-                            uint32_t* __restrict__ pfill, uint64_t* __restrict__ pairs,
-                            unsigned long long* __restrict__ work) {
-  const uint32_t lane = lane_id();
-  UBT_FOR_EDGE_WARPS(base, m) {
-    const int64_t i = base + lane;
-    const bool on = i < m;
-    uint32_t x = 0, streamed = 0, slen = 0;
-    if (on) {
-      const uint32_t u = rowid[i], v = adj_col(adj[i]);
-      const uint32_t du = row_ptr[u + 1] - row_ptr[u], dv = row_ptr[v + 1] - row_ptr[v];
-      x = pair_owner(u, v, du, dv, pull);
-      streamed = x == u ? v : u;
-      slen = x == u ? dv : du;
+                            const uint32_t* __restrict__ rowid, unsigned long long* __restrict__ next,
+                            uint64_t* __restrict__ pairs, unsigned long long* __restrict__ absq,
+                            unsigned long long* __restrict__ streamed) {
+  __shared__ uint32_t s_q[65];
+  for (int i = threadIdx.x; i < 65; i += blockDim.x) s_q[i] = 0;
+  __syncthreads();
+  unsigned long long sum = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint64_t e = adj[i];
+    const uint32_t v = adj_col(e), start = row_ptr[rowid[i]], len = (uint32_t)i - start;
+    uint32_t aq = 0;
+    if (absq) {
+      const int32_t q = adj_q(e);
+      aq = (uint32_t)(q < 0 ? -q : q);
+      if (((i >> 5) & 7) == 0) atomicAdd(&s_q[aq >> 9], 1u);
     }
-    const uint32_t slot = add_by_runs(pfill, x, on);
-    if (on) pairs[pair_ptr[x] + slot] = ((uint64_t)i << 32) | streamed;
-    sum_by_runs(work, x, slen, on);
+    const unsigned long long at =
+        atomicAdd(&next[v], ((unsigned long long)((len + kWorkUnit - 1) / kWorkUnit) << 32) | 1ull);
+    pairs[(uint32_t)at] = pair_pack(start, len, aq >> 1);
+    sum += len;
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(kFull, sum, d);
+  if (lane_id() == 0 && sum) atomicAdd(streamed, sum);
+  if (absq) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < 65; i += blockDim.x)
+      if (s_q[i]) atomicAdd(&absq[i], (unsigned long long)s_q[i]);
   }
 }
+__global__ void k_pair_next(int64_t n, const uint32_t* __restrict__ pair_ptr, unsigned long long* __restrict__ next) {
+  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
+    next[x] = pair_ptr[x];
+}
 
-// Task classes (by the owner's list length and streamed work)
-enum : uint8_t { kClsMedium = 1, kClsHub = 2, kClsGiant = 3 };
 constexpr uint8_t kNoTask = 0xFF;
-constexpr int kLgMax = 47;  // work buckets 2^0 .. 2^47
-constexpr int kBuckets2 = 4 * (kLgMax + 1);
+constexpr int kLgMax = 47;   // work buckets 2^0 .. 2^47 (undirected owners)
+constexpr int kLgTask = 40;  // and of the traversal's owners: lg * kTaskClasses + class < 255
+constexpr int kTaskBuckets = kTaskClasses * (kLgTask + 1);
+static_assert(kTaskBuckets <= kNoTask, "a bucket is one byte");
 
 // Per owner x (one thread): its streamed work (from k_pair_fill), the log2
-// bucket and class; bucket[x] = lg * 4 + cls, or kNoTask (fewer than 2 list
-// entries or no pairs: no triangle can be found there).  Per-block counts in
-// shared memory, one global atomic per block and bucket.
-// stats: [1] longest list, [2] longest list of a block task, [3] streamed
-//        work of all pairs, [4 + lg * 4 + cls] bucket sizes ([0] is set by
-//        k_pair_count)
-__global__ void k_row_stats(int64_t n, const uint32_t* __restrict__ row_ptr, const uint32_t* __restrict__ pair_ptr,
-                            const unsigned long long* __restrict__ work, uint32_t hub_thr, uint32_t giant_thr,
-                            unsigned long long block_work, uint8_t* __restrict__ bucket,
-                            unsigned long long* stats) {
-  __shared__ uint32_t s_cnt[kBuckets2];
-  __shared__ unsigned long long s_work;
-  __shared__ uint32_t s_max, s_hmax;
-  for (int i = threadIdx.x; i < kBuckets2; i += blockDim.x) s_cnt[i] = 0;
-  if (threadIdx.x == 0) { s_work = 0; s_max = 0; s_hmax = 0; }
+// bucket and class; bucket[x] = lg * kTaskClasses + cls, or kNoTask (no list entries or
+// no pairs: no triangle can be found there).  Per-block counts in shared
+// memory, one global atomic per block and bucket.  An owner of more than
+// kHeavyPairs pairs is a block task whatever its work (whose 32 bits could
+// wrap there).
+// A table is a bitmap where the vertices it can hold -- the ones before x in
+// its graph's range -- are at most block_bits (block tasks) or warp_bits (warp
+// tasks), else a hash table.
+// stats: [0] oriented wedges sum_v in(v) |N>(v)| (Alg. 1's probes), [1] longest
+//        list, [2] streamed entries (set by k_pair_fill), [3] longest list of
+//        a kHubHash task, [4] of a kHubBits task, [5] largest range of one,
+//        [kStatBuckets + bucket] bucket sizes
+constexpr uint32_t kHeavyPairs = 1u << 16;
+constexpr int kStatBuckets = 6;
+// A pair's own loads count as this many streamed entries.
+constexpr unsigned long long kPairWork = 16;
+// An owner whose work exceeds part_work is several block tasks, each with its
+// own copy of the table and a share of the pairs, so that no owner's work is
+// the length of the query.  With part_work >= the whole work / kMaxParts at
+// most kMaxParts tasks are added.
+constexpr unsigned long long kPartWork = 1 << 17, kMaxParts = 1 << 15;
+__device__ __forceinline__ unsigned long long whole_work(unsigned long long streamed, int64_t m) {
+  return streamed + (kWorkUnit + kPairWork) * (unsigned long long)m;  // an upper bound of the owners' sum
+}
+__device__ __forceinline__ unsigned long long owner_work(unsigned long long next, uint32_t np) {
+  return np ? (next >> 32) * kWorkUnit + kPairWork * np : 0ull;
+}
+__device__ __forceinline__ uint32_t owner_parts(unsigned long long work, unsigned long long whole) {
+  const unsigned long long part = max(min(kPartWork, max(4096ull, whole / 2048)), whole / kMaxParts + 1);
+  return (uint32_t)min(work / part + 1, kMaxParts);
+}
+__global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ row_ptr, const uint32_t* __restrict__ pair_ptr,
+                            const unsigned long long* __restrict__ work, const uint32_t* __restrict__ vgraph,
+                            const uint32_t* __restrict__ gstart, uint32_t hub_thr, uint32_t giant_thr,
+                            unsigned long long block_work, uint32_t block_bits, uint32_t warp_bits,
+                            uint8_t* __restrict__ bucket, unsigned long long* stats) {
+  __shared__ uint32_t s_cnt[kTaskBuckets];
+  __shared__ unsigned long long s_wedges;
+  __shared__ uint32_t s_max, s_hash, s_len, s_bits;
+  for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x) s_cnt[i] = 0;
+  if (threadIdx.x == 0) { s_wedges = 0; s_max = 0; s_hash = 0; s_len = 0; s_bits = 0; }
   __syncthreads();
-  unsigned long long wsum = 0;
-  uint32_t mx = 0, hmx = 0;
+  // small graphs: smaller block tasks, so that one warp's work is not the whole query's length
+  const unsigned long long whole = whole_work(stats[2], m);
+  block_work = min(block_work, max(2048ull, whole / 4096));
+  unsigned long long wedges = 0;
+  uint32_t mx = 0, hash = 0, blen = 0, bits = 0;
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t len = row_ptr[x + 1] - row_ptr[x];
     const uint32_t np = pair_ptr[x + 1] - pair_ptr[x];
-    const unsigned long long w = np ? work[x] : 0ull;
+    const unsigned long long w = owner_work(work[x], np);
     uint8_t b = kNoTask;
-    if (len >= 2 && np > 0) {
-      const int cls = len > giant_thr ? kClsGiant : ((len > hub_thr || w > block_work) ? kClsHub : kClsMedium);
+    wedges += (unsigned long long)np * len;
+    if (len > 0 && np > 0) {
+      const uint32_t range = (uint32_t)x - (gstart ? gstart[vgraph[x]] : 0u);
+      const bool block = len > hub_thr || w > block_work || np > kHeavyPairs;
+      const int cls = len > giant_thr ? kGiant
+                      : block ? (range <= block_bits && len <= kBitsLen ? kHubBits : kHubHash) : (range <= warp_bits ? kMedBits : kMedHash);
       int lg = w ? 63 - __clzll(w) : 0;
-      lg = lg > kLgMax ? kLgMax : lg;
-      b = (uint8_t)(lg * 4 + cls);
-      atomicAdd(&s_cnt[b], 1u);
-      if (cls == kClsHub) hmx = max(hmx, len);
+      lg = lg > kLgTask ? kLgTask : lg;
+      b = (uint8_t)(lg * kTaskClasses + cls);
+      atomicAdd(&s_cnt[b], cls <= kHubBits ? owner_parts(w, whole) : 1u);
+      if (cls == kHubHash) hash = max(hash, len);
+      if (cls == kHubBits) {
+        blen = max(blen, len);
+        bits = max(bits, range);
+      }
     }
     bucket[x] = b;
-    wsum += w;
     mx = max(mx, len);
   }
-  atomicAdd(&s_work, wsum);
+  atomicAdd(&s_wedges, wedges);
   atomicMax(&s_max, mx);
-  atomicMax(&s_hmax, hmx);
+  atomicMax(&s_hash, hash);
+  atomicMax(&s_len, blen);
+  atomicMax(&s_bits, bits);
   __syncthreads();
-  for (int i = threadIdx.x; i < kBuckets2; i += blockDim.x)
-    if (s_cnt[i]) atomicAdd(&stats[4 + i], (unsigned long long)s_cnt[i]);
+  for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x)
+    if (s_cnt[i]) atomicAdd(&stats[kStatBuckets + i], (unsigned long long)s_cnt[i]);
   if (threadIdx.x == 0) {
-    atomicAdd(&stats[3], s_work);
+    atomicAdd(&stats[0], s_wedges);
     atomicMax(&stats[1], (unsigned long long)s_max);
-    atomicMax(&stats[2], (unsigned long long)s_hmax);
+    atomicMax(&stats[3], (unsigned long long)s_hash);
+    atomicMax(&stats[4], (unsigned long long)s_len);
+    atomicMax(&stats[5], (unsigned long long)s_bits);
   }
 }
 
-// Task lists: every block ranks its owners per bucket in shared memory and
-// reserves one range per bucket with a single global atomic.
-__global__ void k_fill_lists(int64_t n, const uint8_t* __restrict__ bucket, unsigned long long* cursor,
-                             uint32_t* __restrict__ lists) {
-  __shared__ uint32_t s_cnt[kBuckets2];
-  __shared__ unsigned long long s_base[kBuckets2];
+// Task lists: every block ranks its owners' tasks per bucket in shared memory
+// and reserves one range per bucket with a single global atomic.
+__global__ void k_fill_lists(int64_t n, int64_t m, const unsigned long long* __restrict__ work,
+                             const uint32_t* __restrict__ pair_ptr, const uint8_t* __restrict__ bucket,
+                             const unsigned long long* __restrict__ stats, unsigned long long* cursor,
+                             uint64_t* __restrict__ lists) {
+  __shared__ uint32_t s_cnt[kTaskBuckets];
+  __shared__ unsigned long long s_base[kTaskBuckets];
+  const unsigned long long whole = whole_work(stats[2], m);
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
-    for (int i = threadIdx.x; i < kBuckets2; i += blockDim.x) s_cnt[i] = 0;
+    for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x) s_cnt[i] = 0;
     __syncthreads();
     const int64_t x = base + threadIdx.x;
     const uint8_t b = x < n ? bucket[x] : kNoTask;
-    uint32_t rank = 0;
-    if (b != kNoTask) rank = atomicAdd(&s_cnt[b], 1u);
+    uint32_t rank = 0, parts = 1;
+    if (b != kNoTask) {
+      if (b % kTaskClasses <= kHubBits) parts = owner_parts(owner_work(work[x], pair_ptr[x + 1] - pair_ptr[x]), whole);
+      rank = atomicAdd(&s_cnt[b], parts);
+    }
     __syncthreads();
-    for (int i = threadIdx.x; i < kBuckets2; i += blockDim.x)
+    for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x)
       if (s_cnt[i]) s_base[i] = atomicAdd(&cursor[i], (unsigned long long)s_cnt[i]);
     __syncthreads();
-    if (b != kNoTask) lists[s_base[b] + rank] = (uint32_t)x;
+    if (b != kNoTask)
+      for (uint32_t i = 0; i < parts; i++)
+        lists[s_base[b] + rank + i] = (uint32_t)x | ((uint64_t)i << 32) | ((uint64_t)(parts - 1) << 48);
     __syncthreads();
   }
 }
@@ -942,14 +987,19 @@ __global__ void k_max_row(int64_t n, const uint32_t* __restrict__ ptr, unsigned 
 struct BuildLayout {
   // persistent
   Scratch* scratch;
+  uint32_t* vid;
   uint32_t* row_ptr;
   uint64_t* adj;
   uint32_t* eid;
+  uint32_t* rowid;
   uint32_t* ekey;
+  uint32_t* keep;        // pruned queries (FIXED graphs)
+  uint32_t* keep_tmp;
   uint32_t* pair_ptr;
   uint64_t* pairs;
-  uint32_t* lists;       // giant | hub | medium tasks
+  uint64_t* lists;       // tasks by class
   uint32_t* vgraph;
+  uint32_t* gstart;
   uint32_t* uptr;        // undirected AEO adjacency (optional)
   uint64_t* uadj;
   uint32_t* ueid;
@@ -968,16 +1018,21 @@ struct BuildLayout {
   // build temporaries
   uint32_t* deg;
   uint32_t* fill;
+  uint32_t* rank;              // number of every id
+  uint32_t* rank_tmp;          // ids between passes
+  uint32_t* rank_hist;
+  uint32_t* vgraph_id;         // batch: graph of every id
   uint32_t* scan_tmp;
   uint32_t* mid_rows;
   uint32_t* huge_rows;
   uint8_t* bucket;
-  unsigned long long* work;    // streamed work per owner
-  unsigned long long* stats;   // 4 + 4*48 counters, 4*48 cursors, 2 counters
+  unsigned long long* work;    // next pair position and streamed work per owner
+  unsigned long long* stats;   // kStats counters, as many cursors, 4 counters, 65 |q| classes
   char* sort_tmp;
   size_t total;
 };
-constexpr int kStats = 4 + 4 * (kLgMax + 1);
+constexpr int kStats = kStatBuckets + kTaskBuckets;
+static_assert(kStats >= 2 * (kLgMax + 1) + 1, "the undirected owners' cursors share the array");
 
 int64_t list_bound(int64_t n, int64_t m) {
   // a forward list under Node Order holds at most sqrt(2m) entries
@@ -991,7 +1046,8 @@ int64_t pow2_at_least(int64_t x) {
   return p;
 }
 
-BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, const ubt_graph_opts* opts, int sm_count) {
+BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, const ubt_graph_opts* opts,
+                   int sm_count) {
   Carver c(ws, cap);
   BuildLayout L;
   const bool has_key = opts && opts->d_edge_key;
@@ -999,14 +1055,19 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, const ubt_graph_o
   const int64_t ng = batch ? opts->n_graphs : 1;
   const int64_t n1 = std::max<int64_t>(n, 1);
   L.scratch = c.take<Scratch>(1);
+  L.vid = c.take<uint32_t>(n1);
   L.row_ptr = c.take<uint32_t>(n + 1);
   L.adj = c.take<uint64_t>(std::max<int64_t>(m, 1));
   L.eid = c.take<uint32_t>(std::max<int64_t>(m, 1));
+  L.rowid = c.take<uint32_t>(std::max<int64_t>(m, 1));
+  L.keep = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(m + 1) : nullptr;
+  L.keep_tmp = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(scan_tmp_words(m)) : nullptr;
   L.ekey = has_key ? c.take<uint32_t>(std::max<int64_t>(m, 1)) : nullptr;
   L.pair_ptr = c.take<uint32_t>(n + 1);
   L.pairs = c.take<uint64_t>(std::max<int64_t>(m, 1));
-  L.lists = c.take<uint32_t>(n1);
+  L.lists = c.take<uint64_t>(n1 + kMaxParts);
   L.vgraph = batch ? c.take<uint32_t>(n1) : nullptr;
+  L.gstart = batch ? c.take<uint32_t>(ng) : nullptr;
   const bool und = opts && (opts->flags & UBT_OPT_UNDIRECTED);
   L.uptr = und ? c.take<uint32_t>(n + 1) : nullptr;
   L.uadj = und ? c.take<uint64_t>(std::max<int64_t>(2 * m, 1)) : nullptr;
@@ -1028,17 +1089,43 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, const ubt_graph_o
   L.gtab = gslots ? c.take<uint32_t>((size_t)gslots * 3 * (size_t)sm_count) : nullptr;
   L.deg = c.take<uint32_t>(n + 1);
   L.fill = c.take<uint32_t>(n + 1);
-  L.scan_tmp = c.take<uint32_t>(scan_tmp_words(std::max(n, ng)) + 2);
+  L.rank = c.take<uint32_t>(n1);
+  L.rank_tmp = c.take<uint32_t>(n1);
+  const int64_t rank_hist = 256 * ((n + kRankTile - 1) / kRankTile);
+  L.rank_hist = c.take<uint32_t>(rank_hist + 1);
+  L.vgraph_id = batch ? c.take<uint32_t>(n1) : nullptr;
+  L.scan_tmp = c.take<uint32_t>(scan_tmp_words(std::max(std::max(n, ng), rank_hist)) + 2);
   L.mid_rows = c.take<uint32_t>(n1);
   L.huge_rows = c.take<uint32_t>(n1);
   L.bucket = c.take<uint8_t>(n1);
   L.work = c.take<unsigned long long>(n1);
-  L.stats = c.take<unsigned long long>(2 * kStats + 4);
+  L.stats = c.take<unsigned long long>(2 * kStats + 4 + 65);
   const int64_t lb = list_bound(n, m);
   L.sort_tmp = lb > tuning().sort_smem_max
                    ? c.take<char>((size_t)kSortHugeBlocks * (size_t)pow2_at_least(lb) * 24) : nullptr;
   L.total = c.off + 256;
   return L;
+}
+
+// L.vid and L.rank from the degrees (and, for a batch, L.vgraph_id)
+ubt_status rank_vertices(const BuildLayout& L, int64_t n, unsigned long long max_deg, int64_t n_graphs, cudaStream_t s) {
+  RankKey pass[8];
+  int np = 0;
+  for (int sh = 0; sh == 0 || (max_deg >> sh) != 0; sh += 8) pass[np++] = RankKey{L.deg, sh, 255u};
+  if (L.vgraph_id)
+    for (int sh = 0; sh < 32 && ((uint64_t)(n_graphs - 1) >> sh) != 0; sh += 8)
+      pass[np++] = RankKey{L.vgraph_id, sh, 0u};
+  const unsigned tiles = (unsigned)((n + kRankTile - 1) / kRankTile);
+  const uint32_t* in = nullptr;  // the ids n - 1 .. 0
+  for (int i = 0; i < np; i++) {
+    uint32_t* out = (np - 1 - i) % 2 == 0 ? L.vid : L.rank_tmp;  // the last pass ends in vid
+    k_rank_count<<<tiles, kRankThreads, 0, s>>>(n, in, pass[i], L.rank_hist);
+    UBT_CUDA(exclusive_scan_u32(L.rank_hist, L.rank_hist, 256 * (int64_t)tiles, L.scan_tmp, s));
+    k_rank_scatter<<<tiles, kRankThreads, 0, s>>>(n, in, pass[i], L.rank_hist, out, i == np - 1 ? L.rank : nullptr);
+    in = out;
+  }
+  UBT_CUDA(cudaGetLastError());
+  return UBT_OK;
 }
 
 int device_sm_count(int* dev) {
@@ -1073,7 +1160,7 @@ extern "C" ubt_status ubt_graph_workspace_size(int64_t n, int64_t m, int32_t fla
   if (!h_bytes || n < 0 || m < 0 || n >= 0xFFFFFFFFll || m >= 0xFFFFFFFFll) return UBT_ERR_INVALID_ARG;
   if (flags != UBT_GRAPH_FIXED && flags != UBT_GRAPH_REAL) return UBT_ERR_INVALID_ARG;
   if (opts && opts->d_vertex_offsets && opts->n_graphs < 1) return UBT_ERR_INVALID_ARG;
-  BuildLayout L = layout(nullptr, 0, n, m, opts, device_sm_count(nullptr));
+  BuildLayout L = layout(nullptr, 0, n, m, flags, opts, device_sm_count(nullptr));
   *h_bytes = L.total;
   return UBT_OK;
 }
@@ -1104,7 +1191,7 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   const int64_t ng = batch ? opts->n_graphs : 1;
   int dev = 0;
   const int sms = device_sm_count(&dev);
-  BuildLayout L = layout(d_workspace, ws_bytes, n, m, opts, sms);
+  BuildLayout L = layout(d_workspace, ws_bytes, n, m, flags, opts, sms);
   if (ws_bytes < L.total) return UBT_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t s = (cudaStream_t)stream;
   const Tuning& T = tuning();
@@ -1117,37 +1204,45 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   UBT_CUDA(cudaMemsetAsync(&L.scratch->err, 0xFF, sizeof(unsigned long long), s));
   UBT_CUDA(cudaMemsetAsync(L.deg, 0, sizeof(uint32_t) * (n + 1), s));
   UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
-  UBT_CUDA(cudaMemsetAsync(L.stats, 0, sizeof(unsigned long long) * (2 * kStats + 4), s));
+  UBT_CUDA(cudaMemsetAsync(L.stats, 0, sizeof(unsigned long long) * (2 * kStats + 4 + 65), s));
   const int thr = 256;
   const int grid_e = (int)std::min<int64_t>(std::max<int64_t>((m + thr - 1) / thr, 1), (int64_t)sms * 32);
   const int grid_v = (int)std::min<int64_t>(std::max<int64_t>((n + thr - 1) / thr, 1), (int64_t)sms * 32);
   const int grid_w = (int)std::min<int64_t>(std::max<int64_t>((n + 7) / 8, 1), (int64_t)sms * 32);
 
   if (batch) {
-    k_vertex_graph<<<grid_v, thr, 0, s>>>(opts->d_vertex_offsets, opts->n_graphs, n, L.vgraph);
+    k_vertex_graph<<<grid_v, thr, 0, s>>>(opts->d_vertex_offsets, opts->n_graphs, n, L.vgraph_id);
   }
   // 1. validate + degree
   NvtxPhases phase;
   phase.next("build: validate and degree");
   if (m > 0)
-    k_validate_degree<<<grid_e, thr, 0, s>>>(n, m, d_src, d_dst, d_k, d_p, L.vgraph, L.deg, &L.scratch->err);
-  unsigned long long err = 0;
+    k_validate_degree<<<grid_e, thr, 0, s>>>(n, m, d_src, d_dst, d_k, d_p, L.vgraph_id, L.deg, &L.scratch->err);
+  unsigned long long* lcount = L.stats + 2 * kStats;  // row lengths; first the largest degree
+  if (n > 0) k_max_degree<<<grid_v, thr, 0, s>>>(n, L.deg, lcount);
+  unsigned long long err = 0, max_deg = 0;
+  UBT_CUDA(cudaMemcpyAsync(&max_deg, lcount, sizeof(max_deg), cudaMemcpyDeviceToHost, s));
   UBT_CUDA(cudaMemcpyAsync(&err, &L.scratch->err, sizeof(err), cudaMemcpyDeviceToHost, s));
   UBT_CUDA(cudaStreamSynchronize(s));
   ubt_status st = status_from_err(err);
   if (st != UBT_OK) return st;
   // 2. orientation + CSR offsets
   phase.next("build: orient, scatter, sort");
-  if (m > 0) k_out_degree<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, L.deg, L.fill);
+  if (n > 0) {
+    UBT_CUDA(cudaMemsetAsync(lcount, 0, sizeof(unsigned long long), s));
+    st = rank_vertices(L, n, max_deg, ng, s);
+    if (st != UBT_OK) return st;
+    if (batch) k_rank_graphs<<<grid_v, thr, 0, s>>>(n, L.vid, L.vgraph_id, L.vgraph, opts->d_vertex_offsets, ng, L.gstart);
+  }
+  if (m > 0) k_out_degree<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, L.rank, L.fill);
   UBT_CUDA(exclusive_scan_u32(L.fill, L.row_ptr, n, L.scan_tmp, s));
-  UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
+  UBT_CUDA(cudaMemcpyAsync(L.fill, L.row_ptr, sizeof(uint32_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
   if (m > 0)
-    k_scatter<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, d_p, L.deg, L.row_ptr, L.fill, L.adj, L.eid,
+    k_scatter<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, d_p, L.rank, L.fill, L.adj, L.eid,
                                      opts ? opts->d_edge_key : nullptr, L.ekey);
   // 3. sort every forward list
   const int fixed = flags == UBT_GRAPH_FIXED;
-  const int mode = fixed ? kSortByAbsqChecked : kSortById;
-  unsigned long long* lcount = L.stats + 2 * kStats;
+  const int mode = kSortById;
   if (n > 0) {
     k_sort_short_rows<<<grid_w, thr, 0, s>>>(n, L.row_ptr, L.adj, L.eid, L.ekey, mode, &L.scratch->err);
     const uint32_t sort_smem = (uint32_t)tuning().sort_smem_max;
@@ -1169,8 +1264,8 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
     if (lc[1]) {
       const int64_t cap = pow2_at_least(list_bound(n, m));
       const int g = (int)std::min<unsigned long long>(lc[1], (unsigned long long)kSortHugeBlocks);
-      k_sort_long_rows<true><<<g, 1024, 0, s>>>(L.huge_rows, (uint32_t)lc[1], L.row_ptr, L.adj, L.eid, L.ekey,
-                                                fixed, &L.scratch->err, L.sort_tmp, cap);
+      k_sort_long_rows<<<g, 1024, 0, s>>>(L.huge_rows, (uint32_t)lc[1], L.row_ptr, L.adj, L.eid, L.ekey,
+                                          &L.scratch->err, L.sort_tmp, cap);
     }
     UBT_CUDA(cudaGetLastError());
   }
@@ -1180,47 +1275,43 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   if (st != UBT_OK) return st;
   // 4. pairs grouped by owner
   phase.next("build: pairs and work lists");
+  unsigned long long* absq = fixed ? L.stats + 2 * kStats + 4 : nullptr;
   UBT_CUDA(cudaMemsetAsync(L.pair_ptr, 0, sizeof(uint32_t) * (n + 1), s));
   if (n > 0) {
-    UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
-    // the row of every CSR position, in the (not yet used) adjoint accumulators
-    uint32_t* rowid = (uint32_t*)L.gacc;
-    k_row_ids<<<grid_v, thr, 0, s>>>(n, L.row_ptr, rowid);
-    if (m > 0) k_pair_count<<<grid_e, thr, 0, s>>>(m, L.row_ptr, L.adj, rowid, pull, L.fill, &L.stats[0]);
+    k_row_ids<<<grid_v, thr, 0, s>>>(n, L.row_ptr, L.rowid);
+    k_in_degree<<<grid_v, thr, 0, s>>>(n, L.deg, L.vid, L.row_ptr, L.fill);
     UBT_CUDA(exclusive_scan_u32(L.fill, L.pair_ptr, n, L.scan_tmp, s));
-    UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
-    UBT_CUDA(cudaMemsetAsync(L.work, 0, sizeof(unsigned long long) * n, s));
-    if (m > 0)
-      k_pair_fill<<<grid_e, thr, 0, s>>>(m, L.row_ptr, L.adj, rowid, pull, L.pair_ptr, L.fill, L.pairs, L.work);
+    k_pair_next<<<grid_v, thr, 0, s>>>(n, L.pair_ptr, L.work);
+    if (m > 0) k_pair_fill<<<grid_e, thr, 0, s>>>(m, L.row_ptr, L.adj, L.rowid, L.work, L.pairs, absq, &L.stats[2]);
     UBT_CUDA(cudaGetLastError());
   }
-  // 5. work lists: giant | hub | medium tasks, each by decreasing work bucket
-  unsigned long long stats[kStats];
+  // 5. work lists: the owners of every task class by decreasing work bucket
+  unsigned long long stats[kStats], classes[65];
   memset(stats, 0, sizeof(stats));
+  memset(classes, 0, sizeof(classes));
   if (n > 0) {
-    k_row_stats<<<grid_v, thr, 0, s>>>(n, L.row_ptr, L.pair_ptr, L.work, (uint32_t)hub_thr, (uint32_t)giant_thr,
-                                      (unsigned long long)block_work, L.bucket, L.stats);
+    k_row_stats<<<grid_v, thr, 0, s>>>(n, m, L.row_ptr, L.pair_ptr, L.work, L.vgraph, L.gstart, (uint32_t)hub_thr,
+                                      (uint32_t)giant_thr, (unsigned long long)block_work, (uint32_t)T.block_bits,
+                                      (uint32_t)T.warp_bits, L.bucket, L.stats);
     UBT_CUDA(cudaMemcpyAsync(stats, L.stats, sizeof(stats), cudaMemcpyDeviceToHost, s));
+    if (absq) UBT_CUDA(cudaMemcpyAsync(classes, absq, sizeof(classes), cudaMemcpyDeviceToHost, s));
     UBT_CUDA(cudaStreamSynchronize(s));
   }
-  unsigned long long cursor[4 * (kLgMax + 1)];
-  int64_t count_cls[4] = {0, 0, 0, 0};
-  for (int b = 0; b < 4 * (kLgMax + 1); b++) count_cls[b % 4] += (int64_t)stats[4 + b];
-  int64_t run[4] = {0, 0, 0, 0};
-  run[kClsGiant] = 0;
-  run[kClsHub] = count_cls[kClsGiant];
-  run[kClsMedium] = count_cls[kClsGiant] + count_cls[kClsHub];
-  for (int lg = kLgMax; lg >= 0; lg--) {
-    for (int cls = 1; cls < 4; cls++) {
-      const int b = lg * 4 + cls;
-      cursor[b] = (unsigned long long)run[cls];
-      run[cls] += (int64_t)stats[4 + b];
+  unsigned long long cursor[kTaskBuckets];
+  int64_t count_cls[kTaskClasses] = {}, first_cls[kTaskClasses] = {}, run[kTaskClasses] = {};
+  for (int b = 0; b < kTaskBuckets; b++) count_cls[b % kTaskClasses] += (int64_t)stats[kStatBuckets + b];
+  for (int c = 1; c < kTaskClasses; c++) first_cls[c] = first_cls[c - 1] + count_cls[c - 1];
+  for (int lg = kLgTask; lg >= 0; lg--) {
+    for (int c = 0; c < kTaskClasses; c++) {
+      const int b = lg * kTaskClasses + c;
+      cursor[b] = (unsigned long long)(first_cls[c] + run[c]);
+      run[c] += (int64_t)stats[kStatBuckets + b];
     }
   }
   if (n > 0) {
     unsigned long long* dcur = L.stats + kStats;
     UBT_CUDA(cudaMemcpyAsync(dcur, cursor, sizeof(cursor), cudaMemcpyHostToDevice, s));
-    k_fill_lists<<<grid_v, thr, 0, s>>>(n, L.bucket, dcur, L.lists);
+    k_fill_lists<<<grid_v, thr, 0, s>>>(n, m, L.work, L.pair_ptr, L.bucket, L.stats, dcur, L.lists);
     UBT_CUDA(cudaGetLastError());
     UBT_CUDA(cudaStreamSynchronize(s));
   }
@@ -1305,19 +1396,24 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   g->m = m;
   g->kind = flags;
   g->n_graphs = ng;
+  g->vid = L.vid;
   g->row_ptr = L.row_ptr;
   g->adj = L.adj;
   g->eid = L.eid;
+  g->rowid = L.rowid;
+  g->keep = L.keep;
+  g->keep_tmp = L.keep_tmp;
+  for (int b = 64; b >= 0; b--) g->kept[b] = g->kept[b + 1] + (double)classes[b];
+  for (int b = 64; b >= 0; b--) g->kept[b] = g->kept[0] > 0 ? g->kept[b] / g->kept[0] : 1.0;
   g->ekey = L.ekey ? L.ekey : L.eid;
   g->pair_ptr = L.pair_ptr;
   g->pairs = L.pairs;
-  g->giant_list = L.lists;
-  g->n_giant = count_cls[kClsGiant];
-  g->hub_list = L.lists + count_cls[kClsGiant];
-  g->n_hub = count_cls[kClsHub];
-  g->med_list = L.lists + count_cls[kClsGiant] + count_cls[kClsHub];
-  g->n_med = count_cls[kClsMedium];
+  for (int c = 0; c < kTaskClasses; c++) {
+    g->lists[c] = L.lists + first_cls[c];
+    g->n_tasks[c] = count_cls[c];
+  }
   g->vgraph = L.vgraph;
+  g->gstart = L.gstart;
   g->uptr = L.uptr;
   g->uadj = L.uadj;
   g->ueid = L.ueid;
@@ -1345,8 +1441,11 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   g->scratch = L.scratch;
   g->wedges = (int64_t)stats[0];
   g->max_out = (int64_t)stats[1];
-  g->max_hub_len = (int64_t)stats[2];
-  g->probes = (int64_t)stats[3];
+  g->probes = (int64_t)stats[2];
+  g->max_hash_len = (int64_t)stats[3];
+  g->max_bits_len = (int64_t)stats[4];
+  g->max_bits = (int64_t)stats[5];
+  g->warp_bits = T.warp_bits;
   g->hub_threshold = hub_thr;
   g->giant_threshold = giant_thr;
   g->block_work = block_work;
@@ -1368,7 +1467,7 @@ extern "C" ubt_status ubt_graph_get_info(const ubt_graph* g, ubt_graph_info* h_i
   h_info->n = g->n;
   h_info->m = g->m;
   h_info->max_out_degree = g->max_out;
-  h_info->hub_vertices = g->n_hub + g->n_giant;
+  h_info->hub_vertices = g->n_tasks[kGiant] + g->n_tasks[kHubHash] + g->n_tasks[kHubBits];
   h_info->wedges = g->wedges;
   h_info->kind = g->kind;
   h_info->probes = g->probes;

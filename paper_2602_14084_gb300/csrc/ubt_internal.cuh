@@ -12,21 +12,27 @@ namespace ubt {
 
 // ---------------------------------------------------------------- layout
 //
-// Forward CSR under Node Order (Def. Node Order, Sec. 4): row u holds N>(u),
-// the neighbours later than u in (degree, id) order.  Each entry is one
-// 64-bit word: low 32 bits the neighbour id, high 32 bits the edge value:
+// Inside the library a vertex is its position r in reverse Node Order (Def.
+// Node Order, Sec. 4): r = 0 is the last vertex, of the highest degree; the
+// graphs of a batch keep their vertex ranges, each ordered by itself.  vid[r]
+// is the id the caller knows.  A neighbour later in Node Order has a smaller
+// r, so hubs, which most lists contain, have the small numbers.
+//
+// Forward CSR: row u holds N>(u), the neighbours later than u, ascending by
+// r (the last vertex first).  Each entry is one 64-bit word: low 32 bits the
+// neighbour, high 32 bits the edge value:
 //   FIXED graphs: q = 32768 - k as int32 (1 - 2 P+ = q / 2^15)
 //   REAL graphs:  s = 1 - 2 p as int32 fixed point, s * 2^30 rounded
-// FIXED rows are sorted by |q| descending, ties by neighbour id, so the
-// entries a pruning level removes form a suffix of the row (Lemma 2); REAL
-// rows by neighbour id.
-// eid[pos] is the input index of the edge stored at CSR position pos.
+// eid[pos] is the input index of the edge stored at CSR position pos,
+// rowid[pos] its row.
 //
-// Pairs: every forward edge x-s is one pair of the traversal, owned by the
-// endpoint whose list becomes the hash table (the other endpoint's list is
-// streamed through it).  pair_ptr / pairs group the pairs by owner; a pair
-// word holds the streamed vertex s (low 32 bits) and the CSR position of the
-// edge (high 32 bits).
+// Pairs: a triangle u < v < w (Node Order) is found from the edge u -> v: its
+// owner is the later vertex v, whose list N>(v) becomes the table, and w lies
+// in N>(u) after v -- in row u's entries before the position of v.  The pair
+// word of the edge at position pos of row u is
+//   bits 0..31 the start of row u, bits 32..48 pos - start (a forward list
+//   holds fewer than sqrt(2m) < 2^17 entries), bits 49..63 |q| >> 1 (FIXED).
+// pair_ptr / pairs group the pairs by owner.
 
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 constexpr int kWarp = 32;
@@ -52,6 +58,12 @@ __host__ __device__ inline int32_t adj_q(uint64_t e) { return (int32_t)(uint32_t
 __host__ __device__ inline uint32_t adj_valbits(uint64_t e) { return (uint32_t)(e >> 32); }
 __host__ __device__ inline uint64_t adj_pack(uint32_t col, uint32_t valbits) {
   return ((uint64_t)valbits << 32) | col;
+}
+__host__ __device__ inline uint32_t pair_start(uint64_t d) { return (uint32_t)d; }
+__host__ __device__ inline uint32_t pair_len(uint64_t d) { return (uint32_t)(d >> 32) & 0x1FFFFu; }
+__host__ __device__ inline uint32_t pair_absq2(uint64_t d) { return (uint32_t)(d >> 49); }  // |q| >> 1
+__host__ __device__ inline uint64_t pair_pack(uint32_t start, uint32_t len, uint32_t absq2) {
+  return ((uint64_t)absq2 << 49) | ((uint64_t)len << 32) | start;
 }
 
 // Edge index (UBT_OPT_EDGE_INDEX): open addressing with linear probing over
@@ -101,19 +113,24 @@ constexpr int kLongQueue = 1024;
 
 // Query scratch carved from the graph workspace (one per graph).
 struct Scratch {
-  unsigned long long task[4];       // next giant / hub / small task, spare
+  unsigned long long task[8];       // next task of every class, spare
   unsigned long long enum_cursor;   // enumeration append cursor
   unsigned long long tri_count;     // triangles seen (expected counts)
   unsigned long long sum_lo;        // 128-bit two's-complement sum, low word
   unsigned long long sum_hi;        // high word
   unsigned long long err;           // device-side error word (build)
   unsigned long long guard;         // first failed self-check of a query (0 = none)
-  unsigned long long pad[6];
+  unsigned long long pad[2];
   unsigned long long hist[2 * 65];  // per-threshold accumulators (bal [0,64), unbal [64,128))
 };
-constexpr size_t kScratchHeader = 16 * sizeof(unsigned long long);  // zeroed per query
+constexpr size_t kScratchQuery = 12 * sizeof(unsigned long long);  // the words up to err: zeroed per query
 
 }  // namespace ubt
+
+// Task classes of the traversal's owners: what handles them (a block or a
+// warp) and what their table is (ubt_traverse.cuh).
+enum : int { kGiant = 0, kHubHash = 1, kHubBits = 2, kMedHash = 3, kMedBits = 4, kTaskClasses = 5 };
+constexpr uint32_t kBitsLen = 16384;  // longest list of a kHubBits task (list indices are 16 bits there)
 
 // The opaque handle of the public ABI.
 struct ubt_graph {
@@ -121,16 +138,19 @@ struct ubt_graph {
   int32_t kind = 0;
   int64_t n_graphs = 1;
   // device arrays (inside the caller's workspace)
+  uint32_t* vid = nullptr;          // n: the caller's id of every vertex
   uint32_t* row_ptr = nullptr;      // n + 1
   uint64_t* adj = nullptr;          // m
   uint32_t* eid = nullptr;          // m: input edge index per CSR position
+  uint32_t* rowid = nullptr;        // m: row per CSR position
   uint32_t* ekey = nullptr;         // m: Philox key per CSR position
   uint32_t* pair_ptr = nullptr;     // n + 1: pairs of owner x are [pair_ptr[x], pair_ptr[x+1])
-  uint64_t* pairs = nullptr;        // m: streamed vertex | CSR position << 32
-  uint32_t* giant_list = nullptr;   // owners whose list is too long for a shared-memory table
-  uint32_t* hub_list = nullptr;     // long lists or heavy owners: whole-block tasks
-  uint32_t* med_list = nullptr;     // the other owners: one-warp tasks
+  uint64_t* pairs = nullptr;        // m: pair words
+  uint64_t* lists[kTaskClasses] = {};   // tasks by class: owner, part of its pairs (ubt_traverse.cuh)
   uint32_t* vgraph = nullptr;       // batch: graph id of every vertex (or null)
+  uint32_t* gstart = nullptr;       // batch: first vertex of every graph (or null)
+  uint32_t* keep = nullptr;         // FIXED, m + 1: kept entries before a position (pruned queries)
+  uint32_t* keep_tmp = nullptr;     // scan temporaries of keep
   // undirected adjacency in Absolute Edge Order (UBT_OPT_UNDIRECTED; else null):
   // row x holds every edge at x, |q| descending then neighbour id (Def. AEO
   // restricted to the edges at x), packed like adj
@@ -150,16 +170,20 @@ struct ubt_graph {
                                     // 16 bytes, key in the first 8, edge value (valbits) in the next 4
   int64_t eh_slots = 0;             // power of two >= max(4m, 64)
   int eh_shift = 64;                // 64 - log2(eh_slots)
-  unsigned long long* gacc = nullptr;   // m: backward accumulators
+  unsigned long long* gacc = nullptr;   // m: backward accumulators; a pruned query's kept entries
   unsigned long long* bacc = nullptr;   // batch accumulators
   uint32_t* gtab = nullptr;         // global hash tables for very long lists
   int64_t gtab_slots = 0;           // slots per block
   int64_t gtab_blocks = 0;          // blocks that have one
   ubt::Scratch* scratch = nullptr;
   // sizes recorded at build time
-  int64_t n_giant = 0, n_hub = 0, n_med = 0;
-  int64_t max_out = 0, max_hub_len = 0, wedges = 0, probes = 0;
+  int64_t n_tasks[kTaskClasses] = {};
+  int64_t max_out = 0, wedges = 0, probes = 0;
+  int64_t max_hash_len = 0;                 // longest list of a kHubHash task
+  int64_t max_bits_len = 0, max_bits = 0;   // longest list and largest bit range of a kHubBits task
+  int64_t warp_bits = 0;                    // bit range of the kMedBits tasks
   int64_t hub_threshold = 0, giant_threshold = 0, block_work = 0, pull = 1;
+  double kept[66] = {0};  // FIXED: share of the edges with |q| >= 512 b (of a sample; [65] = 0)
   int device = 0, sm_count = 0;
 };
 
@@ -168,7 +192,7 @@ namespace ubt {
 // ---------------------------------------------------------------- tuning
 
 struct Tuning {
-  int64_t pull = 1;               // 1: each pair streams the shorter list; 0: always N>(v) (Alg. 1)
+  int64_t pull = 1;               // ubt_graph_export_pairs: 1 the longer list's endpoint owns, 0 the earlier one
   int64_t count_visitor = 0;      // threshold counts: 0 binned in the finding lane, 1 queued per warp
   int64_t block_work = 1 << 14;   // owners streaming more entries are whole-block tasks
   int64_t hub_threshold = 128;    // owners with longer lists are whole-block tasks
@@ -176,9 +200,11 @@ struct Tuning {
   int64_t warp_threads = 128;     // threads of the warp-task kernel (at most 128)
   int64_t blocks_per_sm = 32;     // cap on resident blocks (occupancy decides below it)
   int64_t smem_table_max = 8192;  // hash slots of a shared-memory table
+  int64_t block_bits = 1 << 18;   // block tasks: largest vertex range of a bitmap table
+  int64_t warp_bits = 1 << 14;    // warp tasks: the same
   int64_t world_words_per_pass = 8;
   int64_t small_batch = 4;        // warp tasks taken per grab
-  int64_t block_unit = 16;        // pairs per warp step in block tasks
+  int64_t block_unit = 32;        // pairs per warp step in block tasks
   int64_t long_min = 64;          // streamed lists this long are streamed by the whole warp
   int64_t long_tail = 1;          // 1: the last < 64 entries of such a list join the short lists
   int64_t edge_index = 1;         // vertex queries: 0 never look pairs up in the edge index, 1 when cheaper, 2 always
@@ -267,5 +293,7 @@ inline int64_t table_slots(int64_t entries) {
 cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp,
                                cudaStream_t s);
 size_t scan_tmp_words(int64_t n);
+cudaError_t keep_entries(const uint64_t* adj, int64_t m, uint32_t qmin, uint32_t* keep, uint64_t* kept, uint32_t* tmp,
+                         cudaStream_t s);
 
 }  // namespace ubt

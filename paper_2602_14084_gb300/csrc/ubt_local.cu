@@ -521,7 +521,7 @@ ubt_status local_counts(ubt_graph* g, const uint32_t* d_items, int64_t k, int ve
   a.sc = g->scratch;
   a.bal = d_bal;
   a.unbal = d_unbal;
-  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchHeader / 2, s));
+  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
   UBT_CUDA(cudaMemsetAsync(a.lq, 0, 2 * sizeof(unsigned long long), s));
   if (k > 0) {
     const int threads = 512;
@@ -814,7 +814,7 @@ extern "C" ubt_status ubt_vertex_topk(ubt_graph* g, const uint32_t* d_vertices, 
   a.sc = g->scratch;
   a.out = d_out;
   a.n_out = d_n_out;
-  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchHeader / 2, s));
+  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
   if (k == 0) return UBT_OK;
   const int threads = 512;
   const size_t smem = 2064 * 4 + (size_t)kTopkCap * (8 + 12) + (size_t)a.cap * 3 * 4;

@@ -77,53 +77,31 @@ struct CountRegP {
   int64_t B[kRegTau], U[kRegTau];
   unsigned long long* out;  // [0, NT) balanced, [NT, 2 NT) unbalanced
 };
-// A warp collects the products P of its triangles in a shared-memory queue
-// and counts them 32 at a time, so the counting runs on full warps.  The
-// queue holds fewer than 32 between steps; a step adds at most 32 and a
-// batched pair of steps at most 64.
-constexpr int kHitQueue = 96;
-
-// Appends the products of two probe steps' hits to a warp queue (q, qn); the
-// caller drains it below 32 afterwards.  All lanes, converged.
-__device__ __forceinline__ void enqueue_pair(long long* q, uint32_t& qn, bool h0, bool h1, uint32_t quv,
-                                             uint32_t quw0, uint32_t qvw0, uint32_t quw1, uint32_t qvw1) {
-  const unsigned lt = lanemask_lt();
-  const unsigned m0 = __ballot_sync(kFull, h0);
-  const unsigned m1 = __ballot_sync(kFull, h1);
-  const uint32_t n0 = qn + __popc(m0);
-  if (h0) q[qn + __popc(m0 & lt)] = tri_product(quv, quw0, qvw0);
-  if (h1) q[n0 + __popc(m1 & lt)] = tri_product(quv, quw1, qvw1);
-  qn = n0 + __popc(m1);
-}
-
-// Moves queue entries [32, qn) (fewer than 64) to the front.
-__device__ __forceinline__ void queue_shift32(long long* q, uint32_t& qn) {
-  const uint32_t lane = lane_id();
-  const uint32_t rest = qn - 32;
-  const long long a = lane < rest ? q[32 + lane] : 0;
-  const long long b = lane + 32 < rest ? q[64 + lane] : 0;
-  __syncwarp();
-  if (lane < rest) q[lane] = a;
-  if (lane + 32 < rest) q[32 + lane] = b;
-  qn = rest;
-  __syncwarp();
+// What is queued of a triangle of a FIXED graph: the product of the pair's and
+// the streamed edge's values (|q| <= 2^15: it fits int32).
+struct ProductItem {
+  using Item = uint2;
+  static constexpr bool kMore = false;
+  static constexpr int kU = 4;
+  __device__ __forceinline__ static uint2 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t, uint32_t, uint32_t) {
+    return make_uint2(slot, (uint32_t)((int32_t)quv * (int32_t)qvw));
+  }
+};
+__device__ __forceinline__ long long item_product(uint32_t pair, uint32_t quw) {
+  return (long long)(int32_t)pair * (long long)(int32_t)quw;
 }
 
 template <int NT>
-struct CountReg {
+struct CountReg : ProductItem {
   using P = CountRegP;
   static constexpr bool kPos = false;
-  static constexpr bool kBatched = true;
   static constexpr int kRegCap = UBT_COUNT_REGCAP;
-  static __host__ __device__ int smem_bytes(int threads) { return (threads / 32) * kHitQueue * 8; }
+  static __host__ __device__ int smem_bytes(int) { return 0; }
   int64_t B[NT], U[NT];
   unsigned long long* out;
-  long long* q;  // this warp's queue of products
-  uint32_t qn = 0;
   uint32_t bal[NT], unbal[NT];
   uint32_t since = 0;
-  __device__ CountReg(const P& p, char* smem) : out(p.out) {
-    q = (long long*)smem + (threadIdx.x >> 5) * kHitQueue;
+  __device__ CountReg(const P& p, char*) : out(p.out) {
 #pragma unroll
     for (int i = 0; i < NT; i++) {
       B[i] = p.B[i];
@@ -140,41 +118,14 @@ struct CountReg {
     }
     since++;
   }
-  // count the first 32 queued products, move the rest to the front
-  __device__ void drain32() {
-    const int lane = (int)lane_id();
-    __syncwarp();
-    const long long mine = q[lane];
-    queue_shift32(q, qn);
-    count(mine);
+  __device__ __forceinline__ void take(bool on, uint32_t, uint2 it, uint32_t, uint32_t, uint32_t quw, uint32_t,
+                                       uint32_t) {
+    if (on) count(item_product(it.y, quw));
   }
-  __device__ void drain_all() {
-    const int lane = (int)lane_id();
-    __syncwarp();
-    if ((uint32_t)lane < qn) count(q[lane]);
-    qn = 0;
-    __syncwarp();
-  }
+  // the Alg. 2 kernels
   __device__ __forceinline__ void step(bool hit, uint32_t, uint32_t, uint32_t, uint32_t quv, uint32_t quw,
                                        uint32_t qvw, uint32_t, uint32_t, uint32_t) {
-    const unsigned m = __ballot_sync(kFull, hit);
-    if (!m) return;
-    const int lane = (int)lane_id();
-    if (hit) q[qn + __popc(m & lanemask_lt())] = tri_product(quv, quw, qvw);
-    qn += __popc(m);
-    if (qn >= 32) drain32();
-  }
-  template <int U>
-  __device__ __forceinline__ void steps(const bool (&hit)[U], uint32_t quv, const uint32_t (&quw)[U],
-                                        const uint32_t (&qvw)[U]) {
-    static_assert(U % 2 == 0, "steps come in pairs");
-#pragma unroll
-    for (int s = 0; s < U; s += 2) {
-      if (__any_sync(kFull, hit[s] || hit[s + 1])) {
-        enqueue_pair(q, qn, hit[s], hit[s + 1], quv, quw[s], qvw[s], quw[s + 1], qvw[s + 1]);
-        while (qn >= 32) drain32();
-      }
-    }
+    if (hit) count(tri_product(quv, quw, qvw));
   }
   __device__ void task_begin(uint32_t) {}
   __device__ void flush() {
@@ -194,10 +145,7 @@ struct CountReg {
   __device__ void task_end(uint32_t) {
     if (__any_sync(kFull, since >= (1u << 26))) flush();
   }
-  __device__ void block_end() {
-    drain_all();
-    flush();
-  }
+  __device__ void block_end() { flush(); }
 };
 
 __global__ void k_finish_reg(const unsigned long long* __restrict__ acc, int nt, int NT, const int* perm_unused,
@@ -213,14 +161,12 @@ __global__ void k_finish_reg(const unsigned long long* __restrict__ acc, int nt,
 // Many thresholds (up to 64), tested all at once.  The 2 nt levels -- every B
 // and every U, sorted ascending (each B <= 0 <= each U) -- cut the integers
 // into 2 nt + 1 intervals; a product P falls in interval r = #{levels < P}.
-// Products are queued per warp as in CountReg; 32 at a time, each lane finds
-// the interval of one product by binary search and adds 1 to that interval's
+// Each lane finds the interval of one product by binary search and adds 1 to that interval's
 // bin (a block-wide shared histogram).  Then, with B_(k) and U_(k) the k-th
 // smallest levels of each kind,
 //   #{P <= B_(k)} = #{r <= k}           (P <= B_(k) iff fewer than k+1 B's are < P)
 //   #{P >  U_(k)} = #{r > nt + k}       (P >  U_(k) iff at least k+1 U's are < P,
 //                                        and then every B is < P too)
-static_assert(UBT_LB_THREADS <= 512, "CountMulti's 32-bit bins assume at most 16 warps a block");
 constexpr int kMultiLevels = 256;  // padded table of levels: 2^K > 2 kMaxTau
 constexpr int kMultiBins = 2 * kMaxTau + 1;
 struct CountMultiP {
@@ -229,26 +175,20 @@ struct CountMultiP {
   int64_t S[2 * kMaxTau];          // the 2 nt levels, ascending
   unsigned long long* out;         // global bins [0, 2 nt]
 };
-struct CountMulti {
+struct CountMulti : ProductItem {
   using P = CountMultiP;
   static constexpr bool kPos = false;
-  static constexpr bool kBatched = true;
   static constexpr int kRegCap = UBT_COUNT_REGCAP;
-  static __host__ __device__ int smem_bytes(int threads) {
-    return kMultiLevels * 8 + ((kMultiBins * 4 + 15) / 16) * 16 + (threads / 32) * kHitQueue * 8;
-  }
+  static __host__ __device__ int smem_bytes(int) { return kMultiLevels * 8 + ((kMultiBins * 4 + 15) / 16) * 16; }
   unsigned long long* out;
   const long long* S;  // shared: levels, padded with INT64_MAX
   uint32_t* bins;      // shared: block histogram
-  long long* q;        // shared: this warp's queue of products
-  uint32_t qn = 0;
   uint32_t since = 0;  // products this warp binned since its last flush (warp-uniform)
   int nt, half;
   __device__ CountMulti(const P& p, char* smem) : out(p.out), nt(p.nt), half(p.half) {
     long long* s = (long long*)smem;
     S = s;
     bins = (uint32_t*)(smem + kMultiLevels * 8);
-    q = (long long*)(smem + kMultiLevels * 8 + ((kMultiBins * 4 + 15) / 16) * 16) + (threadIdx.x >> 5) * kHitQueue;
     for (int i = threadIdx.x; i < kMultiLevels; i += blockDim.x) s[i] = i < 2 * p.nt ? p.S[i] : INT64_MAX;
     for (int i = threadIdx.x; i < kMultiBins; i += blockDim.x) bins[i] = 0;
   }
@@ -273,71 +213,46 @@ struct CountMulti {
     }
     since = 0;
   }
-  __device__ void drain32() {
-    const int lane = (int)lane_id();
-    __syncwarp();
-    const long long mine = q[lane];
-    queue_shift32(q, qn);
-    bin(mine);
-    since += 32;
+  __device__ __forceinline__ void take(bool on, uint32_t n, uint2 it, uint32_t, uint32_t, uint32_t quw, uint32_t,
+                                       uint32_t) {
+    if (on) bin(item_product(it.y, quw));
+    since += n;
     if (since >= (1u << 26)) flush();
   }
-  __device__ void drain_all() {
-    const int lane = (int)lane_id();
-    __syncwarp();
-    if ((uint32_t)lane < qn) bin(q[lane]);
-    since += qn;
-    qn = 0;
-    __syncwarp();
-  }
+  // the Alg. 2 kernels
   __device__ __forceinline__ void step(bool hit, uint32_t, uint32_t, uint32_t, uint32_t quv, uint32_t quw,
                                        uint32_t qvw, uint32_t, uint32_t, uint32_t) {
-    const unsigned m = __ballot_sync(kFull, hit);
-    if (!m) return;
-    if (hit) q[qn + __popc(m & lanemask_lt())] = tri_product(quv, quw, qvw);
-    qn += __popc(m);
-    if (qn >= 32) drain32();
-  }
-  template <int U>
-  __device__ __forceinline__ void steps(const bool (&hit)[U], uint32_t quv, const uint32_t (&quw)[U],
-                                        const uint32_t (&qvw)[U]) {
-    static_assert(U % 2 == 0, "steps come in pairs");
-#pragma unroll
-    for (int s = 0; s < U; s += 2) {
-      if (__any_sync(kFull, hit[s] || hit[s + 1])) {
-        enqueue_pair(q, qn, hit[s], hit[s + 1], quv, quw[s], qvw[s], quw[s + 1], qvw[s + 1]);
-        while (qn >= 32) drain32();
-      }
-    }
+    if (hit) bin(tri_product(quv, quw, qvw));
+    since += 32;
+    if (since >= (1u << 26)) flush();
   }
   __device__ void task_begin(uint32_t) {}
   __device__ void task_end(uint32_t) {}
   __device__ void block_end() {
-    drain_all();
     __syncthreads();
     if (threadIdx.x < 32) flush();
   }
 };
 
-// Any number of thresholds (up to 64), classified in the lane that found the
-// triangle, without a queue.  The 2 nt levels S (every B and every U,
+// Any number of thresholds (up to 64).  The 2 nt levels S (every B and every U,
 // ascending) cut the integers into 2 nt + 1 intervals; P falls in interval
 // r = #{S_j < P}, counted in bin r (finished by k_finish_multi).  r is found
 // with a slice table: P + 2^45 in [0, 2^46] is cut into 2049 slices of 2^35;
-// slice i records b0 = #{S_j < its start} and the number c of levels inside
-// it, so r = b0 + #{S_j < P, b0 <= j < b0 + c} (c is 0 or 1 unless two
-// thresholds lie within 2^35 / 2^45 = 2^-10 of each other).  Bins 0 and 2 nt
-// (P classified at every threshold, the common case for confident edges)
-// are per-lane register counters; the others are 32-bit counters in shared
-// memory, one set per warp, incremented without reading the old value.
+// slice i records r at its start, and whether levels lie inside it, which are
+// then compared (few slices: 2 nt of 2049 at most).  A byte holds both: r, or
+// 128 + r with levels inside (2 nt = 128 is given as 128 + 127, whose one
+// comparison finds it).  Bins 0 and 2 nt (P classified at every threshold, the
+// common case for confident edges) are per-lane register counters, added to
+// without a branch; the others are 32-bit counters in shared memory, one set
+// per warp, incremented without reading the old value.
 //
-// Overflow bound: a warp adds at most one per probed entry, and the bins are
-// moved to the global bins (an atomic exchange with 0, then a 64-bit add;
-// the exchange keeps adds made meanwhile) before a bin can reach 2^32:
+// Overflow bound: a warp adds at most one per probed entry, and the counters
+// are moved to the global bins (an atomic exchange with 0, then a 64-bit add;
+// the exchange keeps adds made meanwhile) before one can reach 2^32:
 //   * degree-ordered traversal (CountBins): the warp counts the entries
 //     of each batch of pairs (probed(n); forward lists are shorter than
-//     sqrt(2m) < 2^17, so a batch of 32 lists counts at most 2^23), and lane
-//     0 moves the bins once the count reaches kWarpFlush = 2^31;
+//     sqrt(2m) < 2^17, so a batch of 32 lists counts at most 2^23), and moves
+//     the counters once the count reaches kWarpFlush = 2^31;
 //   * Alg. 2 kernels (CountBinsAeo, rows of any length): every lane counts
 //     the entries it was handed and moves the bins itself once its count
 //     reaches kBinFlush, so a bin holds fewer than 32 x 2^27 adds.
@@ -358,33 +273,38 @@ struct CountBinsP {
   int nt;
   int64_t S[2 * kMaxTau];   // the 2 nt levels, ascending
   unsigned long long* out;  // global bins [0, 2 nt]
+  bool several = false;     // some slice holds several levels
+  void set_several() {
+    for (int j = 1; j < 2 * nt; j++) several |= ((S[j - 1] + (1ll << 45)) >> 35) == ((S[j] + (1ll << 45)) >> 35);
+  }
 };
-struct CountBins {
+struct CountBins : ProductItem {
   using P = CountBinsP;
   static constexpr bool kPos = false;
-  static constexpr bool kBatched = true;
   static constexpr int kRegCap = UBT_COUNT_REGCAP;
-  static constexpr int kTabBytes = ((kSlices * 2 + 15) / 16) * 16;
+  static constexpr int kTabBytes = ((kSlices + 15) / 16) * 16;
+  static constexpr int kLevelBytes = (2 * kMaxTau + 2) * 8;
   static __host__ __device__ int smem_bytes(int threads) {
-    return kTabBytes + 2 * kMaxTau * 8 + (threads / 32) * kBinStride * 4;
+    return kTabBytes + kLevelBytes + (threads / 32) * kBinStride * 4;
   }
-  const uint16_t* tab;  // shared: slice table, b0 | c << 8
-  const long long* S;   // shared: levels
-  uint32_t* bins;       // shared: this warp's bins
-  uint32_t* all;        // shared: every warp's bins, kBinStride words each
+  const uint8_t* tab;  // shared: slice table
+  const long long* S;  // shared: levels
+  uint32_t* bins;      // shared: this warp's bins
+  uint32_t* all;       // shared: every warp's bins, kBinStride words each
   unsigned long long* out;
-  unsigned long long first = 0, last = 0;  // bins 0 and 2 nt of this lane
-  uint32_t since = 0;                       // entries since the last flush (this lane's or the warp's)
-  int top;                                  // 2 nt
-  __device__ CountBins(const P& p, char* smem) : out(p.out), top(2 * p.nt) {
-    uint16_t* t = (uint16_t*)smem;
+  uint32_t first = 0, last = 0;  // bins 0 and 2 nt of this lane
+  uint32_t since = 0;            // entries since the last flush (this lane's or the warp's)
+  int top;                       // 2 nt
+  bool several;                  // some slice holds several levels
+  __device__ CountBins(const P& p, char* smem) : out(p.out), top(2 * p.nt), several(p.several) {
+    uint8_t* t = (uint8_t*)smem;
     long long* sv = (long long*)(smem + kTabBytes);
-    uint32_t* b = (uint32_t*)(smem + kTabBytes + 2 * kMaxTau * 8);
+    uint32_t* b = (uint32_t*)(smem + kTabBytes + kLevelBytes);
     tab = t;
     S = sv;
     all = b;
     bins = b + (threadIdx.x >> 5) * kBinStride;
-    for (int i = threadIdx.x; i < 2 * p.nt; i += blockDim.x) sv[i] = p.S[i];
+    for (int i = threadIdx.x; i <= 2 * p.nt; i += blockDim.x) sv[i] = i < 2 * p.nt ? p.S[i] : INT64_MAX;
     for (int i = threadIdx.x; i < (int)(blockDim.x >> 5) * kBinStride; i += blockDim.x) b[i] = 0;
     for (int i = threadIdx.x; i < kSlices; i += blockDim.x) {
       const long long start = (long long)i * (1ll << 35) - (1ll << 45);
@@ -394,53 +314,52 @@ struct CountBins {
         b0 += p.S[j] < start ? 1 : 0;
         b1 += p.S[j] < end ? 1 : 0;
       }
-      t[i] = (uint16_t)(b0 | ((b1 - b0) << 8));
+      t[i] = (uint8_t)(b0 == 128 ? 255 : b1 > b0 ? 128 + b0 : b0);
     }
   }
   __device__ void block_init() {}
-  __device__ __forceinline__ void count(long long P) {
-    const uint32_t e = tab[(uint32_t)((unsigned long long)(P + (1ll << 45)) >> 35)];
-    int r = (int)(e & 0xFFu);
-    const int c = (int)(e >> 8);
-    if (c) {
-      const int b0 = r;
-      for (int j = 0; j < c; j++) r += S[b0 + j] < P ? 1 : 0;
-    }
-    if (r == 0) {
-      first++;
-    } else if (r == top) {
-      last++;
-    } else {
-      atomicAdd(&bins[r], 1u);
-    }
+  __device__ __forceinline__ uint32_t slice_entry(long long P) const {
+    return tab[(uint32_t)((int32_t)(P >> 32) + (1 << 13)) >> 3];  // bits 35 and up of P + 2^45
   }
-  __device__ __forceinline__ void step(bool hit, uint32_t, uint32_t, uint32_t, uint32_t quv, uint32_t quw,
-                                       uint32_t qvw, uint32_t, uint32_t, uint32_t) {
-    if (hit) count(tri_product(quv, quw, qvw));
+  __device__ __forceinline__ void bin(bool on, int r) {
+    first += on && r == 0 ? 1u : 0u;
+    last += on && r == top ? 1u : 0u;
+    if (on && r != 0 && r != top) atomicAdd(&bins[r], 1u);
   }
-  template <int U>
-  __device__ __forceinline__ void steps(const bool (&hit)[U], uint32_t quv, const uint32_t (&quw)[U],
-                                        const uint32_t (&qvw)[U]) {
-#pragma unroll
-    for (int s = 0; s < U; s++)
-      if (hit[s]) count(tri_product(quv, quw[s], qvw[s]));
+  // all 32 lanes, converged.  A lane whose slice holds no level finds S[r] > P.
+  __device__ __forceinline__ void take(bool on, uint32_t, uint2 it, uint32_t, uint32_t, uint32_t quw, uint32_t,
+                                       uint32_t) {
+    const long long P = item_product(it.y, quw);
+    const uint32_t e = slice_entry(P);
+    int r = (int)(e & 127u);
+    if (__any_sync(kFull, e & 128u)) {
+      r += S[r] < P ? 1 : 0;
+      if (several)
+        while (r < top && S[r] < P) r++;
+    }
+    bin(on, r);
+  }
+  __device__ __forceinline__ void flush_ends() {
+    const unsigned long long f = warp_sum(first), l = warp_sum(last);
+    if (lane_id() == 0) {
+      if (f) atomicAdd(&out[0], f);
+      if (l) atomicAdd(&out[top], l);
+    }
+    first = last = 0;
   }
   // the degree-ordered traversal's batch count (all lanes, the same n)
   __device__ __forceinline__ void probed(uint32_t n) {
     since += n;
     if (since >= kWarpFlush) {
       if (lane_id() == 0) count_bins_flush(bins, out, top);
+      flush_ends();
       since = 0;
     }
   }
   __device__ void task_begin(uint32_t) {}
   __device__ void task_end(uint32_t) {}
   __device__ void block_end() {
-    const unsigned long long f = warp_sum(first), l = warp_sum(last);
-    if (lane_id() == 0) {
-      if (f) atomicAdd(&out[0], f);
-      if (l) atomicAdd(&out[top], l);
-    }
+    flush_ends();
     __syncthreads();
     const int nw = (int)(blockDim.x >> 5);
     for (int i = threadIdx.x + 1; i < top; i += blockDim.x) {
@@ -455,12 +374,21 @@ struct CountBins {
 // counts the entries it was handed and moves its warp's bins itself
 struct CountBinsAeo : CountBins {
   using CountBins::CountBins;
-  __device__ __forceinline__ void step(bool hit, uint32_t u, uint32_t v, uint32_t w, uint32_t quv, uint32_t quw,
-                                       uint32_t qvw, uint32_t puv, uint32_t puw, uint32_t pvw) {
-    CountBins::step(hit, u, v, w, quv, quw, qvw, puv, puw, pvw);
+  __device__ __forceinline__ void step(bool found, uint32_t, uint32_t, uint32_t, uint32_t quv, uint32_t quw,
+                                       uint32_t qvw, uint32_t, uint32_t, uint32_t) {
+    if (found) {
+      const long long P = tri_product(quv, quw, qvw);
+      const uint32_t e = slice_entry(P);
+      int r = (int)(e & 127u);
+      if (e & 128u)
+        while (r < top && S[r] < P) r++;
+      bin(true, r);
+    }
     if (++since >= kBinFlush) {
       count_bins_flush(bins, out, top);
-      since = 0;
+      if (first) atomicAdd(&out[0], (unsigned long long)first);
+      if (last) atomicAdd(&out[top], (unsigned long long)last);
+      first = last = since = 0;
     }
   }
 };
@@ -492,22 +420,26 @@ struct EnumP {
   unsigned long long cap;
   unsigned long long* cursor;
   int64_t Blo = INT64_MIN, Uhi = INT64_MAX;
+  const uint32_t* vid = nullptr;    // forward traversal: ids of the vertices
+  const uint32_t* rowid = nullptr;  // and the row of the streamed list's position
 };
 struct Enum {
   using P = EnumP;
   static constexpr bool kPos = false;
-  static constexpr bool kBatched = false;
+  using Item = uint4;  // table slot, product of two values, position of the streamed row
+  static constexpr bool kMore = false;
+  static constexpr int kU = 4;
   static constexpr int kRegCap = 64;
   static __host__ __device__ int smem_bytes(int) { return 0; }
   P p;
   __device__ Enum(const P& p_, char*) : p(p_) {}
   __device__ void block_init() {}
-  __device__ __forceinline__ void step(bool hit, uint32_t u, uint32_t v, uint32_t w, uint32_t quv, uint32_t quw,
-                                       uint32_t qvw, uint32_t, uint32_t, uint32_t) {
+  // all 32 lanes, converged: `hit` lanes have a triangle of product P whose
+  // vertices ids(a, b, c) gives
+  template <class F>
+  __device__ __forceinline__ void emit(bool hit, long long P, F&& ids) {
     uint32_t cls = 0;
-    int64_t P = 0;
     if (hit) {
-      P = tri_product(quv, quw, qvw);
       if ((p.which & 1) && P <= p.B && P > p.Blo) cls = 1;
       else if ((p.which & 2) && P > p.U && P <= p.Uhi) cls = 2;
     }
@@ -521,7 +453,8 @@ struct Enum {
     if (cls) {
       const unsigned long long idx = base + __popc(m & lanemask_lt());
       if (idx < p.cap) {
-        uint32_t a = u, b = v, c = w, t;
+        uint32_t a, b, c, t;
+        ids(a, b, c);
         if (a > b) { t = a; a = b; b = t; }
         if (b > c) { t = b; b = c; c = t; }
         if (a > b) { t = a; a = b; b = t; }
@@ -532,6 +465,26 @@ struct Enum {
         p.out[idx] = r;
       }
     }
+  }
+  __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t s, uint32_t, uint32_t) {
+    return make_uint4(slot, (uint32_t)((int32_t)quv * (int32_t)qvw), s, 0u);
+  }
+  __device__ __forceinline__ void take(bool on, uint32_t, uint4 it, uint32_t, uint32_t x, uint32_t quw, uint32_t,
+                                       uint32_t w) {
+    emit(on, item_product(it.y, quw), [&](uint32_t& a, uint32_t& b, uint32_t& c) {
+      a = p.vid[x];
+      b = p.vid[p.rowid[it.z]];
+      c = p.vid[w];
+    });
+  }
+  // the Alg. 2 kernels (u, v, w are ids)
+  __device__ __forceinline__ void step(bool hit, uint32_t u, uint32_t v, uint32_t w, uint32_t quv, uint32_t quw,
+                                       uint32_t qvw, uint32_t, uint32_t, uint32_t) {
+    emit(hit, hit ? tri_product(quv, quw, qvw) : 0ll, [&](uint32_t& a, uint32_t& b, uint32_t& c) {
+      a = u;
+      b = v;
+      c = w;
+    });
   }
   __device__ void task_begin(uint32_t) {}
   __device__ void task_end(uint32_t) {}
@@ -550,7 +503,9 @@ template <bool kReal>
 struct Expect {
   using P = ExpectP;
   static constexpr bool kPos = false;
-  static constexpr bool kBatched = false;
+  using Item = uint4;  // table slot, the pair's and the streamed edge's values
+  static constexpr bool kMore = false;
+  static constexpr int kU = 4;
   static constexpr int kRegCap = 64;
   static __host__ __device__ int smem_bytes(int) { return 0; }
   P p;
@@ -558,9 +513,13 @@ struct Expect {
   unsigned long long cnt = 0;
   __device__ Expect(const P& p_, char*) : p(p_) {}
   __device__ void block_init() {}
-  __device__ __forceinline__ void step(bool hit, uint32_t, uint32_t, uint32_t, uint32_t quv, uint32_t quw,
-                                       uint32_t qvw, uint32_t, uint32_t, uint32_t) {
-    if (!hit) return;
+  __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t, uint32_t, uint32_t) {
+    return make_uint4(slot, quv, qvw, 0u);
+  }
+  __device__ __forceinline__ void take(bool on, uint32_t, uint4 it, uint32_t, uint32_t, uint32_t quw, uint32_t,
+                                       uint32_t) {
+    if (!on) return;
+    const uint32_t quv = it.y, qvw = it.z;
     cnt++;
     if (kReal) {
       const long long a = (long long)(int32_t)quv * (int32_t)quw;          // 2^-60
@@ -615,15 +574,22 @@ template <bool kReal>
 struct Adjoint {
   using P = AdjointP;
   static constexpr bool kPos = true;
-  static constexpr bool kBatched = false;
+  using Item = uint4;  // table slot, the pair's and the streamed edge's values, the pair's position
+  static constexpr bool kMore = true;
+  static constexpr int kU = 2;
   static constexpr int kRegCap = 64;
   static __host__ __device__ int smem_bytes(int) { return 0; }
   P p;
   __device__ Adjoint(const P& p_, char*) : p(p_) {}
   __device__ void block_init() {}
-  __device__ __forceinline__ void step(bool hit, uint32_t, uint32_t, uint32_t, uint32_t quv, uint32_t quw,
-                                       uint32_t qvw, uint32_t puv, uint32_t puw, uint32_t pvw) {
-    if (!hit) return;
+  __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t, uint32_t puv,
+                                               uint32_t) {
+    return make_uint4(slot, quv, qvw, puv);
+  }
+  __device__ __forceinline__ void take(bool on, uint32_t, uint4 it, uint32_t pvw, uint32_t, uint32_t quw, uint32_t puw,
+                                       uint32_t) {
+    if (!on) return;
+    const uint32_t quv = it.y, qvw = it.z, puv = it.w;
     long long a_uv, a_uw, a_vw;
     if (kReal) {
       // products of two 2^-30 fixed-point values are exact in int64 (2^-60);
@@ -656,37 +622,21 @@ __global__ void k_finish_adjoint(int64_t m, const unsigned long long* __restrict
 // traversal sizes (same task and pruning rules as the traversal); one warp
 // per owner.  out: [0] table entries, [1] pairs probed, [2] streamed
 // entries, [3] tasks
-__global__ void k_trav_stats(int64_t n, const uint32_t* __restrict__ row_ptr, const uint64_t* __restrict__ adj,
-                             const uint32_t* __restrict__ pair_ptr, const uint64_t* __restrict__ pairs, int64_t L,
-                             uint32_t light, unsigned long long* out) {
+__global__ void k_trav_stats(TravArgs a, unsigned long long* out) {
   const int lane = (int)lane_id();
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   unsigned long long tab = 0, npairs = 0, str = 0, tasks = 0;
-  for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += warps) {
-    const uint32_t rs = row_ptr[x];
-    uint32_t len = row_ptr[x + 1] - rs;
-    const uint32_t ps = pair_ptr[x], pe = pair_ptr[x + 1];
-    if (len < 2 || pe == ps) continue;
-    int64_t qmax = 0;
-    if (L > 0) {
-      qmax = qabs(adj_valbits(adj[rs]));
-      len = prune_prefix(adj + rs, len, 1ll << 30, L);
-    }
-    if (len == 0) continue;
+  for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < a.n; x += warps) {
+    uint32_t rs = 0, len = 0, ps = 0, np = 0;
+    if (!owner_list(a, (uint32_t)x, rs, len) || !pair_range(a, (uint32_t)x, ps, np) || len == 0 || np == 0) continue;
     if (lane == 0) {
       tab += len;
       tasks += 1;
     }
-    for (uint32_t i = ps + lane; i < pe; i += 32) {
-      const uint64_t d = pairs[i];
-      const uint32_t sv = (uint32_t)d;
-      const int64_t qe = qabs(adj_valbits(adj[(uint32_t)(d >> 32)]));
-      if (L > 0 && qe * (1ll << 30) < L) continue;
-      const uint32_t vs = row_ptr[sv];
-      uint32_t dv = row_ptr[sv + 1] - vs;
-      if (L > 0 && !light) dv = prune_prefix(adj + vs, dv, qe * qmax, L);
-      npairs += 1;
-      str += dv;
+    for (uint32_t i = 0; i < np; i += 32) {
+      const Pair pr = owner_pair(a, (uint32_t)x, ps + i, min(32u, np - i));
+      npairs += pr.dv > 0 ? 1 : 0;
+      str += pr.dv;
     }
   }
   tab = warp_sum(tab);
@@ -705,41 +655,67 @@ __global__ void k_trav_stats(int64_t n, const uint32_t* __restrict__ row_ptr, co
 
 }  // namespace
 
-TravArgs make_trav_args(const ubt_graph* g, int64_t L, bool with_pos) {
-  (void)with_pos;
+// Whether writing the kept entries of level L first pays for itself: with a
+// share f of the edges kept, about f^2 of the probes remain; writing reads
+// every entry twice and writes the kept ones.
+bool prune_pays(const ubt_graph* g, int64_t qmin) {
+  const double f = g->kept[std::min<int64_t>(65, qmin >> 9)];  // an upper bound of the share
+  const double saved_us = (double)g->probes * (1.0 - f * f) / 3.0e5;
+  const double cost_us = 12.0 + (double)g->m * (20.0 + 8.0 * f) / 4.0e6;
+  return saved_us > cost_us;
+}
+
+// The traversal of graph g at prune level L (0: none).  Enqueues the writing
+// of the kept entries where that pays.
+ubt_status make_trav_args(const ubt_graph* g, int64_t L, cudaStream_t s, TravArgs* out) {
   const Tuning& T = tuning();
   TravArgs a;
   a.row_ptr = g->row_ptr;
   a.adj = g->adj;
   a.pair_ptr = g->pair_ptr;
   a.pairs = g->pairs;
-  a.giant_list = g->giant_list;
-  a.hub_list = g->hub_list;
-  a.med_list = g->med_list;
-  a.n_giant = (uint32_t)g->n_giant;
-  a.n_hub = (uint32_t)g->n_hub;
-  a.n_med = (uint32_t)g->n_med;
+  a.keep = nullptr;
+  for (int c = 0; c < kTaskClasses; c++) {
+    a.lists[c] = g->lists[c];
+    a.n_tasks[c] = (uint32_t)g->n_tasks[c];
+  }
+  a.vgraph = g->vgraph;
+  a.gstart = g->gstart;
   a.n = (uint32_t)g->n;
   a.m = (uint32_t)g->m;
   a.sc = g->scratch;
   a.gtab = g->gtab;
   a.gtab_slots = (uint32_t)g->gtab_slots;
-  a.gtab_blocks = g->n_giant ? (uint32_t)g->gtab_blocks : 0u;
-  a.hub_slots = g->n_hub ? (uint32_t)table_slots(g->max_hub_len) : 0u;
+  a.gtab_blocks = g->n_tasks[kGiant] ? (uint32_t)g->gtab_blocks : 0u;
+  a.hub_slots = (uint32_t)table_slots(g->max_hash_len);
+  a.hub_bits = (uint32_t)g->max_bits;
+  a.hub_len = (uint32_t)g->max_bits_len;
   // a warp table holds one medium task's list (at most hub_threshold entries)
-  a.warp_slots = (uint32_t)table_slots(g->hub_threshold);
+  a.warp_slots = (uint32_t)table_slots(std::min(g->hub_threshold, g->max_out));
+  a.warp_len = (uint32_t)std::min(g->hub_threshold, g->max_out);
+  a.warp_bits = (uint32_t)std::min(g->warp_bits, g->n);
   a.unit = (uint32_t)std::min<int64_t>(32, std::max<int64_t>(1, T.block_unit));
   a.batch = (uint32_t)std::max<int64_t>(1, T.small_batch);
   a.long_min = (uint32_t)T.long_min;
   a.long_tail = (uint32_t)T.long_tail;
-  a.L = L;
-  a.light_prune = light_prune_for(L);
-  return a;
+  // Lemma 2: |q| 2^30 >= L
+  const int64_t qmin = L > 0 ? (L + (1ll << 30) - 1) >> 30 : 0;
+  a.qmin2 = (uint32_t)(qmin >> 1);
+  if (qmin > 0 && g->keep && prune_pays(g, qmin)) {
+    UBT_RANGE("prune");
+    UBT_CUDA(keep_entries(g->adj, g->m, (uint32_t)qmin, g->keep, (uint64_t*)g->gacc, g->keep_tmp, s));
+    a.adj = (const uint64_t*)g->gacc;
+    a.keep = g->keep;
+  }
+  *out = a;
+  return UBT_OK;
 }
 
 template <class V>
 ubt_status launch_traverse(const ubt_graph* g, const typename V::P& p, int64_t L, cudaStream_t s) {
-  return launch_traversal<V>(g, make_trav_args(g, L, V::kPos), p, s);
+  TravArgs a;
+  const ubt_status st = make_trav_args(g, L, s, &a);
+  return st != UBT_OK ? st : launch_traversal<V>(g, a, p, s);
 }
 
 // Threshold counts (at most kRegTau thresholds) whose per-call scratch -- the
@@ -764,9 +740,10 @@ ubt_status count_reg_at(const ubt_graph* g, const double* h_tau, int n_tau, int 
     p.U[i] = i < n_tau ? lv[i].U : INT64_MAX;
   }
   p.out = acc;
-  TravArgs a = make_trav_args(g, L, false);
+  TravArgs a;
+  ubt_status st = make_trav_args(g, L, s, &a);
+  if (st != UBT_OK) return st;
   a.sc = sc;
-  ubt_status st = UBT_OK;
   switch (NT) {
     case 1: st = launch_traversal<CountReg<1>>(g, a, p, s); break;
     case 2: st = launch_traversal<CountReg<2>>(g, a, p, s); break;
@@ -825,6 +802,7 @@ ubt_status count_impl(ubt_graph* g, const double* h_tau, int32_t n_tau, int32_t 
       p.S[i] = lv[order[n_tau - 1 - i]].B;  // B ascending: t descending
       p.S[n_tau + i] = lv[order[i]].U;      // U ascending: t ascending
     }
+    p.set_several();
     p.out = g->scratch->hist;
     UBT_CUDA(cudaMemsetAsync(g->scratch->hist, 0, sizeof(g->scratch->hist), s));
     st = aeo ? launch_aeo<CountBinsAeo>(g, L, p, s) : launch_traverse<CountBins>(g, p, L, s);
@@ -902,6 +880,10 @@ ubt_status enumerate_impl(ubt_graph* g, double tau, int32_t which, int32_t prune
   Level lv;
   if (!tau_level(tau, &lv)) return UBT_ERR_TAU_OOB;
   EnumP p{lv.B, lv.U, which, d_out, (unsigned long long)capacity, &g->scratch->enum_cursor};
+  if (!aeo) {
+    p.vid = g->vid;
+    p.rowid = g->rowid;
+  }
   ubt_status st = aeo ? launch_aeo<Enum>(g, lv.L, p, s) : launch_traverse<Enum>(g, p, prune ? lv.L : 0, s);
   if (st != UBT_OK) return st;
   unsigned long long found = 0;
@@ -971,8 +953,11 @@ extern "C" ubt_status ubt_traversal_stats(ubt_graph* g, const double* h_tau, int
   unsigned long long* d = &g->scratch->hist[0];
   UBT_CUDA(cudaMemsetAsync(d, 0, 4 * sizeof(unsigned long long), s));
   if (g->n > 0) {
+    TravArgs a;
+    const ubt_status st = make_trav_args(g, L, s, &a);
+    if (st != UBT_OK) return st;
     const int grid = (int)std::min<int64_t>((g->n + 7) / 8, (int64_t)g->sm_count * 16);
-    k_trav_stats<<<grid, 256, 0, s>>>(g->n, g->row_ptr, g->adj, g->pair_ptr, g->pairs, L, light_prune_for(L), d);
+    k_trav_stats<<<grid, 256, 0, s>>>(a, d);
     UBT_CUDA(cudaGetLastError());
   }
   unsigned long long h[4];
@@ -990,29 +975,6 @@ extern "C" ubt_status ubt_query_guard(ubt_graph* g, int64_t* h_word, void* strea
   UBT_CUDA(cudaMemsetAsync(&g->scratch->guard, 0, sizeof(w), s));
   UBT_CUDA(cudaStreamSynchronize(s));
   *h_word = (int64_t)w;
-  return UBT_OK;
-}
-
-extern "C" ubt_status ubt_graph_export(const ubt_graph* g, uint32_t* h_row_ptr, uint64_t* h_adj, uint32_t* h_eid,
-                                       uint32_t* h_lists, int64_t* h_list_sizes, void* stream) {
-  if (!g) return UBT_ERR_INVALID_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
-  if (h_row_ptr)
-    UBT_CUDA(cudaMemcpyAsync(h_row_ptr, g->row_ptr, sizeof(uint32_t) * (g->n + 1), cudaMemcpyDeviceToHost, s));
-  if (h_adj && g->m)
-    UBT_CUDA(cudaMemcpyAsync(h_adj, g->adj, sizeof(uint64_t) * g->m, cudaMemcpyDeviceToHost, s));
-  if (h_eid && g->m)
-    UBT_CUDA(cudaMemcpyAsync(h_eid, g->eid, sizeof(uint32_t) * g->m, cudaMemcpyDeviceToHost, s));
-  const int64_t tasks = g->n_giant + g->n_hub + g->n_med;
-  if (h_lists && tasks)
-    UBT_CUDA(cudaMemcpyAsync(h_lists, g->giant_list, sizeof(uint32_t) * tasks, cudaMemcpyDeviceToHost, s));
-  if (h_list_sizes) {
-    h_list_sizes[0] = g->n_giant;
-    h_list_sizes[1] = g->n_hub;
-    h_list_sizes[2] = g->n_med;
-    h_list_sizes[3] = 0;
-  }
-  UBT_CUDA(cudaStreamSynchronize(s));
   return UBT_OK;
 }
 
@@ -1064,6 +1026,7 @@ ubt_status count_levels(const ubt_graph* g, const std::vector<int64_t>& lev, int
   CountBinsP p;
   p.nt = (int)lev.size() / 2;
   for (size_t i = 0; i < lev.size(); i++) p.S[i] = lev[i];
+  p.set_several();
   p.out = g->scratch->hist;
   UBT_CUDA(cudaMemsetAsync(g->scratch->hist, 0, sizeof(g->scratch->hist), s));
   ubt_status st = launch_traverse<CountBins>(g, p, L, s);
@@ -1078,7 +1041,8 @@ ubt_status count_levels(const ubt_graph* g, const std::vector<int64_t>& lev, int
 // exist (all of them, even past cap)
 ubt_status enum_range(const ubt_graph* g, int which, int64_t B, int64_t Blo, int64_t U, int64_t Uhi, int64_t L,
                       ubt_tri_rec* r, int64_t cap, int64_t* found, cudaStream_t s) {
-  EnumP p{B, U, which, r, (unsigned long long)std::max<int64_t>(cap, 0), &g->scratch->enum_cursor, Blo, Uhi};
+  EnumP p{B, U, which, r, (unsigned long long)std::max<int64_t>(cap, 0), &g->scratch->enum_cursor, Blo, Uhi,
+          g->vid, g->rowid};
   ubt_status st = launch_traverse<Enum>(g, p, L, s);
   if (st != UBT_OK) return st;
   unsigned long long f = 0;
@@ -1210,18 +1174,6 @@ extern "C" ubt_status ubt_graph_export_undirected(const ubt_graph* g, uint32_t* 
     UBT_CUDA(cudaMemcpyAsync(h_apair_ptr, g->apair_ptr, sizeof(uint32_t) * (g->n + 1), cudaMemcpyDeviceToHost, s));
   if (h_apairs && g->m)
     UBT_CUDA(cudaMemcpyAsync(h_apairs, g->apairs, sizeof(uint64_t) * g->m, cudaMemcpyDeviceToHost, s));
-  UBT_CUDA(cudaStreamSynchronize(s));
-  return UBT_OK;
-}
-
-extern "C" ubt_status ubt_graph_export_pairs(const ubt_graph* g, uint32_t* h_pair_ptr, uint64_t* h_pairs,
-                                             void* stream) {
-  if (!g) return UBT_ERR_INVALID_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
-  if (h_pair_ptr)
-    UBT_CUDA(cudaMemcpyAsync(h_pair_ptr, g->pair_ptr, sizeof(uint32_t) * (g->n + 1), cudaMemcpyDeviceToHost, s));
-  if (h_pairs && g->m)
-    UBT_CUDA(cudaMemcpyAsync(h_pairs, g->pairs, sizeof(uint64_t) * g->m, cudaMemcpyDeviceToHost, s));
   UBT_CUDA(cudaStreamSynchronize(s));
   return UBT_OK;
 }

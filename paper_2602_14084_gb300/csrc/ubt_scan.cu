@@ -99,6 +99,70 @@ __global__ void k_tile_apply(const uint32_t* in, int64_t n, const uint32_t* __re
   }
 }
 
+// The scan of at most kSmallTiles tiles in one launch, total at out[n].
+constexpr int64_t kSmallTiles = 4;
+__global__ void k_scan_small(const uint32_t* in, int64_t n, uint32_t* out) {
+  uint32_t carry = 0;
+  for (int64_t start = 0; start < n; start += kTile) {
+    const int64_t base = start + (int64_t)threadIdx.x * kScanItems;
+    uint32_t v[kScanItems];
+    uint32_t s = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++) {
+      v[i] = (base + i < n) ? in[base + i] : 0;
+      s += v[i];
+    }
+    uint32_t ex;
+    const uint32_t tot = block_exclusive_scan(s, &ex);
+    uint32_t run = carry + ex;
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++) {
+      if (base + i < n) out[base + i] = run;
+      run += v[i];
+    }
+    carry += tot;
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
+// Kept entries (|q| >= qmin) per tile of row entries, and, with the scanned
+// tile counts, keep[i] = kept entries before i and the kept entries themselves
+// in order.  Both stream the rows once (8 bytes an entry); the second pass
+// mostly reads them from L2.
+__device__ __forceinline__ bool entry_kept(uint64_t e, uint32_t qmin) {
+  const int32_t q = adj_q(e);
+  return (uint32_t)(q < 0 ? -q : q) >= qmin;
+}
+__global__ void k_keep_count(const uint64_t* __restrict__ adj, int64_t m, uint32_t qmin, uint32_t* __restrict__ tile_sum) {
+  const int64_t base = (int64_t)blockIdx.x * kTile;
+  uint32_t s = 0;
+#pragma unroll
+  for (int i = 0; i < kScanItems; i++) {
+    const int64_t at = base + i * kScanThreads + threadIdx.x;
+    if (at < m && entry_kept(adj[at], qmin)) s++;
+  }
+  uint32_t ex;
+  const uint32_t tot = block_exclusive_scan(s, &ex);
+  if (threadIdx.x == 0) tile_sum[blockIdx.x] = tot;
+}
+__global__ void k_keep_apply(const uint64_t* __restrict__ adj, int64_t m, uint32_t qmin,
+                             const uint32_t* __restrict__ tile_off, uint32_t* __restrict__ keep,
+                             uint64_t* __restrict__ kept) {
+  uint32_t run = tile_off[blockIdx.x];
+  const int64_t base = (int64_t)blockIdx.x * kTile;
+#pragma unroll
+  for (int i = 0; i < kScanItems; i++) {  // coalesced: kScanThreads consecutive entries at a time
+    const int64_t at = base + i * kScanThreads + threadIdx.x;
+    const uint64_t e = at < m ? adj[at] : 0ull;
+    const uint32_t on = at < m && entry_kept(e, qmin) ? 1u : 0u;
+    uint32_t ex;
+    const uint32_t tot = block_exclusive_scan(on, &ex);
+    if (at < m) keep[at] = run + ex;
+    if (on) kept[run + ex] = e;
+    run += tot;
+  }
+}
+
 __global__ void k_write_total(const uint32_t* tile_off, int64_t ntiles, uint32_t* out, int64_t n) {
   out[n] = tile_off[ntiles];
 }
@@ -111,14 +175,26 @@ size_t scan_tmp_words(int64_t n) { return (size_t)((n + kTile - 1) / kTile) + 2;
 // `out` may alias.  tmp holds scan_tmp_words(n) words.
 cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp, cudaStream_t s) {
   const int64_t ntiles = (n + kTile - 1) / kTile;
-  if (ntiles > 0) {
-    k_tile_sums<<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp);
-    k_scan_tiles<<<1, kScanThreads, 0, s>>>(tmp, ntiles);
-    k_tile_apply<<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp, out);
-  } else {
-    cudaMemsetAsync(tmp, 0, sizeof(uint32_t), s);
+  if (ntiles <= kSmallTiles) {
+    k_scan_small<<<1, kScanThreads, 0, s>>>(in, n, out);
+    return cudaGetLastError();
   }
+  k_tile_sums<<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp);
+  k_scan_tiles<<<1, kScanThreads, 0, s>>>(tmp, ntiles);
+  k_tile_apply<<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp, out);
   k_write_total<<<1, 1, 0, s>>>(tmp, ntiles, out, n);
+  return cudaGetLastError();
+}
+
+// keep[0..m]: kept entries before each position, and the kept entries in
+// order.  tmp holds scan_tmp_words(m) words.
+cudaError_t keep_entries(const uint64_t* adj, int64_t m, uint32_t qmin, uint32_t* keep, uint64_t* kept, uint32_t* tmp,
+                         cudaStream_t s) {
+  const int64_t ntiles = (m + kTile - 1) / kTile;
+  if (ntiles > 0) k_keep_count<<<(unsigned)ntiles, kScanThreads, 0, s>>>(adj, m, qmin, tmp);
+  k_scan_tiles<<<1, kScanThreads, 0, s>>>(tmp, ntiles);
+  if (ntiles > 0) k_keep_apply<<<(unsigned)ntiles, kScanThreads, 0, s>>>(adj, m, qmin, tmp, keep, kept);
+  k_write_total<<<1, 1, 0, s>>>(tmp, ntiles, keep, m);
   return cudaGetLastError();
 }
 

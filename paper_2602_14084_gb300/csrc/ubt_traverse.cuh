@@ -3,48 +3,63 @@
 // Forward edge iteration under Node Order (Alg. 1, Sec. 4): triangle {u,v,w}
 // with u < v < w in Node Order is found exactly once, from its pair (u, v),
 // as w in N>(u) n N>(v).  Every forward edge is one pair.  Alg. 1 streams
-// N>(v) through a table of N>(u); streaming N>(u) through a table of N>(v)
-// intersects the same two lists, and the build gives each pair to the
-// endpoint (its "owner" x) whose list is the longer, so that the shorter list
-// N>(s) is streamed (the pair partition of ubt_build.cu).
+// N>(v) through a table of N>(u); here the later vertex v owns the pair (the
+// "owner" x): the table holds N>(v), and of N>(u) only the part after v is
+// streamed -- the entries of row u before v's position, as the rows are
+// sorted latest vertex first (ubt_internal.cuh).
 //
 // GPU layout of that loop (two persistent kernels, three kinds of task):
-//   * N>(x) is loaded into an open-addressing hash table (neighbour -> edge
-//     value, CSR position) in shared memory: 4-slot buckets read with one
-//     16-byte load, at most 1/4 full, so nearly every probe is one load.
+//   * N>(x) becomes a table in shared memory that answers "is w in N>(x), and
+//     with which edge value and CSR position":
+//       bitmap  one bit per vertex before x in its graph's range, and where a
+//               word's first entry is in the list: membership is one 4-byte
+//               shared load, a hit's entry is found by counting bits (its CSR
+//               position too) and its value loaded from the list's values.
+//               The touched words are cleared after the task, so a table costs
+//               what its list is long, not its range.
+//       hash    neighbour -> edge value, CSR position in 4-slot buckets read
+//               with one 16-byte load, at most 1/4 full: for owners whose range
+//               is too large for a bitmap (low-degree vertices of large graphs)
+//     A shared-memory load serves 32 random 4-byte words in 3-4 cycles and 32
+//     random 16-byte buckets in about 10, which bound the hash form.
 //   * The pairs of x are handed to one warp 32 at a time.  The lists N>(s)
 //     are streamed with coalesced 8-byte loads: long lists one after another
 //     by the whole warp, short lists concatenated ("flattened") so that every
-//     lane has an entry.  Each entry w is probed in x's table; a hit is a
+//     lane has an entry (a "list" is the streamed part of a row).  Each entry w is probed in x's table; a hit is a
 //     triangle and goes to the visitor with the three edge values and CSR
 //     positions.
-//   * Task kinds, by owner:
-//       giant   list longer than the shared-memory table: whole block, table
-//               in a per-block slice of global memory
-//       hub     long list or heavy streamed work: whole block, shared table,
-//               warps take `unit` pairs at a time
-//       medium  the rest: one warp, its own table
-//   * Probability pruning (FIXED graphs, level L > 0): every list is sorted by
-//     |q| descending, so the entries that cannot reach |P| >= L are suffixes:
-//       table and pairs:   |q_e| * 2^30 >= L              (Lemma 2: the other
-//                                                         two factors are at
-//                                                         most 2^15)
-//       streamed N>(s):    |q_sw| * |q_xs| * qmax(x) >= L (order-free form of
-//                                                         Lemma 3: the other
-//                                                         two edges bound it)
-//     qmax(x) is the largest |q| in N>(x) (its first entry).
+//   * Task classes, by owner:
+//       giant   list longer than the shared-memory hash table: whole block, hash
+//               table in a per-block slice of global memory
+//       hub     long list or heavy streamed work: whole block, warps take
+//               `unit` pairs at a time (bitmap or hash table)
+//       medium  the rest: one warp, its own table (bitmap or hash)
+//   * Probability pruning (FIXED graphs, level L > 0): an edge with |q_e| 2^30
+//     < L is in no triangle with |P| >= L (Lemma 2: the other two factors are
+//     at most 2^15).  Where a level removes enough (prune_pays), the query
+//     first writes the kept entries of all rows in order (keep_entries) and
+//     the traversal runs on those: `adj` holds the kept entries and keep[pos]
+//     says how many lie before the unpruned position pos.  A pair that fails
+//     is skipped from its pair word alone.  Otherwise nothing is pruned; the
+//     visitors classify every product exactly either way.
+//
+// Hits go through a queue: a warp appends the triangles that its lanes find --
+// the table slot, the two other edges' values, positions -- to a queue in
+// shared memory and takes them 32 at a time, so that the table lookup of the
+// value, the product and what the query does with it run on full warps
+// instead of the third of the lanes that hits on average (a miss costs only
+// the membership test and its part of the append).
 //
 // Visitors implement: smem_bytes(threads) (shared memory they need) /
-// block_init / task_begin / step (called by all 32 lanes of a warp, converged,
-// once per probed entry with a hit flag) / task_end / block_end.  Visitors
-// with kBatched also take the hits of U probes of one long list at once
-// (steps<U>: hit flags and the two streamed-edge values; the pair's is common).
-// A visitor sees a triangle as (x, s, w): the pair edge x-s, the table edge
-// x-w and the streamed edge s-w; under pull x is the later vertex of the pair,
-// so visitors treat the three edges symmetrically (they all do).  A visitor
-// may also define probed(n): after each batch of at most 32 pairs the whole
-// warp calls it with n >= the number of entries the batch probed (the same n
-// in every lane).
+// block_init / task_begin / task_end / block_end; item (what is queued of a
+// triangle; with kMore the streamed edge's position too) and take (called by
+// all 32 lanes of a warp, converged, with up to 32 queued triangles, `on` in
+// the lanes that have one).  A visitor sees a triangle as
+// (x, s, w): the pair edge x-s, the table edge x-w and the streamed edge s-w;
+// s is given as an (unpruned) CSR position in its row, whose rowid it is.  A
+// visitor may also define probed(n): after each batch of at most 32 pairs the
+// whole warp calls it with n >= the number of entries the batch probed (the
+// same n in every lane).
 #pragma once
 
 #include <algorithm>
@@ -53,18 +68,6 @@
 
 #include "ubt_internal.cuh"
 
-// launch bounds of the traversal kernels: at most UBT_LB_THREADS threads per
-// block, at least UBT_LB_MINB resident blocks per SM (caps the registers)
-#ifndef UBT_LB_THREADS
-#define UBT_LB_THREADS 512
-#endif
-#ifndef UBT_LB_MINB
-#define UBT_LB_MINB 1
-#endif
-// entries per lane of a full chunk of a long list (4 or 8)
-#ifndef UBT_LONG_U
-#define UBT_LONG_U 4
-#endif
 
 namespace ubt {
 
@@ -72,31 +75,27 @@ struct TravArgs {
   const uint32_t* row_ptr;
   const uint64_t* adj;
   const uint32_t* pair_ptr;    // pairs of owner x: [pair_ptr[x], pair_ptr[x + 1])
-  const uint64_t* pairs;       // streamed vertex | CSR position of the pair edge << 32
-  const uint32_t* giant_list;
-  const uint32_t* hub_list;
-  const uint32_t* med_list;
-  uint32_t n_giant, n_hub, n_med;
+  const uint64_t* pairs;       // pair words (ubt_internal.cuh)
+  const uint32_t* keep;        // pruned: kept entries before every position (adj holds the kept ones); else null
+  const uint64_t* lists[kTaskClasses];  // owner | part << 32 | (parts - 1) << 48
+  uint32_t n_tasks[kTaskClasses];
+  const uint32_t* vgraph;      // batch: graph of every vertex and first vertex of every graph (else null)
+  const uint32_t* gstart;
   uint32_t n, m;            // vertices, edges (bounds of the self-checks)
   Scratch* sc;              // task counters (zeroed before launch)
   uint32_t* gtab;           // giant tables: gtab_blocks x gtab_slots x 3 words
   uint32_t gtab_slots;      // power of two
   uint32_t gtab_blocks;
-  uint32_t hub_slots;       // shared-memory hub table capacity (power of two)
-  uint32_t warp_slots;      // per-warp table capacity (power of two)
+  uint32_t hub_slots;       // shared-memory hash table of a hub (power of two)
+  uint32_t warp_slots;      // per-warp hash table (power of two)
+  uint32_t hub_bits, hub_len;    // bitmap table of a hub: range and list
+  uint32_t warp_bits, warp_len;  // and of a medium task
   uint32_t unit;            // pairs per warp step in block tasks
   uint32_t batch;           // warp tasks taken per grab
   uint32_t long_min;        // streamed lists at least this long take the whole-warp path
   uint32_t long_tail;       // 1: a long list's last < 64 entries join the concatenated short lists
-  int64_t L;                // prune level, 0 = none
-  uint32_t light_prune;     // 1: streamed lists kept whole (owner tables and pairs still pruned)
+  uint32_t qmin2;           // pairs with |q| >> 1 below this are skipped (0: none)
 };
-
-// At a low prune level (2t - 1 < 1/10) a streamed list rarely loses more than
-// a few entries, and streaming them costs less than the load of the list's
-// last entry that decides whether any go.  The kept entries form no triangle
-// with |P| >= L, so every query answers the same.
-inline uint32_t light_prune_for(int64_t L) { return L > 0 && L < (1ll << 45) / 10 ? 1u : 0u; }
 
 __device__ __forceinline__ uint32_t hash_slot(uint32_t w, int shift) { return (w * 0x9E3779B1u) >> shift; }
 
@@ -235,20 +234,17 @@ __host__ __device__ constexpr uint32_t table_words(uint32_t slots) {
   return slots * TableWords<V::kPos>::kWords;
 }
 
-// table_find for the 32 converged lanes of a warp (every lane calls it; a
+// The slot of w for the 32 converged lanes of a warp (every lane calls it; a
 // lane without an entry passes any key and ignores the result): the search
 // past a full home bucket -- rare, at most 1/4 of the slots are used -- is
-// entered by the whole warp only when some lane needs it, and the value is
-// read from the slot the bucket search ends at, hit or not, so that the
-// common case runs without a divergent branch.
-template <bool kPos>
-__device__ __forceinline__ bool table_find_warp(const Table& t, uint32_t w, uint32_t& val, uint32_t& pos,
-                                                Scratch* sc) {
+// entered by the whole warp only when some lane needs it, so that the common
+// case runs without a divergent branch.
+__device__ __forceinline__ bool table_slot_warp(const Table& t, uint32_t w, uint32_t& slot, Scratch* sc) {
   uint32_t b = hash_slot(w, t.shift);
   const uint4 k = reinterpret_cast<const uint4*>(t.key)[b];
   const bool m0 = k.x == w, m1 = k.y == w, m2 = k.z == w, m3 = k.w == w;
   bool hit = m0 | m1 | m2 | m3;
-  uint32_t s = 4 * b + (m0 ? 0u : (m1 ? 1u : (m2 ? 2u : 3u)));
+  slot = 4 * b + (m0 ? 0u : (m1 ? 1u : (m2 ? 2u : 3u)));
   const bool more = !hit && k.w != kEmpty;
   if (__any_sync(kFull, more)) {
     if (more) {  // the home bucket is full: continue in the next ones
@@ -259,7 +255,7 @@ __device__ __forceinline__ bool table_find_warp(const Table& t, uint32_t w, uint
         const bool n0 = kk.x == w, n1 = kk.y == w, n2 = kk.z == w, n3 = kk.w == w;
         if (n0 | n1 | n2 | n3) {
           hit = true;
-          s = 4 * b + (n0 ? 0u : (n1 ? 1u : (n2 ? 2u : 3u)));
+          slot = 4 * b + (n0 ? 0u : (n1 ? 1u : (n2 ? 2u : 3u)));
           ended = true;
           break;
         }
@@ -271,77 +267,233 @@ __device__ __forceinline__ bool table_find_warp(const Table& t, uint32_t w, uint
       if (!ended) guard_fail(sc, kGuardFind, w);
     }
   }
-  val = t.val[s];
-  if (kPos) pos = t.pos[s];
   return hit;
 }
 
 // Per-lane description of one pair handed to probe_pairs: owner x (its list
-// is the table), streamed vertex s, CSR position and value of the x-s edge.
+// is the table), position and value of the pair edge, an unpruned position of
+// the streamed row, and the streamed entries [vs, vs + dv) of adj.
 struct Pair {
-  uint32_t x, s, pe, qe;
-  int64_t qmax;  // largest |q| of x's list (pruning)
-  bool ok;
+  uint32_t x, s, pe, qe, vs, dv;
 };
 
-// The whole warp probes entries [off, off + 32 U) of one long list N>(v),
-// U entries per lane, all loads issued before the probes.  kAll: all 32 U
-// entries exist (no bounds tests).
-template <class V, int U, bool kAll>
-__device__ __forceinline__ void long_steps(const uint64_t* __restrict__ adj, Scratch* sc, V& vis, const Table& t,
-                                           int lane, uint32_t uj, uint32_t vj, uint32_t vsj, uint32_t dvj,
-                                           uint32_t qj, uint32_t pj, uint32_t off) {
-  uint64_t e[U];
-  const uint64_t* __restrict__ row = adj + vsj + off + lane;
-#pragma unroll
-  for (int s = 0; s < U; s++) e[s] = (kAll || off + 32 * s + lane < dvj) ? row[32 * s] : 0ull;
-  if constexpr (V::kBatched) {
-    // all U probes first, then the visitor takes their hits together
-    bool hit[U];
-    uint32_t quw[U], qvw[U];
-#pragma unroll
-    for (int s = 0; s < U; s++) {
-      uint32_t puw = 0;
-      qvw[s] = adj_valbits(e[s]);
-      const bool f = table_find_warp<false>(t, adj_col(e[s]), quw[s], puw, sc);
-      hit[s] = (kAll || off + 32 * s + lane < dvj) && f;
-    }
-    vis.template steps<U>(hit, qj, quw, qvw);
-  } else {
-#pragma unroll
-    for (int s = 0; s < U; s++) {
-      const uint32_t i = off + 32 * s + lane;
-      uint32_t quw = 0, puw = 0;
-      const bool f = table_find_warp<V::kPos>(t, adj_col(e[s]), quw, puw, sc);
-      const bool hit = (kAll || i < dvj) && f;
-      if (kAll || off + 32 * s < dvj)
-        vis.step(hit, uj, vj, adj_col(e[s]), qj, quw, adj_valbits(e[s]), pj, puw, vsj + i);
-    }
+// ------------------------------------------------------------ tables
+
+// Bitmap of the list N>(x): a bit for every entry w, pre[word] = the list index
+// of the word's first entry, val[i] the edge value of entry i.  Words are
+// numbered by w >> 5 from the graph's first one, `w0`; the lookups use 32-bit
+// shared-memory addresses of the (possibly unbacked) word 0, which saves the
+// subtraction per probe.
+struct BitTable {
+  uint32_t* bits;   // all zero between tasks
+  uint16_t* pre;
+  uint32_t* val;
+  uint32_t w0;      // first word of the graph's range
+  uint32_t lo;      // first vertex of the graph's range
+  uint32_t rs;      // CSR position of the list
+  uint32_t abits, apre;  // shared addresses of words 0
+};
+#ifdef __CUDACC__
+// the table for a graph that starts at vertex `first`
+__device__ __forceinline__ void bit_table_graph(BitTable& t, uint32_t first) {
+  t.lo = first;
+  t.w0 = first >> 5;
+  t.abits = (uint32_t)__cvta_generic_to_shared(t.bits) - 4u * t.w0;
+  t.apre = (uint32_t)__cvta_generic_to_shared(t.pre) - 2u * t.w0;
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t at) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t lds16(uint32_t at) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(at) : "memory");
+  return v;
+}
+#endif
+__host__ __device__ inline uint32_t bit_words(uint32_t range) { return (range + 31) / 32 + 1; }  // any alignment of the first vertex
+__host__ __device__ inline size_t bit_table_bytes(uint32_t range, uint32_t len) {
+  const size_t w = bit_words(range);
+  return (w * 4 + (w * 2 + 3) / 4 * 4 + (size_t)len * 4 + 15) / 16 * 16;
+}
+__device__ __forceinline__ BitTable bit_table_at(char* base, uint32_t range, uint32_t len) {
+  const uint32_t w = bit_words(range);
+  BitTable t;
+  t.bits = (uint32_t*)base;
+  t.val = t.bits + w;
+  t.pre = (uint16_t*)(t.val + len);
+  t.rs = 0;
+  bit_table_graph(t, 0);
+  return t;
+}
+// entries i0, i0 + step, ... of the list into the table / out of it again
+__device__ __forceinline__ void bit_table_load(const BitTable& t, const uint64_t* __restrict__ adj, uint32_t len,
+                                               uint32_t i0, uint32_t step) {
+  for (uint32_t i = i0; i < len; i += step) {
+    const uint64_t e = adj[t.rs + i];
+    const uint32_t b = adj_col(e), w = (b >> 5) - t.w0;
+    atomicOr(&t.bits[w], 1u << (b & 31));
+    t.val[i] = adj_valbits(e);
+    if (i == 0 || (adj_col(adj[t.rs + i - 1]) >> 5) - t.w0 != w) t.pre[w] = (uint16_t)i;
   }
 }
+__device__ __forceinline__ void bit_table_clear(const BitTable& t, const uint64_t* __restrict__ adj, uint32_t len,
+                                                uint32_t i0, uint32_t step) {
+  for (uint32_t i = i0; i < len; i += step) t.bits[(adj_col(adj[t.rs + i]) >> 5) - t.w0] = 0;
+}
 
-// One warp probes the lists of up to 32 pairs (one per lane, `ok` lanes).
+// Membership of U entries and, for a queued hit, its table entry: the edge
+// value, CSR position and vertex.
+__device__ __forceinline__ uint32_t none(const BitTable& t) { return t.lo; }  // a vertex that may be probed
+template <int U>
+__device__ __forceinline__ void find(const BitTable& t, const uint64_t (&e)[U], const bool (&act)[U], bool (&hit)[U],
+                                     uint32_t (&slot)[U], Scratch*) {
+  uint32_t word[U];
+#pragma unroll
+  for (int i = 0; i < U; i++) {
+    slot[i] = adj_col(e[i]);
+    word[i] = lds32(t.abits + 4u * (slot[i] >> 5));
+  }
+#pragma unroll
+  for (int i = 0; i < U; i++) hit[i] = act[i] && ((word[i] >> (slot[i] & 31)) & 1u);
+}
+template <bool kPos>
+__device__ __forceinline__ void entry(const BitTable& t, uint32_t slot, uint32_t& val, uint32_t& pos, uint32_t& w) {
+  const uint32_t wi = slot >> 5;
+  const uint32_t at = lds16(t.apre + 2u * wi) + __popc(lds32(t.abits + 4u * wi) & ((1u << (slot & 31)) - 1u));
+  val = t.val[at];
+  pos = t.rs + at;
+  w = slot;
+}
+__device__ __forceinline__ uint32_t none(const Table&) { return 0; }
+template <int U>
+__device__ __forceinline__ void find(const Table& t, const uint64_t (&e)[U], const bool (&act)[U], bool (&hit)[U],
+                                     uint32_t (&slot)[U], Scratch* sc) {
+#pragma unroll
+  for (int i = 0; i < U; i++) {
+    const bool found = table_slot_warp(t, adj_col(e[i]), slot[i], sc);
+    hit[i] = act[i] && found;
+  }
+}
+template <bool kPos>
+__device__ __forceinline__ void entry(const Table& t, uint32_t slot, uint32_t& val, uint32_t& pos, uint32_t& w) {
+  val = t.val[slot];
+  pos = kPos ? t.pos[slot] : 0u;
+  w = t.key[slot];
+}
+
+// ------------------------------------------------------------ the queue of hits
+
+// A warp's queue of items (V::Item, 8 or 16 bytes, the table slot in x) and, if
+// V::kMore, one more word each.  Fewer than 32 are queued between steps; a
+// step adds at most 32 V::kU.  Appending is a predicated store per entry, with
+// no branch: most of the traversal's instructions are here.
 template <class V>
-__device__ __forceinline__ void probe_pairs(const TravArgs& a, V& vis, const Table& t, const Pair& pr) {
+struct Queue {
+  static constexpr int kCap = 32 + 32 * V::kU;
+  static constexpr uint32_t kItem = (uint32_t)sizeof(typename V::Item);
+  static constexpr int kBytes = kCap * (int)(kItem + (V::kMore ? 4 : 0));
+  typename V::Item* q;
+  uint32_t* more;
+  uint32_t base, end;  // shared addresses of the first item and past the last
+  __device__ explicit Queue(char* mem)
+      : q((typename V::Item*)mem), more((uint32_t*)(mem + kCap * kItem)),
+        base((uint32_t)__cvta_generic_to_shared(mem)), end(base) {}
+  __device__ __forceinline__ void append(bool hit, const typename V::Item& it, uint32_t extra, uint32_t lt) {
+    const unsigned m = __ballot_sync(kFull, hit);
+    const uint32_t at = end + kItem * __popc(m & lt);
+    if constexpr (kItem == 8)
+      asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.v2.u32 [%1], {%2, %3}; }" ::"r"((uint32_t)hit),
+                   "r"(at), "r"(it.x), "r"(it.y) : "memory");
+    else
+      asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.v4.u32 [%1], {%2, %3, %4, %5}; }" ::"r"(
+                       (uint32_t)hit),
+                   "r"(at), "r"(it.x), "r"(it.y), "r"(it.z), "r"(it.w) : "memory");
+    if constexpr (V::kMore)
+      if (hit) more[(at - base) / kItem] = extra;
+    end += kItem * __popc(m);
+  }
+  // the last `cnt` <= 32 queued triangles to the visitor (kWhole: cnt is 32)
+  template <bool kWhole, class T>
+  __device__ __forceinline__ void take(const T& t, V& vis, uint32_t x, uint32_t cnt) {
+    const uint32_t lane = lane_id();
+    end -= kItem * cnt;
+    const uint32_t first = (end - base) / kItem + lane;
+    const bool on = kWhole || lane < cnt;
+    typename V::Item it = {};
+    uint32_t extra = 0, val = 0, pos = 0, w = 0;
+    if (on) {
+      it = q[first];
+      if constexpr (V::kMore) extra = more[first];
+      entry<V::kPos>(t, it.x, val, pos, w);
+    }
+    __syncwarp();
+    vis.take(on, cnt, it, extra, x, val, pos, w);
+  }
+  template <class T>
+  __device__ __forceinline__ void take_full(const T& t, V& vis, uint32_t x) {
+    if (end - base >= 32 * kItem) {
+      __syncwarp();
+      do take<true>(t, vis, x, 32); while (end - base >= 32 * kItem);
+    }
+  }
+  template <class T>
+  __device__ __forceinline__ void take_all(const T& t, V& vis, uint32_t x) {
+    __syncwarp();
+    if (end != base) take<false>(t, vis, x, (end - base) / kItem);
+  }
+};
+
+// U entries of streamed lists per lane (act: this lane has one; a lane
+// without one passes an entry naming vertex none()): probed, the hits queued.
+// q, pe: value and CSR position of the pair edge, s: the row's position, pos:
+// of the entry.
+template <class V, class T, int U>
+__device__ __forceinline__ void probe(const T& t, V& vis, Queue<V>& queue, const uint64_t (&e)[U], const bool (&act)[U],
+                                      uint32_t x, const uint32_t (&s)[U], const uint32_t (&q)[U],
+                                      const uint32_t (&pe)[U], const uint32_t (&pos)[U], Scratch* sc) {
+  static_assert(U <= V::kU, "the queue has room for kU entries a lane");
+  bool hit[U];
+  uint32_t slot[U];
+  find<U>(t, e, act, hit, slot, sc);
+  const uint32_t lt = lanemask_lt();
+#pragma unroll
+  for (int i = 0; i < U; i++)
+    queue.append(hit[i], V::item(slot[i], q[i], adj_valbits(e[i]), s[i], pe[i], pos[i]), pos[i], lt);
+  queue.take_full(t, vis, x);
+}
+
+// The whole warp probes 32 U entries of one long list, U per lane, all loads
+// issued before the probes: `row` and `pos` are the lane's first entry and its
+// position, `left` the entries from lane 0's on.  kAll: all 32 U exist.
+template <class V, class T, int U, bool kAll>
+__device__ __forceinline__ void long_steps(const uint64_t* __restrict__ row, uint32_t pos0, uint32_t left, Scratch* sc,
+                                           V& vis, Queue<V>& queue, const T& t, int lane, uint32_t x, uint32_t sj,
+                                           uint32_t qj, uint32_t pj) {
+  uint64_t e[U];
+  bool act[U];
+  uint32_t s[U], q[U], pe[U], pos[U];
+#pragma unroll
+  for (int i = 0; i < U; i++) {
+    act[i] = kAll || 32 * i + lane < left;
+    e[i] = act[i] ? row[32 * i] : (uint64_t)none(t);
+    pos[i] = pos0 + 32 * i;
+    s[i] = sj;
+    q[i] = qj;
+    pe[i] = pj;
+  }
+  probe<V, T, U>(t, vis, queue, e, act, x, s, q, pe, pos, sc);
+}
+
+// One warp probes the lists of up to 32 pairs (one per lane; empty ones have dv = 0).
+template <class V, class T>
+__device__ __forceinline__ void probe_pairs(const TravArgs& a, V& vis, Queue<V>& queue, const T& t, const Pair& pr) {
   const int lane = (int)lane_id();
   const uint64_t* __restrict__ adj = a.adj;
   Scratch* const sc = a.sc;
-  uint32_t vs = 0, dv = 0;
-  if (pr.ok) {
-    if (pr.s < a.n) {
-      vs = a.row_ptr[pr.s];
-      const uint32_t ve = a.row_ptr[pr.s + 1];
-      if (ve >= vs && ve <= a.m) {
-        dv = ve - vs;
-        if (a.L > 0 && !a.light_prune) dv = prune_prefix(a.adj + vs, dv, qabs(pr.qe) * pr.qmax, a.L);
-      } else {
-        guard_fail(a.sc, kGuardList, pr.s);
-      }
-    } else {
-      guard_fail(a.sc, kGuardVertex, pr.s);
-    }
-  }
-  // long lists: one at a time, the whole warp streams it, up to four entries per lane
+  uint32_t vs = pr.vs, dv = pr.dv;
+  // long lists: one at a time, the whole warp streams it, V::kU entries per lane
   const uint32_t kLong = a.long_min;
   const bool tail_short = a.long_tail != 0;
   const bool was_long = dv >= kLong;
@@ -350,36 +502,35 @@ __device__ __forceinline__ void probe_pairs(const TravArgs& a, V& vis, const Tab
   while (longm) {
     const int j = __ffs(longm) - 1;
     longm &= longm - 1;
-    const uint32_t uj = __shfl_sync(kFull, pr.x, j);
-    const uint32_t vj = __shfl_sync(kFull, pr.s, j);
+    const uint32_t sj = __shfl_sync(kFull, pr.s, j);
     const uint32_t vsj = __shfl_sync(kFull, vs, j);
     const uint32_t dvj = __shfl_sync(kFull, dv, j);
     if constexpr (HasProbed<V>::value) probed += dvj;
     const uint32_t qj = __shfl_sync(kFull, pr.qe, j);
     const uint32_t pj = __shfl_sync(kFull, pr.pe, j);
-    uint32_t off = 0;
-    while (dvj - off >= 32 * UBT_LONG_U) {
-      long_steps<V, UBT_LONG_U, true>(adj, sc, vis, t, lane, uj, vj, vsj, dvj, qj, pj, off);
-      off += 32 * UBT_LONG_U;
-    }
-    if (UBT_LONG_U > 4 && dvj - off >= 128) {
-      long_steps<V, 4, true>(adj, sc, vis, t, lane, uj, vj, vsj, dvj, qj, pj, off);
-      off += 128;
+    uint32_t left = dvj, pos = vsj + lane;
+    const uint64_t* __restrict__ row = adj + vsj + lane;
+    while (left >= 32 * V::kU) {
+      long_steps<V, T, V::kU, true>(row, pos, left, sc, vis, queue, t, lane, pr.x, sj, qj, pj);
+      row += 32 * V::kU;
+      pos += 32 * V::kU;
+      left -= 32 * V::kU;
     }
     if (tail_short) {
       // full half-chunk, then the rest (< 64 entries) is streamed with the short lists
-      if (dvj - off >= 64) {
-        long_steps<V, 2, true>(adj, sc, vis, t, lane, uj, vj, vsj, dvj, qj, pj, off);
-        off += 64;
+      if (V::kU > 2 && left >= 64) {
+        long_steps<V, T, 2, true>(row, pos, left, sc, vis, queue, t, lane, pr.x, sj, qj, pj);
+        left -= 64;
       }
       if (lane == j) {
-        vs += off;
-        dv -= off;
+        vs += dvj - left;
+        dv = left;
       }
     } else {
-      while (off < dvj) {
-        long_steps<V, 2, false>(adj, sc, vis, t, lane, uj, vj, vsj, dvj, qj, pj, off);
-        off += 64;
+      for (; left; left -= min(left, 64u)) {
+        long_steps<V, T, 2, false>(row, pos, left, sc, vis, queue, t, lane, pr.x, sj, qj, pj);
+        row += 64;
+        pos += 64;
       }
     }
   }
@@ -392,76 +543,82 @@ __device__ __forceinline__ void probe_pairs(const TravArgs& a, V& vis, const Tab
     if (lane >= d) incl += y;
   }
   const uint32_t total = __shfl_sync(kFull, incl, 31);
-  const uint32_t excl = incl - ds;
+  const uint32_t base_pos = vs - (incl - ds);  // position of entry f of the concatenation: base_pos + f
   for (uint32_t base = 0; base < total; base += 64) {
-    uint32_t f[2], jj[2];
-    bool act[2];
     uint64_t e[2];
+    bool act[2];
+    uint32_t sv[2], q[2], pe[2], pos[2];
 #pragma unroll
-    for (int s = 0; s < 2; s++) {
-      f[s] = base + 32 * s + lane;
-      act[s] = f[s] < total;
+    for (int i = 0; i < 2; i++) {
+      const uint32_t f = base + 32 * i + lane;
+      act[i] = f < total;
       // owner: number of lanes whose inclusive end is <= f
       int j = 0;
 #pragma unroll
       for (int b = 16; b > 0; b >>= 1) {
         const uint32_t tj = __shfl_sync(kFull, incl, j + b - 1);
-        if (tj <= f[s]) j += b;
+        if (tj <= f) j += b;
       }
-      jj[s] = (uint32_t)(j > 31 ? 31 : j);
-      const uint32_t vsj = __shfl_sync(kFull, vs, jj[s]);
-      const uint32_t exj = __shfl_sync(kFull, excl, jj[s]);
-      e[s] = act[s] ? adj[vsj + (f[s] - exj)] : 0ull;
-      f[s] = vsj + (f[s] - exj);  // now the CSR position of the entry
+      j = j > 31 ? 31 : j;
+      pos[i] = __shfl_sync(kFull, base_pos, j) + f;
+      e[i] = act[i] ? adj[pos[i]] : (uint64_t)none(t);
+      sv[i] = __shfl_sync(kFull, pr.s, j);
+      q[i] = __shfl_sync(kFull, pr.qe, j);
+      pe[i] = __shfl_sync(kFull, pr.pe, j);
     }
-#pragma unroll
-    for (int s = 0; s < 2; s++) {
-      const int j = (int)jj[s];
-      uint32_t quw = 0, puw = 0;
-      const bool found = table_find_warp<V::kPos>(t, adj_col(e[s]), quw, puw, sc);
-      const bool hit = act[s] && found;
-      const uint32_t uj = __shfl_sync(kFull, pr.x, j);
-      const uint32_t vj = __shfl_sync(kFull, pr.s, j);
-      const uint32_t qj = __shfl_sync(kFull, pr.qe, j);
-      const uint32_t pj = __shfl_sync(kFull, pr.pe, j);
-      if (s == 0 || base + 32 < total)
-        vis.step(hit, uj, vj, adj_col(e[s]), qj, quw, adj_valbits(e[s]), pj, puw, f[s]);
-    }
+    probe<V, T, 2>(t, vis, queue, e, act, pr.x, sv, q, pe, pos, sc);
   }
   // a long list's tail streamed with the short lists is counted twice: an upper bound
   if constexpr (HasProbed<V>::value) vis.probed(probed + total);
 }
 
-// This lane's pair among the pairs [ps, ps + cnt) of owner x.  A pair whose
-// edge fails Lemma 2 (|q_e| 2^30 < L) cannot be in a classified triangle.
-__device__ __forceinline__ Pair owner_pair(const TravArgs& a, uint32_t x, int64_t qmax, uint32_t ps, uint32_t cnt) {
+// This lane's pair among the pairs [ps, ps + cnt) of owner x.  The pair edge's
+// entry is the one right after its streamed entries.
+__device__ __forceinline__ Pair owner_pair(const TravArgs& a, uint32_t x, uint32_t ps, uint32_t cnt) {
   const int lane = (int)lane_id();
   Pair pr;
   pr.x = x;
-  pr.qmax = qmax;
-  pr.ok = (uint32_t)lane < cnt;
-  const uint64_t d = pr.ok ? a.pairs[ps + lane] : 0ull;
-  pr.s = (uint32_t)d;
-  pr.pe = (uint32_t)(d >> 32);
-  if (pr.ok && pr.pe >= a.m) {
+  pr.qe = 0;
+  const uint64_t d = (uint32_t)lane < cnt ? a.pairs[ps + lane] : 0ull;
+  bool ok = (uint32_t)lane < cnt && pair_absq2(d) >= a.qmin2;
+  pr.vs = pair_start(d);
+  pr.dv = pair_len(d);
+  pr.s = pr.pe = pr.vs + pr.dv;
+  if (ok && (pr.pe >= a.m || pr.pe < pr.vs)) {
     guard_fail(a.sc, kGuardList, x);
-    pr.ok = false;
+    ok = false;
   }
-  const uint64_t e = pr.ok ? a.adj[pr.pe] : 0ull;
-  pr.qe = adj_valbits(e);
-  if (a.L > 0 && qabs(pr.qe) * (1ll << 30) < a.L) pr.ok = false;
+  if (ok && a.keep) {
+    pr.vs = a.keep[pr.vs];
+    const uint32_t pe = a.keep[pr.pe];
+    ok = a.keep[pr.pe + 1] > pe;  // the pair edge is kept
+    pr.dv = pe - pr.vs;
+    pr.pe = pe;
+  }
+  if (!ok) pr.dv = 0;
+  if (pr.dv) {
+    const uint64_t e = a.adj[pr.pe];
+    pr.qe = adj_valbits(e);
+    if (adj_col(e) != x) {
+      guard_fail(a.sc, kGuardVertex, x);
+      pr.dv = 0;
+    }
+  }
   return pr;
 }
 
-// Entries of x's list that go into its table (the Lemma 2 prefix) and qmax(x);
-// identical in every calling thread.
-__device__ __forceinline__ uint32_t table_len(const TravArgs& a, uint32_t rs, uint32_t len, int64_t& qmax) {
-  qmax = 0;
-  if (a.L > 0 && len > 0) {
-    qmax = qabs(adj_valbits(a.adj[rs]));
-    return prune_prefix(a.adj + rs, len, 1ll << 30, a.L);
+// Owner x's list: entries [rs, rs + len) of adj; false if the offsets are out of order.
+__device__ __forceinline__ bool owner_list(const TravArgs& a, uint32_t x, uint32_t& rs, uint32_t& len) {
+  rs = a.row_ptr[x];
+  uint32_t re = a.row_ptr[x + 1];
+  if (re < rs || re > a.m) return false;
+  if (a.keep) {
+    rs = a.keep[rs];
+    re = a.keep[re];
+    if (re < rs || re > a.m) return false;
   }
-  return len;
+  len = re - rs;
+  return true;
 }
 
 // Pair range of owner x, checked against the pair array's bounds.
@@ -473,31 +630,73 @@ __device__ __forceinline__ bool pair_range(const TravArgs& a, uint32_t x, uint32
   return true;
 }
 
-// A whole block handles owner x; `tab` is shared memory (hub) or a global
-// slice (giant).
-template <class V>
-__device__ __forceinline__ void block_task(const TravArgs& a, V& vis, uint32_t x, uint32_t* tab, uint32_t cap,
-                                           uint32_t* s_misc) {
-  const int tid = threadIdx.x, lane = tid & 31;
+// ------------------------------------------------------------ tasks
+
+// The pairs [ps, ps + np) of owner x by a whole block whose table is loaded:
+// warps take pairs `unit` at a time, fewer as the pairs run out, so that they
+// reach the closing barrier at about the same time.
+template <class V, class T>
+__device__ __forceinline__ void block_pairs(const TravArgs& a, V& vis, Queue<V>& queue, const T& t, uint32_t x,
+                                            uint32_t ps, uint32_t np, uint32_t* s_misc) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t nw = blockDim.x >> 5;
+  vis.task_begin(x);
+  while (true) {
+    uint32_t c = 0, cnt = 0;
+    if (lane == 0) {
+      const uint32_t seen = *(volatile uint32_t*)&s_misc[1];
+      const uint32_t rem = seen < np ? np - seen : 0u;
+      const uint32_t want = min(a.unit, max(8u, rem / (2 * nw)));
+      c = atomicAdd(&s_misc[1], want);
+      cnt = c < np ? min(want, np - c) : 0u;
+    }
+    c = __shfl_sync(kFull, c, 0);
+    cnt = __shfl_sync(kFull, cnt, 0);
+    if (cnt == 0) break;
+    probe_pairs<V, T>(a, vis, queue, t, owner_pair(a, x, ps + c, cnt));
+  }
+  queue.take_all(t, vis, x);
+  vis.task_end(x);
+}
+
+// Owner x's list and pairs; false: nothing to do (or a failed self-check).
+__device__ __forceinline__ bool owner_task(const TravArgs& a, uint32_t x, uint32_t& rs, uint32_t& len, uint32_t& ps,
+                                           uint32_t& np, bool report) {
   if (x >= a.n) {
-    if (tid == 0) guard_fail(a.sc, kGuardVertex, x);
-    return;
+    if (report) guard_fail(a.sc, kGuardVertex, x);
+    return false;
   }
-  const uint32_t rs = a.row_ptr[x], re = a.row_ptr[x + 1];
-  uint32_t ps = 0, np = 0;
-  if (re < rs || re > a.m || !pair_range(a, x, ps, np)) {
-    if (tid == 0) guard_fail(a.sc, kGuardList, x);
-    return;
+  if (!owner_list(a, x, rs, len) || !pair_range(a, x, ps, np)) {
+    if (report) guard_fail(a.sc, kGuardList, x);
+    return false;
   }
-  int64_t qmax = 0;
-  if (tid == 0) s_misc[0] = table_len(a, rs, re - rs, qmax);
-  __syncthreads();
-  const uint32_t len = s_misc[0];
-  if (a.L > 0 && len > 0) qmax = qabs(adj_valbits(a.adj[rs]));
+  return len > 0 && np > 0;
+}
+// A block task's share of its owner's pairs: part / parts of them.
+__device__ __forceinline__ void task_part(uint64_t task, uint32_t& ps, uint32_t& np) {
+  const uint32_t part = (uint32_t)(task >> 32) & 0xFFFFu, parts = (uint32_t)(task >> 48) + 1u;
+  const uint32_t p0 = (uint32_t)((uint64_t)np * part / parts), p1 = (uint32_t)((uint64_t)np * (part + 1) / parts);
+  ps += p0;
+  np = p1 - p0;
+}
+// first vertex of x's graph
+__device__ __forceinline__ uint32_t graph_start(const TravArgs& a, uint32_t x) {
+  return a.gstart ? a.gstart[a.vgraph[x]] : 0u;
+}
+
+// A whole block handles (a part of) owner x with a hash table in `tab`: shared
+// memory (hub) or a global slice (giant).
+template <class V>
+__device__ __forceinline__ void block_task_hash(const TravArgs& a, V& vis, Queue<V>& queue, uint64_t task,
+                                                uint32_t* tab, uint32_t cap, uint32_t* s_misc) {
+  const int tid = threadIdx.x;
+  const uint32_t x = (uint32_t)task;
+  uint32_t rs = 0, len = 0, ps = 0, np = 0;
+  if (!owner_task(a, x, rs, len, ps, np, tid == 0)) return;
+  task_part(task, ps, np);
   const uint32_t slots = slots_for(len);
-  if (len == 0 || np == 0 || slots > cap) {
-    if (len && np && slots > cap && tid == 0) guard_fail(a.sc, kGuardTable, x);
-    __syncthreads();
+  if (slots > cap) {
+    if (tid == 0) guard_fail(a.sc, kGuardTable, x);
     return;
   }
   const Table t = make_table(tab, cap, slots);
@@ -509,45 +708,38 @@ __device__ __forceinline__ void block_task(const TravArgs& a, V& vis, uint32_t x
     table_insert<V::kPos>(t, adj_col(e), adj_valbits(e), rs + i, a.sc);
   }
   __syncthreads();
-  vis.task_begin(x);
-  // warps take pairs `unit` at a time, fewer as the pairs run out, so that
-  // they reach the closing barrier at about the same time
-  const uint32_t nw = blockDim.x >> 5;
-  while (true) {
-    uint32_t c = 0, cnt = 0;
-    if (lane == 0) {
-      const uint32_t seen = *(volatile uint32_t*)&s_misc[1];
-      const uint32_t rem = seen < np ? np - seen : 0u;
-      const uint32_t want = max(1u, min(a.unit, rem / (2 * nw)));
-      c = atomicAdd(&s_misc[1], want);
-      cnt = c < np ? min(want, np - c) : 0u;
-    }
-    c = __shfl_sync(kFull, c, 0);
-    cnt = __shfl_sync(kFull, cnt, 0);
-    if (cnt == 0) break;
-    probe_pairs<V>(a, vis, t, owner_pair(a, x, qmax, ps + c, cnt));
-  }
-  vis.task_end(x);
+  block_pairs<V, Table>(a, vis, queue, t, x, ps, np, s_misc);
   __syncthreads();
 }
 
-// One warp handles owner x.
+// The same with a bitmap table.
 template <class V>
-__device__ __forceinline__ void warp_task(const TravArgs& a, V& vis, uint32_t x, uint32_t* tab) {
+__device__ __forceinline__ void block_task_bits(const TravArgs& a, V& vis, Queue<V>& queue, uint64_t task, BitTable t,
+                                                uint32_t* s_misc) {
+  const int tid = threadIdx.x;
+  const uint32_t x = (uint32_t)task;
+  uint32_t len = 0, ps = 0, np = 0;
+  if (!owner_task(a, x, t.rs, len, ps, np, tid == 0)) return;
+  task_part(task, ps, np);
+  bit_table_graph(t, graph_start(a, x));
+  if (x - t.lo > a.hub_bits || len > a.hub_len) {
+    if (tid == 0) guard_fail(a.sc, kGuardTable, x);
+    return;
+  }
+  if (tid == 0) s_misc[1] = 0;
+  bit_table_load(t, a.adj, len, tid, blockDim.x);
+  __syncthreads();
+  block_pairs<V, BitTable>(a, vis, queue, t, x, ps, np, s_misc);
+  __syncthreads();
+  bit_table_clear(t, a.adj, len, tid, blockDim.x);  // the next task's first barrier orders it
+}
+
+// One warp handles owner x with its own table.
+template <class V>
+__device__ __forceinline__ void warp_task_hash(const TravArgs& a, V& vis, Queue<V>& queue, uint32_t x, uint32_t* tab) {
   const int lane = (int)lane_id();
-  if (x >= a.n) {
-    if (lane == 0) guard_fail(a.sc, kGuardVertex, x);
-    return;
-  }
-  const uint32_t rs = a.row_ptr[x], re = a.row_ptr[x + 1];
-  uint32_t ps = 0, np = 0;
-  if (re < rs || re > a.m || !pair_range(a, x, ps, np)) {
-    if (lane == 0) guard_fail(a.sc, kGuardList, x);
-    return;
-  }
-  int64_t qmax = 0;
-  const uint32_t len = table_len(a, rs, re - rs, qmax);
-  if (len == 0 || np == 0) return;
+  uint32_t rs = 0, len = 0, ps = 0, np = 0;
+  if (!owner_task(a, x, rs, len, ps, np, lane == 0)) return;
   const uint32_t slots = slots_for(len);
   if (slots > a.warp_slots) {
     if (lane == 0) guard_fail(a.sc, kGuardTable, x);
@@ -563,126 +755,193 @@ __device__ __forceinline__ void warp_task(const TravArgs& a, V& vis, uint32_t x,
   __syncwarp();
   vis.task_begin(x);
   for (uint32_t cs = 0; cs < np; cs += 32)
-    probe_pairs<V>(a, vis, t, owner_pair(a, x, qmax, ps + cs, min(32u, np - cs)));
+    probe_pairs<V, Table>(a, vis, queue, t, owner_pair(a, x, ps + cs, min(32u, np - cs)));
+  queue.take_all(t, vis, x);
   vis.task_end(x);
   __syncwarp();
 }
-
-// The traversal runs as two persistent kernels, so that each can have the
-// block size and shared memory its tasks need: the block kernel (giant and
-// hub tasks, one large table per block) and the warp kernel (medium tasks,
-// one small table per warp).
-enum : int { kBlockTasks = 1, kWarpTasks = 2 };
-
-// Persistent traversal kernel body.  Shared memory: [visitor bytes][tables].
-template <class V, int kPhases>
-__device__ void traverse(const TravArgs& a, V& vis, char* smem_tables) {
-  __shared__ uint32_t s_misc[4];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  uint32_t* tab = (uint32_t*)smem_tables;
-  if (kPhases & kBlockTasks) {
-    // giant lists, tables in global memory (first gtab_blocks blocks)
-    if (blockIdx.x < a.gtab_blocks) {
-      uint32_t* gt = a.gtab + (size_t)blockIdx.x * a.gtab_slots * 3;
-      while (true) {
-        if (tid == 0) s_misc[2] = (uint32_t)atomicAdd(&a.sc->task[0], 1ull);
-        __syncthreads();
-        const uint32_t task = s_misc[2];
-        __syncthreads();
-        if (task >= a.n_giant) break;
-        block_task(a, vis, a.giant_list[task], gt, a.gtab_slots, s_misc);
-      }
-    }
-    // hub lists, block-wide shared-memory tables
-    while (true) {
-      if (tid == 0) s_misc[2] = (uint32_t)atomicAdd(&a.sc->task[1], 1ull);
-      __syncthreads();
-      const uint32_t task = s_misc[2];
-      __syncthreads();
-      if (task >= a.n_hub) break;
-      block_task(a, vis, a.hub_list[task], tab, a.hub_slots, s_misc);
-    }
+template <class V>
+__device__ __forceinline__ void warp_task_bits(const TravArgs& a, V& vis, Queue<V>& queue, uint32_t x, BitTable t) {
+  const int lane = (int)lane_id();
+  uint32_t len = 0, ps = 0, np = 0;
+  if (!owner_task(a, x, t.rs, len, ps, np, lane == 0)) return;
+  bit_table_graph(t, graph_start(a, x));
+  if (x - t.lo > a.warp_bits || len > a.warp_len) {
+    if (lane == 0) guard_fail(a.sc, kGuardTable, x);
+    return;
   }
-  if (kPhases & kWarpTasks) {
-    uint32_t* wtab = tab + (size_t)wid * table_words<V>(a.warp_slots);
-    // medium tasks, one warp each
+  bit_table_load(t, a.adj, len, lane, 32);
+  __syncwarp();
+  vis.task_begin(x);
+  for (uint32_t cs = 0; cs < np; cs += 32)
+    probe_pairs<V, BitTable>(a, vis, queue, t, owner_pair(a, x, ps + cs, min(32u, np - cs)));
+  queue.take_all(t, vis, x);
+  vis.task_end(x);
+  __syncwarp();
+  bit_table_clear(t, a.adj, len, lane, 32);
+  __syncwarp();
+}
+
+// The traversal runs as up to two persistent kernels: the rare block tasks
+// with hash tables, and everything else -- the block tasks with bitmaps, then
+// the warp tasks -- in one, so that a block that finds no more block tasks goes
+// on to warp tasks instead of idling until the last one ends.
+enum : int { kHashKernel = 0, kMainKernel = 1 };
+
+template <class V>
+__host__ __device__ inline size_t warp_table_bytes(const TravArgs& a) {
+  const size_t h = a.n_tasks[kMedHash] ? (size_t)table_words<V>(a.warp_slots) * 4 : 0;
+  const size_t b = a.n_tasks[kMedBits] ? bit_table_bytes(a.warp_bits, a.warp_len) : 0;
+  return h > b ? h : b;
+}
+// Shared memory of a block's tables.
+template <class V>
+inline size_t traverse_table_bytes(const TravArgs& a, int kernel, int threads) {
+  if (kernel == kHashKernel) return a.n_tasks[kHubHash] ? (size_t)table_words<V>(a.hub_slots) * 4 : 0;
+  const size_t hub = a.n_tasks[kHubBits] ? bit_table_bytes(a.hub_bits, a.hub_len) : 0;
+  return std::max(hub, (size_t)(threads / 32) * warp_table_bytes<V>(a));
+}
+template <class V>
+__host__ __device__ inline size_t visitor_bytes(int threads) {
+  return (size_t)((V::smem_bytes(threads) + 15) / 16) * 16 + (size_t)(threads / 32) * Queue<V>::kBytes;
+}
+
+// The next block task of a class (the same in every thread); n_tasks if none.
+__device__ __forceinline__ uint32_t next_block_task(const TravArgs& a, int cls, uint32_t* s_misc) {
+  if (threadIdx.x == 0) s_misc[2] = (uint32_t)atomicAdd(&a.sc->task[cls], 1ull);
+  __syncthreads();
+  const uint32_t task = s_misc[2];
+  __syncthreads();
+  return task;
+}
+
+// Warp tasks [0, n) of a class, the first eighth (the heaviest) one at a time,
+// the others `batch` at a time, from two counters.
+template <class F>
+__device__ __forceinline__ void warp_tasks(const TravArgs& a, int cls, F&& run) {
+  const uint32_t n = a.n_tasks[cls], first = n / 8;
+  for (int light = 0; light < 2; light++) {
+    const uint32_t step = light ? a.batch : 1u, end = light ? n : first;
+    unsigned long long* ctr = &a.sc->task[cls == kMedBits ? (light ? 6 : 4) : (light ? 5 : 3)];
     while (true) {
       unsigned long long t0 = 0;
-      if (lane == 0) t0 = atomicAdd(&a.sc->task[2], (unsigned long long)a.batch);
-      t0 = __shfl_sync(kFull, t0, 0);
-      if (t0 >= a.n_med) break;
-      const uint32_t t1 = (uint32_t)min((unsigned long long)a.n_med, t0 + a.batch);
-      for (uint32_t t = (uint32_t)t0; t < t1; t++) warp_task(a, vis, a.med_list[t], wtab);
+      if (lane_id() == 0) t0 = atomicAdd(ctr, (unsigned long long)step);
+      t0 = __shfl_sync(kFull, t0, 0) + (light ? first : 0u);
+      if (t0 >= end) break;
+      const uint32_t t1 = (uint32_t)min((unsigned long long)end, t0 + step);
+      for (uint32_t t = (uint32_t)t0; t < t1; t++) run((uint32_t)a.lists[cls][t]);
     }
+  }
+}
+
+template <class V, int kKernel>
+__device__ void traverse(const TravArgs& a, V& vis, char* queues, char* tables) {
+  __shared__ uint32_t s_misc[4];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  Queue<V> queue(queues + (size_t)wid * Queue<V>::kBytes);
+  if constexpr (kKernel == kHashKernel) {
+    while (blockIdx.x < a.gtab_blocks) {
+      const uint32_t task = next_block_task(a, kGiant, s_misc);
+      if (task >= a.n_tasks[kGiant]) break;
+      block_task_hash(a, vis, queue, a.lists[kGiant][task], a.gtab + (size_t)blockIdx.x * a.gtab_slots * 3,
+                      a.gtab_slots, s_misc);
+    }
+    while (true) {
+      const uint32_t task = next_block_task(a, kHubHash, s_misc);
+      if (task >= a.n_tasks[kHubHash]) break;
+      block_task_hash(a, vis, queue, a.lists[kHubHash][task], (uint32_t*)tables, a.hub_slots, s_misc);
+    }
+  } else {
+    if (a.n_tasks[kHubBits]) {
+      const BitTable bt = bit_table_at(tables, a.hub_bits, a.hub_len);
+      for (uint32_t i = tid; i < bit_words(a.hub_bits); i += blockDim.x) bt.bits[i] = 0;
+      while (true) {
+        const uint32_t task = next_block_task(a, kHubBits, s_misc);
+        if (task >= a.n_tasks[kHubBits]) break;
+        block_task_bits(a, vis, queue, a.lists[kHubBits][task], bt, s_misc);
+      }
+    }
+    char* mine = tables + (size_t)wid * warp_table_bytes<V>(a);
+    if (a.n_tasks[kMedBits]) {
+      const BitTable bt = bit_table_at(mine, a.warp_bits, a.warp_len);
+      for (uint32_t i = lane; i < bit_words(a.warp_bits); i += 32) bt.bits[i] = 0;
+      __syncwarp();
+      warp_tasks(a, kMedBits, [&](uint32_t x) { warp_task_bits(a, vis, queue, x, bt); });
+      __syncwarp();
+    }
+    if (a.n_tasks[kMedHash])
+      warp_tasks(a, kMedHash, [&](uint32_t x) { warp_task_hash(a, vis, queue, x, (uint32_t*)mine); });
   }
   __syncthreads();
   vis.block_end();
 }
 
-// Shared memory of one block of a traversal kernel: visitor bytes + tables
-// (words 32-bit words per table slot).
-template <class V>
-inline size_t traverse_smem_bytes(const TravArgs& a, int phases, int threads) {
-  const size_t vis_bytes = (size_t)((V::smem_bytes(threads) + 15) / 16) * 16;
-  size_t tables = 0;
-  if (phases & kBlockTasks) tables = std::max(tables, (size_t)table_words<V>(a.hub_slots) * 4);
-  if (phases & kWarpTasks) tables = std::max(tables, (size_t)(threads / 32) * table_words<V>(a.warp_slots) * 4);
-  return vis_bytes + tables;
-}
-
 namespace {
 
-// Launch bounds per kernel: the block kernel runs 512-thread blocks, the warp
-// kernel 128-thread blocks, and a visitor's register cap (V::kRegCap) sets how
-// many of them must fit on one SM (65536 registers).
-template <class V, int kPhases>
+// Launch bounds per kernel: at most kThreads threads a block; a visitor's
+// register cap (V::kRegCap) sets how many blocks must fit on one SM (65536
+// registers).
+template <class V, int kKernel>
 struct Bounds {
-  static constexpr int kThreads = (kPhases & kBlockTasks) ? UBT_LB_THREADS : 128;
+  static constexpr int kThreads = 512;
   static constexpr int kMinBlocks = 65536 / (kThreads * V::kRegCap) > 0 ? 65536 / (kThreads * V::kRegCap) : 1;
 };
 
-template <class V, int kPhases>
-__global__ void __launch_bounds__(Bounds<V, kPhases>::kThreads, Bounds<V, kPhases>::kMinBlocks)
+template <class V, int kKernel>
+__global__ void __launch_bounds__(Bounds<V, kKernel>::kThreads, Bounds<V, kKernel>::kMinBlocks)
     k_traverse(TravArgs a, typename V::P p) {
   extern __shared__ __align__(16) char smem[];
   V vis(p, smem);
   vis.block_init();
   __syncthreads();
-  traverse<V, kPhases>(a, vis, smem + ((V::smem_bytes((int)blockDim.x) + 15) / 16) * 16);
+  char* queues = smem + ((V::smem_bytes((int)blockDim.x) + 15) / 16) * 16;
+  traverse<V, kKernel>(a, vis, queues, smem + visitor_bytes<V>((int)blockDim.x));
 }
 
-template <class V, int kPhases>
-ubt_status launch_phase(const ubt_graph* g, const TravArgs& a, const typename V::P& p, int threads, cudaStream_t s) {
+// Warps of a kernel that fit on an SM: by registers (65536) and shared memory
+// (227 KB, 1 KB of it per block taken by the system).
+template <class V, int kKernel>
+int resident_warps(const TravArgs& a, int threads) {
+  const size_t smem = visitor_bytes<V>(threads) + traverse_table_bytes<V>(a, kKernel, threads) + 1024;
+  const int blocks = (int)std::min<size_t>((227 * 1024 + 1024) / smem, 65536 / (size_t)(threads * V::kRegCap));
+  return blocks * threads / 32;
+}
+
+template <class V, int kKernel>
+ubt_status launch_kernel(const ubt_graph* g, const TravArgs& a, const typename V::P& p, cudaStream_t s) {
   const Tuning& T = tuning();
-  threads = (int)std::min<int64_t>(Bounds<V, kPhases>::kThreads, std::max<int64_t>(64, threads / 32 * 32));
-  const size_t smem = traverse_smem_bytes<V>(a, kPhases, threads);
-  UBT_CUDA(cudaFuncSetAttribute(k_traverse<V, kPhases>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int threads = (int)(kKernel == kHashKernel ? T.block_threads : T.warp_threads);
+  threads = (int)std::min<int64_t>(Bounds<V, kKernel>::kThreads, std::max<int64_t>(64, threads / 32 * 32));
+  // Larger blocks share the block tasks' table among more warps; smaller ones
+  // lose less at its barriers.  Twice the threads where the table's size would
+  // otherwise leave fewer than 7/8 of the warps they make room for (R-MAT scale
+  // 22, tables of 26 KB: 19.8 -> 17.0 ms with 256 threads; Chung-Lu of 1e6
+  // vertices, tables of 4 KB: 1.15 ms with 128, 1.21 with 256).
+  if (kKernel == kMainKernel && 2 * threads <= Bounds<V, kKernel>::kThreads &&
+      8 * resident_warps<V, kKernel>(a, threads) < 7 * resident_warps<V, kKernel>(a, 2 * threads))
+    threads *= 2;
+  const size_t smem = visitor_bytes<V>(threads) + traverse_table_bytes<V>(a, kKernel, threads);
+  UBT_CUDA(cudaFuncSetAttribute(k_traverse<V, kKernel>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse<V, kPhases>, threads, smem));
+  UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse<V, kKernel>, threads, smem));
   if (per_sm < 1) return UBT_ERR_INVALID_ARG;
   per_sm = (int)std::min<int64_t>(per_sm, std::max<int64_t>(1, T.blocks_per_sm));
-  k_traverse<V, kPhases><<<g->sm_count * per_sm, threads, smem, s>>>(a, p);
+  k_traverse<V, kKernel><<<g->sm_count * per_sm, threads, smem, s>>>(a, p);
   UBT_CUDA(cudaGetLastError());
   return UBT_OK;
 }
 
-// One traversal: the task counters in a.sc are cleared, then the block kernel
-// (if the graph has giant or hub lists) and the warp kernel (if it has medium
-// tasks) run one after the other on `s`.
+// One traversal: the task counters in a.sc are cleared, then the kernels that
+// have tasks run one after the other on `s`.
 template <class V>
 ubt_status launch_traversal(const ubt_graph* g, const TravArgs& a, const typename V::P& p, cudaStream_t s) {
   UBT_RANGE("traversal launch");
-  const Tuning& T = tuning();
-  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchHeader / 2, s));
-  if (a.n_giant + a.n_hub > 0) {
-    const ubt_status st = launch_phase<V, kBlockTasks>(g, a, p, (int)T.block_threads, s);
-    if (st != UBT_OK) return st;
-  }
-  if (a.n_med > 0) {
-    const ubt_status st = launch_phase<V, kWarpTasks>(g, a, p, (int)T.warp_threads, s);
-    if (st != UBT_OK) return st;
-  }
-  return UBT_OK;
+  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
+  ubt_status st = UBT_OK;
+  if (a.n_tasks[kGiant] + a.n_tasks[kHubHash]) st = launch_kernel<V, kHashKernel>(g, a, p, s);
+  if (st == UBT_OK && a.n_tasks[kHubBits] + a.n_tasks[kMedHash] + a.n_tasks[kMedBits])
+    st = launch_kernel<V, kMainKernel>(g, a, p, s);
+  return st;
 }
 
 }  // namespace

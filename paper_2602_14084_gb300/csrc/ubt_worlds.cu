@@ -22,7 +22,7 @@
 
 namespace ubt {
 
-TravArgs make_trav_args(const ubt_graph* g, int64_t L, bool with_pos);
+ubt_status make_trav_args(const ubt_graph* g, int64_t L, cudaStream_t s, TravArgs* out);
 
 namespace {
 
@@ -152,22 +152,22 @@ template <int SLOTS>
 struct Worlds {
   using P = WorldsP;
   static constexpr bool kPos = true;
-  static constexpr bool kBatched = false;
+  using Item = uint4;  // table slot, positions of the pair edge and the streamed edge
+  static constexpr bool kMore = false;
+  static constexpr int kU = 2;
   static constexpr int kRegCap = 128;
   static constexpr int K = SLOTS == 1 ? 14 : 12;      // planes per slot
   static constexpr uint32_t kLimit = (1u << K) - 1u;  // increments before a flush
-  static constexpr int kQueue = 64;
-  // counters + one queue per warp
-  static __host__ __device__ int smem_bytes(int threads) { return 64 * 64 * 8 + (threads / 32) * kQueue * 12; }
+  // counters + one list of 32 triangles per warp
+  static __host__ __device__ int smem_bytes(int threads) { return 64 * 64 * 8 + (threads / 32) * 96 * 4; }
   P p;
   unsigned long long* cnt;  // shared: wp * 64 counters
-  uint32_t* q;              // this warp's queue: 3 x kQueue positions
-  uint32_t qn = 0;
+  uint32_t* q;              // shared: this warp's triangles, 3 x 32 positions
   uint32_t since = 0;
   Planes<K> pl[SLOTS];
   __device__ Worlds(const P& p_, char* smem) : p(p_) {
     cnt = (unsigned long long*)smem;
-    q = (uint32_t*)(smem + 64 * 64 * 8) + (threadIdx.x >> 5) * 3 * kQueue;
+    q = (uint32_t*)(smem + 64 * 64 * 8) + (threadIdx.x >> 5) * 96;
 #pragma unroll
     for (int s = 0; s < SLOTS; s++) pl[s].clear();
   }
@@ -191,12 +191,23 @@ struct Worlds {
     }
     since = 0;
   }
-  // The queued triangles one after another, with the next triangle's sign
+  __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t, uint32_t, uint32_t, uint32_t puv, uint32_t pvw) {
+    return make_uint4(slot, puv, pvw, 0u);
+  }
+  // The qn queued triangles one after another, with the next triangle's sign
   // words loaded before the current one's counters are updated, so that a
   // warp's loads overlap its counter updates.
-  __device__ void drain() {
-    __syncwarp();
+  __device__ __forceinline__ void take(bool on, uint32_t qn, uint4 it, uint32_t, uint32_t, uint32_t, uint32_t puw,
+                                       uint32_t) {
+    constexpr int kQueue = 32;
     const int lane = (int)lane_id();
+    __syncwarp();
+    if (on) {
+      q[lane] = puw;
+      q[kQueue + lane] = it.y;
+      q[2 * kQueue + lane] = it.z;
+    }
+    __syncwarp();
     const unsigned long long* X = p.X;
     const uint32_t wp = p.wp;
     if (SLOTS == 2) {
@@ -231,27 +242,10 @@ struct Worlds {
         if (++since == kLimit) flush();
       }
     }
-    qn = 0;
-    __syncwarp();
-  }
-  __device__ __forceinline__ void step(bool hit, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t,
-                                       uint32_t puv, uint32_t puw, uint32_t pvw) {
-    const unsigned m = __ballot_sync(kFull, hit);
-    if (!m) return;
-    const int lane = (int)lane_id();
-    if (hit) {
-      const uint32_t at = qn + __popc(m & lanemask_lt());
-      q[at] = puv;
-      q[kQueue + at] = puw;
-      q[2 * kQueue + at] = pvw;
-    }
-    qn += __popc(m);
-    if (qn >= 32) drain();
   }
   __device__ void task_begin(uint32_t) {}
   __device__ void task_end(uint32_t) {}
   __device__ void block_end() {
-    if (qn) drain();
     flush();
     __syncthreads();
     for (int i = threadIdx.x; i < (int)p.wp * 64; i += blockDim.x)
@@ -292,7 +286,9 @@ struct BatchP {
 struct Batch {
   using P = BatchP;
   static constexpr bool kPos = true;
-  static constexpr bool kBatched = false;
+  using Item = uint4;  // table slot, product of two values, positions of the pair edge and the streamed edge
+  static constexpr bool kMore = false;
+  static constexpr int kU = 2;
   static constexpr int kRegCap = 128;
   static __host__ __device__ int smem_bytes(int) { return 0; }
   static constexpr int K = 8;
@@ -353,10 +349,15 @@ struct Batch {
     }
     reset();
   }
-  __device__ __forceinline__ void step(bool hit, uint32_t, uint32_t, uint32_t, uint32_t quv, uint32_t quw,
-                                       uint32_t qvw, uint32_t puv, uint32_t puw, uint32_t pvw) {
-    if (hit) {
-      const int64_t P = (int64_t)((int32_t)quv * (int32_t)quw) * (int64_t)(int32_t)qvw;
+  __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t, uint32_t puv,
+                                               uint32_t pvw) {
+    return make_uint4(slot, (uint32_t)((int32_t)quv * (int32_t)qvw), puv, pvw);
+  }
+  __device__ __forceinline__ void take(bool on, uint32_t, uint4 it, uint32_t, uint32_t, uint32_t quw, uint32_t puw,
+                                       uint32_t) {
+    if (on) {
+      const uint32_t puv = it.z, pvw = it.w;
+      const int64_t P = (int64_t)(int32_t)it.y * (int64_t)(int32_t)quw;
 #pragma unroll
       for (int i = 0; i < kBatchTau; i++) {
         if (i < p.nt) {
@@ -370,8 +371,8 @@ struct Batch {
       hi += (P < 0 ? ~0ull : 0ull) + (lo < o ? 1ull : 0ull);
       if (p.X) pl.inc(p.X[puv] ^ p.X[puw] ^ p.X[pvw]);
     }
-    // a lane's counters grow by at most one per call that has any hit
-    if (__any_sync(kFull, hit) && ++since == (1u << K) - 1u) {
+    // a lane's counters grow by at most one per call
+    if (++since == (1u << K) - 1u) {
       if (p.X) {
         const int lane = (int)lane_id();
         for (int j = 0; j < 64; j++) {
@@ -407,7 +408,9 @@ __global__ void k_batch_finish(int64_t ng, int nt, const unsigned long long* __r
 
 template <class V>
 ubt_status launch_w(const ubt_graph* g, const typename V::P& p, cudaStream_t s) {
-  return launch_traversal<V>(g, make_trav_args(g, 0, true), p, s);
+  TravArgs a;
+  const ubt_status st = make_trav_args(g, 0, s, &a);
+  return st != UBT_OK ? st : launch_traversal<V>(g, a, p, s);
 }
 
 size_t worlds_table_words(const ubt_graph* g, int64_t W) {
