@@ -529,8 +529,10 @@ ubt_status ubt_topk(ubt_graph* g, int64_t K, int32_t which, ubt_tri_rec* d_out, 
  *                     spread over the warps of all blocks by a second launch
  *                     (at most 1,024 per call; the rest are counted by one
  *                     block each)
- *   "world_words_per_pass"  64-world words per traversal of ubt_sample_worlds
- *                     (1, 2, 4, 8, 16, 32 or 64)
+ *   "world_words_per_pass"  most 64-world words per traversal of
+ *                     ubt_sample_worlds (1, 2, 4, 8, 16, 32 or 64, default
+ *                     64; fewer where the sign table of m x 8 bytes a word
+ *                     would exceed 36 GiB, but not fewer than 8 for that)
  *   "small_batch"     warp tasks taken per grab of a task counter
  *   "sort_smem_max"   longest list sorted in shared memory during the
  *                     build (power of two, 64..4096); longer lists are sorted

@@ -202,7 +202,7 @@ struct Tuning {
   int64_t smem_table_max = 8192;  // hash slots of a shared-memory table
   int64_t block_bits = 1 << 18;   // block tasks: largest vertex range of a bitmap table
   int64_t warp_bits = 1 << 14;    // warp tasks: the same
-  int64_t world_words_per_pass = 8;
+  int64_t world_words_per_pass = 64;
   int64_t small_batch = 4;        // warp tasks taken per grab
   int64_t block_unit = 32;        // pairs per warp step in block tasks
   int64_t long_min = 64;          // streamed lists this long are streamed by the whole warp

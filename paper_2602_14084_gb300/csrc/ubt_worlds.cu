@@ -32,17 +32,29 @@ struct U64x4 {
   unsigned long long x[4];
 };
 
-__device__ __forceinline__ U64x4 philox4x64_10(U64x4 c, unsigned long long k0, unsigned long long k1) {
-  const unsigned long long M0 = 0xD2E7470EE14C6C93ull, M1 = 0xCA5A826395121157ull;
+// Philox4x64-10 of counter (key, w, call, 0) with key (seed, 0), given the
+// product of its first round that the four calls of an edge share.
+struct FirstRound {
+  unsigned long long lo, hi;  // M0 * key
+};
+constexpr unsigned long long kPhiloxM0 = 0xD2E7470EE14C6C93ull, kPhiloxM1 = 0xCA5A826395121157ull;
+__device__ __forceinline__ FirstRound philox_first(uint32_t key) {
+  return FirstRound{kPhiloxM0 * key, __umul64hi(kPhiloxM0, key)};
+}
+__device__ __forceinline__ U64x4 philox_call(const FirstRound& f, uint32_t w, uint32_t call, unsigned long long seed) {
   const unsigned long long W0 = 0x9E3779B97F4A7C15ull, W1 = 0xBB67AE8584CAA73Bull;
+  unsigned long long k0 = seed, k1 = 0;
+  U64x4 c;  // after the first round
+  c.x[0] = __umul64hi(kPhiloxM1, (unsigned long long)call) ^ (unsigned long long)w ^ k0;
+  c.x[1] = kPhiloxM1 * call;
+  c.x[2] = f.hi ^ k1;
+  c.x[3] = f.lo;
 #pragma unroll
-  for (int r = 0; r < 10; r++) {
-    if (r) {
-      k0 += W0;
-      k1 += W1;
-    }
-    const unsigned long long lo0 = M0 * c.x[0], hi0 = __umul64hi(M0, c.x[0]);
-    const unsigned long long lo1 = M1 * c.x[2], hi1 = __umul64hi(M1, c.x[2]);
+  for (int r = 1; r < 10; r++) {
+    k0 += W0;
+    k1 += W1;
+    const unsigned long long lo0 = kPhiloxM0 * c.x[0], hi0 = __umul64hi(kPhiloxM0, c.x[0]);
+    const unsigned long long lo1 = kPhiloxM1 * c.x[2], hi1 = __umul64hi(kPhiloxM1, c.x[2]);
     U64x4 n;
     n.x[0] = hi1 ^ c.x[1] ^ k0;
     n.x[1] = lo1;
@@ -53,50 +65,86 @@ __device__ __forceinline__ U64x4 philox4x64_10(U64x4 c, unsigned long long k0, u
   return c;
 }
 
-// 64 sign draws of one edge in world word w: bit j = 1 iff positive in world 64w+j
-__device__ __forceinline__ unsigned long long sign_word(unsigned long long seed, uint32_t key, uint32_t w,
-                                                        uint32_t k) {
-  if (k >= 65536u) return ~0ull;
-  if (k == 0u) return 0ull;
-  // u < k on the 16 bit planes, most significant first: call c gives planes
-  // 4c .. 4c + 3.  A world is decided at the first plane where u and k
-  // differ; once every world of the word is decided (eq = 0) the lower planes
-  // change nothing, so their calls are skipped (after two calls about 78 % of
-  // the words are decided, after three 98 %).
-  unsigned long long lt = 0, eq = ~0ull;
-#pragma unroll 1
-  for (int c = 3; c >= 0 && eq; c--) {
-    U64x4 ctr;
-    ctr.x[0] = key;
-    ctr.x[1] = w;
-    ctr.x[2] = (unsigned long long)c;
-    ctr.x[3] = 0;
-    const U64x4 o = philox4x64_10(ctr, seed, 0ull);
+// u < k on the bit planes 4 call .. 4 call + 3, most significant first: lt are
+// the worlds decided positive, eq the undecided ones
+__device__ __forceinline__ void sign_planes(const U64x4& o, uint32_t call, uint32_t k, unsigned long long& lt,
+                                            unsigned long long& eq) {
 #pragma unroll
-    for (int i = 3; i >= 0; i--) {
-      const unsigned long long r = o.x[i];
-      if ((k >> (4 * c + i)) & 1u) {
-        lt |= eq & ~r;
-        eq &= r;
-      } else {
-        eq &= ~r;
-      }
-    }
+  for (int i = 3; i >= 0; i--) {
+    const unsigned long long r = o.x[i];
+    const unsigned long long bit = 0ull - (unsigned long long)((k >> (4 * call + i)) & 1u);  // all ones if set
+    lt |= eq & ~r & bit;
+    eq &= ~(r ^ bit);
   }
-  return lt;
 }
 
-// X[pos * wp + i] = sign word (w0 + i) of the edge at CSR position pos
-__global__ void k_sign_table(int64_t m, const uint64_t* __restrict__ adj, const uint32_t* __restrict__ ekey,
-                             unsigned long long seed, uint32_t w0, uint32_t wp, unsigned long long* __restrict__ X) {
-  const int64_t total = m * (int64_t)wp;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t pos = i / wp;
-    const uint32_t w = w0 + (uint32_t)(i - pos * wp);
-    const int32_t q = adj_q(adj[pos]);
-    const uint32_t k = (uint32_t)(32768 - q);
-    X[i] = sign_word(seed, ekey[pos], w, k);
+// X[pos * wp + i] = sign word (w0 + i) of the edge at CSR position pos, i < valid
+// (wp a power of two): bit j = 1 iff positive in world 64 (w0 + i) + j.
+//
+// A world is decided at the first plane where u and k differ, so the lower
+// planes' calls are needed for few words: after the first two calls (planes
+// 15..8) 22 % of the words have an undecided world, after three 2 %.  Every
+// word gets the first two calls, independent of each other; the undecided ones
+// are queued per warp and finished 32 at a time, on full warps (2.4 calls a
+// word; calling until a warp's 32 words are all decided took 3.4).  Bound by
+// the 64-bit products' multiply instructions.
+constexpr int kSignThreads = 256;
+constexpr int kSignQueue = 64;
+struct SignQueue {
+  unsigned long long at[kSignQueue], lt[kSignQueue], eq[kSignQueue];
+  uint32_t key[kSignQueue], w[kSignQueue], k[kSignQueue];
+};
+__global__ void __launch_bounds__(kSignThreads)
+k_sign_table(int64_t m, const uint64_t* __restrict__ adj, const uint32_t* __restrict__ ekey, unsigned long long seed,
+             uint32_t w0, uint32_t wp, uint32_t valid, unsigned long long* __restrict__ X) {
+  __shared__ SignQueue queues[kSignThreads / 32];
+  SignQueue& q = queues[threadIdx.x >> 5];
+  const uint32_t lane = lane_id();
+  uint32_t n = 0;  // queued words (warp-uniform, fewer than 32 between steps)
+  auto finish = [&](uint32_t cnt) {  // the last cnt queued words
+    __syncwarp();
+    n -= cnt;
+    if (lane < cnt) {
+      const uint32_t i = n + lane, k = q.k[i];
+      unsigned long long lt = q.lt[i], eq = q.eq[i];
+      const FirstRound f = philox_first(q.key[i]);
+#pragma unroll 1
+      for (int call = 1; call >= 0 && eq; call--) sign_planes(philox_call(f, q.w[i], call, seed), call, k, lt, eq);
+      X[q.at[i]] = lt;
+    }
+    __syncwarp();
+  };
+  const int lg = 31 - __clz((int)wp);
+  const int64_t total = m << lg;
+  for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; base < total;
+       base += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = base + lane, pos = i >> lg;
+    const uint32_t wi = (uint32_t)i & (wp - 1);
+    const bool on = i < total && wi < valid;
+    const uint32_t k = on ? (uint32_t)(32768 - adj_q(adj[pos])) : 0u, key = on ? ekey[pos] : 0u, w = w0 + wi;
+    unsigned long long lt = k >= 65536u ? ~0ull : 0ull, eq = k == 0u || k >= 65536u ? 0ull : ~0ull;
+    if (__any_sync(kFull, eq != 0ull)) {
+      const FirstRound f = philox_first(key);
+      const U64x4 o3 = philox_call(f, w, 3, seed), o2 = philox_call(f, w, 2, seed);
+      sign_planes(o3, 3, k, lt, eq);
+      sign_planes(o2, 2, k, lt, eq);
+    }
+    const bool more = on && eq != 0ull;
+    if (on && !more) X[i] = lt;
+    const unsigned mask = __ballot_sync(kFull, more);
+    if (more) {
+      const uint32_t at = n + __popc(mask & lanemask_lt());
+      q.at[at] = (unsigned long long)i;
+      q.lt[at] = lt;
+      q.eq[at] = eq;
+      q.key[at] = key;
+      q.w[at] = w;
+      q.k[at] = k;
+    }
+    n += __popc(mask);
+    if (n >= 32) finish(32);
   }
+  if (n) finish(n);
 }
 
 // ------------------------------------------------------------ bit-sliced counters
@@ -117,18 +165,31 @@ struct Planes {
       if (!b) break;
     }
   }
-  // two counters at once: one carry chain per counter, interleaved, ending
-  // when both carries are spent
-  __device__ __forceinline__ static void inc2(Planes& p0, Planes& p1, unsigned long long b0, unsigned long long b1) {
+  // eight words at once (K > 3): a carry-save tree, three full adders' worth of
+  // logic per word instead of a carry chain through every plane, whose carry of
+  // weight 8 goes up the planes once
+  __device__ __forceinline__ void add8(const unsigned long long (&w)[8]) {
+    unsigned long long a, b, f0, f1, e;
+    csa(a, c[0], w[0], w[1]);
+    csa(b, c[0], w[2], w[3]);
+    csa(f0, c[1], a, b);
+    csa(a, c[0], w[4], w[5]);
+    csa(b, c[0], w[6], w[7]);
+    csa(f1, c[1], a, b);
+    csa(e, c[2], f0, f1);
 #pragma unroll
-    for (int t = 0; t < K; t++) {
-      const unsigned long long c0 = p0.c[t] & b0, c1 = p1.c[t] & b1;
-      p0.c[t] ^= b0;
-      p1.c[t] ^= b1;
-      b0 = c0;
-      b1 = c1;
-      if (!(b0 | b1)) break;
+    for (int t = 3; t < K; t++) {
+      const unsigned long long carry = c[t] & e;
+      c[t] ^= e;
+      e = carry;
     }
+  }
+  // sum + x + y: the sum bit stays, the carry goes out
+  __device__ __forceinline__ static void csa(unsigned long long& carry, unsigned long long& sum, unsigned long long x,
+                                             unsigned long long y) {
+    const unsigned long long s = sum;
+    carry = (s & x) | (s & y) | (x & y);
+    sum = s ^ x ^ y;
   }
   // per-lane count of world j
   __device__ __forceinline__ uint32_t count(int j) const {
@@ -144,17 +205,18 @@ struct Planes {
 struct WorldsP {
   const unsigned long long* X;  // sign table of this pass: m x wp words
   uint32_t wp;                  // words per pass (1..64, power of two)
-  unsigned long long* out;      // counts of this pass's worlds: wp * 64
+  uint32_t valid;               // of them wanted
+  unsigned long long* out;      // counts of this pass's worlds: valid * 64
 };
 
 // SLOTS = words per lane: 1 when wp <= 32 (lanes grouped by word), 2 when wp = 64
 template <int SLOTS>
 struct Worlds {
   using P = WorldsP;
-  static constexpr bool kPos = true;
   using Item = uint4;  // table slot, positions of the pair edge and the streamed edge
   static constexpr bool kMore = false;
   static constexpr int kU = 2;
+  static constexpr bool kPos = true;
   static constexpr int kRegCap = 128;
   static constexpr int K = SLOTS == 1 ? 14 : 12;      // planes per slot
   static constexpr uint32_t kLimit = (1u << K) - 1u;  // increments before a flush
@@ -178,7 +240,7 @@ struct Worlds {
     const int lane = (int)lane_id();
     return SLOTS == 2 ? (uint32_t)(2 * lane + s) : (uint32_t)lane % p.wp;
   }
-  __device__ void flush() {
+  __device__ __forceinline__ void flush() {
 #pragma unroll
     for (int s = 0; s < SLOTS; s++) {
       const uint32_t w = word_of(s);
@@ -194,61 +256,75 @@ struct Worlds {
   __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t, uint32_t, uint32_t, uint32_t puv, uint32_t pvw) {
     return make_uint4(slot, puv, pvw, 0u);
   }
-  // The qn queued triangles one after another, with the next triangle's sign
-  // words loaded before the current one's counters are updated, so that a
-  // warp's loads overlap its counter updates.
+  // The queued triangles' sign rows, 8 words a lane at a time (their loads all
+  // issued before the adder tree); the streamed edge's row is not kept in L1,
+  // so that the owner's and the pair's rows, which the next triangles reuse, stay.
   __device__ __forceinline__ void take(bool on, uint32_t qn, uint4 it, uint32_t, uint32_t, uint32_t, uint32_t puw,
                                        uint32_t) {
-    constexpr int kQueue = 32;
     const int lane = (int)lane_id();
     __syncwarp();
     if (on) {
       q[lane] = puw;
-      q[kQueue + lane] = it.y;
-      q[2 * kQueue + lane] = it.z;
+      q[32 + lane] = it.y;
+      q[64 + lane] = it.z;
     }
     __syncwarp();
-    const unsigned long long* X = p.X;
     const uint32_t wp = p.wp;
     if (SLOTS == 2) {
       // a row is 64 words = 32 16-byte pairs: lane l holds words 2l and 2l + 1
-      const ulonglong2* __restrict__ X2 = reinterpret_cast<const ulonglong2*>(X);
-      auto word2 = [&](uint32_t t) -> ulonglong2 {
-        const ulonglong2 a = X2[(size_t)q[t] * 32 + lane], b = X2[(size_t)q[kQueue + t] * 32 + lane],
-                         c = X2[(size_t)q[2 * kQueue + t] * 32 + lane];
-        return make_ulonglong2(a.x ^ b.x ^ c.x, a.y ^ b.y ^ c.y);
-      };
-      ulonglong2 nx = make_ulonglong2(0ull, 0ull);  // the next triangle's XOR words
-      if (qn) nx = word2(0);
-      for (uint32_t t = 0; t < qn; t++) {
-        const ulonglong2 cx = nx;
-        if (t + 1 < qn) nx = word2(t + 1);  // the same for every lane (qn is)
-        Planes<K>::inc2(pl[0], pl[1], cx.x, cx.y);
-        if (++since == kLimit) flush();
+      const ulonglong2* __restrict__ X2 = reinterpret_cast<const ulonglong2*>(p.X) + lane;
+#pragma unroll 1
+      for (uint32_t t0 = 0; t0 < qn; t0 += 8) {
+        unsigned long long w0[8], w1[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+          const uint32_t t = min(t0 + i, qn - 1);  // past the end: loaded again and not counted
+          const ulonglong2 a = X2[(size_t)q[t] * 32], b = X2[(size_t)q[32 + t] * 32],
+                           c = load_once(X2 + (size_t)q[64 + t] * 32);
+          w0[i] = t0 + i < qn ? a.x ^ b.x ^ c.x : 0ull;
+          w1[i] = t0 + i < qn ? a.y ^ b.y ^ c.y : 0ull;
+        }
+        if (since + 8 > kLimit) flush();
+        pl[0].add8(w0);
+        pl[SLOTS - 1].add8(w1);
+        since += 8;
       }
     } else {
-      const uint32_t per = 32 / wp;  // triangles per iteration
+      const uint32_t per = 32 / wp;  // triangles per word of a lane
       const uint32_t grp = (uint32_t)lane / wp, w = (uint32_t)lane % wp;
-      auto word = [&](uint32_t t) -> unsigned long long {
-        return t < qn ? X[(size_t)q[t] * wp + w] ^ X[(size_t)q[kQueue + t] * wp + w] ^
-                            X[(size_t)q[2 * kQueue + t] * wp + w]
-                      : 0ull;
-      };
-      unsigned long long nb = word(grp);
-      for (uint32_t t0 = 0; t0 < qn; t0 += per) {
-        const unsigned long long bw = nb;
-        nb = word(t0 + per + grp);
-        pl[0].inc(bw);
-        if (++since == kLimit) flush();
+      const unsigned long long* __restrict__ X = p.X + w;
+#pragma unroll 1
+      for (uint32_t t0 = grp; t0 < qn + grp; t0 += 8 * per) {  // as often in every lane
+        unsigned long long x[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+          const uint32_t at = t0 + i * per, t = min(at, qn - 1);
+          const unsigned long long v =
+              X[(size_t)q[t] * wp] ^ X[(size_t)q[32 + t] * wp] ^ load_once(X + (size_t)q[64 + t] * wp);
+          x[i] = at < qn ? v : 0ull;
+        }
+        if (since + 8 > kLimit) flush();
+        pl[0].add8(x);
+        since += 8;
       }
     }
+  }
+  __device__ __forceinline__ static unsigned long long load_once(const unsigned long long* a) {
+    unsigned long long v;
+    asm("ld.global.nc.L1::no_allocate.u64 %0, [%1];" : "=l"(v) : "l"(a));
+    return v;
+  }
+  __device__ __forceinline__ static ulonglong2 load_once(const ulonglong2* a) {
+    ulonglong2 v;
+    asm("ld.global.nc.L1::no_allocate.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(a));
+    return v;
   }
   __device__ void task_begin(uint32_t) {}
   __device__ void task_end(uint32_t) {}
   __device__ void block_end() {
     flush();
     __syncthreads();
-    for (int i = threadIdx.x; i < (int)p.wp * 64; i += blockDim.x)
+    for (int i = threadIdx.x; i < (int)p.valid * 64; i += blockDim.x)
       if (cnt[i]) atomicAdd(&p.out[i], cnt[i]);
   }
 };
@@ -406,6 +482,15 @@ __global__ void k_batch_finish(int64_t ng, int nt, const unsigned long long* __r
   }
 }
 
+ubt_status launch_sign_table(const ubt_graph* g, uint64_t seed, int64_t w0, int64_t wp, int64_t valid,
+                             unsigned long long* X, cudaStream_t s) {
+  if (g->m == 0) return UBT_OK;
+  const int grid = (int)std::min<int64_t>((g->m * wp + kSignThreads - 1) / kSignThreads, (int64_t)g->sm_count * 32);
+  k_sign_table<<<grid, kSignThreads, 0, s>>>(g->m, g->adj, g->ekey, seed, (uint32_t)w0, (uint32_t)wp, (uint32_t)valid, X);
+  UBT_CUDA(cudaGetLastError());
+  return UBT_OK;
+}
+
 template <class V>
 ubt_status launch_w(const ubt_graph* g, const typename V::P& p, cudaStream_t s) {
   TravArgs a;
@@ -413,10 +498,22 @@ ubt_status launch_w(const ubt_graph* g, const typename V::P& p, cudaStream_t s) 
   return st != UBT_OK ? st : launch_traversal<V>(g, a, p, s);
 }
 
+// Words of a pass over `left` words: a power of two (lanes are grouped by
+// word), at most the tuning's, whose table (8 m bytes a word) takes at most an
+// eighth of the HBM or, for larger graphs, 8 words.  More words a pass list the
+// triangles fewer times and read longer rows (R-MAT scale 20, 64 words: one pass of 64 85 ms, eight
+// of 8 143 ms).  The last pass may have words to spare rather than be cut into
+// several.
+constexpr int64_t kSignTableBytes = 36ll << 30;
+int64_t pass_words(const ubt_graph* g, int64_t left) {
+  int64_t wp = tuning().world_words_per_pass;
+  while (wp > 8 && g->m * wp * 8 > kSignTableBytes) wp >>= 1;
+  while (wp > 1 && 4 * left < 3 * wp) wp >>= 1;
+  return wp;
+}
+
 size_t worlds_table_words(const ubt_graph* g, int64_t W) {
-  const int64_t words = W / 64;
-  const int64_t wp = std::min<int64_t>(words, tuning().world_words_per_pass);
-  return (size_t)std::max<int64_t>(g->m, 1) * (size_t)wp;
+  return (size_t)std::max<int64_t>(g->m, 1) * (size_t)pass_words(g, W / 64);
 }
 
 // the workspace ubt_sample_worlds_workspace_size reports and ubt_sample_worlds requires
@@ -442,19 +539,16 @@ extern "C" ubt_status ubt_sample_worlds(ubt_graph* g, uint64_t seed, int64_t W, 
   if (ws_bytes < worlds_workspace_bytes(g, W)) return UBT_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t words = W / 64;
-  int64_t wp = std::min<int64_t>(words, tuning().world_words_per_pass);
-  while (words % wp) wp >>= 1;  // passes of equal size
   unsigned long long* X = (unsigned long long*)d_workspace;
   UBT_CUDA(cudaMemsetAsync(d_bal_per_world, 0, sizeof(int64_t) * W, s));
-  for (int64_t w0 = 0; w0 < words; w0 += wp) {
-    if (g->m > 0) {
-      const int grid = (int)std::min<int64_t>((g->m * wp + 255) / 256, (int64_t)g->sm_count * 32);
-      k_sign_table<<<grid, 256, 0, s>>>(g->m, g->adj, g->ekey, seed, (uint32_t)w0, (uint32_t)wp, X);
-      UBT_CUDA(cudaGetLastError());
-    }
-    WorldsP p{X, (uint32_t)wp, (unsigned long long*)(d_bal_per_world + w0 * 64)};
+  for (int64_t w0 = 0; w0 < words;) {
+    const int64_t wp = pass_words(g, words - w0), valid = std::min(wp, words - w0);
+    const ubt_status sst = launch_sign_table(g, seed, w0, wp, valid, X, s);
+    if (sst != UBT_OK) return sst;
+    WorldsP p{X, (uint32_t)wp, (uint32_t)valid, (unsigned long long*)(d_bal_per_world + w0 * 64)};
     const ubt_status st = wp == 64 ? launch_w<Worlds<2>>(g, p, s) : launch_w<Worlds<1>>(g, p, s);
     if (st != UBT_OK) return st;
+    w0 += valid;
   }
   if (d_total) {
     k_world_total<<<1, 1024, 0, s>>>((const unsigned long long*)d_bal_per_world, W, d_total);
@@ -490,11 +584,8 @@ extern "C" ubt_status ubt_batch_query(ubt_graph* g, const double* h_tau, int32_t
   if (d_worlds) {
     UBT_CUDA(cudaMemsetAsync(d_worlds, 0, sizeof(int64_t) * ng * 64, s));
     // one sign word per CSR position, kept in the backward accumulators
-    if (g->m > 0) {
-      const int grid = (int)std::min<int64_t>((g->m + 255) / 256, (int64_t)g->sm_count * 32);
-      k_sign_table<<<grid, 256, 0, s>>>(g->m, g->adj, g->ekey, seed, 0u, 1u, g->gacc);
-      UBT_CUDA(cudaGetLastError());
-    }
+    const ubt_status sst = launch_sign_table(g, seed, 0, 1, 1, g->gacc, s);
+    if (sst != UBT_OK) return sst;
     p.X = g->gacc;
   }
   ubt_status st = launch_w<Batch>(g, p, s);

@@ -120,3 +120,23 @@ def test_batch_with_either_table(ubt, warp_bits):
         assert abs(expect[gi, 0] - S / float(1 << 48)) <= 1e-12 * max(1.0, T), gi
         assert np.array_equal(worlds[gi], oracle.world_counts(v1 - v0, ls, ld, lk, 5, [0], ekey=eg["eid"][e0:e1])), gi
     assert G.guard() == 0
+
+
+@pytest.mark.parametrize("W", [64, 192, 448, 640, 3008, 4160])
+def test_worlds_in_passes_of_every_size(ubt, W):
+    """World counts whose words do not divide into passes of one size: last
+    passes of other sizes, and with words to spare, under every largest pass."""
+    s, d = core_graph(400, 2500, 60, 9)
+    k = synth.k_uniform(s.size, 10)
+    k[:50], k[50:100] = 0, 65536
+    want = oracle.world_counts(400, s, d, k, 21, list(range(W // 64)))
+    G = ubt.Graph(400, s, d, k=k)
+    old = ubt.get_tuning("world_words_per_pass")
+    try:
+        for wpp in (1, 2, 8, 16, 64):
+            ubt.set_tuning("world_words_per_pass", wpp)
+            got, tot = G.sample_worlds(seed=21, W=W)
+            assert np.array_equal(got, want) and tot == int(want.sum()), wpp
+    finally:
+        ubt.set_tuning("world_words_per_pass", old)
+    assert G.guard() == 0
