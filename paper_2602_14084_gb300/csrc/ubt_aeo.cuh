@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(512, 2) k_aeo(AeoArgs a, typename V::P p) {
   V vis(p, smem);
   vis.block_init();
   __syncthreads();
-  uint32_t* tab = (uint32_t*)(smem + ((V::smem_bytes((int)blockDim.x) + 15) / 16) * 16);
+  uint32_t* tab = (uint32_t*)(smem + ((V::smem_bytes(p, (int)blockDim.x) + 15) / 16) * 16);
   while (true) {
     if (threadIdx.x == 0) s_misc[2] = (uint32_t)atomicAdd(&a.sc->task[0], 1ull);
     __syncthreads();
@@ -506,7 +506,7 @@ ubt_status launch_aeo(const ubt_graph* g, int64_t L, const typename V::P& p, cud
       UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
       if (g->m == 0) return UBT_OK;
       const int threads = 512;
-      const size_t smem = (size_t)((V::smem_bytes(threads) + 15) / 16) * 16;
+      const size_t smem = (size_t)((V::smem_bytes(p, threads) + 15) / 16) * 16;
       UBT_CUDA(cudaFuncSetAttribute(k_aeo_index<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       int per_sm = 0;
       UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_aeo_index<V>, threads, smem));
@@ -538,7 +538,7 @@ ubt_status launch_aeo(const ubt_graph* g, int64_t L, const typename V::P& p, cud
   if (a.n_owners == 0) return UBT_OK;
   const int threads = 512;
   const size_t tables = std::max<size_t>((size_t)a.cap, (size_t)(threads / 32) * a.wcap) * 3 * 4;
-  const size_t smem = (size_t)((V::smem_bytes(threads) + 15) / 16) * 16 + tables;
+  const size_t smem = (size_t)((V::smem_bytes(p, threads) + 15) / 16) * 16 + tables;
   UBT_CUDA(cudaFuncSetAttribute(k_aeo<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_aeo<V>, threads, smem));

@@ -101,12 +101,20 @@ __global__ void k_validate_degree(int64_t n, int64_t m, const uint32_t* __restri
   }
 }
 
-__global__ void k_max_degree(int64_t n, const uint32_t* __restrict__ deg, unsigned long long* out) {
-  uint32_t best = 0;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+// out: [0] the largest degree, [1] the vertices of degree > kMergeDegree
+constexpr uint32_t kMergeDegree = 32;
+__global__ void k_degree_stats(int64_t n, const uint32_t* __restrict__ deg, unsigned long long* out) {
+  uint32_t best = 0, large = 0;
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     best = max(best, deg[v]);
+    large += deg[v] > kMergeDegree ? 1u : 0u;
+  }
   best = __reduce_max_sync(kFull, best);
-  if (lane_id() == 0) atomicMax(out, (unsigned long long)best);
+  large = __reduce_add_sync(kFull, large);
+  if (lane_id() == 0) {
+    atomicMax(&out[0], (unsigned long long)best);
+    if (large) atomicAdd(&out[1], (unsigned long long)large);
+  }
 }
 
 // ---------------------------------------------------------------- vertex numbers
@@ -702,9 +710,10 @@ static_assert(kTaskBuckets <= kNoTask, "a bucket is one byte");
 // stats: [0] oriented wedges sum_v in(v) |N>(v)| (Alg. 1's probes), [1] longest
 //        list, [2] streamed entries (set by k_pair_fill), [3] longest list of
 //        a kHubHash task, [4] of a kHubBits task, [5] largest range of one,
+//        [6] first pair of a vertex from merge_from on,
 //        [kStatBuckets + bucket] bucket sizes
 constexpr uint32_t kHeavyPairs = 1u << 16;
-constexpr int kStatBuckets = 6;
+constexpr int kStatBuckets = 7;
 // A pair's own loads count as this many streamed entries.
 constexpr unsigned long long kPairWork = 16;
 // An owner whose work exceeds part_work is several block tasks, each with its
@@ -725,7 +734,7 @@ __device__ __forceinline__ uint32_t owner_parts(unsigned long long work, unsigne
 __global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ row_ptr, const uint32_t* __restrict__ pair_ptr,
                             const unsigned long long* __restrict__ work, const uint32_t* __restrict__ vgraph,
                             const uint32_t* __restrict__ gstart, uint32_t hub_thr, uint32_t giant_thr,
-                            unsigned long long block_work, uint32_t block_bits, uint32_t warp_bits,
+                            unsigned long long block_work, uint32_t block_bits, uint32_t warp_bits, int64_t merge_from,
                             uint8_t* __restrict__ bucket, unsigned long long* stats) {
   __shared__ uint32_t s_cnt[kTaskBuckets];
   __shared__ unsigned long long s_wedges;
@@ -744,7 +753,8 @@ __global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ r
     const unsigned long long w = owner_work(work[x], np);
     uint8_t b = kNoTask;
     wedges += (unsigned long long)np * len;
-    if (len > 0 && np > 0) {
+    if (x == merge_from) stats[6] = pair_ptr[x];
+    if (len > 0 && np > 0 && x < merge_from) {
       const uint32_t range = (uint32_t)x - (gstart ? gstart[vgraph[x]] : 0u);
       const bool block = len > hub_thr || w > block_work || np > kHeavyPairs;
       const int cls = len > giant_thr ? kGiant
@@ -1219,9 +1229,9 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   if (m > 0)
     k_validate_degree<<<grid_e, thr, 0, s>>>(n, m, d_src, d_dst, d_k, d_p, L.vgraph_id, L.deg, &L.scratch->err);
   unsigned long long* lcount = L.stats + 2 * kStats;  // row lengths; first the largest degree
-  if (n > 0) k_max_degree<<<grid_v, thr, 0, s>>>(n, L.deg, lcount);
-  unsigned long long err = 0, max_deg = 0;
-  UBT_CUDA(cudaMemcpyAsync(&max_deg, lcount, sizeof(max_deg), cudaMemcpyDeviceToHost, s));
+  if (n > 0) k_degree_stats<<<grid_v, thr, 0, s>>>(n, L.deg, lcount);
+  unsigned long long err = 0, deg_stats[2] = {0, 0};
+  UBT_CUDA(cudaMemcpyAsync(deg_stats, lcount, sizeof(deg_stats), cudaMemcpyDeviceToHost, s));
   UBT_CUDA(cudaMemcpyAsync(&err, &L.scratch->err, sizeof(err), cudaMemcpyDeviceToHost, s));
   UBT_CUDA(cudaStreamSynchronize(s));
   ubt_status st = status_from_err(err);
@@ -1229,8 +1239,8 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   // 2. orientation + CSR offsets
   phase.next("build: orient, scatter, sort");
   if (n > 0) {
-    UBT_CUDA(cudaMemsetAsync(lcount, 0, sizeof(unsigned long long), s));
-    st = rank_vertices(L, n, max_deg, ng, s);
+    UBT_CUDA(cudaMemsetAsync(lcount, 0, sizeof(deg_stats), s));
+    st = rank_vertices(L, n, deg_stats[0], ng, s);
     if (st != UBT_OK) return st;
     if (batch) k_rank_graphs<<<grid_v, thr, 0, s>>>(n, L.vid, L.vgraph_id, L.vgraph, opts->d_vertex_offsets, ng, L.gstart);
   }
@@ -1289,10 +1299,13 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   unsigned long long stats[kStats], classes[65];
   memset(stats, 0, sizeof(stats));
   memset(classes, 0, sizeof(classes));
+  // vertices of degree <= kMergeDegree are the last ones (of a batch, every
+  // graph's last ones: its pairs all go to tables)
+  const int64_t merge_from = batch ? n : (int64_t)deg_stats[1];
   if (n > 0) {
     k_row_stats<<<grid_v, thr, 0, s>>>(n, m, L.row_ptr, L.pair_ptr, L.work, L.vgraph, L.gstart, (uint32_t)hub_thr,
                                       (uint32_t)giant_thr, (unsigned long long)block_work, (uint32_t)T.block_bits,
-                                      (uint32_t)T.warp_bits, L.bucket, L.stats);
+                                      (uint32_t)T.warp_bits, merge_from, L.bucket, L.stats);
     UBT_CUDA(cudaMemcpyAsync(stats, L.stats, sizeof(stats), cudaMemcpyDeviceToHost, s));
     if (absq) UBT_CUDA(cudaMemcpyAsync(classes, absq, sizeof(classes), cudaMemcpyDeviceToHost, s));
     UBT_CUDA(cudaStreamSynchronize(s));
@@ -1446,6 +1459,7 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   g->max_bits_len = (int64_t)stats[4];
   g->max_bits = (int64_t)stats[5];
   g->warp_bits = T.warp_bits;
+  g->merge_first = merge_from < n ? (int64_t)stats[6] : m;
   g->hub_threshold = hub_thr;
   g->giant_threshold = giant_thr;
   g->block_work = block_work;

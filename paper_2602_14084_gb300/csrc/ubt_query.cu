@@ -96,7 +96,7 @@ struct CountReg : ProductItem {
   using P = CountRegP;
   static constexpr bool kPos = false;
   static constexpr int kRegCap = UBT_COUNT_REGCAP;
-  static __host__ __device__ int smem_bytes(int) { return 0; }
+  static __host__ __device__ int smem_bytes(const P&, int) { return 0; }
   int64_t B[NT], U[NT];
   unsigned long long* out;
   uint32_t bal[NT], unbal[NT];
@@ -179,7 +179,7 @@ struct CountMulti : ProductItem {
   using P = CountMultiP;
   static constexpr bool kPos = false;
   static constexpr int kRegCap = UBT_COUNT_REGCAP;
-  static __host__ __device__ int smem_bytes(int) { return kMultiLevels * 8 + ((kMultiBins * 4 + 15) / 16) * 16; }
+  static __host__ __device__ int smem_bytes(const P&, int) { return kMultiLevels * 8 + ((kMultiBins * 4 + 15) / 16) * 16; }
   unsigned long long* out;
   const long long* S;  // shared: levels, padded with INT64_MAX
   uint32_t* bins;      // shared: block histogram
@@ -266,7 +266,6 @@ static __device__ __noinline__ void count_bins_flush(uint32_t* bins, unsigned lo
     if (v) atomicAdd(&out[i], (unsigned long long)v);
   }
 }
-constexpr int kBinStride = 144;                  // 32-bit words per warp's bins (>= 2 kMaxTau + 1)
 constexpr uint32_t kBinFlush = (1u << 27) - 64;  // entries per lane between flushes (Alg. 2 kernels)
 constexpr uint32_t kWarpFlush = 1u << 31;         // entries per warp between flushes (batch counts)
 struct CountBinsP {
@@ -284,13 +283,15 @@ struct CountBins : ProductItem {
   static constexpr int kRegCap = UBT_COUNT_REGCAP;
   static constexpr int kTabBytes = ((kSlices + 15) / 16) * 16;
   static constexpr int kLevelBytes = (2 * kMaxTau + 2) * 8;
-  static __host__ __device__ int smem_bytes(int threads) {
-    return kTabBytes + kLevelBytes + (threads / 32) * kBinStride * 4;
+  // one warp's bins: 2 nt - 1 of them are used, [1, 2 nt)
+  static __host__ __device__ int bin_stride(int nt) { return (2 * nt + 3) / 4 * 4; }
+  static __host__ __device__ int smem_bytes(const P& p, int threads) {
+    return kTabBytes + kLevelBytes + (threads / 32) * bin_stride(p.nt) * 4;
   }
   const uint8_t* tab;  // shared: slice table
   const long long* S;  // shared: levels
   uint32_t* bins;      // shared: this warp's bins
-  uint32_t* all;       // shared: every warp's bins, kBinStride words each
+  uint32_t* all;       // shared: every warp's bins
   unsigned long long* out;
   uint32_t first = 0, last = 0;  // bins 0 and 2 nt of this lane
   uint32_t since = 0;            // entries since the last flush (this lane's or the warp's)
@@ -303,9 +304,10 @@ struct CountBins : ProductItem {
     tab = t;
     S = sv;
     all = b;
-    bins = b + (threadIdx.x >> 5) * kBinStride;
+    const int stride = bin_stride(p.nt);
+    bins = b + (threadIdx.x >> 5) * stride;
     for (int i = threadIdx.x; i <= 2 * p.nt; i += blockDim.x) sv[i] = i < 2 * p.nt ? p.S[i] : INT64_MAX;
-    for (int i = threadIdx.x; i < (int)(blockDim.x >> 5) * kBinStride; i += blockDim.x) b[i] = 0;
+    for (int i = threadIdx.x; i < (int)(blockDim.x >> 5) * stride; i += blockDim.x) b[i] = 0;
     for (int i = threadIdx.x; i < kSlices; i += blockDim.x) {
       const long long start = (long long)i * (1ll << 35) - (1ll << 45);
       const long long end = start + (1ll << 35);
@@ -364,7 +366,7 @@ struct CountBins : ProductItem {
     const int nw = (int)(blockDim.x >> 5);
     for (int i = threadIdx.x + 1; i < top; i += blockDim.x) {
       unsigned long long v = 0;
-      for (int w = 0; w < nw; w++) v += all[w * kBinStride + i];
+      for (int w = 0; w < nw; w++) v += all[w * bin_stride(top / 2) + i];
       if (v) atomicAdd(&out[i], v);
     }
   }
@@ -421,7 +423,8 @@ struct EnumP {
   unsigned long long* cursor;
   int64_t Blo = INT64_MIN, Uhi = INT64_MAX;
   const uint32_t* vid = nullptr;    // forward traversal: ids of the vertices
-  const uint32_t* rowid = nullptr;  // and the row of the streamed list's position
+  const uint32_t* rowid = nullptr;  // the row of the pair edge's position
+  const uint64_t* adj = nullptr;    // and the (unpruned) entry there
 };
 struct Enum {
   using P = EnumP;
@@ -430,7 +433,7 @@ struct Enum {
   static constexpr bool kMore = false;
   static constexpr int kU = 4;
   static constexpr int kRegCap = 64;
-  static __host__ __device__ int smem_bytes(int) { return 0; }
+  static __host__ __device__ int smem_bytes(const P&, int) { return 0; }
   P p;
   __device__ Enum(const P& p_, char*) : p(p_) {}
   __device__ void block_init() {}
@@ -469,10 +472,10 @@ struct Enum {
   __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t s, uint32_t, uint32_t) {
     return make_uint4(slot, (uint32_t)((int32_t)quv * (int32_t)qvw), s, 0u);
   }
-  __device__ __forceinline__ void take(bool on, uint32_t, uint4 it, uint32_t, uint32_t x, uint32_t quw, uint32_t,
+  __device__ __forceinline__ void take(bool on, uint32_t, uint4 it, uint32_t, uint32_t, uint32_t quw, uint32_t,
                                        uint32_t w) {
     emit(on, item_product(it.y, quw), [&](uint32_t& a, uint32_t& b, uint32_t& c) {
-      a = p.vid[x];
+      a = p.vid[adj_col(p.adj[it.z])];
       b = p.vid[p.rowid[it.z]];
       c = p.vid[w];
     });
@@ -496,39 +499,34 @@ struct ExpectP {
   unsigned long long* sum_lo;   // 128-bit sum
   unsigned long long* sum_hi;
 };
-// FIXED: sum of P exactly.  REAL: sum of S = s_uv s_uw s_vw, each s a 2^-30
-// fixed-point integer: s_uv s_uw is exact in int64 (2^-60), rounded to 2^-30,
-// times s_vw exact (2^-60), rounded to 2^-32; summed in 128-bit integers.
+// FIXED: sum of P exactly.  REAL: sum of S = s_uv s_vw s_uw, each s a 2^-30
+// fixed-point integer: s_uv s_vw is exact in int64 (2^-60), rounded to 2^-30,
+// times s_uw exact (2^-60), rounded to 2^-32; summed in 128-bit integers.
 template <bool kReal>
 struct Expect {
   using P = ExpectP;
   static constexpr bool kPos = false;
-  using Item = uint4;  // table slot, the pair's and the streamed edge's values
+  using Item = uint2;  // table slot, the product of the pair's and the streamed edge's values
   static constexpr bool kMore = false;
   static constexpr int kU = 4;
   static constexpr int kRegCap = 64;
-  static __host__ __device__ int smem_bytes(int) { return 0; }
+  static __host__ __device__ int smem_bytes(const P&, int) { return 0; }
   P p;
   Acc128 acc;
   unsigned long long cnt = 0;
   __device__ Expect(const P& p_, char*) : p(p_) {}
   __device__ void block_init() {}
-  __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t, uint32_t, uint32_t) {
-    return make_uint4(slot, quv, qvw, 0u);
+  __device__ __forceinline__ static uint2 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t, uint32_t, uint32_t) {
+    if (!kReal) return make_uint2(slot, (uint32_t)((int32_t)quv * (int32_t)qvw));
+    const long long p60 = (long long)(int32_t)quv * (int32_t)qvw;  // 2^-60
+    return make_uint2(slot, (uint32_t)(int32_t)((p60 + (1ll << 29)) >> 30));  // 2^-30, |.| <= 2^30
   }
-  __device__ __forceinline__ void take(bool on, uint32_t, uint4 it, uint32_t, uint32_t, uint32_t quw, uint32_t,
+  __device__ __forceinline__ void take(bool on, uint32_t, uint2 it, uint32_t, uint32_t, uint32_t quw, uint32_t,
                                        uint32_t) {
     if (!on) return;
-    const uint32_t quv = it.y, qvw = it.z;
     cnt++;
-    if (kReal) {
-      const long long a = (long long)(int32_t)quv * (int32_t)quw;          // 2^-60
-      const long long a30 = (a + (1ll << 29)) >> 30;                        // 2^-30
-      const long long s60 = a30 * (long long)(int32_t)qvw;                  // 2^-60
-      acc.add((s60 + (1ll << 27)) >> 28);                                   // 2^-32
-    } else {
-      acc.add(tri_product(quv, quw, qvw));
-    }
+    const long long x = item_product(it.y, quw);  // FIXED: P; REAL: 2^-60
+    acc.add(kReal ? (x + (1ll << 27)) >> 28 : x);  // REAL: 2^-32
   }
   __device__ void task_begin(uint32_t) {}
   __device__ void task_end(uint32_t) {}
@@ -578,7 +576,7 @@ struct Adjoint {
   static constexpr bool kMore = true;
   static constexpr int kU = 2;
   static constexpr int kRegCap = 64;
-  static __host__ __device__ int smem_bytes(int) { return 0; }
+  static __host__ __device__ int smem_bytes(const P&, int) { return 0; }
   P p;
   __device__ Adjoint(const P& p_, char*) : p(p_) {}
   __device__ void block_init() {}
@@ -630,7 +628,7 @@ __global__ void k_trav_stats(TravArgs a, unsigned long long* out) {
     uint32_t rs = 0, len = 0, ps = 0, np = 0;
     if (!owner_list(a, (uint32_t)x, rs, len) || !pair_range(a, (uint32_t)x, ps, np) || len == 0 || np == 0) continue;
     if (lane == 0) {
-      tab += len;
+      tab += ps < a.merge_first ? len : 0u;  // merged pairs have no table
       tasks += 1;
     }
     for (uint32_t i = 0; i < np; i += 32) {
@@ -681,6 +679,7 @@ ubt_status make_trav_args(const ubt_graph* g, int64_t L, cudaStream_t s, TravArg
   }
   a.vgraph = g->vgraph;
   a.gstart = g->gstart;
+  a.merge_first = (uint32_t)g->merge_first;
   a.n = (uint32_t)g->n;
   a.m = (uint32_t)g->m;
   a.sc = g->scratch;
@@ -883,6 +882,7 @@ ubt_status enumerate_impl(ubt_graph* g, double tau, int32_t which, int32_t prune
   if (!aeo) {
     p.vid = g->vid;
     p.rowid = g->rowid;
+    p.adj = g->adj;
   }
   ubt_status st = aeo ? launch_aeo<Enum>(g, lv.L, p, s) : launch_traverse<Enum>(g, p, prune ? lv.L : 0, s);
   if (st != UBT_OK) return st;
@@ -1042,7 +1042,7 @@ ubt_status count_levels(const ubt_graph* g, const std::vector<int64_t>& lev, int
 ubt_status enum_range(const ubt_graph* g, int which, int64_t B, int64_t Blo, int64_t U, int64_t Uhi, int64_t L,
                       ubt_tri_rec* r, int64_t cap, int64_t* found, cudaStream_t s) {
   EnumP p{B, U, which, r, (unsigned long long)std::max<int64_t>(cap, 0), &g->scratch->enum_cursor, Blo, Uhi,
-          g->vid, g->rowid};
+          g->vid, g->rowid, g->adj};
   ubt_status st = launch_traverse<Enum>(g, p, L, s);
   if (st != UBT_OK) return st;
   unsigned long long f = 0;

@@ -34,6 +34,12 @@
 //       hub     long list or heavy streamed work: whole block, warps take
 //               `unit` pairs at a time (bitmap or hash table)
 //       medium  the rest: one warp, its own table (bitmap or hash)
+//   * Owners of degree at most 32, the last in the numbering, have no table:
+//     their pairs, consecutive in the pair array, are merged, one pair a lane
+//     (both lists hold at most 32 entries).  They are most of the owners -- 2.1
+//     of 2.5 million tasks, but 20 % of the pairs, of a Chung-Lu graph of 4e6
+//     vertices -- and a warp task costs some 700 instructions before its first
+//     probe.
 //   * Probability pruning (FIXED graphs, level L > 0): an edge with |q_e| 2^30
 //     < L is in no triangle with |P| >= L (Lemma 2: the other two factors are
 //     at most 2^15).  Where a level removes enough (prune_pays), the query
@@ -50,7 +56,7 @@
 // instead of the third of the lanes that hits on average (a miss costs only
 // the membership test and its part of the append).
 //
-// Visitors implement: smem_bytes(threads) (shared memory they need) /
+// Visitors implement: smem_bytes(params, threads) (shared memory they need) /
 // block_init / task_begin / task_end / block_end; item (what is queued of a
 // triangle; with kMore the streamed edge's position too) and take (called by
 // all 32 lanes of a warp, converged, with up to 32 queued triangles, `on` in
@@ -81,6 +87,7 @@ struct TravArgs {
   uint32_t n_tasks[kTaskClasses];
   const uint32_t* vgraph;      // batch: graph of every vertex and first vertex of every graph (else null)
   const uint32_t* gstart;
+  uint32_t merge_first;     // pairs [merge_first, m) are merged
   uint32_t n, m;            // vertices, edges (bounds of the self-checks)
   Scratch* sc;              // task counters (zeroed before launch)
   uint32_t* gtab;           // giant tables: gtab_blocks x gtab_slots x 3 words
@@ -104,6 +111,16 @@ template <class V, class = void>
 struct HasProbed : std::false_type {};
 template <class V>
 struct HasProbed<V, std::void_t<decltype(std::declval<V&>().probed(0u))>> : std::true_type {};
+
+// the fewest threads of the main kernel's blocks a visitor wants (kMinThreads)
+template <class V, class = void>
+struct MinThreads {
+  static constexpr int value = 64;
+};
+template <class V>
+struct MinThreads<V, std::void_t<decltype(V::kMinThreads)>> {
+  static constexpr int value = V::kMinThreads;
+};
 
 // Self-checks record the first violated invariant in Scratch::guard and skip
 // the offending access: 1 probe limit (find), 2 probe limit (insert),
@@ -239,7 +256,8 @@ __host__ __device__ constexpr uint32_t table_words(uint32_t slots) {
 // past a full home bucket -- rare, at most 1/4 of the slots are used -- is
 // entered by the whole warp only when some lane needs it, so that the common
 // case runs without a divergent branch.
-__device__ __forceinline__ bool table_slot_warp(const Table& t, uint32_t w, uint32_t& slot, Scratch* sc) {
+template <class T>
+__device__ __forceinline__ bool table_slot_warp(const T& t, uint32_t w, uint32_t& slot, Scratch* sc) {
   uint32_t b = hash_slot(w, t.shift);
   const uint4 k = reinterpret_cast<const uint4*>(t.key)[b];
   const bool m0 = k.x == w, m1 = k.y == w, m2 = k.z == w, m3 = k.w == w;
@@ -366,6 +384,62 @@ __device__ __forceinline__ void entry(const BitTable& t, uint32_t slot, uint32_t
   pos = t.rs + at;
   w = slot;
 }
+// A warp task's hash table: keys in 4-slot buckets and every key's list index;
+// values come from the list itself, in L1 (6 bytes a slot instead of 8, or 12
+// with CSR positions: the warp tables' shared memory is taken from L1, which
+// the streamed rows need; Chung-Lu of 4e6 vertices, forward + backward: 7.4 -> 6.5 ms).
+struct ListTable {
+  uint32_t* key;
+  uint16_t* at;
+  const uint64_t* list;
+  uint32_t rs;     // CSR position of the list
+  uint32_t bmask;  // buckets - 1
+  int shift;
+};
+__host__ __device__ inline size_t list_table_bytes(uint32_t slots) { return (size_t)slots * 6; }
+__device__ __forceinline__ ListTable list_table_at(uint32_t* base, uint32_t slots, const uint64_t* adj, uint32_t rs) {
+  ListTable t;
+  t.key = base;
+  t.at = (uint16_t*)(base + slots);
+  t.list = adj + rs;
+  t.rs = rs;
+  const uint32_t nb = slots >> 2;
+  t.bmask = nb - 1;
+  t.shift = 32 - (31 - __clz((int)nb));
+  return t;
+}
+__device__ __forceinline__ void list_table_insert(const ListTable& t, uint32_t i, Scratch* sc) {
+  const uint32_t w = adj_col(t.list[i]);
+  uint32_t b = hash_slot(w, t.shift);
+  for (uint32_t it = 0; it <= t.bmask; it++) {
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (atomicCAS(&t.key[4 * b + k], kEmpty, w) == kEmpty) {
+        t.at[4 * b + k] = (uint16_t)i;
+        return;
+      }
+    }
+    b = (b + 1) & t.bmask;
+  }
+  guard_fail(sc, kGuardInsert, w);
+}
+template <bool kPos>
+__device__ __forceinline__ void entry(const ListTable& t, uint32_t slot, uint32_t& val, uint32_t& pos, uint32_t& w) {
+  const uint32_t i = t.at[slot];
+  val = adj_valbits(t.list[i]);
+  pos = t.rs + i;
+  w = t.key[slot];
+}
+__device__ __forceinline__ uint32_t none(const ListTable&) { return 0; }
+template <int U>
+__device__ __forceinline__ void find(const ListTable& t, const uint64_t (&e)[U], const bool (&act)[U], bool (&hit)[U],
+                                     uint32_t (&slot)[U], Scratch* sc) {
+#pragma unroll
+  for (int i = 0; i < U; i++) {
+    const bool found = table_slot_warp(t, adj_col(e[i]), slot[i], sc);
+    hit[i] = act[i] && found;
+  }
+}
 __device__ __forceinline__ uint32_t none(const Table&) { return 0; }
 template <int U>
 __device__ __forceinline__ void find(const Table& t, const uint64_t (&e)[U], const bool (&act)[U], bool (&hit)[U],
@@ -382,6 +456,12 @@ __device__ __forceinline__ void entry(const Table& t, uint32_t slot, uint32_t& v
   pos = kPos ? t.pos[slot] : 0u;
   w = t.key[slot];
 }
+
+// entries a lane probes at a time in a long list, at most
+template <class T>
+struct ProbeWidth {
+  static constexpr int value = 4;
+};
 
 // ------------------------------------------------------------ the queue of hits
 
@@ -510,15 +590,16 @@ __device__ __forceinline__ void probe_pairs(const TravArgs& a, V& vis, Queue<V>&
     const uint32_t pj = __shfl_sync(kFull, pr.pe, j);
     uint32_t left = dvj, pos = vsj + lane;
     const uint64_t* __restrict__ row = adj + vsj + lane;
-    while (left >= 32 * V::kU) {
-      long_steps<V, T, V::kU, true>(row, pos, left, sc, vis, queue, t, lane, pr.x, sj, qj, pj);
-      row += 32 * V::kU;
-      pos += 32 * V::kU;
-      left -= 32 * V::kU;
+    constexpr int kU = V::kU < ProbeWidth<T>::value ? V::kU : ProbeWidth<T>::value;
+    while (left >= 32 * kU) {
+      long_steps<V, T, kU, true>(row, pos, left, sc, vis, queue, t, lane, pr.x, sj, qj, pj);
+      row += 32 * kU;
+      pos += 32 * kU;
+      left -= 32 * kU;
     }
     if (tail_short) {
       // full half-chunk, then the rest (< 64 entries) is streamed with the short lists
-      if (V::kU > 2 && left >= 64) {
+      if (kU > 2 && left >= 64) {
         long_steps<V, T, 2, true>(row, pos, left, sc, vis, queue, t, lane, pr.x, sj, qj, pj);
         left -= 64;
       }
@@ -572,8 +653,8 @@ __device__ __forceinline__ void probe_pairs(const TravArgs& a, V& vis, Queue<V>&
   if constexpr (HasProbed<V>::value) vis.probed(probed + total);
 }
 
-// This lane's pair among the pairs [ps, ps + cnt) of owner x.  The pair edge's
-// entry is the one right after its streamed entries.
+// This lane's pair among the pairs [ps, ps + cnt) of owner x (kEmpty: of any
+// owner).  The pair edge's entry is the one right after its streamed entries.
 __device__ __forceinline__ Pair owner_pair(const TravArgs& a, uint32_t x, uint32_t ps, uint32_t cnt) {
   const int lane = (int)lane_id();
   Pair pr;
@@ -599,7 +680,8 @@ __device__ __forceinline__ Pair owner_pair(const TravArgs& a, uint32_t x, uint32
   if (pr.dv) {
     const uint64_t e = a.adj[pr.pe];
     pr.qe = adj_valbits(e);
-    if (adj_col(e) != x) {
+    if (x == kEmpty) pr.x = adj_col(e);
+    if (adj_col(e) != pr.x) {
       guard_fail(a.sc, kGuardVertex, x);
       pr.dv = 0;
     }
@@ -745,17 +827,14 @@ __device__ __forceinline__ void warp_task_hash(const TravArgs& a, V& vis, Queue<
     if (lane == 0) guard_fail(a.sc, kGuardTable, x);
     return;
   }
-  const Table t = make_table(tab, a.warp_slots, slots);
+  const ListTable t = list_table_at(tab, slots, a.adj, rs);
   for (uint32_t i = lane; i < slots; i += 32) t.key[i] = kEmpty;
   __syncwarp();
-  for (uint32_t i = lane; i < len; i += 32) {
-    const uint64_t e = a.adj[rs + i];
-    table_insert<V::kPos>(t, adj_col(e), adj_valbits(e), rs + i, a.sc);
-  }
+  for (uint32_t i = lane; i < len; i += 32) list_table_insert(t, i, a.sc);
   __syncwarp();
   vis.task_begin(x);
   for (uint32_t cs = 0; cs < np; cs += 32)
-    probe_pairs<V, Table>(a, vis, queue, t, owner_pair(a, x, ps + cs, min(32u, np - cs)));
+    probe_pairs<V, ListTable>(a, vis, queue, t, owner_pair(a, x, ps + cs, min(32u, np - cs)));
   queue.take_all(t, vis, x);
   vis.task_end(x);
   __syncwarp();
@@ -782,15 +861,64 @@ __device__ __forceinline__ void warp_task_bits(const TravArgs& a, V& vis, Queue<
   __syncwarp();
 }
 
+// Pairs merged lane by lane: the "slot" of a hit is the position of x-w in
+// x's list.
+struct MergeTable {
+  const uint64_t* adj;
+};
+template <bool kPos>
+__device__ __forceinline__ void entry(const MergeTable& t, uint32_t slot, uint32_t& val, uint32_t& pos, uint32_t& w) {
+  const uint64_t e = t.adj[slot];
+  val = adj_valbits(e);
+  pos = slot;
+  w = adj_col(e);
+}
+constexpr uint32_t kMergeGrab = 256;  // pairs a warp takes at a time
+template <class V>
+__device__ __forceinline__ void merge_tasks(const TravArgs& a, V& vis, Queue<V>& queue) {
+  const uint32_t lane = lane_id(), lt = lanemask_lt(), npairs = a.m - a.merge_first;
+  const MergeTable t{a.adj};
+  const uint64_t* __restrict__ adj = a.adj;
+  while (true) {
+    unsigned long long t0 = 0;
+    if (lane == 0) t0 = atomicAdd(&a.sc->task[7], (unsigned long long)kMergeGrab);
+    t0 = __shfl_sync(kFull, t0, 0);
+    if (t0 >= npairs) break;
+    for (uint32_t p0 = (uint32_t)t0; p0 < min((unsigned long long)npairs, t0 + kMergeGrab); p0 += 32) {
+      const Pair pr = owner_pair(a, kEmpty, a.merge_first + p0, min(32u, npairs - p0));
+      uint32_t dv = pr.dv, rs = 0, len = 0, i = 0, j = 0;
+      if (dv && (pr.x >= a.n || !owner_list(a, pr.x, rs, len))) {
+        guard_fail(a.sc, kGuardList, pr.x);
+        len = 0;
+      }
+      uint64_t ea = dv ? adj[pr.vs] : 0ull, eb = len ? adj[rs] : 0ull;
+      uint32_t steps = 0;  // at most the entries of both lists, which the queue's appends bound
+      while (__any_sync(kFull, i < dv && j < len)) {
+        const bool act = i < dv && j < len;
+        const uint32_t ca = adj_col(ea), cb = adj_col(eb);
+        const bool hit = act && ca == cb;
+        if (__any_sync(kFull, hit)) {
+          queue.append(hit, V::item(rs + j, pr.qe, adj_valbits(ea), pr.s, pr.pe, pr.vs + i), pr.vs + i, lt);
+          queue.take_full(t, vis, pr.x);
+        }
+        if (act && ca <= cb && ++i < dv) ea = adj[pr.vs + i];
+        if (act && cb <= ca && ++j < len) eb = adj[rs + j];
+        steps++;
+      }
+      if constexpr (HasProbed<V>::value) vis.probed(32 * steps);
+    }
+  }
+  queue.take_all(t, vis, kEmpty);
+}
+
 // The traversal runs as up to two persistent kernels: the rare block tasks
 // with hash tables, and everything else -- the block tasks with bitmaps, then
 // the warp tasks -- in one, so that a block that finds no more block tasks goes
 // on to warp tasks instead of idling until the last one ends.
 enum : int { kHashKernel = 0, kMainKernel = 1 };
 
-template <class V>
 __host__ __device__ inline size_t warp_table_bytes(const TravArgs& a) {
-  const size_t h = a.n_tasks[kMedHash] ? (size_t)table_words<V>(a.warp_slots) * 4 : 0;
+  const size_t h = a.n_tasks[kMedHash] ? list_table_bytes(a.warp_slots) : 0;
   const size_t b = a.n_tasks[kMedBits] ? bit_table_bytes(a.warp_bits, a.warp_len) : 0;
   return h > b ? h : b;
 }
@@ -799,11 +927,11 @@ template <class V>
 inline size_t traverse_table_bytes(const TravArgs& a, int kernel, int threads) {
   if (kernel == kHashKernel) return a.n_tasks[kHubHash] ? (size_t)table_words<V>(a.hub_slots) * 4 : 0;
   const size_t hub = a.n_tasks[kHubBits] ? bit_table_bytes(a.hub_bits, a.hub_len) : 0;
-  return std::max(hub, (size_t)(threads / 32) * warp_table_bytes<V>(a));
+  return std::max(hub, (size_t)(threads / 32) * warp_table_bytes(a));
 }
 template <class V>
-__host__ __device__ inline size_t visitor_bytes(int threads) {
-  return (size_t)((V::smem_bytes(threads) + 15) / 16) * 16 + (size_t)(threads / 32) * Queue<V>::kBytes;
+__host__ __device__ inline size_t visitor_bytes(const typename V::P& p, int threads) {
+  return (size_t)((V::smem_bytes(p, threads) + 15) / 16) * 16 + (size_t)(threads / 32) * Queue<V>::kBytes;
 }
 
 // The next block task of a class (the same in every thread); n_tasks if none.
@@ -861,7 +989,7 @@ __device__ void traverse(const TravArgs& a, V& vis, char* queues, char* tables) 
         block_task_bits(a, vis, queue, a.lists[kHubBits][task], bt, s_misc);
       }
     }
-    char* mine = tables + (size_t)wid * warp_table_bytes<V>(a);
+    char* mine = tables + (size_t)wid * warp_table_bytes(a);
     if (a.n_tasks[kMedBits]) {
       const BitTable bt = bit_table_at(mine, a.warp_bits, a.warp_len);
       for (uint32_t i = lane; i < bit_words(a.warp_bits); i += 32) bt.bits[i] = 0;
@@ -871,6 +999,7 @@ __device__ void traverse(const TravArgs& a, V& vis, char* queues, char* tables) 
     }
     if (a.n_tasks[kMedHash])
       warp_tasks(a, kMedHash, [&](uint32_t x) { warp_task_hash(a, vis, queue, x, (uint32_t*)mine); });
+    if (a.merge_first < a.m) merge_tasks(a, vis, queue);
   }
   __syncthreads();
   vis.block_end();
@@ -883,7 +1012,7 @@ namespace {
 // registers).
 template <class V, int kKernel>
 struct Bounds {
-  static constexpr int kThreads = 512;
+  static constexpr int kThreads = kKernel == kHashKernel ? 512 : 256;
   static constexpr int kMinBlocks = 65536 / (kThreads * V::kRegCap) > 0 ? 65536 / (kThreads * V::kRegCap) : 1;
 };
 
@@ -894,15 +1023,15 @@ __global__ void __launch_bounds__(Bounds<V, kKernel>::kThreads, Bounds<V, kKerne
   V vis(p, smem);
   vis.block_init();
   __syncthreads();
-  char* queues = smem + ((V::smem_bytes((int)blockDim.x) + 15) / 16) * 16;
-  traverse<V, kKernel>(a, vis, queues, smem + visitor_bytes<V>((int)blockDim.x));
+  char* queues = smem + ((V::smem_bytes(p, (int)blockDim.x) + 15) / 16) * 16;
+  traverse<V, kKernel>(a, vis, queues, smem + visitor_bytes<V>(p, (int)blockDim.x));
 }
 
 // Warps of a kernel that fit on an SM: by registers (65536) and shared memory
 // (227 KB, 1 KB of it per block taken by the system).
 template <class V, int kKernel>
-int resident_warps(const TravArgs& a, int threads) {
-  const size_t smem = visitor_bytes<V>(threads) + traverse_table_bytes<V>(a, kKernel, threads) + 1024;
+int resident_warps(const TravArgs& a, const typename V::P& p, int threads) {
+  const size_t smem = visitor_bytes<V>(p, threads) + traverse_table_bytes<V>(a, kKernel, threads) + 1024;
   const int blocks = (int)std::min<size_t>((227 * 1024 + 1024) / smem, 65536 / (size_t)(threads * V::kRegCap));
   return blocks * threads / 32;
 }
@@ -911,16 +1040,16 @@ template <class V, int kKernel>
 ubt_status launch_kernel(const ubt_graph* g, const TravArgs& a, const typename V::P& p, cudaStream_t s) {
   const Tuning& T = tuning();
   int threads = (int)(kKernel == kHashKernel ? T.block_threads : T.warp_threads);
-  threads = (int)std::min<int64_t>(Bounds<V, kKernel>::kThreads, std::max<int64_t>(64, threads / 32 * 32));
+  threads = (int)std::min<int64_t>(Bounds<V, kKernel>::kThreads, std::max<int64_t>(MinThreads<V>::value, threads / 32 * 32));
   // Larger blocks share the block tasks' table among more warps; smaller ones
   // lose less at its barriers.  Twice the threads where the table's size would
   // otherwise leave fewer than 7/8 of the warps they make room for (R-MAT scale
   // 22, tables of 26 KB: 19.8 -> 17.0 ms with 256 threads; Chung-Lu of 1e6
   // vertices, tables of 4 KB: 1.15 ms with 128, 1.21 with 256).
   if (kKernel == kMainKernel && 2 * threads <= Bounds<V, kKernel>::kThreads &&
-      8 * resident_warps<V, kKernel>(a, threads) < 7 * resident_warps<V, kKernel>(a, 2 * threads))
+      8 * resident_warps<V, kKernel>(a, p, threads) < 7 * resident_warps<V, kKernel>(a, p, 2 * threads))
     threads *= 2;
-  const size_t smem = visitor_bytes<V>(threads) + traverse_table_bytes<V>(a, kKernel, threads);
+  const size_t smem = visitor_bytes<V>(p, threads) + traverse_table_bytes<V>(a, kKernel, threads);
   UBT_CUDA(cudaFuncSetAttribute(k_traverse<V, kKernel>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse<V, kKernel>, threads, smem));
@@ -939,7 +1068,7 @@ ubt_status launch_traversal(const ubt_graph* g, const TravArgs& a, const typenam
   UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
   ubt_status st = UBT_OK;
   if (a.n_tasks[kGiant] + a.n_tasks[kHubHash]) st = launch_kernel<V, kHashKernel>(g, a, p, s);
-  if (st == UBT_OK && a.n_tasks[kHubBits] + a.n_tasks[kMedHash] + a.n_tasks[kMedBits])
+  if (st == UBT_OK && a.n_tasks[kHubBits] + a.n_tasks[kMedHash] + a.n_tasks[kMedBits] + (a.m - a.merge_first))
     st = launch_kernel<V, kMainKernel>(g, a, p, s);
   return st;
 }

@@ -156,13 +156,31 @@ struct Planes {
 #pragma unroll
     for (int t = 0; t < K; t++) c[t] = 0;
   }
-  __device__ __forceinline__ void inc(unsigned long long b) {
+  // one word of weight 2^from
+  __device__ __forceinline__ void inc(unsigned long long b, int from) {
 #pragma unroll
     for (int t = 0; t < K; t++) {
+      if (t < from) continue;
       const unsigned long long carry = c[t] & b;
       c[t] ^= b;
       b = carry;
-      if (!b) break;
+    }
+  }
+  // All lanes' counters summed (32 lanes: 5 more planes), bit-sliced all the way:
+  // every lane ends with the totals of all 64 counters in t[0 .. K + 4].
+  __device__ __forceinline__ void warp_total(unsigned long long (&t)[K + 5]) const {
+#pragma unroll
+    for (int i = 0; i < K + 5; i++) t[i] = i < K ? c[i] : 0ull;
+#pragma unroll
+    for (int r = 0; r < 5; r++) {
+      unsigned long long carry = 0;
+#pragma unroll
+      for (int i = 0; i < K + r; i++) {
+        const unsigned long long o = __shfl_xor_sync(kFull, t[i], 1 << r), x = t[i];
+        t[i] = x ^ o ^ carry;
+        carry = (x & o) | (x & carry) | (o & carry);
+      }
+      t[K + r] = carry;
     }
   }
   // eight words at once (K > 3): a carry-save tree, three full adders' worth of
@@ -218,10 +236,13 @@ struct Worlds {
   static constexpr int kU = 2;
   static constexpr bool kPos = true;
   static constexpr int kRegCap = 128;
+  // a block's counters are 32 KB that L1, where the owner's sign rows stay, loses
+  // (R-MAT scale 20, 4,096 worlds: 94.7 ms in blocks of 128 threads, 76.7 of 256)
+  static constexpr int kMinThreads = 256;
   static constexpr int K = SLOTS == 1 ? 14 : 12;      // planes per slot
   static constexpr uint32_t kLimit = (1u << K) - 1u;  // increments before a flush
   // counters + one list of 32 triangles per warp
-  static __host__ __device__ int smem_bytes(int threads) { return 64 * 64 * 8 + (threads / 32) * 96 * 4; }
+  static __host__ __device__ int smem_bytes(const P&, int threads) { return 64 * 64 * 8 + (threads / 32) * 96 * 4; }
   P p;
   unsigned long long* cnt;  // shared: wp * 64 counters
   uint32_t* q;              // shared: this warp's triangles, 3 x 32 positions
@@ -365,29 +386,70 @@ struct Batch {
   using Item = uint4;  // table slot, product of two values, positions of the pair edge and the streamed edge
   static constexpr bool kMore = false;
   static constexpr int kU = 2;
-  static constexpr int kRegCap = 128;
-  static __host__ __device__ int smem_bytes(int) { return 0; }
-  static constexpr int K = 8;
+  // 24 warps an SM instead of 16: the triangles' sign words and list entries are
+  // waited on (batch of 1,000 graphs: 9.9 ms with up to 128 registers, 8.7 with 85, 9.0 with 64)
+  static constexpr int kRegCap = 85;
+  static __host__ __device__ int smem_bytes(const P&, int) { return 0; }
+  static constexpr int K = 8;                        // planes: fewer than 256 words between two flushes
+  static constexpr uint32_t kSumLimit = 1u << 17;    // |P| <= 2^45: so many fit a signed 64-bit sum
   P p;
   uint32_t g = kEmpty;
   uint32_t bal[kBatchTau], unbal[kBatchTau];
   uint32_t tri = 0;
-  unsigned long long lo = 0, hi = 0;
+  long long sum = 0;
   Planes<K> pl;
-  uint32_t since = 0;
-  __device__ Batch(const P& p_, char*) : p(p_) { reset(); }
-  __device__ void reset() {
+  unsigned long long ones = 0, twos = 0, fours = 0;  // words of weight 1, 2, 4 waiting for their second
+  uint32_t since = 0, sums = 0;                      // triangles taken since the last flush (warp-uniform)
+  __device__ Batch(const P& p_, char*) : p(p_) {
 #pragma unroll
     for (int i = 0; i < kBatchTau; i++) bal[i] = unbal[i] = 0;
-    tri = 0;
-    lo = hi = 0;
+    pl.clear();
+  }
+  __device__ void block_init() {}
+  // the world counters to the graph's counts: words still waiting go in first
+  __device__ __forceinline__ void flush_worlds() {
+    if (!since) return;
+    pl.inc(since & 1u ? ones : 0ull, 0);
+    pl.inc(since & 2u ? twos : 0ull, 1);
+    pl.inc(since & 4u ? fours : 0ull, 2);
+    unsigned long long t[K + 5];
+    pl.warp_total(t);
+    const int lane = (int)lane_id();
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const int j = lane + 32 * h;
+      uint32_t v = 0;
+#pragma unroll
+      for (int i = 0; i < K + 5; i++) v |= (uint32_t)((t[i] >> j) & 1ull) << i;
+      if (v) atomicAdd(&p.worlds[(size_t)g * 64 + j], (unsigned long long)v);
+    }
     pl.clear();
     since = 0;
   }
-  __device__ void block_init() {}
+  __device__ __forceinline__ void flush_sums() {
+    const uint32_t t = __reduce_add_sync(kFull, tri);
+    unsigned long long lo = (unsigned long long)sum, hi = sum < 0 ? ~0ull : 0ull;  // 128-bit warp sum
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const unsigned long long l = __shfl_xor_sync(kFull, lo, d);
+      const unsigned long long h = __shfl_xor_sync(kFull, hi, d);
+      const unsigned long long o = lo;
+      lo += l;
+      hi += h + (lo < o ? 1ull : 0ull);
+    }
+    if (lane_id() == 0 && t) {
+      unsigned long long* a = p.acc + (size_t)g * 3;
+      atomicAdd(&a[0], (unsigned long long)t);
+      const unsigned long long o = atomicAdd(&a[1], lo);
+      atomicAdd(&a[2], hi + ((o + lo < o) ? 1ull : 0ull));
+    }
+    tri = 0;
+    sum = 0;
+    sums = 0;
+  }
   __device__ void flush() {
-    const int lane = (int)lane_id();
     if (g == kEmpty) return;
+    const int lane = (int)lane_id();
 #pragma unroll
     for (int i = 0; i < kBatchTau; i++) {
       if (i < p.nt) {
@@ -397,42 +459,24 @@ struct Batch {
           if (b) atomicAdd(&p.counts[(size_t)g * 2 * p.nt + i], (unsigned long long)b);
           if (u) atomicAdd(&p.counts[(size_t)g * 2 * p.nt + p.nt + i], (unsigned long long)u);
         }
+        bal[i] = unbal[i] = 0;
       }
     }
-    if (p.acc) {
-      const uint32_t t = __reduce_add_sync(kFull, tri);
-      // 128-bit warp sum
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) {
-        const unsigned long long l = __shfl_xor_sync(kFull, lo, d);
-        const unsigned long long h = __shfl_xor_sync(kFull, hi, d);
-        const unsigned long long o = lo;
-        lo += l;
-        hi += h + (lo < o ? 1ull : 0ull);
-      }
-      if (lane == 0 && t) {
-        unsigned long long* a = p.acc + (size_t)g * 3;
-        atomicAdd(&a[0], (unsigned long long)t);
-        const unsigned long long o = atomicAdd(&a[1], lo);
-        atomicAdd(&a[2], hi + ((o + lo < o) ? 1ull : 0ull));
-      }
-    }
-    if (p.worlds) {
-      for (int j = 0; j < 64; j++) {
-        const uint32_t v = __reduce_add_sync(kFull, pl.count(j));
-        if (lane == (j & 31) && v) atomicAdd(&p.worlds[(size_t)g * 64 + j], (unsigned long long)v);
-      }
-    }
-    reset();
+    if (p.acc) flush_sums();
+    if (p.worlds) flush_worlds();
   }
   __device__ __forceinline__ static uint4 item(uint32_t slot, uint32_t quv, uint32_t qvw, uint32_t, uint32_t puv,
                                                uint32_t pvw) {
     return make_uint4(slot, (uint32_t)((int32_t)quv * (int32_t)qvw), puv, pvw);
   }
+  // One triangle a lane.  The world words go through carry-save adders a pair
+  // at a time (`since` says which weights wait for their second word), so a
+  // word costs two adders on average instead of a carry chain up the planes.
   __device__ __forceinline__ void take(bool on, uint32_t, uint4 it, uint32_t, uint32_t, uint32_t quw, uint32_t puw,
                                        uint32_t) {
+    unsigned long long x = 0ull;
     if (on) {
-      const uint32_t puv = it.z, pvw = it.w;
+      if (p.X) x = p.X[it.z] ^ p.X[puw] ^ p.X[it.w];
       const int64_t P = (int64_t)(int32_t)it.y * (int64_t)(int32_t)quw;
 #pragma unroll
       for (int i = 0; i < kBatchTau; i++) {
@@ -442,22 +486,27 @@ struct Batch {
         }
       }
       tri++;
-      const unsigned long long o = lo;
-      lo += (unsigned long long)P;
-      hi += (P < 0 ? ~0ull : 0ull) + (lo < o ? 1ull : 0ull);
-      if (p.X) pl.inc(p.X[puv] ^ p.X[puw] ^ p.X[pvw]);
+      sum += P;
     }
-    // a lane's counters grow by at most one per call
-    if (++since == (1u << K) - 1u) {
-      if (p.X) {
-        const int lane = (int)lane_id();
-        for (int j = 0; j < 64; j++) {
-          const uint32_t v = __reduce_add_sync(kFull, pl.count(j));
-          if (lane == (j & 31) && v && g != kEmpty) atomicAdd(&p.worlds[(size_t)g * 64 + j], (unsigned long long)v);
+    if (++sums == kSumLimit && p.acc) flush_sums();
+    if (p.X) {
+      if (!(since & 1u)) {
+        ones = x;
+      } else {
+        Planes<K>::csa(x, pl.c[0], ones, x);
+        if (!(since & 2u)) {
+          twos = x;
+        } else {
+          Planes<K>::csa(x, pl.c[1], twos, x);
+          if (!(since & 4u)) {
+            fours = x;
+          } else {
+            Planes<K>::csa(x, pl.c[2], fours, x);
+            pl.inc(x, 3);
+          }
         }
-        pl.clear();
       }
-      since = 0;
+      if (++since == (1u << K) - 8u) flush_worlds();  // a multiple of 8: nothing waits
     }
   }
   __device__ void task_begin(uint32_t u) {
