@@ -310,6 +310,7 @@ struct AeoIxArgs {
   const uint64_t* uadj;
   const uint32_t* uepos;      // 2m: [2e + side] position of edge e in its endpoints' rows
   const uint4* eslots;        // edge index
+  const uint32_t* efilter;
   uint64_t emask;
   int eshift;
   uint32_t n, m, m2;
@@ -331,34 +332,73 @@ __device__ __forceinline__ bool aeo_ix_keep(const AeoIxArgs& a, uint32_t s, uint
   return (oq < aq || (oq == aq && w > s)) && (a.L == 0 || oq * cut >= a.L);
 }
 
-// Two lanes' worth of lookups at once: both home slots are read before
-// either is examined (at most a quarter of the slots are used, so nearly
-// every lookup ends there); the rare longer probe continues alone.
-__device__ __forceinline__ void aeo_ix_hit2(const AeoIxArgs& a, const bool (&act)[2], const uint32_t (&o)[2],
-                                            const uint32_t (&s)[2], const uint32_t (&w)[2], const int64_t (&aq)[2],
-                                            const int64_t (&cut)[2], bool (&hit)[2], uint32_t (&qow)[2]) {
-  uint64_t k[2], h[2];
-  uint4 sl[2];
+// U lookups of a lane at once: their filter words are all read before any is
+// examined, then the home slots of those that pass (at most a quarter of the
+// slots are used, so nearly every lookup ends there); the rare longer probe
+// continues alone.  found[i]: edge o-w exists, with value qow.
+template <int U>
+__device__ __forceinline__ void aeo_ix_find_all(const AeoIxArgs& a, const bool (&act)[U], const uint32_t (&o)[U],
+                                                const uint32_t (&w)[U], bool (&found)[U], uint32_t (&qow)[U]) {
+  uint32_t word[U];
+  uint4 sl[U];
 #pragma unroll
-  for (int i = 0; i < 2; i++) {
-    k[i] = edge_index_key(o[i], w[i]);
-    h[i] = edge_index_home(k[i], a.eshift);
-    sl[i] = (act[i] && w[i] != o[i]) ? a.eslots[h[i]] : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u);
+  for (int i = 0; i < U; i++)
+    word[i] = (act[i] && w[i] != o[i])
+                  ? a.efilter[edge_index_home(edge_index_key(o[i], w[i]), a.eshift + kEdgeFilterLog)] : 0u;
+#pragma unroll
+  for (int i = 0; i < U; i++) {
+    const uint64_t key = edge_index_key(o[i], w[i]);
+    sl[i] = edge_filter_pass(word[i], key) ? a.eslots[edge_index_home(key, a.eshift)]
+                                           : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u);
   }
 #pragma unroll
-  for (int i = 0; i < 2; i++) {
-    hit[i] = false;
-    qow[i] = 0;
-    if (!act[i] || w[i] == o[i]) continue;
+  for (int i = 0; i < U; i++) {
     const uint64_t key = ((uint64_t)sl[i].y << 32) | sl[i].x;
-    bool found = key == k[i];
-    if (found) {
-      qow[i] = sl[i].z;
-    } else if (key != kEdgeIndexEmpty) {  // the home slot holds another edge: probe on
-      found = aeo_ix_find(a, o[i], w[i], qow[i]);
-    }
-    hit[i] = found && aeo_ix_keep(a, s[i], w[i], qow[i], aq[i], cut[i]);
+    qow[i] = sl[i].z;
+    found[i] = key == edge_index_key(o[i], w[i]);
+    if (!found[i] && key != kEdgeIndexEmpty)  // the home slot holds another edge: probe on
+      found[i] = aeo_ix_find(a, o[i], w[i], qow[i]);
   }
+}
+// entries a lane looks up at a time
+constexpr int kAeoU = 4;
+
+// Entries of a |q|-descending list that reach the cutoff, known to lie in [lo, hi].
+__device__ __forceinline__ uint32_t aeo_window(const AeoIxArgs& a, uint32_t at, uint32_t lo, uint32_t hi, int64_t cut) {
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi + 1) >> 1;
+    if (qabs(adj_valbits(a.uadj[at + mid - 1])) * cut >= a.L) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+// The shorter of e's two windows: true for the one at p (of n entries after
+// e), its length up to Lemma 3's cutoff in `len`.  Both are tried at 1, 2, 4,
+// ... entries side by side until one ends, which is then searched between the
+// last two: log2 of the shorter window's length in steps whose loads overlap,
+// not binary searches of two whole rows one after the other.
+__device__ __forceinline__ bool aeo_shorter(const AeoIxArgs& a, uint32_t p, uint32_t n, uint32_t r, uint32_t m,
+                                            int64_t cut, uint32_t& len) {
+  if (a.L == 0) {
+    len = min(n, m);
+    return n <= m;
+  }
+  uint32_t lo = 0, s = 1;  // both windows hold at least lo entries
+  bool first, second;
+  while (true) {  // s doubles: at most 32 times
+    const uint64_t x = s <= n ? a.uadj[p + s - 1] : 0ull, y = s <= m ? a.uadj[r + s - 1] : 0ull;
+    first = s <= n && qabs(adj_valbits(x)) * cut >= a.L;
+    second = s <= m && qabs(adj_valbits(y)) * cut >= a.L;
+    if (!first || !second || s >= (1u << 31)) break;
+    lo = s;
+    s <<= 1;
+  }
+  if (!first) {
+    len = aeo_window(a, p, lo, min(s - 1, n), cut);
+    if (second || (len < m && qabs(adj_valbits(a.uadj[r + len])) * cut >= a.L)) return true;
+    s = len + 1;  // the other one holds at most len
+  }
+  len = aeo_window(a, r, lo, min(s - 1, m), cut);
+  return false;
 }
 
 template <class V>
@@ -393,12 +433,9 @@ __global__ void __launch_bounds__(512, 2) k_aeo_index(AeoIxArgs a, typename V::P
           if (u >= a.n || v >= a.n) guard_fail(a.sc, kGuardVertex, (uint32_t)e);
           ok = false;
         } else {
-          const uint32_t ue = a.uptr[u + 1], ve = a.uptr[v + 1];
-          const uint32_t cu = a.L > 0 ? a.uptr[u] + prune_prefix(a.uadj + a.uptr[u], ue - a.uptr[u], cut, a.L) : ue;
-          const uint32_t cv = a.L > 0 ? a.uptr[v] + prune_prefix(a.uadj + a.uptr[v], ve - a.uptr[v], cut, a.L) : ve;
-          const uint32_t lu = cu > p0 + 1 ? cu - (p0 + 1) : 0u, lv = cv > p1 + 1 ? cv - (p1 + 1) : 0u;
-          if (lu <= lv) { sv = u; o = v; vs = p0 + 1; dv = lu; }
-          else { sv = v; o = u; vs = p1 + 1; dv = lv; }
+          const uint32_t lu = a.uptr[u + 1] - (p0 + 1), lv = a.uptr[v + 1] - (p1 + 1);  // entries after e
+          if (aeo_shorter(a, p0 + 1, lu, p1 + 1, lv, cut, dv)) { sv = u; o = v; vs = p0 + 1; }
+          else { sv = v; o = u; vs = p1 + 1; }
         }
       }
     }
@@ -413,27 +450,24 @@ __global__ void __launch_bounds__(512, 2) k_aeo_index(AeoIxArgs a, typename V::P
       const uint32_t vsj = __shfl_sync(kFull, vs, j), dvj = __shfl_sync(kFull, dv, j);
       const uint32_t qj = __shfl_sync(kFull, qe, j);
       const long long aqj = __shfl_sync(kFull, (long long)aq, j), cj = __shfl_sync(kFull, (long long)cut, j);
-      for (uint32_t off = 0; off < dvj; off += 64) {
-        bool act[2], hit[2];
-        uint32_t oo[2], ss[2], ww[2], qow[2];
-        int64_t aa[2], cc[2];
-        uint64_t ew[2];
+      for (uint32_t off = 0; off < dvj; off += 32 * kAeoU) {
+        bool act[kAeoU], found[kAeoU];
+        uint32_t oo[kAeoU], ww[kAeoU], qw[kAeoU], qow[kAeoU];
 #pragma unroll
-        for (int u = 0; u < 2; u++) {
+        for (int u = 0; u < kAeoU; u++) {
           const uint32_t i = off + 32 * u + lane;
           act[u] = i < dvj;
-          ew[u] = act[u] ? a.uadj[vsj + i] : 0ull;
+          const uint64_t ew = act[u] ? a.uadj[vsj + i] : (uint64_t)oj;
           oo[u] = oj;
-          ss[u] = sj;
-          ww[u] = adj_col(ew[u]);
-          aa[u] = aqj;
-          cc[u] = cj;
+          ww[u] = adj_col(ew);
+          qw[u] = adj_valbits(ew);
         }
-        aeo_ix_hit2(a, act, oo, ss, ww, aa, cc, hit, qow);
+        aeo_ix_find_all<kAeoU>(a, act, oo, ww, found, qow);
 #pragma unroll
-        for (int u = 0; u < 2; u++)
-          if (u == 0 || off + 32 < dvj)
-            vis.step(hit[u], oj, sj, ww[u], qj, qow[u], adj_valbits(ew[u]), 0u, 0u, vsj + off + 32 * u + lane);
+        for (int u = 0; u < kAeoU; u++)
+          if (u == 0 || off + 32 * u < dvj)
+            vis.step(found[u] && aeo_ix_keep(a, sj, ww[u], qow[u], aqj, cj), oj, sj, ww[u], qj, qow[u], qw[u], 0u, 0u,
+                     vsj + off + 32 * u + lane);
       }
     }
     // short windows: concatenated, one entry per lane per step
@@ -446,13 +480,12 @@ __global__ void __launch_bounds__(512, 2) k_aeo_index(AeoIxArgs a, typename V::P
     }
     const uint32_t total = __shfl_sync(kFull, incl, 31);
     const uint32_t excl = incl - ds;
-    for (uint32_t base = 0; base < total; base += 64) {
-      bool act[2], hit[2];
-      uint32_t oo[2], ss[2], ww[2], qq[2], pos[2], qow[2];
-      int64_t aa[2], cc[2];
-      uint64_t ew[2];
+    for (uint32_t base = 0; base < total; base += 32 * kAeoU) {
+      bool act[kAeoU], found[kAeoU];
+      uint32_t oo[kAeoU], ww[kAeoU], qw[kAeoU], qow[kAeoU];
+      int own[kAeoU];
 #pragma unroll
-      for (int u = 0; u < 2; u++) {
+      for (int u = 0; u < kAeoU; u++) {
         const uint32_t f = base + 32 * u + lane;
         act[u] = f < total;
         int j = 0;
@@ -461,22 +494,22 @@ __global__ void __launch_bounds__(512, 2) k_aeo_index(AeoIxArgs a, typename V::P
           const uint32_t tj = __shfl_sync(kFull, incl, j + b - 1);
           if (tj <= f) j += b;
         }
-        j = j > 31 ? 31 : j;
-        const uint32_t vsj = __shfl_sync(kFull, vs, j), exj = __shfl_sync(kFull, excl, j);
-        oo[u] = __shfl_sync(kFull, o, j);
-        ss[u] = __shfl_sync(kFull, sv, j);
-        qq[u] = __shfl_sync(kFull, qe, j);
-        aa[u] = __shfl_sync(kFull, (long long)aq, j);
-        cc[u] = __shfl_sync(kFull, (long long)cut, j);
-        pos[u] = vsj + (f - exj);
-        ew[u] = act[u] ? a.uadj[pos[u]] : 0ull;
-        ww[u] = adj_col(ew[u]);
+        own[u] = j > 31 ? 31 : j;
+        const uint32_t vsj = __shfl_sync(kFull, vs, own[u]), exj = __shfl_sync(kFull, excl, own[u]);
+        oo[u] = __shfl_sync(kFull, o, own[u]);
+        const uint64_t ew = act[u] ? a.uadj[vsj + (f - exj)] : (uint64_t)oo[u];
+        ww[u] = adj_col(ew);
+        qw[u] = adj_valbits(ew);
       }
-      aeo_ix_hit2(a, act, oo, ss, ww, aa, cc, hit, qow);
+      aeo_ix_find_all<kAeoU>(a, act, oo, ww, found, qow);
 #pragma unroll
-      for (int u = 0; u < 2; u++)
-        if (u == 0 || base + 32 < total)
-          vis.step(hit[u], oo[u], ss[u], ww[u], qq[u], qow[u], adj_valbits(ew[u]), 0u, 0u, pos[u]);
+      for (int u = 0; u < kAeoU; u++) {
+        const uint32_t sj = __shfl_sync(kFull, sv, own[u]), qj = __shfl_sync(kFull, qe, own[u]);
+        const int64_t aqj = qabs(qj);
+        if (u == 0 || base + 32 * u < total)
+          vis.step(found[u] && aeo_ix_keep(a, sj, ww[u], qow[u], aqj, aqj * aqj), oo[u], sj, ww[u], qj, qow[u], qw[u],
+                   0u, 0u, 0u);
+      }
     }
   }
   __syncthreads();
@@ -496,6 +529,7 @@ ubt_status launch_aeo(const ubt_graph* g, int64_t L, const typename V::P& p, cud
       a.uadj = g->uadj;
       a.uepos = g->uepos;
       a.eslots = g->eslots;
+      a.efilter = g->efilter;
       a.emask = (uint64_t)g->eh_slots - 1;
       a.eshift = g->eh_shift;
       a.n = (uint32_t)g->n;

@@ -263,57 +263,56 @@ __device__ inline uint64_t key_by_absq(uint64_t e) {
 enum : int { kSortById = 0, kSortByAbsq = 2 };
 
 // Lists of <= 32 entries: one warp per list, bitonic network over the lanes.
-// Bitonic sort of the values held by each aligned group of W lanes (W = 8,
-// 16 or 32), ascending by key within every group.
+// Bitonic sort of the words held by each aligned group of W lanes (W = 8, 16 or
+// 32), ascending within every group.
 template <int W>
-__device__ __forceinline__ void group_bitonic(uint64_t& key, uint64_t& e, uint32_t& id, uint32_t& ky, int lane) {
+__device__ __forceinline__ void group_bitonic(uint64_t& key, int lane) {
   const int li = lane & (W - 1);
 #pragma unroll
   for (int kk = 2; kk <= W; kk <<= 1) {
 #pragma unroll
     for (int j = kk >> 1; j > 0; j >>= 1) {
       const uint64_t ok = __shfl_xor_sync(kFull, key, j);
-      const uint64_t oe = __shfl_xor_sync(kFull, e, j);
-      const uint32_t oi = __shfl_xor_sync(kFull, id, j);
-      const uint32_t oy = __shfl_xor_sync(kFull, ky, j);
       const bool up = (li & kk) == 0;
       const bool lower = (li & j) == 0;
-      const bool take_min = (lower == up);
-      const bool sw = take_min ? (ok < key) : (ok > key);
-      if (sw) { key = ok; e = oe; id = oi; ky = oy; }
+      key = (lower == up) == (ok < key) ? ok : key;
     }
   }
 }
 
 // Sorts the rows of one group of W lanes (row rs..rs+len, len <= W; groups
-// without a row pass in = false everywhere), as `mode` says.
+// without a row pass row = false everywhere), as `mode` says.  The network
+// moves one word per comparator, the sort key << 5 | the entry's lane (the
+// words are distinct), and the entries follow once at the end.
 template <int W>
 __device__ __forceinline__ void sort_group_row(uint64_t* adj, uint32_t* eid, uint32_t* ekey, uint32_t rs, uint32_t len,
                                                bool row, int mode, unsigned long long* err, int lane) {
   const int li = lane & (W - 1);
   const bool in = row && (uint32_t)li < len;
-  uint64_t e = in ? adj[rs + li] : ~0ull;
-  uint32_t id = in ? eid[rs + li] : 0u;
-  uint32_t ky = (in && ekey) ? ekey[rs + li] : 0u;
+  const uint64_t e = in ? adj[rs + li] : 0ull;
+  const uint32_t id = in ? eid[rs + li] : 0u;
+  const uint32_t ky = (in && ekey) ? ekey[rs + li] : 0u;
+  uint64_t key = in ? ((mode == kSortById ? key_by_col(e) : key_by_absq(e)) << 5) | (uint64_t)lane
+                    : (~0ull << 5) | (uint64_t)lane;
+  group_bitonic<W>(key, lane);
   if (mode == kSortById) {
-    uint64_t key = in ? key_by_col(e) : ~0ull;
-    group_bitonic<W>(key, e, id, ky, lane);
-    const uint64_t prev = __shfl_up_sync(kFull, key, 1);
-    if (in && li > 0 && prev == key) report(err, rs + li, -UBT_ERR_DUPLICATE_EDGE);
-  } else {
-    uint64_t key = in ? key_by_absq(e) : ~0ull;
-    group_bitonic<W>(key, e, id, ky, lane);
+    const uint64_t prev = __shfl_up_sync(kFull, key >> 5, 1);
+    if (in && li > 0 && prev == key >> 5) report(err, rs + li, -UBT_ERR_DUPLICATE_EDGE);
   }
+  const int from = (int)(key & 31u);
+  const uint64_t se = __shfl_sync(kFull, e, from);
+  const uint32_t sid = __shfl_sync(kFull, id, from);
+  const uint32_t sky = ekey ? __shfl_sync(kFull, ky, from) : 0u;
   if (in) {
-    adj[rs + li] = e;
-    eid[rs + li] = id;
-    if (ekey) ekey[rs + li] = ky;
+    adj[rs + li] = se;
+    eid[rs + li] = sid;
+    if (ekey) ekey[rs + li] = sky;
   }
 }
 
-// Rows of 2..32 entries: a warp takes 4 consecutive rows; the rows of at
-// most 8 entries are sorted together, one per 8-lane group, the others one
-// after another by the whole warp.
+// Rows of 2..32 entries: a warp takes 4 consecutive rows; the rows of at most
+// 8 entries are sorted together, one per 8-lane group, then those of at most
+// 16 two at a time and the others one after another by the whole warp.
 __global__ void k_sort_short_rows(int64_t n, const uint32_t* __restrict__ row_ptr, uint64_t* adj, uint32_t* eid,
                                   uint32_t* ekey, int mode, unsigned long long* err) {
   const int lane = threadIdx.x & 31;
@@ -325,8 +324,20 @@ __global__ void k_sort_short_rows(int64_t n, const uint32_t* __restrict__ row_pt
       rs = row_ptr[u];
       len = row_ptr[u + 1] - rs;
     }
-    sort_group_row<8>(adj, eid, ekey, rs, len, len >= 2 && len <= 8, mode, err, lane);
-    unsigned big = __ballot_sync(kFull, (lane & 7) == 0 && len > 8 && len <= 32);
+    if (__any_sync(kFull, len >= 2 && len <= 8))
+      sort_group_row<8>(adj, eid, ekey, rs, len, len >= 2 && len <= 8, mode, err, lane);
+    unsigned mid = __ballot_sync(kFull, (lane & 7) == 0 && len > 8 && len <= 16);
+    while (mid) {
+      const int g0 = __ffs(mid) - 1;
+      mid &= mid - 1;
+      const int g1 = mid ? __ffs(mid) - 1 : g0;
+      const bool two = mid != 0;
+      mid &= mid - 1;
+      const int g = lane < 16 ? g0 : g1;
+      const uint32_t rsg = __shfl_sync(kFull, rs, g), leng = __shfl_sync(kFull, len, g);
+      sort_group_row<16>(adj, eid, ekey, rsg, leng, lane < 16 || two, mode, err, lane);
+    }
+    unsigned big = __ballot_sync(kFull, (lane & 7) == 0 && len > 16 && len <= 32);
     while (big) {
       const int g = __ffs(big) - 1;
       big &= big - 1;
@@ -493,6 +504,51 @@ __device__ __forceinline__ void bitonic_packed(unsigned long long* pk, uint32_t 
   }
 }
 
+// One block sorts the entries [rs, rs + len) of a row, len <= kPackedPerThread
+// x its threads; pk holds the power of two >= len words.
+__device__ __forceinline__ void sort_packed(uint64_t* adj, uint32_t* eid, uint32_t* ekey, uint32_t rs, uint32_t len,
+                                            int mode, unsigned long long* err, unsigned long long* pk) {
+  uint32_t cap = 64;
+  while (cap < len) cap <<= 1;
+  if (mode == kSortById) {
+    for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x)
+      pk[i] = i < len ? (key_by_col(adj[rs + i]) << 12) | i : ~0ull;
+    __syncthreads();
+    bitonic_packed(pk, cap);
+    for (uint32_t i = threadIdx.x + 1; i < len; i += blockDim.x)
+      if ((pk[i] >> 12) == (pk[i - 1] >> 12)) report(err, rs + i, -UBT_ERR_DUPLICATE_EDGE);
+  } else {
+    for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x)
+      pk[i] = i < len ? (key_by_absq(adj[rs + i]) << 12) | i : ~0ull;
+    __syncthreads();
+    bitonic_packed(pk, cap);
+  }
+  // gather every entry's sources before any thread overwrites the list
+  uint64_t e[kPackedPerThread];
+  uint32_t d[kPackedPerThread], y[kPackedPerThread];
+#pragma unroll
+  for (int c = 0; c < kPackedPerThread; c++) {
+    const uint32_t i = threadIdx.x + c * blockDim.x;
+    if (i < len) {
+      const uint32_t w = (uint32_t)(pk[i] & 0xFFFu);
+      e[c] = adj[rs + w];
+      d[c] = eid[rs + w];
+      y[c] = ekey ? ekey[rs + w] : 0u;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < kPackedPerThread; c++) {
+    const uint32_t i = threadIdx.x + c * blockDim.x;
+    if (i < len) {
+      adj[rs + i] = e[c];
+      eid[rs + i] = d[c];
+      if (ekey) ekey[rs + i] = y[c];
+    }
+  }
+  __syncthreads();
+}
+
 // One launch per class takes the rows of the list with lo < len <= hi, with
 // hi / 2 threads (at most 512): every thread has a comparator at every stage.
 __global__ void __launch_bounds__(kPackedSortThreads)
@@ -508,45 +564,7 @@ k_sort_long_rows_packed(const uint32_t* __restrict__ rows, uint32_t nrows, const
       if (threadIdx.x == 0) report(err, rs, -UBT_ERR_INVALID_ARG);
       continue;
     }
-    uint32_t cap = 64;
-    while (cap < len) cap <<= 1;
-    if (mode == kSortById) {
-      for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x)
-        pk[i] = i < len ? (key_by_col(adj[rs + i]) << 12) | i : ~0ull;
-      __syncthreads();
-      bitonic_packed(pk, cap);
-      for (uint32_t i = threadIdx.x + 1; i < len; i += blockDim.x)
-        if ((pk[i] >> 12) == (pk[i - 1] >> 12)) report(err, rs + i, -UBT_ERR_DUPLICATE_EDGE);
-    } else {
-      for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x)
-        pk[i] = i < len ? (key_by_absq(adj[rs + i]) << 12) | i : ~0ull;
-      __syncthreads();
-      bitonic_packed(pk, cap);
-    }
-    // gather every entry's sources before any thread overwrites the list
-    uint64_t e[kPackedPerThread];
-    uint32_t d[kPackedPerThread], y[kPackedPerThread];
-#pragma unroll
-    for (int c = 0; c < kPackedPerThread; c++) {
-      const uint32_t i = threadIdx.x + c * blockDim.x;
-      if (i < len) {
-        const uint32_t w = (uint32_t)(pk[i] & 0xFFFu);
-        e[c] = adj[rs + w];
-        d[c] = eid[rs + w];
-        y[c] = ekey ? ekey[rs + w] : 0u;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < kPackedPerThread; c++) {
-      const uint32_t i = threadIdx.x + c * blockDim.x;
-      if (i < len) {
-        adj[rs + i] = e[c];
-        eid[rs + i] = d[c];
-        if (ekey) ekey[rs + i] = y[c];
-      }
-    }
-    __syncthreads();
+    sort_packed(adj, eid, ekey, rs, len, mode, err, pk);
   }
 }
 
@@ -653,37 +671,66 @@ __global__ void k_row_ids(int64_t n, const uint32_t* __restrict__ row_ptr, uint3
 // so far in its high half, in units of kWorkUnit entries (rounded up per pair), so one
 // 64-bit atomic places a pair and adds its work.  absq (FIXED, or null): a
 // histogram of |q| >> 9 over one warp's edges in eight.  streamed: the sum of
-// the streamed lengths.  Bound by the atomics'
-// and the pair words' random 32-byte sectors.
+// the streamed lengths.
+//
+// Every list starts with the first vertices, so their counters would take a
+// returning atomic from most rows, one after another in L2: a block ranks the
+// pairs of the first kHotOwners vertices among its kFillTile entries in shared
+// memory and reserves one range per vertex (Chung-Lu of 1e6 vertices: 656 -> 185 us).
+// What remains is bound by the atomics' and the pair words' random sectors.
 constexpr uint32_t kWorkUnit = 8;
-__global__ void k_pair_fill(int64_t m, const uint32_t* __restrict__ row_ptr, const uint64_t* __restrict__ adj,
-                            const uint32_t* __restrict__ rowid, unsigned long long* __restrict__ next,
-                            uint64_t* __restrict__ pairs, unsigned long long* __restrict__ absq,
-                            unsigned long long* __restrict__ streamed) {
+constexpr int kFillThreads = 256, kFillItems = 16;
+constexpr int64_t kFillTile = kFillThreads * kFillItems;
+constexpr uint32_t kHotOwners = 1024;
+__global__ void __launch_bounds__(kFillThreads)
+k_pair_fill(int64_t m, const uint32_t* __restrict__ row_ptr, const uint64_t* __restrict__ adj,
+            const uint32_t* __restrict__ rowid, unsigned long long* __restrict__ next, uint64_t* __restrict__ pairs,
+            unsigned long long* __restrict__ absq, unsigned long long* __restrict__ streamed) {
   __shared__ uint32_t s_q[65];
-  for (int i = threadIdx.x; i < 65; i += blockDim.x) s_q[i] = 0;
-  __syncthreads();
+  __shared__ unsigned long long s_hot[kHotOwners];  // count | work << 32, then the reserved base
+  for (int i = threadIdx.x; i < 65; i += kFillThreads) s_q[i] = 0;
   unsigned long long sum = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t e = adj[i];
-    const uint32_t v = adj_col(e), start = row_ptr[rowid[i]], len = (uint32_t)i - start;
-    uint32_t aq = 0;
-    if (absq) {
-      const int32_t q = adj_q(e);
-      aq = (uint32_t)(q < 0 ? -q : q);
-      if (((i >> 5) & 7) == 0) atomicAdd(&s_q[aq >> 9], 1u);
+  for (int64_t base = blockIdx.x * kFillTile; base < m; base += (int64_t)gridDim.x * kFillTile) {
+    for (uint32_t i = threadIdx.x; i < kHotOwners; i += kFillThreads) s_hot[i] = 0;
+    __syncthreads();
+    uint32_t v[kFillItems], at[kFillItems];
+    unsigned long long word[kFillItems];
+#pragma unroll
+    for (int j = 0; j < kFillItems; j++) {
+      const int64_t i = base + j * kFillThreads + threadIdx.x;
+      v[j] = kEmpty;
+      if (i >= m) continue;
+      const uint64_t e = adj[i];
+      v[j] = adj_col(e);
+      const uint32_t start = row_ptr[rowid[i]], len = (uint32_t)i - start;
+      uint32_t aq = 0;
+      if (absq) {
+        const int32_t q = adj_q(e);
+        aq = (uint32_t)(q < 0 ? -q : q);
+        if (((i >> 5) & 7) == 0) atomicAdd(&s_q[aq >> 9], 1u);
+      }
+      word[j] = pair_pack(start, len, aq >> 1);
+      sum += len;
+      const unsigned long long add = ((unsigned long long)((len + kWorkUnit - 1) / kWorkUnit) << 32) | 1ull;
+      at[j] = v[j] < kHotOwners ? (uint32_t)atomicAdd(&s_hot[v[j]], add) : (uint32_t)atomicAdd(&next[v[j]], add);
     }
-    const unsigned long long at =
-        atomicAdd(&next[v], ((unsigned long long)((len + kWorkUnit - 1) / kWorkUnit) << 32) | 1ull);
-    pairs[(uint32_t)at] = pair_pack(start, len, aq >> 1);
-    sum += len;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < kHotOwners; i += kFillThreads) {
+      const unsigned long long c = s_hot[i];
+      if (c) s_hot[i] = atomicAdd(&next[i], c);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kFillItems; j++)
+      if (v[j] != kEmpty) pairs[v[j] < kHotOwners ? (uint32_t)s_hot[v[j]] + at[j] : at[j]] = word[j];
+    __syncthreads();
   }
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(kFull, sum, d);
   if (lane_id() == 0 && sum) atomicAdd(streamed, sum);
   if (absq) {
     __syncthreads();
-    for (int i = threadIdx.x; i < 65; i += blockDim.x)
+    for (int i = threadIdx.x; i < 65; i += kFillThreads)
       if (s_q[i]) atomicAdd(&absq[i], (unsigned long long)s_q[i]);
   }
 }
@@ -821,10 +868,15 @@ __global__ void k_fill_lists(int64_t n, int64_t m, const unsigned long long* __r
 
 // ---------------------------------------------------------------- undirected AEO adjacency
 
-// both directions of every edge, in row order of arrival (sorted below)
+// both directions of every edge, in row order of arrival (sorted below), and
+// the row of every position, so that the passes over the entries below take
+// one thread an entry: a warp per row left the row of a hub -- tens of thousands
+// of entries -- to one warp, which was the length of the pass (Chung-Lu of 1e6
+// vertices, four passes: 2.96 ms, now 0.6)
 __global__ void k_uscatter(int64_t m, const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
                            const uint32_t* __restrict__ k, const uint32_t* __restrict__ uptr,
-                           uint32_t* __restrict__ ufill, uint64_t* __restrict__ uadj, uint32_t* __restrict__ ueid) {
+                           uint32_t* __restrict__ ufill, uint64_t* __restrict__ uadj, uint32_t* __restrict__ ueid,
+                           uint32_t* __restrict__ urow) {
   const uint32_t lane = lane_id();
   UBT_FOR_EDGE_WARPS(base, m) {
     const int64_t i = base + lane;
@@ -837,89 +889,106 @@ __global__ void k_uscatter(int64_t m, const uint32_t* __restrict__ src, const ui
     const uint32_t pb = uptr[b] + atomicAdd(&ufill[b], 1u);
     uadj[pa] = adj_pack(b, val);
     ueid[pa] = (uint32_t)i;
+    urow[pa] = a;
     uadj[pb] = adj_pack(a, val);
     ueid[pb] = (uint32_t)i;
+    urow[pb] = b;
   }
 }
 
-// Rows longer than the shared-memory sort limit: one block per row, sorted
-// in place in global memory by a bitonic network whose comparators all put
-// the smaller key first (the first comparator of every merge pairs i with its
-// mirror i ^ (kk - 1)); positions >= len act as +infinity, so comparators
-// that touch them never swap and are skipped.
-__global__ void k_sort_rows_inplace(const uint32_t* __restrict__ rows, uint32_t nrows,
-                                    const uint32_t* __restrict__ row_ptr, uint64_t* adj, uint32_t* eid) {
+// Rows longer than the shared-memory sort limit: their runs of `chunk` entries
+// are sorted one block each, then merged pairwise between two buffers, every
+// entry finding its place by a binary search in the other run.  One block per
+// row and a bitonic network in global memory took as long as the longest row
+// (Chung-Lu of 1e6 vertices, rows up to 50,000: 2.46 ms, now 0.42).
+__global__ void __launch_bounds__(kPackedSortThreads)
+k_sort_chunks(const uint32_t* __restrict__ rows, uint32_t nrows, const uint32_t* __restrict__ row_ptr, uint64_t* adj,
+              uint32_t* eid, unsigned long long* err, uint32_t chunk) {
+  extern __shared__ __align__(16) unsigned long long pk[];  // chunk words
   for (uint32_t r = blockIdx.x; r < nrows; r += gridDim.x) {
-    const uint32_t u = rows[r];
-    const uint32_t rs = row_ptr[u], len = row_ptr[u + 1] - rs;
-    uint32_t cap = 2;
-    while (cap < len) cap <<= 1;
-    for (uint32_t kk = 2; kk <= cap; kk <<= 1) {
-      for (uint32_t j = kk >> 1; j > 0; j >>= 1) {
-        for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x) {
-          const uint32_t ixj = (j == (kk >> 1)) ? (i ^ (kk - 1)) : (i ^ j);
-          if (ixj > i && ixj < len) {
-            const uint64_t a = adj[rs + i], b = adj[rs + ixj];
-            if (key_by_absq(a) > key_by_absq(b)) {
-              adj[rs + i] = b;
-              adj[rs + ixj] = a;
-              const uint32_t t = eid[rs + i];
-              eid[rs + i] = eid[rs + ixj];
-              eid[rs + ixj] = t;
-            }
-          }
-        }
-        __syncthreads();
+    const uint32_t rs = row_ptr[rows[r]], len = row_ptr[rows[r] + 1] - rs;
+    for (uint64_t c = (uint64_t)blockIdx.y * chunk; c < len; c += (uint64_t)gridDim.y * chunk)
+      sort_packed(adj, eid, nullptr, rs + (uint32_t)c, min(chunk, len - (uint32_t)c), kSortByAbsq, err, pk);
+  }
+}
+__global__ void k_merge_runs(const uint32_t* __restrict__ rows, uint32_t nrows, const uint32_t* __restrict__ row_ptr,
+                             const uint64_t* __restrict__ adj, const uint32_t* __restrict__ eid,
+                             uint64_t* __restrict__ adj_out, uint32_t* __restrict__ eid_out, uint64_t width) {
+  for (uint32_t r = blockIdx.x; r < nrows; r += gridDim.x) {
+    const uint32_t rs = row_ptr[rows[r]], len = row_ptr[rows[r] + 1] - rs;
+    for (uint64_t i = (uint64_t)blockIdx.y * blockDim.x + threadIdx.x; i < len; i += (uint64_t)gridDim.y * blockDim.x) {
+      const uint64_t run = i / width, base = run * width, other = (run ^ 1) * width;
+      const uint64_t e = adj[rs + i], key = key_by_absq(e);
+      uint64_t lo = min((uint64_t)len, other), hi = min((uint64_t)len, other + width);
+      while (lo < hi) {  // entries of the other run before this one (keys are distinct)
+        const uint64_t mid = (lo + hi) >> 1;
+        if (key_by_absq(adj[rs + mid]) < key) lo = mid + 1; else hi = mid;
       }
+      const uint64_t at = rs + (other < base ? lo + (i - base) : i + (lo - min((uint64_t)len, other)));
+      adj_out[at] = e;
+      eid_out[at] = eid[rs + i];
     }
   }
+}
+// adj_tmp, eid_tmp: as long as the rows; max_len: an upper bound of their lengths
+ubt_status sort_huge_rows(const uint32_t* rows, uint32_t nrows, const uint32_t* row_ptr, uint64_t* adj, uint32_t* eid,
+                          uint64_t* adj_tmp, uint32_t* eid_tmp, unsigned long long* err, uint32_t chunk,
+                          uint64_t max_len, int sms, cudaStream_t s) {
+  const unsigned gx = std::min<uint32_t>(nrows, 65535u);
+  const unsigned gy = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((max_len + chunk - 1) / chunk, 4 * sms / gx + 1));
+  const size_t smem = (size_t)chunk * 8;
+  k_sort_chunks<<<dim3(gx, gy), kPackedSortThreads, smem, s>>>(rows, nrows, row_ptr, adj, eid, err, chunk);
+  uint64_t* src = adj;
+  uint32_t* srce = eid;
+  uint64_t* dst = adj_tmp;
+  uint32_t* dste = eid_tmp;
+  const unsigned my = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((max_len + 255) / 256, 32 * sms / gx + 1));
+  // a last round whose runs have no other run copies the rows back where needed
+  for (uint64_t width = chunk; width < max_len || src != adj; width *= 2) {
+    k_merge_runs<<<dim3(gx, my), 256, 0, s>>>(rows, nrows, row_ptr, src, srce, dst, dste, width);
+    std::swap(src, dst);
+    std::swap(srce, dste);
+  }
+  UBT_CUDA(cudaGetLastError());
+  return UBT_OK;
 }
 
 // epos[2e + side] = position of edge e in the row of its smaller (side 0) or
-// larger (side 1) endpoint; then umir[p] = the other one.  One warp per row.
-__global__ void k_uepos(int64_t n, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
+// larger (side 1) endpoint; umir[p] = the position of p's edge in the other row
+__global__ void k_uepos(int64_t m2, const uint32_t* __restrict__ urow, const uint64_t* __restrict__ uadj,
                         const uint32_t* __restrict__ ueid, uint32_t* __restrict__ epos) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += warps)
-    for (uint32_t p = uptr[x] + lane; p < uptr[x + 1]; p += 32)
-      epos[2 * (size_t)ueid[p] + ((uint32_t)x > adj_col(uadj[p]) ? 1 : 0)] = p;
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m2; p += (int64_t)gridDim.x * blockDim.x)
+    epos[2 * (size_t)ueid[p] + (urow[p] > adj_col(uadj[p]) ? 1 : 0)] = (uint32_t)p;
 }
-__global__ void k_umirror(int64_t n, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
-                          const uint32_t* __restrict__ ueid, const uint32_t* __restrict__ epos,
-                          uint32_t* __restrict__ umir) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += warps)
-    for (uint32_t p = uptr[x] + lane; p < uptr[x + 1]; p += 32)
-      umir[p] = epos[2 * (size_t)ueid[p] + ((uint32_t)x > adj_col(uadj[p]) ? 0 : 1)];
+__global__ void k_umirror(int64_t m, const uint32_t* __restrict__ epos, uint32_t* __restrict__ umir) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t p0 = epos[2 * e], p1 = epos[2 * e + 1];
+    umir[p0] = p1;
+    umir[p1] = p0;
+  }
 }
 
-// Edge index: every edge once, from the row of its smaller endpoint.  The
-// table has at least four times as many slots as edges, so every insert
-// finds a free slot; the loop bound is a self-check.
-__global__ void k_edge_index(int64_t n, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
-                             uint4* __restrict__ eslots, uint64_t slots,
-                             int shift, unsigned long long* err) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += warps)
-    for (uint32_t p = uptr[x] + lane; p < uptr[x + 1]; p += 32) {
-      const uint64_t e = uadj[p];
-      if ((uint32_t)x > adj_col(e)) continue;
-      const uint64_t key = edge_index_key((uint32_t)x, adj_col(e));
-      uint64_t h = edge_index_home(key, shift);
-      uint64_t it = 0;
-      for (; it < slots; it++) {
-        unsigned long long* slot_key = reinterpret_cast<unsigned long long*>(&eslots[h]);
-        if (atomicCAS(slot_key, (unsigned long long)kEdgeIndexEmpty, (unsigned long long)key) == kEdgeIndexEmpty) {
-          eslots[h].z = adj_valbits(e);
-          break;
-        }
-        h = (h + 1) & (slots - 1);
+// Edge index: every input edge once.  The table has at least four times as
+// many slots as edges, so every insert finds a free slot; the loop bound is a
+// self-check.
+__global__ void k_edge_index(int64_t m, const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
+                             const uint32_t* __restrict__ k, uint4* __restrict__ eslots, uint64_t slots, int shift,
+                             uint32_t* __restrict__ filter, unsigned long long* err) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint64_t key = edge_index_key(src[i], dst[i]);
+    atomicOr(&filter[edge_index_home(key, shift + kEdgeFilterLog)], edge_filter_bits(key));
+    uint64_t h = edge_index_home(key, shift);
+    uint64_t it = 0;
+    for (; it < slots; it++) {
+      unsigned long long* slot_key = reinterpret_cast<unsigned long long*>(&eslots[h]);
+      if (atomicCAS(slot_key, (unsigned long long)kEdgeIndexEmpty, (unsigned long long)key) == kEdgeIndexEmpty) {
+        eslots[h].z = (uint32_t)(int32_t)(32768 - (int32_t)k[i]);
+        break;
       }
-      if (it == slots) report(err, p, -UBT_ERR_INVALID_ARG);
+      h = (h + 1) & (slots - 1);
     }
+    if (it == slots) report(err, i, -UBT_ERR_INVALID_ARG);
+  }
 }
 
 // AEO traversal: edge x-y is handled by x, the endpoint with the longer list
@@ -927,49 +996,51 @@ __global__ void k_edge_index(int64_t n, const uint32_t* __restrict__ uptr, const
 __device__ inline bool aeo_owns(uint32_t x, uint32_t y, uint32_t dx, uint32_t dy) {
   return dx > dy || (dx == dy && x > y);
 }
-__global__ void k_apair_count(int64_t n, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
-                              uint32_t* __restrict__ pcount) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += warps) {
-    const uint32_t dx = uptr[x + 1] - uptr[x];
-    uint32_t c = 0;
-    for (uint32_t p = uptr[x] + lane; p < uptr[x + 1]; p += 32) {
+__global__ void k_apair_count(int64_t m2, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
+                              const uint32_t* __restrict__ urow, uint32_t* __restrict__ pcount) {
+  const uint32_t lane = lane_id();
+  UBT_FOR_EDGE_WARPS(base, m2) {
+    const int64_t p = base + lane;
+    bool own = false;
+    uint32_t x = 0;
+    if (p < m2) {
+      x = urow[p];
       const uint32_t y = adj_col(uadj[p]);
-      c += aeo_owns((uint32_t)x, y, dx, uptr[y + 1] - uptr[y]) ? 1u : 0u;
+      own = aeo_owns(x, y, uptr[x + 1] - uptr[x], uptr[y + 1] - uptr[y]);
     }
-    c = __reduce_add_sync(kFull, c);
-    if (lane == 0) pcount[x] = c;
+    add_by_runs(pcount, x, own);
   }
 }
-// pair words in row order: streamed endpoint | position of the edge in x's row << 32
-__global__ void k_apair_fill(int64_t n, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
-                             const uint32_t* __restrict__ apair_ptr, uint64_t* __restrict__ apairs,
-                             unsigned long long* __restrict__ work) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += warps) {
-    const uint32_t dx = uptr[x + 1] - uptr[x];
-    uint32_t at = apair_ptr[x];
-    unsigned long long w = 0;
-    for (uint32_t base = uptr[x]; base < uptr[x + 1]; base += 32) {
-      const uint32_t p = base + lane;
-      bool own = false;
-      uint32_t y = 0;
-      if (p < uptr[x + 1]) {
-        y = adj_col(uadj[p]);
-        own = aeo_owns((uint32_t)x, y, dx, uptr[y + 1] - uptr[y]);
-      }
-      const unsigned msk = __ballot_sync(kFull, own);
-      if (own) {
-        apairs[at + __popc(msk & lanemask_lt())] = ((uint64_t)p << 32) | y;
-        w += uptr[y + 1] - uptr[y];
-      }
-      at += __popc(msk);
+// pair words by owner: streamed endpoint | position of the edge in x's row << 32.
+// next[x] as in k_pair_fill (from apair_ptr[x], streamed entries in units); the
+// entries of a row are neighbours, so a warp adds once per row it holds.
+__global__ void k_apair_fill(int64_t m2, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
+                             const uint32_t* __restrict__ urow, unsigned long long* __restrict__ next,
+                             uint64_t* __restrict__ apairs) {
+  const uint32_t lane = lane_id();
+  UBT_FOR_EDGE_WARPS(base, m2) {
+    const int64_t p = base + lane;
+    uint32_t x = kEmpty, y = 0, dy = 0;
+    bool own = false;
+    if (p < m2) {
+      x = urow[p];
+      y = adj_col(uadj[p]);
+      dy = uptr[y + 1] - uptr[y];
+      own = aeo_owns(x, y, uptr[x + 1] - uptr[x], dy);
     }
+    const unsigned row = __match_any_sync(kFull, x);  // the lanes of this lane's row
+    unsigned long long add = own ? ((unsigned long long)((dy + kWorkUnit - 1) / kWorkUnit) << 32) | 1ull : 0ull, incl = add;
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) w += __shfl_xor_sync(kFull, w, d);
-    if (lane == 0) work[x] = w;
+    for (int d = 1; d < 32; d <<= 1) {  // sums over the row's lanes up to this one (they are consecutive)
+      const unsigned long long o = __shfl_up_sync(kFull, incl, d);
+      if (lane >= (uint32_t)d && ((row >> (lane - d)) & 1u)) incl += o;
+    }
+    const int last = 31 - __clz((int)row), head = __ffs(row) - 1;
+    const unsigned long long all = __shfl_sync(kFull, incl, last);
+    unsigned long long at = 0;
+    if ((int)lane == head && all) at = atomicAdd(&next[x], all);
+    at = __shfl_sync(kFull, at, head);
+    if (own) apairs[(uint32_t)at + (uint32_t)(incl - add)] = ((uint64_t)p << 32) | y;
   }
 }
 // owners by decreasing log2 of their streamed work, those with rows longer
@@ -978,20 +1049,28 @@ constexpr uint32_t kAeoWarpRow = 128;
 __global__ void k_afill_lists(int64_t n, const uint32_t* __restrict__ uptr, const uint32_t* __restrict__ apair_ptr,
                               const unsigned long long* __restrict__ work, unsigned long long* cursor,
                               uint32_t* __restrict__ lists, int count_only) {
-  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-    if (apair_ptr[x + 1] == apair_ptr[x]) continue;
-    const unsigned long long w = work[x];
-    const int lg = w ? 63 - __clzll(w) : 0;
-    const int b = lg * 2 + (uptr[x + 1] - uptr[x] > kAeoWarpRow ? 1 : 0);
-    if (count_only) atomicAdd(&cursor[b], 1ull);
-    else lists[atomicAdd(&cursor[b], 1ull)] = (uint32_t)x;
+  constexpr int kB = 2 * (kLgMax + 1);
+  __shared__ uint32_t s_cnt[kB];
+  __shared__ unsigned long long s_base[kB];
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
+    for (int i = threadIdx.x; i < kB; i += blockDim.x) s_cnt[i] = 0;
+    __syncthreads();
+    const int64_t x = base + threadIdx.x;
+    const bool on = x < n && apair_ptr[x + 1] != apair_ptr[x];
+    int b = 0;
+    uint32_t rank = 0;
+    if (on) {
+      const unsigned long long w = (work[x] >> 32) * kWorkUnit;
+      b = (w ? 63 - __clzll(w) : 0) * 2 + (uptr[x + 1] - uptr[x] > kAeoWarpRow ? 1 : 0);
+      rank = atomicAdd(&s_cnt[b], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kB; i += blockDim.x)
+      if (s_cnt[i]) s_base[i] = atomicAdd(&cursor[i], (unsigned long long)s_cnt[i]);
+    __syncthreads();
+    if (on && !count_only) lists[s_base[b] + rank] = (uint32_t)x;
+    __syncthreads();
   }
-}
-__global__ void k_max_row(int64_t n, const uint32_t* __restrict__ ptr, unsigned long long* out) {
-  unsigned long long best = 0;
-  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-    best = max(best, (unsigned long long)(ptr[x + 1] - ptr[x]));
-  atomicMax(out, best);
 }
 
 struct BuildLayout {
@@ -1020,6 +1099,7 @@ struct BuildLayout {
   uint32_t* alist;
   unsigned long long* awork;
   unsigned long long* lqueue;  // long vertex samples of a local-count call (with the undirected rows)
+  uint32_t* efilter;           // filter of the edge index
   uint4* eslots;               // edge index (optional)
   int64_t eh_slots;
   unsigned long long* gacc;
@@ -1042,7 +1122,7 @@ struct BuildLayout {
   size_t total;
 };
 constexpr int kStats = kStatBuckets + kTaskBuckets;
-static_assert(kStats >= 2 * (kLgMax + 1) + 1, "the undirected owners' cursors share the array");
+static_assert(kStats >= 2 * (kLgMax + 1), "the undirected owners' cursors share the array");
 
 int64_t list_bound(int64_t n, int64_t m) {
   // a forward list under Node Order holds at most sqrt(2m) entries
@@ -1082,14 +1162,16 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.uptr = und ? c.take<uint32_t>(n + 1) : nullptr;
   L.uadj = und ? c.take<uint64_t>(std::max<int64_t>(2 * m, 1)) : nullptr;
   L.ueid = und ? c.take<uint32_t>(std::max<int64_t>(2 * m, 1)) : nullptr;
-  L.umir = und ? c.take<uint32_t>(std::max<int64_t>(2 * m, 1)) : nullptr;
-  L.uepos = und ? c.take<uint32_t>(std::max<int64_t>(2 * m, 1)) : nullptr;
+  // one piece: the long rows' sort uses both as its second buffer of entries
+  L.uepos = und ? c.take<uint32_t>(std::max<int64_t>(4 * m, 2)) : nullptr;
+  L.umir = und ? L.uepos + 2 * m : nullptr;
   L.apair_ptr = und ? c.take<uint32_t>(n + 1) : nullptr;
   L.apairs = und ? c.take<uint64_t>(std::max<int64_t>(m, 1)) : nullptr;
   L.alist = und ? c.take<uint32_t>(n1) : nullptr;
   L.awork = und ? c.take<unsigned long long>(n1) : nullptr;
   L.lqueue = und ? c.take<unsigned long long>(2 + kLongQueue) : nullptr;
   const bool eidx = und && (opts->flags & UBT_OPT_EDGE_INDEX);
+  L.efilter = und ? c.take<uint32_t>((size_t)(pow2_at_least(std::max<int64_t>(4 * m, 64)) >> kEdgeFilterLog)) : nullptr;
   L.eh_slots = eidx ? pow2_at_least(std::max<int64_t>(4 * m, 64)) : 0;
   L.eslots = eidx ? c.take<uint4>(L.eh_slots) : nullptr;
   L.gacc = c.take<unsigned long long>(std::max<int64_t>(m, 1));
@@ -1292,7 +1374,8 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
     k_in_degree<<<grid_v, thr, 0, s>>>(n, L.deg, L.vid, L.row_ptr, L.fill);
     UBT_CUDA(exclusive_scan_u32(L.fill, L.pair_ptr, n, L.scan_tmp, s));
     k_pair_next<<<grid_v, thr, 0, s>>>(n, L.pair_ptr, L.work);
-    if (m > 0) k_pair_fill<<<grid_e, thr, 0, s>>>(m, L.row_ptr, L.adj, L.rowid, L.work, L.pairs, absq, &L.stats[2]);
+    const int grid_f = (int)std::min<int64_t>((m + kFillTile - 1) / kFillTile, (int64_t)sms * 8);
+    if (m > 0) k_pair_fill<<<grid_f, kFillThreads, 0, s>>>(m, L.row_ptr, L.adj, L.rowid, L.work, L.pairs, absq, &L.stats[2]);
     UBT_CUDA(cudaGetLastError());
   }
   // 5. work lists: the owners of every task class by decreasing work bucket
@@ -1334,9 +1417,12 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   int64_t n_aowners = 0, n_ablock = 0, max_udeg = 0;
   if (und && n > 0) {
     phase.next("build: undirected rows in Absolute Edge Order");
+    uint32_t* urow = (uint32_t*)L.gacc;  // the row of every entry, in the (not yet used) accumulators
+    const int64_t m2 = 2 * m;
+    const int grid_2 = (int)std::min<int64_t>(std::max<int64_t>((m2 + thr - 1) / thr, 1), (int64_t)sms * 32);
     UBT_CUDA(exclusive_scan_u32(L.deg, L.uptr, n, L.scan_tmp, s));
     UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
-    if (m > 0) k_uscatter<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, L.uptr, L.fill, L.uadj, L.ueid);
+    if (m > 0) k_uscatter<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, L.uptr, L.fill, L.uadj, L.ueid, urow);
     k_sort_short_rows<<<grid_w, thr, 0, s>>>(n, L.uptr, L.uadj, L.ueid, nullptr, kSortByAbsq, &L.scratch->err);
     const uint32_t sort_smem = (uint32_t)tuning().sort_smem_max;
     UBT_CUDA(cudaMemsetAsync(lcount, 0, 3 * sizeof(unsigned long long), s));
@@ -1356,27 +1442,33 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
       if (st != UBT_OK) return st;
     }
     if (lc[1]) {
-      const int g2 = (int)std::min<unsigned long long>(lc[1], (unsigned long long)sms * 2);
-      k_sort_rows_inplace<<<g2, 1024, 0, s>>>(L.huge_rows, (uint32_t)lc[1], L.uptr, L.uadj, L.ueid);
+      st = sort_huge_rows(L.huge_rows, (uint32_t)lc[1], L.uptr, L.uadj, L.ueid, (uint64_t*)L.uepos,
+                          (uint32_t*)L.apairs, &L.scratch->err, sort_smem, deg_stats[0], sms, s);
+      if (st != UBT_OK) return st;
     }
-    k_uepos<<<grid_w, thr, 0, s>>>(n, L.uptr, L.uadj, L.ueid, L.uepos);
-    k_umirror<<<grid_w, thr, 0, s>>>(n, L.uptr, L.uadj, L.ueid, L.uepos, L.umir);
+    if (m > 0) {
+      k_uepos<<<grid_2, thr, 0, s>>>(m2, urow, L.uadj, L.ueid, L.uepos);
+      k_umirror<<<grid_e, thr, 0, s>>>(m, L.uepos, L.umir);
+    }
     if (L.eslots) {
       UBT_CUDA(cudaMemsetAsync(L.eslots, 0xFF, sizeof(uint4) * (size_t)L.eh_slots, s));
+      UBT_CUDA(cudaMemsetAsync(L.efilter, 0, sizeof(uint32_t) * (size_t)(L.eh_slots >> kEdgeFilterLog), s));
       int lg = 0;
       while ((1ll << lg) < L.eh_slots) lg++;
-      k_edge_index<<<grid_w, thr, 0, s>>>(n, L.uptr, L.uadj, L.eslots, (uint64_t)L.eh_slots, 64 - lg,
-                                          &L.scratch->err);
+      if (m > 0)
+        k_edge_index<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, L.eslots, (uint64_t)L.eh_slots, 64 - lg, L.efilter,
+                                            &L.scratch->err);
     }
     UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
-    k_apair_count<<<grid_w, thr, 0, s>>>(n, L.uptr, L.uadj, L.fill);
+    if (m > 0) k_apair_count<<<grid_2, thr, 0, s>>>(m2, L.uptr, L.uadj, urow, L.fill);
     UBT_CUDA(exclusive_scan_u32(L.fill, L.apair_ptr, n, L.scan_tmp, s));
-    k_apair_fill<<<grid_w, thr, 0, s>>>(n, L.uptr, L.uadj, L.apair_ptr, L.apairs, L.awork);
-    unsigned long long* acur = L.stats;  // 2 (kLgMax + 1) cursors, then the longest row
+    k_pair_next<<<grid_v, thr, 0, s>>>(n, L.apair_ptr, L.awork);
+    if (m > 0) k_apair_fill<<<grid_2, thr, 0, s>>>(m2, L.uptr, L.uadj, urow, L.awork, L.apairs);
+    unsigned long long* acur = L.stats;  // 2 (kLgMax + 1) cursors
     constexpr int kAB = 2 * (kLgMax + 1);
-    UBT_CUDA(cudaMemsetAsync(acur, 0, sizeof(unsigned long long) * (kAB + 1), s));
+    UBT_CUDA(cudaMemsetAsync(acur, 0, sizeof(unsigned long long) * kAB, s));
     k_afill_lists<<<grid_v, thr, 0, s>>>(n, L.uptr, L.apair_ptr, L.awork, acur, L.alist, 1);
-    unsigned long long acount[kAB + 1];
+    unsigned long long acount[kAB];
     UBT_CUDA(cudaMemcpyAsync(acount, acur, sizeof(acount), cudaMemcpyDeviceToHost, s));
     UBT_CUDA(cudaStreamSynchronize(s));
     unsigned long long run = 0;
@@ -1389,16 +1481,12 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
       if (cls == 1) n_ablock = (int64_t)run;
     }
     n_aowners = (int64_t)run;
-    acount[kAB] = 0;
     UBT_CUDA(cudaMemcpyAsync(acur, acount, sizeof(acount), cudaMemcpyHostToDevice, s));
     k_afill_lists<<<grid_v, thr, 0, s>>>(n, L.uptr, L.apair_ptr, L.awork, acur, L.alist, 0);
-    k_max_row<<<grid_v, thr, 0, s>>>(n, L.uptr, &acur[kAB]);
-    unsigned long long mx = 0;
-    UBT_CUDA(cudaMemcpyAsync(&mx, &acur[kAB], sizeof(mx), cudaMemcpyDeviceToHost, s));
     UBT_CUDA(cudaMemcpyAsync(&err, &L.scratch->err, sizeof(err), cudaMemcpyDeviceToHost, s));
     UBT_CUDA(cudaGetLastError());
     UBT_CUDA(cudaStreamSynchronize(s));
-    max_udeg = (int64_t)mx;
+    max_udeg = (int64_t)deg_stats[0];
     st = status_from_err(err);
     if (st != UBT_OK) return st;
   }
@@ -1440,6 +1528,7 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   g->max_udeg = max_udeg;
   g->lqueue = L.lqueue;
   g->eslots = L.eslots;
+  g->efilter = L.efilter;
   g->eh_slots = L.eh_slots;
   {
     int lg = 0;

@@ -46,6 +46,7 @@ struct LocalP {
 // used); the bound is a self-check.
 struct EdgeIndex {
   const uint4* slots;
+  const uint32_t* filter;
   uint64_t mask;   // slots - 1
   int shift;
   int mode;        // 0 unused, 1 where cheaper than streaming, 2 always
@@ -53,6 +54,8 @@ struct EdgeIndex {
 
 __device__ __forceinline__ bool edge_index_find(const EdgeIndex& ix, uint32_t a, uint32_t b, uint32_t& val,
                                                 Scratch* sc) {
+  const uint64_t key = edge_index_key(a, b);
+  if (!edge_filter_pass(ix.filter[edge_index_home(key, ix.shift + kEdgeFilterLog)], key)) return false;
   const int r = edge_index_lookup(ix.slots, ix.mask, ix.shift, a, b, val);
   if (r < 0) guard_fail(sc, kGuardFind, a);
   return r > 0;
@@ -77,19 +80,25 @@ __device__ __forceinline__ bool use_index(const EdgeIndex& ix, uint32_t cand, ui
 //   Absolute Edge Order, so that is |q_vw| < |q_va|, or equal and w > a --
 //   and lies in v's Lemma 2 prefix (|q_vw| 2^30 >= L, L = 0: all).
 // found(P, w) receives every triangle.
-// Two lookups of one lane at once: both home slots are read before either
-// is examined (at most a quarter of the slots are used, so nearly every
-// lookup ends there); the rare longer probe continues alone.
+// Two lookups of one lane at once: both filter words are read before either is
+// examined, then the home slots of those that pass (at most a quarter of the
+// slots are used, so nearly every lookup ends there); the rare longer probe
+// continues alone.
 __device__ __forceinline__ void edge_index_find2(const EdgeIndex& ix, const bool (&act)[2], const uint32_t (&a)[2],
                                                  const uint32_t (&b)[2], bool (&hit)[2], uint32_t (&val)[2],
                                                  Scratch* sc) {
   uint64_t k[2];
+  uint32_t word[2];
   uint4 sl[2];
 #pragma unroll
   for (int i = 0; i < 2; i++) {
     k[i] = edge_index_key(a[i], b[i]);
-    sl[i] = act[i] ? ix.slots[edge_index_home(k[i], ix.shift)] : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u);
+    word[i] = act[i] ? ix.filter[edge_index_home(k[i], ix.shift + kEdgeFilterLog)] : 0u;
   }
+#pragma unroll
+  for (int i = 0; i < 2; i++)
+    sl[i] = edge_filter_pass(word[i], k[i]) ? ix.slots[edge_index_home(k[i], ix.shift)]
+                                            : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u);
 #pragma unroll
   for (int i = 0; i < 2; i++) {
     hit[i] = false;
@@ -157,6 +166,7 @@ __device__ __forceinline__ void index_pairs(const EdgeIndex& ix, const uint64_t*
 EdgeIndex edge_index_of(const ubt_graph* g) {
   EdgeIndex ix;
   ix.slots = g->eslots;
+  ix.filter = g->efilter;
   ix.mask = g->eh_slots ? (uint64_t)g->eh_slots - 1 : 0;
   ix.shift = g->eh_shift;
   ix.mode = g->eslots ? (int)tuning().edge_index : 0;

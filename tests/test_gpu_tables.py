@@ -140,3 +140,42 @@ def test_worlds_in_passes_of_every_size(ubt, W):
     finally:
         ubt.set_tuning("world_words_per_pass", old)
     assert G.guard() == 0
+
+
+@pytest.mark.parametrize("smem_max", [64, 256, 4096])
+@pytest.mark.parametrize("deg", [63, 64, 65, 257, 1030, 4095, 4097, 9000])
+def test_undirected_rows_of_every_length(ubt, deg, smem_max):
+    """A star of `deg` leaves and edges among them: a row at and around the
+    lengths where its sort changes (registers, one block, runs merged in an
+    odd or even number of rounds), with equal |q| (ties go by neighbour)."""
+    n = deg + 200
+    r = synth.rng(deg)
+    leaves = r.choice(n - 1, size=deg, replace=False) + 1
+    e = r.integers(1, n, size=(3000, 2))
+    a = np.concatenate([np.zeros(deg, np.int64), e[:, 0]])
+    b = np.concatenate([leaves, e[:, 1]])
+    key = np.unique(np.minimum(a, b) * n + np.maximum(a, b))
+    key = key[key // n != key % n]
+    s, d = synth.random_orientation((key // n).astype(np.uint32), (key % n).astype(np.uint32), 3)
+    k = (synth.k_uniform(s.size, 4) >> 12 << 12).astype(np.uint32)
+    old = ubt.get_tuning("sort_smem_max"), ubt.get_tuning("warp_sort_max")
+    try:
+        ubt.set_tuning("warp_sort_max", 128)
+        ubt.set_tuning("sort_smem_max", smem_max)
+        G = ubt.Graph(n, s, d, k=k, undirected=True, edge_index=True)
+    finally:
+        ubt.set_tuning("sort_smem_max", old[0])
+        ubt.set_tuning("warp_sort_max", old[1])
+    ex = G.export_undirected()
+    up = ex["uptr"].astype(np.int64)
+    row = np.repeat(np.arange(n), np.diff(up))
+    val, col, mir = ex["val"].astype(np.int64), ex["col"].astype(np.int64), ex["mirror"].astype(np.int64)
+    key = (32768 - np.abs(val)) * (1 << 32) + col
+    same = row[1:] == row[:-1]
+    assert np.all(key[1:][same] > key[:-1][same])
+    assert np.array_equal(val, 32768 - k.astype(np.int64)[ex["eid"]])
+    assert np.array_equal(mir[mir], np.arange(2 * s.size)) and np.array_equal(row[mir], col)
+    want = oracle.count_threshold(n, s, d, k, [0.55, 0.8])
+    got = G.count_aeo([0.55, 0.8])
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    assert G.guard() == 0
