@@ -26,6 +26,8 @@ LIB_PATH = os.path.join(_HERE, "libubt.so")
 FIXED, REAL = 0, 1
 UBT_OPT_UNDIRECTED = 1
 UBT_OPT_EDGE_INDEX = 2
+# records an enumeration without a given capacity has room for at first (24 MiB)
+_ENUM_GUESS = 1 << 20
 
 # ubt_tri_rec: {uint32 u, v, w, cls; double p_bal}
 TRI_REC_DTYPE = np.dtype([("u", "<u4"), ("v", "<u4"), ("w", "<u4"), ("cls", "<u4"), ("p_bal", "<f8")])
@@ -283,15 +285,16 @@ class Graph:
         torch = _torch()
         L = lib()
         found = ctypes.c_int64(0)
-        if capacity is None:
-            st = L.ubt_enumerate(self._h, float(tau), int(which), int(bool(prune)), None, 0, ctypes.byref(found),
-                                 _stream(stream))
-            if st not in (0, -7):
-                _check(st, "ubt_enumerate")
-            capacity = int(found.value)
-        buf = torch.empty(max(capacity, 1) * TRI_REC_DTYPE.itemsize, dtype=torch.uint8, device=self.device)
-        st = L.ubt_enumerate(self._h, float(tau), int(which), int(bool(prune)), _ptr(buf), int(capacity),
-                             ctypes.byref(found), _stream(stream))
+        exact = capacity is not None
+        if not exact:
+            capacity = _ENUM_GUESS  # most answers fit; one that does not has said its size
+        while True:
+            buf = torch.empty(max(capacity, 1) * TRI_REC_DTYPE.itemsize, dtype=torch.uint8, device=self.device)
+            st = L.ubt_enumerate(self._h, float(tau), int(which), int(bool(prune)), _ptr(buf), int(capacity),
+                                 ctypes.byref(found), _stream(stream))
+            if st != -7 or exact:
+                break
+            capacity, exact = int(found.value), True
         if st == -7:
             raise UbtError(st, "ubt_enumerate needs capacity %d" % found.value)
         _check(st, "ubt_enumerate")
@@ -336,14 +339,14 @@ class Graph:
         it = _dev_u32(items, self.device)
         t = np.ascontiguousarray(np.atleast_1d(np.asarray(taus, dtype=np.float64)))
         k = int(it.numel())
-        bal = torch.empty(max(k, 1) * t.size, dtype=torch.int64, device=self.device)
-        unb = torch.empty(max(k, 1) * t.size, dtype=torch.int64, device=self.device)
-        est = torch.empty(2 * t.size, dtype=torch.float64, device=self.device)
-        _check(fn(self._h, _ptr(it), k, t.ctypes.data_as(ctypes.c_void_p), t.size, _ptr(bal), _ptr(unb), _ptr(est),
-                  _stream(stream)), "local counts")
         nt = t.size
-        return (bal.cpu().numpy()[: k * nt].reshape(k, nt), unb.cpu().numpy()[: k * nt].reshape(k, nt),
-                est.cpu().numpy().reshape(2, nt))
+        size = max(k, 1) * nt
+        out = torch.empty(2 * size + 2 * nt, dtype=torch.int64, device=self.device)  # both counts, the estimates
+        _check(fn(self._h, _ptr(it), k, t.ctypes.data_as(ctypes.c_void_p), nt, _ptr(out[:size]),
+                  _ptr(out[size: 2 * size]), _ptr(out[2 * size:]), _stream(stream)), "local counts")
+        h = out.cpu().numpy()
+        return (h[: k * nt].reshape(k, nt), h[size: size + k * nt].reshape(k, nt),
+                h[2 * size:].view(np.float64).reshape(2, nt))
 
     def edge_local_counts(self, edges, taus, stream=None):
         """Edge sampling (Algs. 5-6): per sampled edge (input index) the
@@ -450,10 +453,10 @@ class Graph:
     def sample_worlds(self, seed, W, stream=None):
         """Balanced-triangle count in each of W sign worlds: (int64[W], total)."""
         torch = _torch()
-        out = torch.empty(int(W), dtype=torch.int64, device=self.device)
-        tot = torch.empty(1, dtype=torch.int64, device=self.device)
-        self.sample_worlds_(seed, W, out, tot, stream=stream)
-        return out.cpu().numpy(), int(tot.cpu().item())
+        out = torch.empty(int(W) + 1, dtype=torch.int64, device=self.device)
+        self.sample_worlds_(seed, W, out[:-1], out[-1:], stream=stream)
+        h = out.cpu().numpy()
+        return h[:-1], int(h[-1])
 
     def batch_query_(self, taus, seed, counts, expect=None, worlds=None, stream=None):
         t = np.ascontiguousarray(np.atleast_1d(np.asarray(taus, dtype=np.float64)))
@@ -466,12 +469,13 @@ class Graph:
         torch = _torch()
         nt = int(np.atleast_1d(taus).size)
         G = self.n_graphs
-        c = torch.empty(G * 2 * nt, dtype=torch.int64, device=self.device)
-        e = torch.empty(G * 2, dtype=torch.float64, device=self.device) if expect else None
-        w = torch.empty(G * 64, dtype=torch.int64, device=self.device) if worlds else None
-        self.batch_query_(taus, seed, c, e, w, stream)
-        return (c.cpu().numpy().reshape(G, 2, nt), None if e is None else e.cpu().numpy().reshape(G, 2),
-                None if w is None else w.cpu().numpy().reshape(G, 64))
+        nc, ne = G * 2 * nt, G * 2 if expect else 0
+        out = torch.empty(nc + ne + (G * 64 if worlds else 0), dtype=torch.int64, device=self.device)
+        self.batch_query_(taus, seed, out[:nc], out[nc: nc + ne] if expect else None,
+                          out[nc + ne:] if worlds else None, stream)
+        h = out.cpu().numpy()
+        return (h[:nc].reshape(G, 2, nt), h[nc: nc + ne].view(np.float64).reshape(G, 2) if expect else None,
+                h[nc + ne:].reshape(G, 64) if worlds else None)
 
 
 class _ExpectedCountsFn:

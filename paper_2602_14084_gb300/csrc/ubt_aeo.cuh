@@ -537,13 +537,12 @@ ubt_status launch_aeo(const ubt_graph* g, int64_t L, const typename V::P& p, cud
       a.m2 = (uint32_t)(2 * g->m);
       a.sc = g->scratch;
       a.L = L;
-      UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
+      UBT_CUDA(cudaMemsetAsync(a.sc->task, 0, kScratchQuery, s));
       if (g->m == 0) return UBT_OK;
       const int threads = 512;
       const size_t smem = (size_t)((V::smem_bytes(p, threads) + 15) / 16) * 16;
-      UBT_CUDA(cudaFuncSetAttribute(k_aeo_index<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       int per_sm = 0;
-      UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_aeo_index<V>, threads, smem));
+      UBT_CUDA(resident_blocks((const void*)k_aeo_index<V>, g->device, threads, smem, &per_sm));
       if (per_sm < 1) return UBT_ERR_INVALID_ARG;
       per_sm = (int)std::min<int64_t>(per_sm, std::max<int64_t>(1, T.blocks_per_sm));
       k_aeo_index<V><<<g->sm_count * per_sm, threads, smem, s>>>(a, p);
@@ -568,14 +567,13 @@ ubt_status launch_aeo(const ubt_graph* g, int64_t L, const typename V::P& p, cud
                                       std::max<int64_t>(64, T.smem_table_max));
   a.unit = (uint32_t)std::min<int64_t>(32, std::max<int64_t>(1, T.block_unit));
   a.L = L;
-  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
+  UBT_CUDA(cudaMemsetAsync(a.sc->task, 0, kScratchQuery, s));
   if (a.n_owners == 0) return UBT_OK;
   const int threads = 512;
   const size_t tables = std::max<size_t>((size_t)a.cap, (size_t)(threads / 32) * a.wcap) * 3 * 4;
   const size_t smem = (size_t)((V::smem_bytes(p, threads) + 15) / 16) * 16 + tables;
-  UBT_CUDA(cudaFuncSetAttribute(k_aeo<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_aeo<V>, threads, smem));
+  UBT_CUDA(resident_blocks((const void*)k_aeo<V>, g->device, threads, smem, &per_sm));
   if (per_sm < 1) return UBT_ERR_INVALID_ARG;
   per_sm = (int)std::min<int64_t>(per_sm, std::max<int64_t>(1, T.blocks_per_sm));
   k_aeo<V><<<g->sm_count * per_sm, threads, smem, s>>>(a, p);

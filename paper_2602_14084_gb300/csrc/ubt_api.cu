@@ -5,6 +5,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "ubt_internal.cuh"
 
@@ -57,6 +58,38 @@ extern "C" const char* ubt_status_str(ubt_status s) {
     default: return "unknown status";
   }
 }
+
+namespace ubt {
+
+// A fixed table of launch shapes, by a hash of the kernel and its shape; a
+// shape that meets another one's place replaces it.  Shared memory is allowed
+// up to the device's limit at once, so no later call lowers it.
+cudaError_t resident_blocks(const void* kernel, int device, int threads, size_t smem, int* per_sm) {
+  struct Shape {
+    const void* kernel;
+    int device, threads;
+    size_t smem;
+    int per_sm;
+  };
+  constexpr size_t kShapes = 256;
+  static std::mutex mu;
+  static Shape shapes[kShapes];
+  const size_t at = (((uintptr_t)kernel >> 4) * 31 + smem * 7 + (size_t)threads + (size_t)device * 131) % kShapes;
+  std::lock_guard<std::mutex> lock(mu);
+  Shape& x = shapes[at];
+  if (x.kernel != kernel || x.device != device || x.threads != threads || x.smem != smem) {
+    const size_t most = std::max(smem, (size_t)226 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    int n = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem);
+    if (e != cudaSuccess) return e;
+    x = Shape{kernel, device, threads, smem, n};
+  }
+  *per_sm = x.per_sm;
+  return cudaSuccess;
+}
+
+}  // namespace ubt
 
 extern "C" int32_t ubt_version(void) { return 1 * 10000 + 0 * 100 + 0; }
 

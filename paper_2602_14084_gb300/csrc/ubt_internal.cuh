@@ -125,19 +125,23 @@ __device__ __forceinline__ uint32_t real_valbits(float p) {
 // Entries of the queue of long vertex samples (ubt_graph::lqueue).
 constexpr int kLongQueue = 1024;
 
-// Query scratch carved from the graph workspace (one per graph).
+// Query scratch carved from the graph workspace (one per graph).  From `task`
+// on it is zeroed per query, the threshold counts with their accumulators.
 struct Scratch {
+  unsigned long long err;           // device-side error word (build)
+  unsigned long long guard;         // first failed self-check of a query (0 = none)
+  unsigned long long pad[2];
   unsigned long long task[8];       // next task of every class, spare
   unsigned long long enum_cursor;   // enumeration append cursor
   unsigned long long tri_count;     // triangles seen (expected counts)
   unsigned long long sum_lo;        // 128-bit two's-complement sum, low word
   unsigned long long sum_hi;        // high word
-  unsigned long long err;           // device-side error word (build)
-  unsigned long long guard;         // first failed self-check of a query (0 = none)
-  unsigned long long pad[2];
+  unsigned long long done;          // blocks of the query's last kernel that have added their counts
+  unsigned long long pad2;
   unsigned long long hist[2 * 65];  // per-threshold accumulators (bal [0,64), unbal [64,128))
 };
-constexpr size_t kScratchQuery = 12 * sizeof(unsigned long long);  // the words up to err: zeroed per query
+constexpr size_t kScratchQuery = 14 * sizeof(unsigned long long);                       // from task: before hist
+constexpr size_t kScratchCounts = kScratchQuery + 2 * 65 * sizeof(unsigned long long);  // with hist
 
 }  // namespace ubt
 
@@ -304,6 +308,12 @@ inline int64_t table_slots(int64_t entries) {
   while (s < 4 * entries) s <<= 1;
   return s;
 }
+
+// Resident blocks per SM of a kernel on the current device (`device`) with
+// `threads` threads and `smem` bytes of dynamic shared memory, which the kernel
+// is allowed afterwards.  The last answers are kept (ubt_api.cu): asking the
+// runtime costs several microseconds a launch.
+cudaError_t resident_blocks(const void* kernel, int device, int threads, size_t smem, int* per_sm);
 
 // launch helpers implemented in ubt_scan.cu
 cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp,

@@ -531,14 +531,13 @@ ubt_status local_counts(ubt_graph* g, const uint32_t* d_items, int64_t k, int ve
   a.sc = g->scratch;
   a.bal = d_bal;
   a.unbal = d_unbal;
-  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
+  UBT_CUDA(cudaMemsetAsync(a.sc->task, 0, kScratchQuery, s));
   UBT_CUDA(cudaMemsetAsync(a.lq, 0, 2 * sizeof(unsigned long long), s));
   if (k > 0) {
     const int threads = 512;
     const size_t smem = 256 * 8 + 144 * 8 + (size_t)a.cap * 3 * 4;
-    UBT_CUDA(cudaFuncSetAttribute(k_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_local, threads, smem));
+    UBT_CUDA(resident_blocks((const void*)k_local, g->device, threads, smem, &per_sm));
     if (per_sm < 1) return UBT_ERR_INVALID_ARG;
     const int64_t blocks = std::min<int64_t>((int64_t)g->sm_count * per_sm, k);
     k_local<<<(int)blocks, threads, smem, s>>>(a, p);
@@ -824,13 +823,12 @@ extern "C" ubt_status ubt_vertex_topk(ubt_graph* g, const uint32_t* d_vertices, 
   a.sc = g->scratch;
   a.out = d_out;
   a.n_out = d_n_out;
-  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
+  UBT_CUDA(cudaMemsetAsync(a.sc->task, 0, kScratchQuery, s));
   if (k == 0) return UBT_OK;
   const int threads = 512;
   const size_t smem = 2064 * 4 + (size_t)kTopkCap * (8 + 12) + (size_t)a.cap * 3 * 4;
-  UBT_CUDA(cudaFuncSetAttribute(k_vertex_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_vertex_topk, threads, smem));
+  UBT_CUDA(resident_blocks((const void*)k_vertex_topk, g->device, threads, smem, &per_sm));
   if (per_sm < 1) return UBT_ERR_INVALID_ARG;
   const int64_t blocks = std::min<int64_t>((int64_t)g->sm_count * per_sm, k);
   k_vertex_topk<<<(int)blocks, threads, smem, s>>>(a);

@@ -272,7 +272,9 @@ struct CountBinsP {
   int nt;
   int64_t S[2 * kMaxTau];   // the 2 nt levels, ascending
   unsigned long long* out;  // global bins [0, 2 nt]
-  bool several = false;     // some slice holds several levels
+  int64_t* counts = nullptr;    // the answer (null: the bins are)
+  uint8_t perm[kMaxTau] = {0};  // caller index of the i-th smallest threshold
+  bool several = false;         // some slice holds several levels
   void set_several() {
     for (int j = 1; j < 2 * nt; j++) several |= ((S[j - 1] + (1ll << 45)) >> 35) == ((S[j] + (1ll << 45)) >> 35);
   }
@@ -282,7 +284,7 @@ struct CountBins : ProductItem {
   static constexpr bool kPos = false;
   static constexpr int kRegCap = UBT_COUNT_REGCAP;
   static constexpr int kTabBytes = ((kSlices + 15) / 16) * 16;
-  static constexpr int kLevelBytes = (2 * kMaxTau + 2) * 8;
+  static constexpr int kLevelBytes = (2 * kMaxTau + 2) * 8 + kMaxTau;
   // one warp's bins: 2 nt - 1 of them are used, [1, 2 nt)
   static __host__ __device__ int bin_stride(int nt) { return (2 * nt + 3) / 4 * 4; }
   static __host__ __device__ int smem_bytes(const P& p, int threads) {
@@ -296,8 +298,10 @@ struct CountBins : ProductItem {
   uint32_t first = 0, last = 0;  // bins 0 and 2 nt of this lane
   uint32_t since = 0;            // entries since the last flush (this lane's or the warp's)
   int top;                       // 2 nt
+  int64_t* counts;
+  const uint8_t* perm;           // shared
   bool several;                  // some slice holds several levels
-  __device__ CountBins(const P& p, char* smem) : out(p.out), top(2 * p.nt), several(p.several) {
+  __device__ CountBins(const P& p, char* smem) : out(p.out), top(2 * p.nt), counts(p.counts), several(p.several) {
     uint8_t* t = (uint8_t*)smem;
     long long* sv = (long long*)(smem + kTabBytes);
     uint32_t* b = (uint32_t*)(smem + kTabBytes + kLevelBytes);
@@ -306,7 +310,10 @@ struct CountBins : ProductItem {
     all = b;
     const int stride = bin_stride(p.nt);
     bins = b + (threadIdx.x >> 5) * stride;
+    uint8_t* pm = (uint8_t*)(sv + 2 * kMaxTau + 2);
+    perm = pm;
     for (int i = threadIdx.x; i <= 2 * p.nt; i += blockDim.x) sv[i] = i < 2 * p.nt ? p.S[i] : INT64_MAX;
+    for (int i = threadIdx.x; i < p.nt; i += blockDim.x) pm[i] = p.perm[i];
     for (int i = threadIdx.x; i < (int)(blockDim.x >> 5) * stride; i += blockDim.x) b[i] = 0;
     for (int i = threadIdx.x; i < kSlices; i += blockDim.x) {
       const long long start = (long long)i * (1ll << 35) - (1ll << 45);
@@ -369,6 +376,18 @@ struct CountBins : ProductItem {
       for (int w = 0; w < nw; w++) v += all[w * bin_stride(top / 2) + i];
       if (v) atomicAdd(&out[i], v);
     }
+  }
+  // bins -> counts, by the last block: the i-th smallest t has the
+  // (nt-1-i)-th smallest B and the i-th smallest U
+  __device__ void finish() {
+    const int i = (int)threadIdx.x, nt = top / 2;
+    if (!counts || i >= nt) return;
+    const volatile unsigned long long* b = out;
+    unsigned long long bal = 0, unbal = 0;
+    for (int r = 0; r <= nt - 1 - i; r++) bal += b[r];
+    for (int r = nt + i + 1; r <= top; r++) unbal += b[r];
+    counts[perm[i]] = (int64_t)bal;
+    counts[nt + perm[i]] = (int64_t)unbal;
   }
 };
 
@@ -803,8 +822,13 @@ ubt_status count_impl(ubt_graph* g, const double* h_tau, int32_t n_tau, int32_t 
     }
     p.set_several();
     p.out = g->scratch->hist;
+    if (!aeo) {
+      p.counts = d_counts;
+      for (int i = 0; i < n_tau; i++) p.perm[i] = (uint8_t)order[i];
+      return launch_traverse<CountBins>(g, p, L, s);
+    }
     UBT_CUDA(cudaMemsetAsync(g->scratch->hist, 0, sizeof(g->scratch->hist), s));
-    st = aeo ? launch_aeo<CountBinsAeo>(g, L, p, s) : launch_traverse<CountBins>(g, p, L, s);
+    st = launch_aeo<CountBinsAeo>(g, L, p, s);
     if (st != UBT_OK) return st;
     FinishMulti f;
     f.nt = n_tau;
@@ -1028,7 +1052,6 @@ ubt_status count_levels(const ubt_graph* g, const std::vector<int64_t>& lev, int
   for (size_t i = 0; i < lev.size(); i++) p.S[i] = lev[i];
   p.set_several();
   p.out = g->scratch->hist;
-  UBT_CUDA(cudaMemsetAsync(g->scratch->hist, 0, sizeof(g->scratch->hist), s));
   ubt_status st = launch_traverse<CountBins>(g, p, L, s);
   if (st != UBT_OK) return st;
   UBT_CUDA(cudaMemcpyAsync(h_bins, g->scratch->hist, sizeof(unsigned long long) * (lev.size() + 1),

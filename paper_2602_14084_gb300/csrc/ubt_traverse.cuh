@@ -112,6 +112,12 @@ struct HasProbed : std::false_type {};
 template <class V>
 struct HasProbed<V, std::void_t<decltype(std::declval<V&>().probed(0u))>> : std::true_type {};
 
+// visitors with a finish() member write their answer in the traversal's last block
+template <class V, class = void>
+struct HasFinish : std::false_type {};
+template <class V>
+struct HasFinish<V, std::void_t<decltype(std::declval<V&>().finish())>> : std::true_type {};
+
 // the fewest threads of the main kernel's blocks a visitor wants (kMinThreads)
 template <class V, class = void>
 struct MinThreads {
@@ -873,18 +879,21 @@ __device__ __forceinline__ void entry(const MergeTable& t, uint32_t slot, uint32
   pos = slot;
   w = adj_col(e);
 }
-constexpr uint32_t kMergeGrab = 256;  // pairs a warp takes at a time
+constexpr uint32_t kMergeGrab = 256;  // pairs a warp takes at a time, at most
 template <class V>
 __device__ __forceinline__ void merge_tasks(const TravArgs& a, V& vis, Queue<V>& queue) {
   const uint32_t lane = lane_id(), lt = lanemask_lt(), npairs = a.m - a.merge_first;
   const MergeTable t{a.adj};
   const uint64_t* __restrict__ adj = a.adj;
+  // few pairs: spread over all warps, 32 each, or a graph of 20,000 edges is 78
+  // warps' work (count of three thresholds 137 us a call, 104 spread)
+  const uint32_t grab = min(kMergeGrab, npairs / (gridDim.x * (blockDim.x >> 5)) / 32 * 32 + 32);
   while (true) {
     unsigned long long t0 = 0;
-    if (lane == 0) t0 = atomicAdd(&a.sc->task[7], (unsigned long long)kMergeGrab);
+    if (lane == 0) t0 = atomicAdd(&a.sc->task[7], (unsigned long long)grab);
     t0 = __shfl_sync(kFull, t0, 0);
     if (t0 >= npairs) break;
-    for (uint32_t p0 = (uint32_t)t0; p0 < min((unsigned long long)npairs, t0 + kMergeGrab); p0 += 32) {
+    for (uint32_t p0 = (uint32_t)t0; p0 < min((unsigned long long)npairs, t0 + grab); p0 += 32) {
       const Pair pr = owner_pair(a, kEmpty, a.merge_first + p0, min(32u, npairs - p0));
       uint32_t dv = pr.dv, rs = 0, len = 0, i = 0, j = 0;
       if (dv && (pr.x >= a.n || !owner_list(a, pr.x, rs, len))) {
@@ -1003,6 +1012,17 @@ __device__ void traverse(const TravArgs& a, V& vis, char* queues, char* tables) 
   }
   __syncthreads();
   vis.block_end();
+  // the last block of the main kernel turns the accumulators into the answer
+  if constexpr (kKernel == kMainKernel && HasFinish<V>::value) {
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_misc[3] = atomicAdd(&a.sc->done, 1ull) + 1 == gridDim.x ? 1u : 0u;
+    __syncthreads();
+    if (s_misc[3]) {
+      __threadfence();
+      vis.finish();
+    }
+  }
 }
 
 namespace {
@@ -1050,25 +1070,31 @@ ubt_status launch_kernel(const ubt_graph* g, const TravArgs& a, const typename V
       8 * resident_warps<V, kKernel>(a, p, threads) < 7 * resident_warps<V, kKernel>(a, p, 2 * threads))
     threads *= 2;
   const size_t smem = visitor_bytes<V>(p, threads) + traverse_table_bytes<V>(a, kKernel, threads);
-  UBT_CUDA(cudaFuncSetAttribute(k_traverse<V, kKernel>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  UBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse<V, kKernel>, threads, smem));
+  UBT_CUDA(resident_blocks((const void*)k_traverse<V, kKernel>, g->device, threads, smem, &per_sm));
   if (per_sm < 1) return UBT_ERR_INVALID_ARG;
   per_sm = (int)std::min<int64_t>(per_sm, std::max<int64_t>(1, T.blocks_per_sm));
-  k_traverse<V, kKernel><<<g->sm_count * per_sm, threads, smem, s>>>(a, p);
+  int64_t blocks = (int64_t)g->sm_count * per_sm;
+  if (kKernel == kMainKernel) {  // no more blocks than there is work for: each sets up its visitor's tables
+    const int64_t warps = a.n_tasks[kMedHash] + a.n_tasks[kMedBits] + (a.m - a.merge_first + 31) / 32;
+    blocks = std::min(blocks, std::max<int64_t>(1, a.n_tasks[kHubBits] + (warps + threads / 32 - 1) / (threads / 32)));
+  }
+  k_traverse<V, kKernel><<<(int)blocks, threads, smem, s>>>(a, p);
   UBT_CUDA(cudaGetLastError());
   return UBT_OK;
 }
 
 // One traversal: the task counters in a.sc are cleared, then the kernels that
-// have tasks run one after the other on `s`.
+// have tasks run one after the other on `s` (the main one always where the
+// visitor's answer is written by its last block).
 template <class V>
 ubt_status launch_traversal(const ubt_graph* g, const TravArgs& a, const typename V::P& p, cudaStream_t s) {
   UBT_RANGE("traversal launch");
-  UBT_CUDA(cudaMemsetAsync(a.sc, 0, kScratchQuery, s));
+  UBT_CUDA(cudaMemsetAsync(a.sc->task, 0, HasFinish<V>::value ? kScratchCounts : kScratchQuery, s));
   ubt_status st = UBT_OK;
   if (a.n_tasks[kGiant] + a.n_tasks[kHubHash]) st = launch_kernel<V, kHashKernel>(g, a, p, s);
-  if (st == UBT_OK && a.n_tasks[kHubBits] + a.n_tasks[kMedHash] + a.n_tasks[kMedBits] + (a.m - a.merge_first))
+  if (st == UBT_OK && (HasFinish<V>::value || a.n_tasks[kHubBits] + a.n_tasks[kMedHash] + a.n_tasks[kMedBits] +
+                                                  (a.m - a.merge_first)))
     st = launch_kernel<V, kMainKernel>(g, a, p, s);
   return st;
 }
