@@ -104,11 +104,12 @@ typedef struct {
      * ubt_edge_local_counts and ubt_vertex_local_counts need.
      * UBT_OPT_EDGE_INDEX (with UBT_OPT_UNDIRECTED): also build a hash index
      * of the edges ({u, w} -> edge value; 16 bytes per slot, the power of two
-     * >= 4m slots).  Same results, different work: ubt_vertex_local_counts
-     * and ubt_vertex_topk look a neighbour pair up in it instead of streaming
-     * a neighbour's row when that row is much longer than the pairs left to
-     * check; ubt_count_aeo and ubt_enumerate_aeo stream, for each edge, the
-     * shorter of its two Lemma 3 windows and look the closing edge up, with
+     * >= 4m slots).  Same results, different work: ubt_edge_local_counts and
+     * ubt_vertex_local_counts look every closing edge up instead of building a
+     * table per sample; ubt_vertex_topk looks a neighbour pair up instead of
+     * streaming a neighbour's row when that row is much longer than the pairs
+     * left to check; ubt_count_aeo and ubt_enumerate_aeo stream, for each edge,
+     * the shorter of its two Lemma 3 windows and look the closing edge up, with
      * no owner tables (knob "edge_index" = 0 keeps the table forms). */
     int64_t flags;
 } ubt_graph_opts;
@@ -519,16 +520,17 @@ ubt_status ubt_topk(ubt_graph* g, int64_t K, int32_t which, ubt_tri_rec* d_out, 
  *                     concatenated with the short lists; 0: the warp streams
  *                     them itself with idle lanes
  *   "edge_index"      on a graph with UBT_OPT_EDGE_INDEX: 0 never use the
- *                     index; 1 (default) vertex local counts / per-vertex
- *                     top-k use it for a neighbour whose row is more than 8
- *                     times longer than the pairs left to check, and the AEO
- *                     calls use its form; 2 as 1, the vertex queries for every
+ *                     index; 1 (default) local counts and the AEO calls
+ *                     use its form, and per-vertex top-k uses it for a
+ *                     neighbour whose row is more than 8 times longer than the
+ *                     pairs left to check; 2 as 1, per-vertex top-k for every
  *                     neighbour
  *   "vertex_split"    ubt_vertex_local_counts on a graph with the edge index:
- *                     samples whose pruned row is longer (default 64) are
+ *                     samples whose pruned row is longer (default 32) are
  *                     spread over the warps of all blocks by a second launch
- *                     (at most 1,024 per call; the rest are counted by one
- *                     block each)
+ *                     (at most 3,072 per call, and 1,024 with rows of more
+ *                     than 1,024 entries; the rest are counted by one warp
+ *                     each)
  *   "world_words_per_pass"  most 64-world words per traversal of
  *                     ubt_sample_worlds (1, 2, 4, 8, 16, 32 or 64, default
  *                     64; fewer where the sign table of m x 8 bytes a word

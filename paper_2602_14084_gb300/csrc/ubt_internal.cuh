@@ -122,8 +122,11 @@ __device__ __forceinline__ uint32_t real_valbits(float p) {
 }
 #endif
 
-// Entries of the queue of long vertex samples (ubt_graph::lqueue).
-constexpr int kLongQueue = 1024;
+// Entries of the queue of long samples (ubt_graph::lqueue), the last
+// kLongest of them kept for samples of more than kLongestRow entries.
+constexpr int kLongest = 1024;
+constexpr uint32_t kLongestRow = 1024;
+constexpr int kLongQueue = 4096;
 
 // Query scratch carved from the graph workspace (one per graph).  From `task`
 // on it is zeroed per query, the threshold counts with their accumulators.
@@ -182,7 +185,7 @@ struct ubt_graph {
   uint64_t* apairs = nullptr;       // m: streamed endpoint | position of the edge in x's row << 32
   uint32_t* alist = nullptr;        // owners, by decreasing streamed work
   int64_t n_aowners = 0, n_ablock = 0, max_udeg = 0;  // owners; the first n_ablock are block tasks
-  unsigned long long* lqueue = nullptr;  // with the undirected rows: 2 + kLongQueue words, the vertex
+  unsigned long long* lqueue = nullptr;  // with the undirected rows: 3 + kLongQueue words, the long
                                          // samples a local-count call spreads over all blocks
   uint4* eslots = nullptr;          // edge index (UBT_OPT_EDGE_INDEX; else null): eh_slots slots of
                                     // 16 bytes, key in the first 8, edge value (valbits) in the next 4
@@ -228,7 +231,7 @@ struct Tuning {
   int64_t long_min = 64;          // streamed lists this long are streamed by the whole warp
   int64_t long_tail = 1;          // 1: the last < 64 entries of such a list join the short lists
   int64_t edge_index = 1;         // vertex queries: 0 never look pairs up in the edge index, 1 when cheaper, 2 always
-  int64_t vertex_split = 64;      // vertex samples with longer pruned rows are spread over all blocks (edge index)
+  int64_t vertex_split = 32;      // vertex samples with longer pruned rows are spread over all blocks (edge index)
   int64_t sort_smem_max = 4096;   // longer forward lists are sorted in global memory
   int64_t warp_sort_max = 256;    // lists up to this long are sorted by one warp in registers
 };

@@ -33,6 +33,7 @@ namespace {
 
 constexpr int kLocalTau = 64;
 constexpr int kLocalSub = 256;  // streamed entries per warp task of an edge sample
+constexpr uint32_t kEdgeSplit = 512;  // with the edge index: entries of an edge sample one warp looks up
 
 struct LocalP {
   int nt;
@@ -173,13 +174,16 @@ EdgeIndex edge_index_of(const ubt_graph* g) {
   return ix;
 }
 
-// Vertex samples whose pruned row is longer than `split` (with the edge
-// index) are not counted by one block: the sampling kernel queues them (at
-// most kLongCap per query; more are counted in place) and a second launch
-// spreads their neighbours over the warps of all blocks.  The queue
-// (ubt_graph::lqueue): [0] queued, [1] next warp task, [2 + i] entry i =
-// row length << 32 | sample index.
+// Samples with more entries than `split` (vertices) or kEdgeSplit (edges) are
+// not counted by one warp: the sampling kernel queues them and a second launch
+// spreads their work over the warps of all blocks.  The queue
+// (ubt_graph::lqueue): [0] queued with at most kLongestRow entries, [1] next
+// warp task, [2] queued with more, [3 + i] entry i = row length << 32 | sample
+// index.  The longest have room of their own, so that a large call's many
+// moderate samples cannot leave a hub to one warp; what finds no room is
+// counted in place.
 constexpr int kLongCap = kLongQueue;
+constexpr int kLongFirst = kLongCap - kLongest;
 
 struct LocalArgs {
   const uint32_t* uptr;
@@ -225,6 +229,149 @@ __device__ __forceinline__ void index_neighbours(const LocalArgs& a, const Local
     if (a.L > 0) len = prune_prefix(a.uadj + s0, len, qabs(qp) * qmax, a.L);
     index_pairs(a.ix, a.uadj, x, av, qp, rs + j, rs + tlen, s0, len, a.L, lane, a.sc,
                 [&](long long P, uint32_t) { atomicAdd(&bins[level_of(S, p.half, P)], 1ull); });
+  }
+}
+
+// The endpoints and value of sampled edge `id` and the range of the shorter
+// row that can hold a classified triangle: x the other endpoint, entries [s0,
+// s0 + len) of the shorter row up to |q| |q_e| 2^15 >= L.  False: none, or
+// (reported by the caller's lane 0) not an edge.
+__device__ __forceinline__ bool edge_sample(const LocalArgs& a, uint32_t id, uint32_t& x, uint32_t& qe, uint32_t& s0,
+                                            uint32_t& len, bool report) {
+  if (id >= a.m) {
+    if (report) guard_fail(a.sc, kGuardList, id);
+    return false;
+  }
+  const uint32_t p0 = a.uepos[2 * (size_t)id], p1 = a.uepos[2 * (size_t)id + 1];
+  const uint64_t e0 = a.uadj[p0], e1 = a.uadj[p1];
+  const uint32_t lo = adj_col(e1), hi = adj_col(e0);
+  qe = adj_valbits(e0);
+  if (a.L > 0 && qabs(qe) * (1ll << 30) < a.L) return false;  // Lemma 2 on e
+  const uint32_t slo = a.uptr[lo], shi = a.uptr[hi], dlo = a.uptr[lo + 1] - slo, dhi = a.uptr[hi + 1] - shi;
+  x = dhi >= dlo ? hi : lo;
+  s0 = dhi >= dlo ? slo : shi;
+  len = min(dlo, dhi);
+  if (a.L > 0) len = prune_prefix(a.uadj + s0, len, qabs(qe) * 32768, a.L);
+  return len > 0;
+}
+// Triangles through edge x-y: every entry y-w of [s0, s1), the closing edge
+// x-w looked up.  (Where x-w is beyond its own cutoff, |P| < L: no threshold
+// counts it.)
+__device__ __forceinline__ void edge_entries(const LocalArgs& a, const LocalP& p, const long long* S,
+                                             unsigned long long* bins, uint32_t x, uint32_t qe, uint32_t s0, uint32_t s1,
+                                             int lane) {
+  for (uint32_t b0 = s0; b0 < s1; b0 += 64) {
+    bool act[2], hit[2];
+    uint32_t oo[2], ww[2], qxw[2];
+    uint64_t ew[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const uint32_t pos = b0 + 32 * u + lane;
+      ew[u] = pos < s1 ? a.uadj[pos] : 0ull;
+      ww[u] = adj_col(ew[u]);
+      oo[u] = x;
+      act[u] = pos < s1 && ww[u] != x;
+    }
+    edge_index_find2(a.ix, act, oo, ww, hit, qxw, a.sc);
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+      if (hit[u])
+        atomicAdd(&bins[level_of(S, p.half, (long long)((int32_t)qe * (int32_t)adj_valbits(ew[u])) *
+                                                 (long long)(int32_t)qxw[u])], 1ull);
+  }
+}
+
+// Samples on a graph with the edge index: one warp each, no table -- a sampled
+// edge streams its shorter row, a sampled vertex takes the pairs of its row's
+// prefix, and every closing edge is looked up.  A sample with more than
+// `split` entries is queued for the split launch (kLongCap of them; more are
+// counted here).  A block and its table per sample, as without the index, kept
+// an SM at two samples at a time (Chung-Lu of 1e6 vertices, 10,000 samples:
+// edges 301 -> 59 us with the split launch, vertices 718 -> 580).
+constexpr int kSampleThreads = 128;
+__global__ void __launch_bounds__(kSampleThreads) k_sample_warps(LocalArgs a, LocalP p) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ long long S[256];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  unsigned long long* bins = (unsigned long long*)smem + (size_t)wid * (2 * p.nt + 1);
+  for (int i = tid; i < 256; i += kSampleThreads) S[i] = i < 2 * p.nt ? p.S[i] : INT64_MAX;
+  for (int r = lane; r <= 2 * p.nt; r += 32) bins[r] = 0;
+  __syncthreads();
+  while (true) {
+    unsigned long long t = 0;
+    if (lane == 0) t = atomicAdd(&a.sc->task[0], 1ull);
+    t = __shfl_sync(kFull, t, 0);
+    if (t >= a.n_items) break;
+    const uint32_t item = (uint32_t)t, id = a.items[item];
+    uint32_t x = 0, qe = 0, s0 = 0, len = 0;
+    int64_t qmax = 0;
+    bool ok = true;
+    if (!a.vertex_mode) {
+      ok = edge_sample(a, id, x, qe, s0, len, lane == 0);
+    } else if (id >= a.n) {
+      if (lane == 0) guard_fail(a.sc, kGuardVertex, id);
+      ok = false;
+    } else {
+      x = id;
+      s0 = a.uptr[x];
+      len = a.uptr[x + 1] - s0;
+      if (a.L > 0 && len > 0) {
+        qmax = qabs(adj_valbits(a.uadj[s0]));
+        len = prune_prefix(a.uadj + s0, len, 1ll << 30, a.L);  // Lemma 2
+      }
+      ok = len > 1;
+    }
+    if (ok && len > (a.vertex_mode ? a.split : kEdgeSplit)) {
+      uint32_t queued = 0;
+      if (lane == 0) {
+        const bool longest = len > kLongestRow;
+        const unsigned long long slot = atomicAdd(&a.lq[longest ? 2 : 0], 1ull);
+        if (slot < (unsigned long long)(longest ? kLongest : kLongFirst)) {
+          a.lq[3 + (longest ? kLongFirst : 0) + slot] = ((unsigned long long)len << 32) | item;
+          queued = 1;
+        }
+      }
+      if (__shfl_sync(kFull, queued, 0)) ok = false;  // its counts here stay 0
+    }
+    if (ok) {
+      if (!a.vertex_mode) {
+        edge_entries(a, p, S, bins, x, qe, s0, s0 + len, lane);
+      } else if (len <= 64) {
+        // the row's prefix in two registers; for every first neighbour all later ones
+        const uint64_t r0 = (uint32_t)lane < len ? a.uadj[s0 + lane] : 0ull;
+        const uint64_t r1 = (uint32_t)lane + 32 < len ? a.uadj[s0 + 32 + lane] : 0ull;
+        for (uint32_t i = 0; i + 1 < len; i++) {
+          const uint64_t ea = i < 32 ? __shfl_sync(kFull, r0, (int)i) : __shfl_sync(kFull, r1, (int)(i - 32));
+          const bool act[2] = {(uint32_t)lane > i && (uint32_t)lane < len,
+                               (uint32_t)lane + 32 > i && (uint32_t)lane + 32 < len};
+          const uint32_t oo[2] = {adj_col(ea), adj_col(ea)}, ww[2] = {adj_col(r0), adj_col(r1)};
+          bool hit[2];
+          uint32_t q[2];
+          edge_index_find2(a.ix, act, oo, ww, hit, q, a.sc);
+#pragma unroll
+          for (int u = 0; u < 2; u++)
+            if (hit[u])
+              atomicAdd(&bins[level_of(S, p.half, (long long)((int32_t)adj_valbits(ea) *
+                                                              (int32_t)adj_valbits(u ? r1 : r0)) *
+                                                      (long long)(int32_t)q[u])], 1ull);
+        }
+      } else {
+        index_neighbours(a, p, S, bins, x, s0, len, qmax, 0, len - 1, 1, lane);
+      }
+    }
+    __syncwarp();
+    // histogram -> counts: the i-th smallest t has the (nt-1-i)-th smallest B
+    // and the i-th smallest U
+    for (int i = lane; i < p.nt; i += 32) {
+      unsigned long long b = 0, u = 0;
+      for (int r = 0; r <= p.nt - 1 - i; r++) b += bins[r];
+      for (int r = p.nt + i + 1; r <= 2 * p.nt; r++) u += bins[r];
+      a.bal[(size_t)item * p.nt + p.perm[i]] = (int64_t)b;
+      a.unbal[(size_t)item * p.nt + p.perm[i]] = (int64_t)u;
+    }
+    __syncwarp();
+    for (int r = lane; r <= 2 * p.nt; r += 32) bins[r] = 0;
+    __syncwarp();
   }
 }
 
@@ -286,24 +433,6 @@ __global__ void __launch_bounds__(512, 2) k_local(LocalArgs a, LocalP p) {
     }
     const uint32_t rs = a.uptr[x];
     const uint32_t chunk = a.cap / 4;
-    if (ok && a.vertex_mode && a.ix.mode != 0 && (tlen > chunk || tlen > a.split)) {
-      // a long row: no table, every pair from the edge index -- counted by the
-      // split launch when the queue has room (its counts here stay 0), else here
-      if (tid == 0) {
-        uint32_t queued = 0;
-        if (tlen > a.split) {
-          const unsigned long long slot = atomicAdd(&a.lq[0], 1ull);
-          if (slot < (unsigned long long)kLongCap) {
-            a.lq[2 + slot] = ((unsigned long long)tlen << 32) | item;
-            queued = 1;
-          }
-        }
-        s_misc[1] = queued;
-      }
-      __syncthreads();
-      if (!s_misc[1]) index_neighbours(a, p, S, bins, x, rs, tlen, qmax, wid, tlen ? tlen - 1 : 0, nw, lane);
-      ok = false;  // skip the table chunks
-    }
     for (uint32_t c0 = 0; ok && c0 < tlen; c0 += chunk) {
       const uint32_t c1 = min(tlen, c0 + chunk);
       const uint32_t slots = slots_for(c1 - c0);
@@ -336,23 +465,6 @@ __global__ void __launch_bounds__(512, 2) k_local(LocalArgs a, LocalP p) {
           uint32_t len = a.uptr[av + 1] - s0;
           if (a.L > 0) len = prune_prefix(a.uadj + s0, len, qabs(qp) * qmax, a.L);
           s1 = s0 + len;
-          // the same triangles from v's side: b after a in this chunk of v's
-          // row, each pair a-b looked up in the edge index
-          const uint32_t b_lo = max(pp + 1, rs + c0), b_hi = rs + c1;
-          if (use_index(a.ix, b_hi - b_lo, len)) {
-            for (uint32_t b0 = b_lo; b0 < b_hi; b0 += 32) {
-              const uint32_t pos = b0 + lane;
-              const bool act = pos < b_hi;
-              const uint64_t eb = act ? a.uadj[pos] : 0ull;
-              uint32_t qab = 0;
-              const bool hit = act && edge_index_find(a.ix, av, adj_col(eb), qab, a.sc);
-              if (hit) {
-                const long long P = (long long)((int32_t)qp * (int32_t)adj_valbits(eb)) * (long long)(int32_t)qab;
-                atomicAdd(&bins[level_of(S, p.half, P)], 1ull);
-              }
-            }
-            continue;
-          }
         }
         for (uint32_t b0 = s0; b0 < s1; b0 += 32) {
           const uint32_t pos = b0 + lane;
@@ -385,11 +497,18 @@ __global__ void __launch_bounds__(512, 2) k_local(LocalArgs a, LocalP p) {
 }
 
 // The split launch: the queued vertex samples' neighbours, kWarpNb per warp
-// task from one counter over all queued samples, no block barriers.  Each
+// task, or the queued edge samples' entries, kEdgeSplit per warp task, from one
+// counter over all queued samples, no block barriers.  Each
 // warp bins into its own shared histogram and adds its per-threshold counts
 // to the sample's outputs (zero after the sampling kernel) when it moves on
 // to another sample or runs out of tasks.
 constexpr uint32_t kWarpNb = 4;
+
+// warp tasks of a queued sample of `len` entries
+__device__ __forceinline__ uint32_t split_tasks(const LocalArgs& a, uint32_t len) {
+  return a.vertex_mode ? (len - 1 + kWarpNb - 1) / kWarpNb  // neighbours 0 .. len - 2
+                       : (len + kEdgeSplit - 1) / kEdgeSplit;
+}
 
 __device__ __forceinline__ void flush_bins(const LocalArgs& a, const LocalP& p, unsigned long long* wb,
                                            uint32_t item, int lane) {
@@ -414,27 +533,31 @@ __global__ void __launch_bounds__(512, 2) k_local_split(LocalArgs a, LocalP p) {
   unsigned long long* wb = (unsigned long long*)smem + (size_t)wid * (2 * p.nt + 1);  // this warp's bins
   for (int i = tid; i < 256; i += blockDim.x) S[i] = i < 2 * p.nt ? p.S[i] : INT64_MAX;
   for (int r = lane; r <= 2 * p.nt; r += 32) wb[r] = 0;
-  const uint32_t nq = (uint32_t)min(a.lq[0], (unsigned long long)kLongCap);
-  if (wid == 0) {
-    // first warp task of every entry: lane l sums entries [l * seg, (l + 1) * seg),
-    // a warp scan gives each lane its segment's start
-    constexpr uint32_t seg = (kLongCap + 31) / 32;
-    const uint32_t b0 = lane * seg, b1 = min(nq, b0 + seg);
+  const uint32_t n0 = (uint32_t)min(a.lq[0], (unsigned long long)kLongFirst);
+  const uint32_t nq = n0 + (uint32_t)min(a.lq[2], (unsigned long long)kLongest);
+  if (nq == 0) return;
+  auto queued = [&](uint32_t i) { return a.lq[3 + (i < n0 ? i : kLongFirst + (i - n0))]; };
+  {  // first warp task of every entry: a thread sums its segment, the block scans the sums
+    __shared__ uint32_t s_warp[16];
+    constexpr uint32_t seg = (kLongCap + 511) / 512;
+    const uint32_t b0 = min(nq, tid * seg), b1 = min(nq, b0 + seg);
     uint32_t mine = 0;
-    for (uint32_t i = b0; i < b1; i++)
-      mine += ((uint32_t)(a.lq[2 + i] >> 32) - 1 + kWarpNb - 1) / kWarpNb;  // neighbours 0 .. tlen - 2
+    for (uint32_t i = b0; i < b1; i++) mine += split_tasks(a, (uint32_t)(queued(i) >> 32));
     uint32_t incl = mine;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const uint32_t y = __shfl_up_sync(kFull, incl, d);
       if (lane >= d) incl += y;
     }
+    if (lane == 31) s_warp[wid] = incl;
+    __syncthreads();
     uint32_t acc = incl - mine;
+    for (int w = 0; w < wid; w++) acc += s_warp[w];
     for (uint32_t i = b0; i < b1; i++) {
       pref[i] = acc;
-      acc += ((uint32_t)(a.lq[2 + i] >> 32) - 1 + kWarpNb - 1) / kWarpNb;
+      acc += split_tasks(a, (uint32_t)(queued(i) >> 32));
     }
-    if (lane == 31) pref[nq] = incl;
+    if (tid == 511) pref[nq] = acc;
   }
   __syncthreads();
   const uint32_t total = pref[nq];
@@ -450,12 +573,20 @@ __global__ void __launch_bounds__(512, 2) k_local_split(LocalArgs a, LocalP p) {
       const uint32_t mid = (e + hi + 1) >> 1;
       if (pref[mid] <= task) e = mid; else hi = mid - 1;
     }
-    const unsigned long long ent = a.lq[2 + e];
+    const unsigned long long ent = queued(e);
     const uint32_t item = (uint32_t)ent, tlen = (uint32_t)(ent >> 32);
     if (e != cur) {
       if (cur != 0xFFFFFFFFu) flush_bins(a, p, wb, cur_item, lane);
       cur = e;
       cur_item = item;
+    }
+    if (!a.vertex_mode) {
+      uint32_t x = 0, qe = 0, s0 = 0, len = 0;
+      if (edge_sample(a, a.items[item], x, qe, s0, len, false)) {
+        const uint32_t b0 = min(len, (task - pref[e]) * kEdgeSplit);
+        edge_entries(a, p, S, wb, x, qe, s0 + b0, s0 + min(len, b0 + kEdgeSplit), lane);
+      }
+      continue;
     }
     const uint32_t x = a.items[item], rs = a.uptr[x];
     const int64_t qmax = a.L > 0 ? qabs(adj_valbits(a.uadj[rs])) : 0;
@@ -474,7 +605,7 @@ __global__ void k_local_estimate(const int64_t* __restrict__ bal, const int64_t*
     sb += (double)bal[(size_t)i * nt + t];
     su += (double)unbal[(size_t)i * nt + t];
   }
-  __shared__ double rb[256], ru[256];
+  __shared__ double rb[1024], ru[1024];
   rb[threadIdx.x] = sb;
   ru[threadIdx.x] = su;
   __syncthreads();
@@ -532,25 +663,29 @@ ubt_status local_counts(ubt_graph* g, const uint32_t* d_items, int64_t k, int ve
   a.bal = d_bal;
   a.unbal = d_unbal;
   UBT_CUDA(cudaMemsetAsync(a.sc->task, 0, kScratchQuery, s));
-  UBT_CUDA(cudaMemsetAsync(a.lq, 0, 2 * sizeof(unsigned long long), s));
+  UBT_CUDA(cudaMemsetAsync(a.lq, 0, 3 * sizeof(unsigned long long), s));
   if (k > 0) {
     const int threads = 512;
-    const size_t smem = 256 * 8 + 144 * 8 + (size_t)a.cap * 3 * 4;
-    int per_sm = 0;
-    UBT_CUDA(resident_blocks((const void*)k_local, g->device, threads, smem, &per_sm));
-    if (per_sm < 1) return UBT_ERR_INVALID_ARG;
-    const int64_t blocks = std::min<int64_t>((int64_t)g->sm_count * per_sm, k);
-    k_local<<<(int)blocks, threads, smem, s>>>(a, p);
-    UBT_CUDA(cudaGetLastError());
-    if (vertex_mode && a.ix.mode != 0) {
-      const size_t wbytes = (size_t)(threads / 32) * (2 * n_tau + 1) * 8;  // per-warp bins
-      k_local_split<<<(int)(g->sm_count * 2), threads, wbytes, s>>>(a, p);
+    if (a.ix.mode != 0) {
+      const size_t wbins = (size_t)(2 * n_tau + 1) * 8;  // bytes of a warp's bins
+      const int64_t blocks = std::min<int64_t>((k + kSampleThreads / 32 - 1) / (kSampleThreads / 32), (int64_t)g->sm_count * 12);
+      k_sample_warps<<<(int)blocks, kSampleThreads, (kSampleThreads / 32) * wbins, s>>>(a, p);
+      UBT_CUDA(cudaGetLastError());
+      k_local_split<<<(int)(g->sm_count * 2), threads, (threads / 32) * wbins, s>>>(a, p);
+      UBT_CUDA(cudaGetLastError());
+    } else {
+      const size_t smem = 256 * 8 + 144 * 8 + (size_t)a.cap * 3 * 4;
+      int per_sm = 0;
+      UBT_CUDA(resident_blocks((const void*)k_local, g->device, threads, smem, &per_sm));
+      if (per_sm < 1) return UBT_ERR_INVALID_ARG;
+      const int64_t blocks = std::min<int64_t>((int64_t)g->sm_count * per_sm, k);
+      k_local<<<(int)blocks, threads, smem, s>>>(a, p);
       UBT_CUDA(cudaGetLastError());
     }
   }
   if (d_est) {
     const double scale = (vertex_mode ? (double)g->n : (double)g->m) / 3.0;
-    k_local_estimate<<<n_tau, 256, 0, s>>>(d_bal, d_unbal, (uint32_t)k, n_tau, scale, d_est);
+    k_local_estimate<<<n_tau, 1024, 0, s>>>(d_bal, d_unbal, (uint32_t)k, n_tau, scale, d_est);
     UBT_CUDA(cudaGetLastError());
   }
   return UBT_OK;
