@@ -168,9 +168,9 @@ def merge_model_bytes(n, src, dst):
 
 def alg_bytes_of(st):
     """Algorithmic bytes of one traversal (ubt_traversal_stats sizes): 8 B per
-    table entry, 24 B per pair (its pair word, its edge's CSR entry and the
-    streamed list's two offsets), 8 B per streamed entry."""
-    return 8 * st["table_entries"] + 24 * st["pairs"] + 8 * st["streamed"]
+    table entry, 16 B per pair (its pair word, which says where the streamed
+    entries lie, and its edge's CSR entry), 8 B per streamed entry."""
+    return 8 * st["table_entries"] + 16 * st["pairs"] + 8 * st["streamed"]
 
 
 def ncu_traffic(kernel, workload):
@@ -459,8 +459,8 @@ def main():
     times_unpruned = time_steps(step_unpruned, max(3, args.steps // 4), 1, flush)
 
     # roofline of the dominant kernel (the traversal): algorithmic bytes =
-    # 8 B per table entry loaded + 24 B per pair (pair word, its edge's entry,
-    # the streamed list's offsets) + 8 B per streamed entry
+    # 8 B per table entry loaded + 16 B per pair (pair word, its edge's entry)
+    # + 8 B per streamed entry
     st = G.traversal_stats(TAUS, prune=True)
     alg_bytes = alg_bytes_of(st)
     pk, pk_kind = peaks()
@@ -549,10 +549,11 @@ def main():
                 "ms_per_step_min": 1e3 * float(np.min(e2e_times)),
                 "ms_per_step_all": [round(1e3 * x, 2) for x in e2e_times], "h2d_ms": h2d_ms, "clocks": e2e_clk,
                 "includes": "H2D of src/dst/k, graph build (validate, orient, CSR, sort), query, D2H"},
-        # per query: the block-task traversal (giant / hub owners), the
-        # warp-task traversal (medium owners; this workload has both) and the
-        # kernel that turns the bins into counts
-        "gpu_launches": args.steps * ((1 if info["hub_vertices"] > 0 else 0) + 1 + 1),
+        # per query one kernel: all owners of this workload that are tasks of
+        # a block have bitmap tables (no hash kernel), the lowest level keeps
+        # nearly every edge (no kept entries are written), and the last block
+        # of the traversal turns the bins into counts
+        "gpu_launches": args.steps,
         "clocks": clk,
         "build_ms": build_ms,
         "tuning": {k: tuning[k] for k in ("source", "config", "key") if k in tuning},

@@ -7,10 +7,9 @@ they only move work between task kinds, warps and blocks -- but the best
 setting depends on the graph's degree distribution, the query and the GPU.
 This module picks them by measurement:
 
-* knobs that act when a graph is built (``BUILD_KNOBS``: the pair
-  partition, the block-task limits on list length and streamed work, the
-  shared-memory table limit) and knobs that
-  act on every query (``RUN_KNOBS``: block shapes, blocks per SM, work-grab
+* knobs that act when a graph is built (``BUILD_KNOBS``: the
+  limits on a warp task's list length and streamed work, the shared-memory
+  table limit) and knobs that act on every query (``RUN_KNOBS``: block shapes, blocks per SM, work-grab
   sizes, sign-world words per pass);
 * coordinate descent over a small candidate list per knob, starting from the
   current settings: one knob at a time, every candidate timed with CUDA events
@@ -40,7 +39,6 @@ import numpy as np
 
 # candidate values per knob (the library validates each against its limits)
 BUILD_KNOBS: Dict[str, List[int]] = {
-    "pull": [1, 0],
     "hub_threshold": [32, 64, 128, 256, 512],
     "block_work": [1 << 12, 1 << 14, 1 << 16, 1 << 18, 1 << 20],
     "smem_table_max": [4096, 8192, 16384],
@@ -50,7 +48,7 @@ RUN_KNOBS: Dict[str, List[int]] = {
     "block_unit": [1, 2, 4, 8, 16, 32],
     "small_batch": [1, 2, 4, 8, 16],
     "block_threads": [128, 256, 512],
-    "warp_threads": [64, 128],
+    "warp_threads": [64, 128, 256],
     "blocks_per_sm": [1, 2, 4, 32],
     "world_words_per_pass": [1, 2, 4, 8, 16, 32, 64],
     "long_min": [32, 48, 64, 96, 128],
@@ -59,9 +57,9 @@ RUN_KNOBS: Dict[str, List[int]] = {
 # knobs that matter per query kind (others are left as they are)
 QUERY_KNOBS: Dict[str, List[str]] = {
     "count": ["count_visitor", "hub_threshold", "block_work", "block_unit", "small_batch", "blocks_per_sm",
-              "block_threads", "warp_threads", "smem_table_max", "pull", "long_min", "long_tail"],
+              "block_threads", "warp_threads", "smem_table_max", "long_min", "long_tail"],
     "expected": ["hub_threshold", "block_work", "block_unit", "small_batch", "blocks_per_sm", "block_threads",
-                 "warp_threads", "smem_table_max", "pull"],
+                 "warp_threads", "smem_table_max"],
     "worlds": ["world_words_per_pass", "hub_threshold", "block_work", "block_unit", "small_batch",
                "blocks_per_sm", "long_tail", "long_min"],
     "batch": ["block_threads", "hub_threshold", "block_work", "block_unit", "small_batch", "warp_threads",

@@ -16,9 +16,10 @@
 //   vertex v:      its row's Lemma 2 prefix; for each a there, a's row up to
 //                  |q_ab| |q_va| qmax(v) >= L, and b counts once, at the later
 //                  of the two positions in v's row
-// One block per sample: the longer list (edge) or v's row (vertex) becomes a
-// shared-memory hash table, in chunks when it is longer than one table, and
-// the other lists are streamed through it.  Every triangle found is placed
+// With the edge index a warp takes a sample and looks the closing edges up
+// (k_sample_warps).  Without it one block per sample: the longer list (edge)
+// or v's row (vertex) becomes a shared-memory hash table, in chunks when it is
+// longer than one table, and the other lists are streamed through it.  Every triangle found is placed
 // among the sorted threshold levels by binary search and counted in a
 // per-sample shared histogram, turned into per-threshold counts at the end.
 #include <algorithm>

@@ -179,3 +179,23 @@ def test_undirected_rows_of_every_length(ubt, deg, smem_max):
     got = G.count_aeo([0.55, 0.8])
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
     assert G.guard() == 0
+
+
+@pytest.mark.parametrize("core,taus", [(640, [0.6, 0.95]), (1100, [0.5, 0.8])])
+def test_edge_and_vertex_samples_of_long_rows_with_the_index(ubt, core, taus):
+    """Samples looked up in the edge index by one warp (rows up to 512 entries of
+    an edge, 32 of a vertex) or by many (longer rows, queued; rows of more than
+    1,024 entries in a part of the queue kept for them): both sides of each
+    limit, more samples than either part of the queue holds, repeats."""
+    n = core + 900
+    s, d = core_graph(n, 6000, core, 11)
+    k = synth.k_uniform(s.size, 12)
+    eb, eu, vb, vu = oracle.local_counts(n, s, d, k, taus)
+    G = ubt.Graph(n, s, d, k=k, undirected=True, edge_index=True)
+    es = synth.rng(13).integers(0, s.size, size=9000).astype(np.uint32)
+    gb, gu, _ = G.edge_local_counts(es, taus)
+    assert np.array_equal(gb, eb[es]) and np.array_equal(gu, eu[es])
+    vs = synth.rng(14).integers(0, n, size=7000).astype(np.uint32)
+    gb, gu, _ = G.vertex_local_counts(vs, taus)
+    assert np.array_equal(gb, vb[vs]) and np.array_equal(gu, vu[vs])
+    assert G.guard() == 0
