@@ -206,3 +206,31 @@ def test_vertex_topk_every_vertex(ubt, table_max, n_list):
         assert G.guard() == 0
     finally:
         ubt.set_tuning("smem_table_max", old)
+
+
+@pytest.mark.parametrize("p", ["strong", "weak", "one_sign"])
+def test_topk_first_range_and_candidate_sorts(ubt, p):
+    """The first range counted follows the edges' |q| (many strong edges; none;
+    strong edges whose triangles are nearly all of one sign, where the other
+    sign's search starts over), and the candidates' sort crosses its chunks:
+    the records are the oracle's, in its order."""
+    n = 1 << 12
+    s, d = synth.rmat(12, 40, 0.57, 0.19, 0.19, 21)
+    k = synth.k_uniform(s.size, 22)
+    if p == "strong":
+        k = synth.quantise(synth.p_beta(s.size, 0.5, 0.5, 23))
+    elif p == "weak":
+        k = 32768 + (k >> 6) - 512
+    else:  # all edges surely positive but some weak ones
+        k = np.where(k < 20000, 30000 + (k >> 4), 65535 - (k >> 8)).astype(np.uint32)
+    G = ubt.Graph(n, s, d, k=k.astype(np.uint32))
+    for which in (1, 2):
+        want_uvw, want_pb = oracle_topk(n, s, d, k.astype(np.uint32), 20000, which)
+        for K in (1, 1000, 2047, 2049, 6000, 20000):
+            rec = G.topk(K, which)
+            got_uvw = np.stack([rec["u"], rec["v"], rec["w"]], axis=1).astype(np.uint32)
+            assert np.array_equal(rec["p_bal"], want_pb[:K]), (K, which)
+            tied = want_pb == want_pb[min(K, want_pb.size) - 1]   # ties of the last value: any of them
+            sure = int(np.argmax(tied))
+            assert np.array_equal(got_uvw[:sure], want_uvw[:sure]), (K, which)
+    assert G.guard() == 0
