@@ -217,13 +217,6 @@ __global__ void k_out_degree(int64_t m, const uint32_t* __restrict__ src, const 
   }
 }
 
-// forward entries that name a vertex: its degree less its own list (in place)
-__global__ void k_in_degree(int64_t n, const uint32_t* __restrict__ deg, const uint32_t* __restrict__ vid,
-                            const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ indeg) {
-  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
-    indeg[r] = deg[vid[r]] - (row_ptr[r + 1] - row_ptr[r]);
-}
-
 __global__ void k_scatter(int64_t m, const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
                           const uint32_t* __restrict__ k, const float* __restrict__ p,
                           const uint32_t* __restrict__ rank, uint32_t* __restrict__ next,
@@ -588,7 +581,9 @@ ubt_status launch_block_sorts(const uint32_t* rows, uint32_t nrows, const uint32
 }
 
 // Longer lists: one block per list, bitonic network in a per-block global
-// slice (lists longer than the "sort_smem_max" tuning).
+// slice (lists longer than the "sort_smem_max" tuning).  A list longer than a
+// slice names a vertex twice: each of its vertices has at least its length as
+// degree, so distinct ones are at most sqrt(2m).
 __global__ void k_sort_long_rows(const uint32_t* __restrict__ rows, uint32_t nrows, const uint32_t* __restrict__ row_ptr,
                                  uint64_t* adj, uint32_t* eid, uint32_t* ekey, unsigned long long* err,
                                  char* gtmp, int64_t gtmp_cap) {
@@ -596,6 +591,10 @@ __global__ void k_sort_long_rows(const uint32_t* __restrict__ rows, uint32_t nro
     const uint32_t u = rows[r];
     const uint32_t rs = row_ptr[u], re = row_ptr[u + 1];
     const uint32_t len = re - rs;
+    if ((int64_t)len > gtmp_cap) {
+      if (threadIdx.x == 0) report(err, rs, -UBT_ERR_DUPLICATE_EDGE);
+      continue;
+    }
     uint32_t cap = 64;
     while (cap < len) cap <<= 1;
     char* base = gtmp + (size_t)blockIdx.x * (size_t)gtmp_cap * 24;
@@ -660,10 +659,15 @@ __global__ void k_collect_long(int64_t n, const uint32_t* __restrict__ row_ptr, 
   }
 }
 
-// rowid[p] = the row that holds CSR position p (one thread per row)
-__global__ void k_row_ids(int64_t n, const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ rowid) {
-  for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x)
-    for (uint32_t p = row_ptr[u]; p < row_ptr[u + 1]; p++) rowid[p] = (uint32_t)u;
+// rowid[p] = the row that holds CSR position p, and the forward entries that
+// name a vertex: its degree less its own list (one thread per row)
+__global__ void k_row_ids(int64_t n, const uint32_t* __restrict__ row_ptr, const uint32_t* __restrict__ deg,
+                          const uint32_t* __restrict__ vid, uint32_t* __restrict__ rowid, uint32_t* __restrict__ indeg) {
+  for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t b = row_ptr[u], e = row_ptr[u + 1];
+    indeg[u] = deg[vid[u]] - (e - b);
+    for (uint32_t p = b; p < e; p++) rowid[p] = (uint32_t)u;
+  }
 }
 
 // Pair words grouped by owner.  next[v] holds the next free position of owner
@@ -733,10 +737,6 @@ k_pair_fill(int64_t m, const uint32_t* __restrict__ row_ptr, const uint64_t* __r
     for (int i = threadIdx.x; i < 65; i += kFillThreads)
       if (s_q[i]) atomicAdd(&absq[i], (unsigned long long)s_q[i]);
   }
-}
-__global__ void k_pair_next(int64_t n, const uint32_t* __restrict__ pair_ptr, unsigned long long* __restrict__ next) {
-  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-    next[x] = pair_ptr[x];
 }
 
 constexpr uint8_t kNoTask = 0xFF;
@@ -836,15 +836,36 @@ __global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ r
   }
 }
 
-// Task lists: every block ranks its owners' tasks per bucket in shared memory
-// and reserves one range per bucket with a single global atomic.
+// Task lists, by class and in a class by falling bucket: every block ranks its
+// owners' tasks per bucket in shared memory and reserves one range per bucket
+// with a single global atomic.  Where a bucket starts follows from the bucket
+// sizes, summed up by each block: a copy of them to the host and the starts
+// back, with a wait between, was 15 us of every build.  cursor: zero before.
 __global__ void k_fill_lists(int64_t n, int64_t m, const unsigned long long* __restrict__ work,
                              const uint32_t* __restrict__ pair_ptr, const uint8_t* __restrict__ bucket,
                              const unsigned long long* __restrict__ stats, unsigned long long* cursor,
                              uint64_t* __restrict__ lists) {
   __shared__ uint32_t s_cnt[kTaskBuckets];
   __shared__ unsigned long long s_base[kTaskBuckets];
+  __shared__ uint32_t s_first[kTaskBuckets], s_all[kTaskClasses], s_class[kTaskClasses];
   const unsigned long long whole = whole_work(stats[2], m);
+  for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x) s_first[i] = (uint32_t)stats[kStatBuckets + i];
+  __syncthreads();
+  if (threadIdx.x < kTaskClasses) {  // a class's buckets, the largest work first
+    uint32_t run = 0;
+    for (int b = kLgTask * kTaskClasses + threadIdx.x; b >= 0; b -= kTaskClasses) {
+      const uint32_t size = s_first[b];
+      s_first[b] = run;
+      run += size;
+    }
+    s_all[threadIdx.x] = run;
+  }
+  __syncthreads();
+  if (threadIdx.x < kTaskClasses) {
+    uint32_t run = 0;
+    for (int c = 0; c < (int)threadIdx.x; c++) run += s_all[c];
+    s_class[threadIdx.x] = run;
+  }
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
     for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x) s_cnt[i] = 0;
     __syncthreads();
@@ -857,7 +878,7 @@ __global__ void k_fill_lists(int64_t n, int64_t m, const unsigned long long* __r
     }
     __syncthreads();
     for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x)
-      if (s_cnt[i]) s_base[i] = atomicAdd(&cursor[i], (unsigned long long)s_cnt[i]);
+      if (s_cnt[i]) s_base[i] = s_class[i % kTaskClasses] + s_first[i] + atomicAdd(&cursor[i], (unsigned long long)s_cnt[i]);
     __syncthreads();
     if (b != kNoTask)
       for (uint32_t i = 0; i < parts; i++)
@@ -1122,6 +1143,7 @@ struct BuildLayout {
   size_t total;
 };
 constexpr int kStats = kStatBuckets + kTaskBuckets;
+constexpr int kLengths = 2 * kStats, kClasses = kLengths + 4, kBuildWords = kClasses + 65;
 static_assert(kStats >= 2 * (kLgMax + 1), "the undirected owners' cursors share the array");
 
 int64_t list_bound(int64_t n, int64_t m) {
@@ -1191,7 +1213,7 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.huge_rows = c.take<uint32_t>(n1);
   L.bucket = c.take<uint8_t>(n1);
   L.work = c.take<unsigned long long>(n1);
-  L.stats = c.take<unsigned long long>(2 * kStats + 4 + 65);
+  L.stats = c.take<unsigned long long>(kBuildWords);
   const int64_t lb = list_bound(n, m);
   L.sort_tmp = lb > tuning().sort_smem_max
                    ? c.take<char>((size_t)kSortHugeBlocks * (size_t)pow2_at_least(lb) * 24) : nullptr;
@@ -1293,10 +1315,14 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   const int64_t block_work = std::max<int64_t>(1, T.block_work);
 
   UBT_CUDA(cudaMemsetAsync(L.scratch, 0, sizeof(Scratch), s));
-  UBT_CUDA(cudaMemsetAsync(&L.scratch->err, 0xFF, sizeof(unsigned long long), s));
-  UBT_CUDA(cudaMemsetAsync(L.deg, 0, sizeof(uint32_t) * (n + 1), s));
-  UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
-  UBT_CUDA(cudaMemsetAsync(L.stats, 0, sizeof(unsigned long long) * (2 * kStats + 4 + 65), s));
+  UBT_CUDA(cudaMemsetAsync(L.deg, 0, (size_t)((char*)(L.fill + n + 1) - (char*)L.deg), s));  // deg and fill
+  UBT_CUDA(cudaMemsetAsync(L.stats, 0, sizeof(unsigned long long) * kBuildWords, s));
+  // what the host reads lies together, as a copy to the host is 15 us: bucket
+  // statistics, list cursors, row lengths (first the largest degree), the
+  // first error, |q| classes
+  unsigned long long* const lcount = L.stats + kLengths;
+  unsigned long long* const derr = lcount + 3;
+  UBT_CUDA(cudaMemsetAsync(derr, 0xFF, sizeof(unsigned long long), s));
   const int thr = 256;
   const int grid_e = (int)std::min<int64_t>(std::max<int64_t>((m + thr - 1) / thr, 1), (int64_t)sms * 32);
   const int grid_v = (int)std::min<int64_t>(std::max<int64_t>((n + thr - 1) / thr, 1), (int64_t)sms * 32);
@@ -1309,26 +1335,23 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   NvtxPhases phase;
   phase.next("build: validate and degree");
   if (m > 0)
-    k_validate_degree<<<grid_e, thr, 0, s>>>(n, m, d_src, d_dst, d_k, d_p, L.vgraph_id, L.deg, &L.scratch->err);
-  unsigned long long* lcount = L.stats + 2 * kStats;  // row lengths; first the largest degree
+    k_validate_degree<<<grid_e, thr, 0, s>>>(n, m, d_src, d_dst, d_k, d_p, L.vgraph_id, L.deg, derr);
   if (n > 0) k_degree_stats<<<grid_v, thr, 0, s>>>(n, L.deg, lcount);
-  unsigned long long err = 0, deg_stats[2] = {0, 0};
+  unsigned long long deg_stats[4] = {0, 0, 0, 0};
   UBT_CUDA(cudaMemcpyAsync(deg_stats, lcount, sizeof(deg_stats), cudaMemcpyDeviceToHost, s));
-  UBT_CUDA(cudaMemcpyAsync(&err, &L.scratch->err, sizeof(err), cudaMemcpyDeviceToHost, s));
   UBT_CUDA(cudaStreamSynchronize(s));
-  ubt_status st = status_from_err(err);
+  ubt_status st = status_from_err(deg_stats[3]);
   if (st != UBT_OK) return st;
   // 2. orientation + CSR offsets
   phase.next("build: orient, scatter, sort");
   if (n > 0) {
-    UBT_CUDA(cudaMemsetAsync(lcount, 0, sizeof(deg_stats), s));
+    UBT_CUDA(cudaMemsetAsync(lcount, 0, 3 * sizeof(unsigned long long), s));
     st = rank_vertices(L, n, deg_stats[0], ng, s);
     if (st != UBT_OK) return st;
     if (batch) k_rank_graphs<<<grid_v, thr, 0, s>>>(n, L.vid, L.vgraph_id, L.vgraph, opts->d_vertex_offsets, ng, L.gstart);
   }
   if (m > 0) k_out_degree<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, L.rank, L.fill);
-  UBT_CUDA(exclusive_scan_u32(L.fill, L.row_ptr, n, L.scan_tmp, s));
-  UBT_CUDA(cudaMemcpyAsync(L.fill, L.row_ptr, sizeof(uint32_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
+  UBT_CUDA(exclusive_scan_u32(L.fill, L.row_ptr, n, L.scan_tmp, s, L.fill));
   if (m > 0)
     k_scatter<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, d_p, L.rank, L.fill, L.adj, L.eid,
                                      opts ? opts->d_edge_key : nullptr, L.ekey);
@@ -1336,7 +1359,7 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   const int fixed = flags == UBT_GRAPH_FIXED;
   const int mode = kSortById;
   if (n > 0) {
-    k_sort_short_rows<<<grid_w, thr, 0, s>>>(n, L.row_ptr, L.adj, L.eid, L.ekey, mode, &L.scratch->err);
+    k_sort_short_rows<<<grid_w, thr, 0, s>>>(n, L.row_ptr, L.adj, L.eid, L.ekey, mode, derr);
     const uint32_t sort_smem = (uint32_t)tuning().sort_smem_max;
     const uint32_t warp_max = (uint32_t)tuning().warp_sort_max;
     k_collect_long<<<grid_v, thr, 0, s>>>(n, L.row_ptr, sort_smem, warp_max, L.mid_rows, L.huge_rows, lcount);
@@ -1345,43 +1368,37 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
     UBT_CUDA(cudaStreamSynchronize(s));
     if (lc[2]) {
       st = launch_mid_sorts(L.mid_rows + (n - (int64_t)lc[2]), (uint32_t)lc[2], L.row_ptr, L.adj, L.eid, L.ekey, mode,
-                            &L.scratch->err, warp_max, sms, thr, s);
+                            derr, warp_max, sms, thr, s);
       if (st != UBT_OK) return st;
     }
     if (lc[0]) {
-      st = launch_block_sorts(L.mid_rows, (uint32_t)lc[0], L.row_ptr, L.adj, L.eid, L.ekey, mode, &L.scratch->err,
+      st = launch_block_sorts(L.mid_rows, (uint32_t)lc[0], L.row_ptr, L.adj, L.eid, L.ekey, mode, derr,
                               warp_max, sort_smem, sms, s);
       if (st != UBT_OK) return st;
     }
     if (lc[1]) {
-      const int64_t cap = pow2_at_least(list_bound(n, m));
+      const int64_t cap = L.sort_tmp ? pow2_at_least(list_bound(n, m)) : 0;
       const int g = (int)std::min<unsigned long long>(lc[1], (unsigned long long)kSortHugeBlocks);
       k_sort_long_rows<<<g, 1024, 0, s>>>(L.huge_rows, (uint32_t)lc[1], L.row_ptr, L.adj, L.eid, L.ekey,
-                                          &L.scratch->err, L.sort_tmp, cap);
+                                          derr, L.sort_tmp, cap);
     }
     UBT_CUDA(cudaGetLastError());
   }
-  UBT_CUDA(cudaMemcpyAsync(&err, &L.scratch->err, sizeof(err), cudaMemcpyDeviceToHost, s));
-  UBT_CUDA(cudaStreamSynchronize(s));
-  st = status_from_err(err);
-  if (st != UBT_OK) return st;
-  // 4. pairs grouped by owner
+  // 4. pairs grouped by owner.  (Rows with a duplicate are known by now, but
+  // not here: the host looks once, at the end.  Nothing below reads more of
+  // such rows than their lengths.)
   phase.next("build: pairs and work lists");
-  unsigned long long* absq = fixed ? L.stats + 2 * kStats + 4 : nullptr;
-  UBT_CUDA(cudaMemsetAsync(L.pair_ptr, 0, sizeof(uint32_t) * (n + 1), s));
+  unsigned long long* absq = fixed ? L.stats + kClasses : nullptr;
+  if (n == 0) UBT_CUDA(cudaMemsetAsync(L.pair_ptr, 0, sizeof(uint32_t), s));
   if (n > 0) {
-    k_row_ids<<<grid_v, thr, 0, s>>>(n, L.row_ptr, L.rowid);
-    k_in_degree<<<grid_v, thr, 0, s>>>(n, L.deg, L.vid, L.row_ptr, L.fill);
-    UBT_CUDA(exclusive_scan_u32(L.fill, L.pair_ptr, n, L.scan_tmp, s));
-    k_pair_next<<<grid_v, thr, 0, s>>>(n, L.pair_ptr, L.work);
+    k_row_ids<<<grid_v, thr, 0, s>>>(n, L.row_ptr, L.deg, L.vid, L.rowid, L.fill);
+    UBT_CUDA(exclusive_scan_u32(L.fill, L.pair_ptr, n, L.scan_tmp, s, nullptr, L.work));
     const int grid_f = (int)std::min<int64_t>((m + kFillTile - 1) / kFillTile, (int64_t)sms * 8);
     if (m > 0) k_pair_fill<<<grid_f, kFillThreads, 0, s>>>(m, L.row_ptr, L.adj, L.rowid, L.work, L.pairs, absq, &L.stats[2]);
     UBT_CUDA(cudaGetLastError());
   }
   // 5. work lists: the owners of every task class by decreasing work bucket
-  unsigned long long stats[kStats], classes[65];
-  memset(stats, 0, sizeof(stats));
-  memset(classes, 0, sizeof(classes));
+  unsigned long long stats[kBuildWords];
   // vertices of degree <= kMergeDegree are the last ones (of a batch, every
   // graph's last ones: its pairs all go to tables)
   const int64_t merge_from = batch ? n : (int64_t)deg_stats[1];
@@ -1389,29 +1406,16 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
     k_row_stats<<<grid_v, thr, 0, s>>>(n, m, L.row_ptr, L.pair_ptr, L.work, L.vgraph, L.gstart, (uint32_t)hub_thr,
                                       (uint32_t)giant_thr, (unsigned long long)block_work, (uint32_t)T.block_bits,
                                       (uint32_t)T.warp_bits, merge_from, L.bucket, L.stats);
-    UBT_CUDA(cudaMemcpyAsync(stats, L.stats, sizeof(stats), cudaMemcpyDeviceToHost, s));
-    if (absq) UBT_CUDA(cudaMemcpyAsync(classes, absq, sizeof(classes), cudaMemcpyDeviceToHost, s));
-    UBT_CUDA(cudaStreamSynchronize(s));
+    k_fill_lists<<<grid_v, thr, 0, s>>>(n, m, L.work, L.pair_ptr, L.bucket, L.stats, L.stats + kStats, L.lists);
+    UBT_CUDA(cudaGetLastError());
   }
-  unsigned long long cursor[kTaskBuckets];
-  int64_t count_cls[kTaskClasses] = {}, first_cls[kTaskClasses] = {}, run[kTaskClasses] = {};
+  UBT_CUDA(cudaMemcpyAsync(stats, L.stats, sizeof(stats), cudaMemcpyDeviceToHost, s));
+  UBT_CUDA(cudaStreamSynchronize(s));
+  st = status_from_err(stats[kLengths + 3]);
+  if (st != UBT_OK) return st;
+  int64_t count_cls[kTaskClasses] = {}, first_cls[kTaskClasses] = {};
   for (int b = 0; b < kTaskBuckets; b++) count_cls[b % kTaskClasses] += (int64_t)stats[kStatBuckets + b];
   for (int c = 1; c < kTaskClasses; c++) first_cls[c] = first_cls[c - 1] + count_cls[c - 1];
-  for (int lg = kLgTask; lg >= 0; lg--) {
-    for (int c = 0; c < kTaskClasses; c++) {
-      const int b = lg * kTaskClasses + c;
-      cursor[b] = (unsigned long long)(first_cls[c] + run[c]);
-      run[c] += (int64_t)stats[kStatBuckets + b];
-    }
-  }
-  if (n > 0) {
-    unsigned long long* dcur = L.stats + kStats;
-    UBT_CUDA(cudaMemcpyAsync(dcur, cursor, sizeof(cursor), cudaMemcpyHostToDevice, s));
-    k_fill_lists<<<grid_v, thr, 0, s>>>(n, m, L.work, L.pair_ptr, L.bucket, L.stats, dcur, L.lists);
-    UBT_CUDA(cudaGetLastError());
-    UBT_CUDA(cudaStreamSynchronize(s));
-  }
-  (void)ng;
   // 6. undirected adjacency in Absolute Edge Order, its mirror positions and
   //    the AEO pair partition (optional)
   int64_t n_aowners = 0, n_ablock = 0, max_udeg = 0;
@@ -1423,7 +1427,7 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
     UBT_CUDA(exclusive_scan_u32(L.deg, L.uptr, n, L.scan_tmp, s));
     UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
     if (m > 0) k_uscatter<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, L.uptr, L.fill, L.uadj, L.ueid, urow);
-    k_sort_short_rows<<<grid_w, thr, 0, s>>>(n, L.uptr, L.uadj, L.ueid, nullptr, kSortByAbsq, &L.scratch->err);
+    k_sort_short_rows<<<grid_w, thr, 0, s>>>(n, L.uptr, L.uadj, L.ueid, nullptr, kSortByAbsq, derr);
     const uint32_t sort_smem = (uint32_t)tuning().sort_smem_max;
     UBT_CUDA(cudaMemsetAsync(lcount, 0, 3 * sizeof(unsigned long long), s));
     const uint32_t warp_max = (uint32_t)tuning().warp_sort_max;
@@ -1433,17 +1437,17 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
     UBT_CUDA(cudaStreamSynchronize(s));
     if (lc[2]) {
       st = launch_mid_sorts(L.mid_rows + (n - (int64_t)lc[2]), (uint32_t)lc[2], L.uptr, L.uadj, L.ueid, nullptr,
-                            kSortByAbsq, &L.scratch->err, warp_max, sms, thr, s);
+                            kSortByAbsq, derr, warp_max, sms, thr, s);
       if (st != UBT_OK) return st;
     }
     if (lc[0]) {
       st = launch_block_sorts(L.mid_rows, (uint32_t)lc[0], L.uptr, L.uadj, L.ueid, nullptr, kSortByAbsq,
-                              &L.scratch->err, warp_max, sort_smem, sms, s);
+                              derr, warp_max, sort_smem, sms, s);
       if (st != UBT_OK) return st;
     }
     if (lc[1]) {
       st = sort_huge_rows(L.huge_rows, (uint32_t)lc[1], L.uptr, L.uadj, L.ueid, (uint64_t*)L.uepos,
-                          (uint32_t*)L.apairs, &L.scratch->err, sort_smem, deg_stats[0], sms, s);
+                          (uint32_t*)L.apairs, derr, sort_smem, deg_stats[0], sms, s);
       if (st != UBT_OK) return st;
     }
     if (m > 0) {
@@ -1457,12 +1461,11 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
       while ((1ll << lg) < L.eh_slots) lg++;
       if (m > 0)
         k_edge_index<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, L.eslots, (uint64_t)L.eh_slots, 64 - lg, L.efilter,
-                                            &L.scratch->err);
+                                            derr);
     }
     UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
     if (m > 0) k_apair_count<<<grid_2, thr, 0, s>>>(m2, L.uptr, L.uadj, urow, L.fill);
-    UBT_CUDA(exclusive_scan_u32(L.fill, L.apair_ptr, n, L.scan_tmp, s));
-    k_pair_next<<<grid_v, thr, 0, s>>>(n, L.apair_ptr, L.awork);
+    UBT_CUDA(exclusive_scan_u32(L.fill, L.apair_ptr, n, L.scan_tmp, s, nullptr, L.awork));
     if (m > 0) k_apair_fill<<<grid_2, thr, 0, s>>>(m2, L.uptr, L.uadj, urow, L.awork, L.apairs);
     unsigned long long* acur = L.stats;  // 2 (kLgMax + 1) cursors
     constexpr int kAB = 2 * (kLgMax + 1);
@@ -1483,7 +1486,8 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
     n_aowners = (int64_t)run;
     UBT_CUDA(cudaMemcpyAsync(acur, acount, sizeof(acount), cudaMemcpyHostToDevice, s));
     k_afill_lists<<<grid_v, thr, 0, s>>>(n, L.uptr, L.apair_ptr, L.awork, acur, L.alist, 0);
-    UBT_CUDA(cudaMemcpyAsync(&err, &L.scratch->err, sizeof(err), cudaMemcpyDeviceToHost, s));
+    unsigned long long err = 0;
+    UBT_CUDA(cudaMemcpyAsync(&err, derr, sizeof(err), cudaMemcpyDeviceToHost, s));
     UBT_CUDA(cudaGetLastError());
     UBT_CUDA(cudaStreamSynchronize(s));
     max_udeg = (int64_t)deg_stats[0];
@@ -1504,7 +1508,7 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   g->rowid = L.rowid;
   g->keep = L.keep;
   g->keep_tmp = L.keep_tmp;
-  for (int b = 64; b >= 0; b--) g->kept[b] = g->kept[b + 1] + (double)classes[b];
+  for (int b = 64; b >= 0; b--) g->kept[b] = g->kept[b + 1] + (double)stats[kClasses + b];
   for (int b = 64; b >= 0; b--) g->kept[b] = g->kept[0] > 0 ? g->kept[b] / g->kept[0] : 1.0;
   g->ekey = L.ekey ? L.ekey : L.eid;
   g->pair_ptr = L.pair_ptr;

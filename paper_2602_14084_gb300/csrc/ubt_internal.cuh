@@ -319,8 +319,8 @@ inline int64_t table_slots(int64_t entries) {
 cudaError_t resident_blocks(const void* kernel, int device, int threads, size_t smem, int* per_sm);
 
 // launch helpers implemented in ubt_scan.cu
-cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp,
-                               cudaStream_t s);
+cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp, cudaStream_t s,
+                               uint32_t* copy = nullptr, unsigned long long* wide = nullptr);
 size_t scan_tmp_words(int64_t n);
 cudaError_t keep_entries(const uint64_t* adj, int64_t m, uint32_t qmin, uint32_t* keep, uint64_t* kept, uint32_t* tmp,
                          cudaStream_t s);

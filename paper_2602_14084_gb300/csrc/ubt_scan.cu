@@ -79,8 +79,20 @@ __global__ void k_scan_tiles(uint32_t* tile_sum, int64_t ntiles) {
   if (threadIdx.x == 0) tile_sum[ntiles] = carry;
 }
 
-__global__ void k_tile_apply(const uint32_t* in, int64_t n, const uint32_t* __restrict__ tile_off,
-                             uint32_t* out) {
+// The sums also go to `copy` and, as 64-bit words, to `wide` (either may be
+// null): the build's fill cursors start as its offsets.
+struct ScanOut {
+  uint32_t* out;
+  uint32_t* copy;
+  unsigned long long* wide;
+  __device__ __forceinline__ void put(int64_t i, uint32_t v) const {
+    out[i] = v;
+    if (copy) copy[i] = v;
+    if (wide) wide[i] = v;
+  }
+};
+
+__global__ void k_tile_apply(const uint32_t* in, int64_t n, const uint32_t* __restrict__ tile_off, ScanOut out) {
   const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kScanItems;
   uint32_t v[kScanItems];
   uint32_t s = 0;
@@ -94,14 +106,14 @@ __global__ void k_tile_apply(const uint32_t* in, int64_t n, const uint32_t* __re
   uint32_t run = tile_off[blockIdx.x] + ex;
 #pragma unroll
   for (int i = 0; i < kScanItems; i++) {
-    if (base + i < n) out[base + i] = run;
+    if (base + i < n) out.put(base + i, run);
     run += v[i];
   }
 }
 
 // The scan of at most kSmallTiles tiles in one launch, total at out[n].
 constexpr int64_t kSmallTiles = 4;
-__global__ void k_scan_small(const uint32_t* in, int64_t n, uint32_t* out) {
+__global__ void k_scan_small(const uint32_t* in, int64_t n, ScanOut out) {
   uint32_t carry = 0;
   for (int64_t start = 0; start < n; start += kTile) {
     const int64_t base = start + (int64_t)threadIdx.x * kScanItems;
@@ -117,12 +129,12 @@ __global__ void k_scan_small(const uint32_t* in, int64_t n, uint32_t* out) {
     uint32_t run = carry + ex;
 #pragma unroll
     for (int i = 0; i < kScanItems; i++) {
-      if (base + i < n) out[base + i] = run;
+      if (base + i < n) out.put(base + i, run);
       run += v[i];
     }
     carry += tot;
   }
-  if (threadIdx.x == 0) out[n] = carry;
+  if (threadIdx.x == 0) out.out[n] = carry;
 }
 
 // Kept entries (|q| >= qmin) per tile of row entries, and, with the scanned
@@ -171,17 +183,20 @@ __global__ void k_write_total(const uint32_t* tile_off, int64_t ntiles, uint32_t
 
 size_t scan_tmp_words(int64_t n) { return (size_t)((n + kTile - 1) / kTile) + 2; }
 
-// out[0..n] = exclusive prefix sums of in[0..n), out[n] = total.  `in` and
-// `out` may alias.  tmp holds scan_tmp_words(n) words.
-cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp, cudaStream_t s) {
+// out[0..n] = exclusive prefix sums of in[0..n), out[n] = total; copy[0..n) and
+// wide[0..n), where given, the sums again.  `in` may alias `out` or `copy`.
+// tmp holds scan_tmp_words(n) words.
+cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* tmp, cudaStream_t s,
+                               uint32_t* copy, unsigned long long* wide) {
+  const ScanOut to{out, copy, wide};
   const int64_t ntiles = (n + kTile - 1) / kTile;
   if (ntiles <= kSmallTiles) {
-    k_scan_small<<<1, kScanThreads, 0, s>>>(in, n, out);
+    k_scan_small<<<1, kScanThreads, 0, s>>>(in, n, to);
     return cudaGetLastError();
   }
   k_tile_sums<<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp);
   k_scan_tiles<<<1, kScanThreads, 0, s>>>(tmp, ntiles);
-  k_tile_apply<<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp, out);
+  k_tile_apply<<<(unsigned)ntiles, kScanThreads, 0, s>>>(in, n, tmp, to);
   k_write_total<<<1, 1, 0, s>>>(tmp, ntiles, out, n);
   return cudaGetLastError();
 }

@@ -189,3 +189,14 @@ def test_layout_under_other_partitions(ubt, knobs):
     finally:
         for k, v in old.items():
             ubt.set_tuning(k, v)
+
+
+@pytest.mark.parametrize("copies", [4090, 4097, 9000])
+def test_one_edge_many_times(ubt, copies):
+    """A forward row longer than any simple graph's, and longer than a shared
+    memory sort takes, is refused as a duplicate edge."""
+    s = np.concatenate([np.zeros(copies, np.uint32), np.array([1, 2], np.uint32)])
+    d = np.concatenate([np.ones(copies, np.uint32), np.array([2, 3], np.uint32)])
+    with pytest.raises(ubt.UbtError) as err:
+        ubt.Graph(4, s, d, k=synth.k_uniform(s.size, 20))
+    assert err.value.status == -3
