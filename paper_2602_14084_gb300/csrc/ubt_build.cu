@@ -1191,7 +1191,7 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.apairs = und ? c.take<uint64_t>(std::max<int64_t>(m, 1)) : nullptr;
   L.alist = und ? c.take<uint32_t>(n1) : nullptr;
   L.awork = und ? c.take<unsigned long long>(n1) : nullptr;
-  L.lqueue = und ? c.take<unsigned long long>(3 + kLongQueue) : nullptr;
+  L.lqueue = und ? c.take<unsigned long long>(kLongHead + kLongQueue) : nullptr;
   const bool eidx = und && (opts->flags & UBT_OPT_EDGE_INDEX);
   L.efilter = und ? c.take<uint32_t>((size_t)(pow2_at_least(std::max<int64_t>(4 * m, 64)) >> kEdgeFilterLog)) : nullptr;
   L.eh_slots = eidx ? pow2_at_least(std::max<int64_t>(4 * m, 64)) : 0;

@@ -127,6 +127,7 @@ __device__ __forceinline__ uint32_t real_valbits(float p) {
 constexpr int kLongest = 1024;
 constexpr uint32_t kLongestRow = 1024;
 constexpr int kLongQueue = 4096;
+constexpr int kLongHead = 5;  // counters in front of them
 
 // Query scratch carved from the graph workspace (one per graph).  From `task`
 // on it is zeroed per query, the threshold counts with their accumulators.
@@ -185,7 +186,7 @@ struct ubt_graph {
   uint64_t* apairs = nullptr;       // m: streamed endpoint | position of the edge in x's row << 32
   uint32_t* alist = nullptr;        // owners, by decreasing streamed work
   int64_t n_aowners = 0, n_ablock = 0, max_udeg = 0;  // owners; the first n_ablock are block tasks
-  unsigned long long* lqueue = nullptr;  // with the undirected rows: 3 + kLongQueue words, the long
+  unsigned long long* lqueue = nullptr;  // with the undirected rows: kLongHead + kLongQueue words, the long
                                          // samples a local-count call spreads over all blocks
   uint4* eslots = nullptr;          // edge index (UBT_OPT_EDGE_INDEX; else null): eh_slots slots of
                                     // 16 bytes, key in the first 8, edge value (valbits) in the next 4

@@ -179,12 +179,19 @@ EdgeIndex edge_index_of(const ubt_graph* g) {
 // not counted by one warp: the sampling kernel queues them and a second launch
 // spreads their work over the warps of all blocks.  The queue
 // (ubt_graph::lqueue): [0] queued with at most kLongestRow entries, [1] next
-// warp task, [2] queued with more, [3 + i] entry i = row length << 32 | sample
+// warp task, [2] queued with more, [3] samples left over, [4] next sample to
+// look at for one of them, [kLongHead + i] entry i = row length << 32 | sample
 // index.  The longest have room of their own, so that a large call's many
-// moderate samples cannot leave a hub to one warp; what finds no room is
-// counted in place.
+// moderate samples cannot leave a hub to one warp.  What finds no room is
+// counted in place by its warp up to kLeftVertex / kLeftEdge entries; a longer
+// one is marked (kLeftOver as its first balanced count) and counted by a whole
+// block of the split launch, whose 16 warps share its entries: a hub left to
+// one warp was the length of the call (the 2,400-clique's vertex behind a full
+// queue: 148.6 ms, now 13.5).
 constexpr int kLongCap = kLongQueue;
 constexpr int kLongFirst = kLongCap - kLongest;
+constexpr uint32_t kLeftVertex = 256, kLeftEdge = kLongestRow;
+constexpr int64_t kLeftOver = -1;
 
 struct LocalArgs {
   const uint32_t* uptr;
@@ -285,8 +292,7 @@ __device__ __forceinline__ void edge_entries(const LocalArgs& a, const LocalP& p
 // Samples on a graph with the edge index: one warp each, no table -- a sampled
 // edge streams its shorter row, a sampled vertex takes the pairs of its row's
 // prefix, and every closing edge is looked up.  A sample with more than
-// `split` entries is queued for the split launch (kLongCap of them; more are
-// counted here).  A block and its table per sample, as without the index, kept
+// `split` entries is queued for the split launch (kLongCap of them).  A block and its table per sample, as without the index, kept
 // an SM at two samples at a time (Chung-Lu of 1e6 vertices, 10,000 samples:
 // edges 301 -> 59 us with the split launch, vertices 718 -> 580).
 constexpr int kSampleThreads = 128;
@@ -322,17 +328,20 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_warps(LocalArgs a, Lo
       }
       ok = len > 1;
     }
+    bool left = false;
     if (ok && len > (a.vertex_mode ? a.split : kEdgeSplit)) {
       uint32_t queued = 0;
       if (lane == 0) {
         const bool longest = len > kLongestRow;
         const unsigned long long slot = atomicAdd(&a.lq[longest ? 2 : 0], 1ull);
         if (slot < (unsigned long long)(longest ? kLongest : kLongFirst)) {
-          a.lq[3 + (longest ? kLongFirst : 0) + slot] = ((unsigned long long)len << 32) | item;
+          a.lq[kLongHead + (longest ? kLongFirst : 0) + slot] = ((unsigned long long)len << 32) | item;
           queued = 1;
         }
       }
-      if (__shfl_sync(kFull, queued, 0)) ok = false;  // its counts here stay 0
+      left = !__shfl_sync(kFull, queued, 0) && len > (a.vertex_mode ? kLeftVertex : kLeftEdge);
+      if (left && lane == 0) atomicAdd(&a.lq[3], 1ull);
+      ok = !left && !__shfl_sync(kFull, queued, 0);  // counted by the split launch: its counts here stay 0
     }
     if (ok) {
       if (!a.vertex_mode) {
@@ -367,7 +376,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_warps(LocalArgs a, Lo
       unsigned long long b = 0, u = 0;
       for (int r = 0; r <= p.nt - 1 - i; r++) b += bins[r];
       for (int r = p.nt + i + 1; r <= 2 * p.nt; r++) u += bins[r];
-      a.bal[(size_t)item * p.nt + p.perm[i]] = (int64_t)b;
+      a.bal[(size_t)item * p.nt + p.perm[i]] = left && p.perm[i] == 0 ? kLeftOver : (int64_t)b;
       a.unbal[(size_t)item * p.nt + p.perm[i]] = (int64_t)u;
     }
     __syncwarp();
@@ -537,7 +546,7 @@ __global__ void __launch_bounds__(512, 2) k_local_split(LocalArgs a, LocalP p) {
   const uint32_t n0 = (uint32_t)min(a.lq[0], (unsigned long long)kLongFirst);
   const uint32_t nq = n0 + (uint32_t)min(a.lq[2], (unsigned long long)kLongest);
   if (nq == 0) return;
-  auto queued = [&](uint32_t i) { return a.lq[3 + (i < n0 ? i : kLongFirst + (i - n0))]; };
+  auto queued = [&](uint32_t i) { return a.lq[kLongHead + (i < n0 ? i : kLongFirst + (i - n0))]; };
   {  // first warp task of every entry: a thread sums its segment, the block scans the sums
     __shared__ uint32_t s_warp[16];
     constexpr uint32_t seg = (kLongCap + 511) / 512;
@@ -595,6 +604,50 @@ __global__ void __launch_bounds__(512, 2) k_local_split(LocalArgs a, LocalP p) {
     index_neighbours(a, p, S, wb, x, rs, tlen, qmax, j0, j1, 1, lane);
   }
   if (cur != 0xFFFFFFFFu) flush_bins(a, p, wb, cur_item, lane);
+  if (a.lq[3] == 0) return;
+  // the samples left over, 32 looked at a time: the whole block counts each
+  __shared__ unsigned long long s_first;
+  __shared__ unsigned s_left;
+  const uint32_t nw = blockDim.x >> 5;
+  while (true) {
+    __syncthreads();
+    if (wid == 0) {
+      unsigned long long first = 0;
+      if (lane == 0) first = atomicAdd(&a.lq[4], 32ull);
+      first = __shfl_sync(kFull, first, 0);
+      const unsigned m = __ballot_sync(kFull, first + lane < a.n_items && a.bal[(first + lane) * p.nt] == kLeftOver);
+      if (lane == 0) {
+        s_first = first;
+        s_left = m;
+      }
+    }
+    __syncthreads();
+    const unsigned long long first = s_first;
+    unsigned left = s_left;
+    if (first >= a.n_items) break;
+    if (tid < 32 && ((left >> tid) & 1u)) a.bal[(first + tid) * p.nt] = 0;  // before any warp adds to it
+    __syncthreads();
+    while (left) {
+      const uint32_t item = (uint32_t)first + (uint32_t)__ffs(left) - 1u;
+      left &= left - 1;
+      if (!a.vertex_mode) {
+        uint32_t x = 0, qe = 0, s0 = 0, len = 0;
+        if (edge_sample(a, a.items[item], x, qe, s0, len, false))
+          for (uint32_t b = wid * kEdgeSplit; b < len; b += nw * kEdgeSplit)
+            edge_entries(a, p, S, wb, x, qe, s0 + b, s0 + min(len, b + kEdgeSplit), lane);
+      } else {
+        const uint32_t x = a.items[item], rs = a.uptr[x];
+        uint32_t len = a.uptr[x + 1] - rs;
+        int64_t qmax = 0;
+        if (a.L > 0) {
+          qmax = qabs(adj_valbits(a.uadj[rs]));
+          len = prune_prefix(a.uadj + rs, len, 1ll << 30, a.L);
+        }
+        index_neighbours(a, p, S, wb, x, rs, len, qmax, wid, len - 1, nw, lane);
+      }
+      flush_bins(a, p, wb, item, lane);
+    }
+  }
 }
 
 // estimate[t] = scale / k * sum over samples of the local count
@@ -664,7 +717,7 @@ ubt_status local_counts(ubt_graph* g, const uint32_t* d_items, int64_t k, int ve
   a.bal = d_bal;
   a.unbal = d_unbal;
   UBT_CUDA(cudaMemsetAsync(a.sc->task, 0, kScratchQuery, s));
-  UBT_CUDA(cudaMemsetAsync(a.lq, 0, 3 * sizeof(unsigned long long), s));
+  UBT_CUDA(cudaMemsetAsync(a.lq, 0, kLongHead * sizeof(unsigned long long), s));
   if (k > 0) {
     const int threads = 512;
     if (a.ix.mode != 0) {
