@@ -295,7 +295,15 @@ ubt_status ubt_set_edge_values(ubt_graph* g, const float* d_p, void* stream);
  * u_j = sum_b bit j of r_b * 2^b; the edge is positive iff u_j < k_e.
  *   d_bal_per_world  device int64[W].
  *   d_total          device int64[1]: sum over worlds (may be NULL).
- *   d_workspace      >= the queried bytes (sign table of one pass + counters).
+ *   d_workspace      256-byte aligned.  The queried size holds the sign table
+ *                    of the largest pass, m x 8 bytes a word (the knob
+ *                    "world_words_per_pass"; fewer where the table would take
+ *                    more than 36 GiB or, above 1 GiB, than 7/8 of the memory
+ *                    free at the query).  A smaller one serves too, in passes
+ *                    of as many words as fit and with the same counts, down to
+ *                    max(m, 1) x 8 x w + 256 bytes, w the largest power of two
+ *                    <= min(8, W / 64, the knob); less returns
+ *                    UBT_ERR_WORKSPACE_TOO_SMALL.
  * Graph kind: FIXED only.
  */
 ubt_status ubt_sample_worlds_workspace_size(const ubt_graph* g, int64_t W, size_t* h_bytes);
@@ -534,8 +542,7 @@ ubt_status ubt_topk(ubt_graph* g, int64_t K, int32_t which, ubt_tri_rec* d_out, 
  *                     by one warp each)
  *   "world_words_per_pass"  most 64-world words per traversal of
  *                     ubt_sample_worlds (1, 2, 4, 8, 16, 32 or 64, default
- *                     64; fewer where the sign table of m x 8 bytes a word
- *                     would exceed 36 GiB, but not fewer than 8 for that)
+ *                     64; fewer where the workspace holds fewer)
  *   "small_batch"     warp tasks taken per grab of a task counter
  *   "sort_smem_max"   longest list sorted in shared memory during the
  *                     build (power of two, 64..4096); longer lists are sorted

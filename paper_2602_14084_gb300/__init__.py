@@ -442,10 +442,23 @@ class Graph:
                "ubt_sample_worlds_workspace_size")
         return int(nb.value)
 
+    def _worlds_workspace(self, W):
+        """A workspace of the size asked for or, where the allocator has no room
+        for it, of a half, a quarter, ... of its words an edge, down to 8."""
+        torch = _torch()
+        nbytes = self.sample_worlds_workspace(W)
+        while True:
+            try:
+                return torch.empty(nbytes, dtype=torch.uint8, device=self.device)
+            except torch.cuda.OutOfMemoryError:
+                if nbytes - 256 <= 64 * max(self.m, 1):
+                    raise
+                nbytes = (nbytes - 256) // 2 + 256
+
     def sample_worlds_(self, seed, W, out, total=None, workspace=None, stream=None):
         torch = _torch()
         if workspace is None:
-            workspace = torch.empty(self.sample_worlds_workspace(W), dtype=torch.uint8, device=self.device)
+            workspace = self._worlds_workspace(W)
         _check(lib().ubt_sample_worlds(self._h, ctypes.c_uint64(int(seed)), int(W), _ptr(out), _ptr(total),
                                        _ptr(workspace), workspace.numel(), _stream(stream)), "ubt_sample_worlds")
         return out

@@ -548,25 +548,49 @@ ubt_status launch_w(const ubt_graph* g, const typename V::P& p, cudaStream_t s) 
 }
 
 // Words of a pass over `left` words: a power of two (lanes are grouped by
-// word), at most the tuning's, whose table (8 m bytes a word) takes at most an
-// eighth of the HBM or, for larger graphs, 8 words.  More words a pass list the
-// triangles fewer times and read longer rows (R-MAT scale 20, 64 words: one pass of 64 85 ms, eight
-// of 8 143 ms).  The last pass may have words to spare rather than be cut into
+// word), at most `most`.  More words a pass list the triangles fewer times and
+// read longer rows (R-MAT scale 20, 64 words: one pass of 64 85 ms, eight of 8
+// 143 ms).  The last pass may have words to spare rather than be cut into
 // several.
-constexpr int64_t kSignTableBytes = 36ll << 30;
-int64_t pass_words(const ubt_graph* g, int64_t left) {
-  int64_t wp = tuning().world_words_per_pass;
-  while (wp > 8 && g->m * wp * 8 > kSignTableBytes) wp >>= 1;
+int64_t pass_words(int64_t left, int64_t most) {
+  int64_t wp = most;
   while (wp > 1 && 4 * left < 3 * wp) wp >>= 1;
   return wp;
 }
 
-size_t worlds_table_words(const ubt_graph* g, int64_t W) {
-  return (size_t)std::max<int64_t>(g->m, 1) * (size_t)pass_words(g, W / 64);
+// bytes of a workspace whose sign table has `words` words an edge
+size_t worlds_workspace_bytes(const ubt_graph* g, int64_t words) {
+  return (size_t)std::max<int64_t>(g->m, 1) * (size_t)words * 8 + 256;
 }
 
-// the workspace ubt_sample_worlds_workspace_size reports and ubt_sample_worlds requires
-size_t worlds_workspace_bytes(const ubt_graph* g, int64_t W) { return worlds_table_words(g, W) * 8 + 256; }
+// The most words a call needs room for: every workspace from this size on
+// serves (the passes are the largest that fit it, with the same counts).
+constexpr int64_t kLeastWords = 8;
+int64_t least_words(int64_t words) {
+  int64_t wp = std::min(kLeastWords, tuning().world_words_per_pass);
+  while (wp > words) wp >>= 1;
+  return wp;
+}
+
+// What ubt_sample_worlds_workspace_size asks for: the tuning's words, unless
+// the table would take more than an eighth of the HBM or, above 1 GiB (where a
+// call lasts long enough for the question to cost nothing), than 7/8 of the
+// memory that is free now: a call beside other tenants of the GPU runs in
+// smaller passes instead of failing to allocate.
+constexpr int64_t kSignTableBytes = 36ll << 30, kSmallTableBytes = 1ll << 30;
+int64_t wanted_words(const ubt_graph* g, int64_t words) {
+  int64_t wp = pass_words(words, tuning().world_words_per_pass);
+  const int64_t word_bytes = g->m * 8;
+  if (wp <= kLeastWords || wp * word_bytes <= kSmallTableBytes) return wp;
+  size_t free_bytes = 0, all = 0;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // the question is harmless inside a capture
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (cudaMemGetInfo(&free_bytes, &all) != cudaSuccess) free_bytes = (size_t)kSignTableBytes;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const int64_t room = std::min<int64_t>(kSignTableBytes, (int64_t)(free_bytes / 8 * 7));
+  while (wp > kLeastWords && wp * word_bytes > room) wp >>= 1;
+  return wp;
+}
 
 }  // namespace
 }  // namespace ubt
@@ -575,7 +599,7 @@ using namespace ubt;
 
 extern "C" ubt_status ubt_sample_worlds_workspace_size(const ubt_graph* g, int64_t W, size_t* h_bytes) {
   if (!g || !h_bytes || W < 64 || W % 64) return UBT_ERR_INVALID_ARG;
-  *h_bytes = worlds_workspace_bytes(g, W);
+  *h_bytes = worlds_workspace_bytes(g, wanted_words(g, W / 64));
   return UBT_OK;
 }
 
@@ -585,13 +609,15 @@ extern "C" ubt_status ubt_sample_worlds(ubt_graph* g, uint64_t seed, int64_t W, 
   if (!g || !d_bal_per_world || W < 64 || W % 64 || W / 64 > 0xFFFFFFFFll) return UBT_ERR_INVALID_ARG;
   if (g->kind != UBT_GRAPH_FIXED) return UBT_ERR_UNSUPPORTED;
   if (!d_workspace || ((uintptr_t)d_workspace & 255)) return UBT_ERR_INVALID_ARG;
-  if (ws_bytes < worlds_workspace_bytes(g, W)) return UBT_ERR_WORKSPACE_TOO_SMALL;
-  cudaStream_t s = (cudaStream_t)stream;
   const int64_t words = W / 64;
+  int64_t most = least_words(words);
+  if (ws_bytes < worlds_workspace_bytes(g, most)) return UBT_ERR_WORKSPACE_TOO_SMALL;
+  while (2 * most <= tuning().world_words_per_pass && ws_bytes >= worlds_workspace_bytes(g, 2 * most)) most *= 2;
+  cudaStream_t s = (cudaStream_t)stream;
   unsigned long long* X = (unsigned long long*)d_workspace;
   UBT_CUDA(cudaMemsetAsync(d_bal_per_world, 0, sizeof(int64_t) * W, s));
   for (int64_t w0 = 0; w0 < words;) {
-    const int64_t wp = pass_words(g, words - w0), valid = std::min(wp, words - w0);
+    const int64_t wp = pass_words(words - w0, most), valid = std::min(wp, words - w0);
     const ubt_status sst = launch_sign_table(g, seed, w0, wp, valid, X, s);
     if (sst != UBT_OK) return sst;
     WorldsP p{X, (uint32_t)wp, (uint32_t)valid, (unsigned long long*)(d_bal_per_world + w0 * 64)};
