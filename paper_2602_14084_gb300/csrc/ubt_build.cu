@@ -1120,7 +1120,7 @@ struct BuildLayout {
   uint32_t* alist;
   unsigned long long* awork;
   unsigned long long* lqueue;  // long vertex samples of a local-count call (with the undirected rows)
-  uint32_t* efilter;           // filter of the edge index
+  uint32_t* efilter;           // filter of the edge index, in the build temporaries' place
   uint4* eslots;               // edge index (optional)
   int64_t eh_slots;
   unsigned long long* gacc;
@@ -1193,7 +1193,6 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.awork = und ? c.take<unsigned long long>(n1) : nullptr;
   L.lqueue = und ? c.take<unsigned long long>(kLongHead + kLongQueue) : nullptr;
   const bool eidx = und && (opts->flags & UBT_OPT_EDGE_INDEX);
-  L.efilter = und ? c.take<uint32_t>((size_t)(pow2_at_least(std::max<int64_t>(4 * m, 64)) >> kEdgeFilterLog)) : nullptr;
   L.eh_slots = eidx ? pow2_at_least(std::max<int64_t>(4 * m, 64)) : 0;
   L.eslots = eidx ? c.take<uint4>(L.eh_slots) : nullptr;
   L.gacc = c.take<unsigned long long>(std::max<int64_t>(m, 1));
@@ -1201,6 +1200,8 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.bacc = c.take<unsigned long long>(3 * std::max<int64_t>(ng, 1));
   const int64_t gslots = gtab_slots_for(m);
   L.gtab = gslots ? c.take<uint32_t>((size_t)gslots * 3 * (size_t)sm_count) : nullptr;
+  L.stats = c.take<unsigned long long>(kBuildWords);
+  const size_t temporaries = c.off;
   L.deg = c.take<uint32_t>(n + 1);
   L.fill = c.take<uint32_t>(n + 1);
   L.rank = c.take<uint32_t>(n1);
@@ -1213,10 +1214,17 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.huge_rows = c.take<uint32_t>(n1);
   L.bucket = c.take<uint8_t>(n1);
   L.work = c.take<unsigned long long>(n1);
-  L.stats = c.take<unsigned long long>(kBuildWords);
   const int64_t lb = list_bound(n, m);
   L.sort_tmp = lb > tuning().sort_smem_max
                    ? c.take<char>((size_t)kSortHugeBlocks * (size_t)pow2_at_least(lb) * 24) : nullptr;
+  // the filter takes the temporaries' place: the index is the last thing built
+  L.efilter = nullptr;
+  if (eidx) {
+    const size_t end = c.off;
+    c.off = temporaries;
+    L.efilter = c.take<uint32_t>((size_t)(L.eh_slots >> kEdgeFilterLog));
+    c.off = std::max(c.off, end);
+  }
   L.total = c.off + 256;
   return L;
 }
@@ -1454,15 +1462,6 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
       k_uepos<<<grid_2, thr, 0, s>>>(m2, urow, L.uadj, L.ueid, L.uepos);
       k_umirror<<<grid_e, thr, 0, s>>>(m, L.uepos, L.umir);
     }
-    if (L.eslots) {
-      UBT_CUDA(cudaMemsetAsync(L.eslots, 0xFF, sizeof(uint4) * (size_t)L.eh_slots, s));
-      UBT_CUDA(cudaMemsetAsync(L.efilter, 0, sizeof(uint32_t) * (size_t)(L.eh_slots >> kEdgeFilterLog), s));
-      int lg = 0;
-      while ((1ll << lg) < L.eh_slots) lg++;
-      if (m > 0)
-        k_edge_index<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, L.eslots, (uint64_t)L.eh_slots, 64 - lg, L.efilter,
-                                            derr);
-    }
     UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
     if (m > 0) k_apair_count<<<grid_2, thr, 0, s>>>(m2, L.uptr, L.uadj, urow, L.fill);
     UBT_CUDA(exclusive_scan_u32(L.fill, L.apair_ptr, n, L.scan_tmp, s, nullptr, L.awork));
@@ -1486,6 +1485,15 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
     n_aowners = (int64_t)run;
     UBT_CUDA(cudaMemcpyAsync(acur, acount, sizeof(acount), cudaMemcpyHostToDevice, s));
     k_afill_lists<<<grid_v, thr, 0, s>>>(n, L.uptr, L.apair_ptr, L.awork, acur, L.alist, 0);
+    if (L.eslots) {  // last: the filter lies where the build's temporaries were
+      UBT_CUDA(cudaMemsetAsync(L.eslots, 0xFF, sizeof(uint4) * (size_t)L.eh_slots, s));
+      UBT_CUDA(cudaMemsetAsync(L.efilter, 0, sizeof(uint32_t) * (size_t)(L.eh_slots >> kEdgeFilterLog), s));
+      int lg = 0;
+      while ((1ll << lg) < L.eh_slots) lg++;
+      if (m > 0)
+        k_edge_index<<<grid_e, thr, 0, s>>>(m, d_src, d_dst, d_k, L.eslots, (uint64_t)L.eh_slots, 64 - lg, L.efilter,
+                                            derr);
+    }
     unsigned long long err = 0;
     UBT_CUDA(cudaMemcpyAsync(&err, derr, sizeof(err), cudaMemcpyDeviceToHost, s));
     UBT_CUDA(cudaGetLastError());
