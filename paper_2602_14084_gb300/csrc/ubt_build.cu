@@ -1171,7 +1171,7 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.row_ptr = c.take<uint32_t>(n + 1);
   L.adj = c.take<uint64_t>(std::max<int64_t>(m, 1));
   L.eid = c.take<uint32_t>(std::max<int64_t>(m, 1));
-  L.rowid = c.take<uint32_t>(std::max<int64_t>(m, 1));
+  L.rowid = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(std::max<int64_t>(m, 1)) : nullptr;
   L.keep = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(m + 1) : nullptr;
   L.keep_tmp = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(scan_tmp_words(m)) : nullptr;
   L.ekey = has_key ? c.take<uint32_t>(std::max<int64_t>(m, 1)) : nullptr;
@@ -1196,6 +1196,9 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.eh_slots = eidx ? pow2_at_least(std::max<int64_t>(4 * m, 64)) : 0;
   L.eslots = eidx ? c.take<uint4>(L.eh_slots) : nullptr;
   L.gacc = c.take<unsigned long long>(std::max<int64_t>(m, 1));
+  // only enumeration (FIXED graphs) reads the row ids of a built graph; the
+  // build of a REAL one keeps them in the accumulators
+  if (!L.rowid) L.rowid = (uint32_t*)L.gacc;
   // per graph: T, sum_lo, sum_hi (expected counts) of a batch
   L.bacc = c.take<unsigned long long>(3 * std::max<int64_t>(ng, 1));
   const int64_t gslots = gtab_slots_for(m);
@@ -1513,7 +1516,7 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   g->row_ptr = L.row_ptr;
   g->adj = L.adj;
   g->eid = L.eid;
-  g->rowid = L.rowid;
+  g->rowid = flags == UBT_GRAPH_FIXED ? L.rowid : nullptr;
   g->keep = L.keep;
   g->keep_tmp = L.keep_tmp;
   for (int b = 64; b >= 0; b--) g->kept[b] = g->kept[b + 1] + (double)stats[kClasses + b];

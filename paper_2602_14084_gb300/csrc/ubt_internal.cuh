@@ -24,7 +24,7 @@ namespace ubt {
 //   FIXED graphs: q = 32768 - k as int32 (1 - 2 P+ = q / 2^15)
 //   REAL graphs:  s = 1 - 2 p as int32 fixed point, s * 2^30 rounded
 // eid[pos] is the input index of the edge stored at CSR position pos,
-// rowid[pos] its row.
+// rowid[pos] (FIXED graphs) its row.
 //
 // Pairs: a triangle u < v < w (Node Order) is found from the edge u -> v: its
 // owner is the later vertex v, whose list N>(v) becomes the table, and w lies
@@ -164,7 +164,7 @@ struct ubt_graph {
   uint32_t* row_ptr = nullptr;      // n + 1
   uint64_t* adj = nullptr;          // m
   uint32_t* eid = nullptr;          // m: input edge index per CSR position
-  uint32_t* rowid = nullptr;        // m: row per CSR position
+  uint32_t* rowid = nullptr;        // FIXED, m: row per CSR position (enumeration)
   uint32_t* ekey = nullptr;         // m: Philox key per CSR position
   uint32_t* pair_ptr = nullptr;     // n + 1: pairs of owner x are [pair_ptr[x], pair_ptr[x+1])
   uint64_t* pairs = nullptr;        // m: pair words

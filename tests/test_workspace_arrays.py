@@ -37,3 +37,8 @@ def test_index_is_its_slots_and_a_filter_in_place_of_the_build_arrays(ubt, n, m)
     slots = max(64, 1 << (4 * m - 1).bit_length())
     build_arrays = 33 * n  # at least: what only the build uses
     assert 16 * slots <= idx - und <= 16 * slots + max(0, slots // 4 - build_arrays) + 4096
+
+
+@pytest.mark.parametrize("n,m", [(100000, 1000000), (1000000, 9119924)])
+def test_real_graph_holds_no_row_ids_and_no_kept_counts(ubt, n, m):
+    assert size(ubt, n, m, FIXED) - size(ubt, n, m, REAL) >= 8 * m
