@@ -79,7 +79,7 @@ typedef struct {
     int64_t n;                /* vertices */
     int64_t m;                /* undirected edges */
     int64_t max_out_degree;   /* largest forward list under Node Order */
-    int64_t hub_vertices;     /* vertices handled by a whole thread block */
+    int64_t hub_vertices;     /* vertices handled by whole thread blocks */
     int64_t wedges;           /* sum over forward edges (u,v) of |N>(v)|: the
                                  entries Alg. 1 probes */
     int64_t kind;             /* UBT_GRAPH_FIXED or UBT_GRAPH_REAL */

@@ -757,10 +757,11 @@ static_assert(kTaskBuckets <= kNoTask, "a bucket is one byte");
 // stats: [0] oriented wedges sum_v in(v) |N>(v)| (Alg. 1's probes), [1] longest
 //        list, [2] streamed entries (set by k_pair_fill), [3] longest list of
 //        a kHubHash task, [4] of a kHubBits task, [5] largest range of one,
-//        [6] first pair of a vertex from merge_from on,
+//        [6] first pair of a vertex from merge_from on, [7] owners whose tasks
+//        are block tasks,
 //        [kStatBuckets + bucket] bucket sizes
 constexpr uint32_t kHeavyPairs = 1u << 16;
-constexpr int kStatBuckets = 7;
+constexpr int kStatBuckets = 8;
 // A pair's own loads count as this many streamed entries.
 constexpr unsigned long long kPairWork = 16;
 // An owner whose work exceeds part_work is several block tasks, each with its
@@ -785,15 +786,15 @@ __global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ r
                             uint8_t* __restrict__ bucket, unsigned long long* stats) {
   __shared__ uint32_t s_cnt[kTaskBuckets];
   __shared__ unsigned long long s_wedges;
-  __shared__ uint32_t s_max, s_hash, s_len, s_bits;
+  __shared__ uint32_t s_max, s_hash, s_len, s_bits, s_hubs;
   for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x) s_cnt[i] = 0;
-  if (threadIdx.x == 0) { s_wedges = 0; s_max = 0; s_hash = 0; s_len = 0; s_bits = 0; }
+  if (threadIdx.x == 0) { s_wedges = 0; s_max = 0; s_hash = 0; s_len = 0; s_bits = 0; s_hubs = 0; }
   __syncthreads();
   // small graphs: smaller block tasks, so that one warp's work is not the whole query's length
   const unsigned long long whole = whole_work(stats[2], m);
   block_work = min(block_work, max(2048ull, whole / 4096));
   unsigned long long wedges = 0;
-  uint32_t mx = 0, hash = 0, blen = 0, bits = 0;
+  uint32_t mx = 0, hash = 0, blen = 0, bits = 0, hubs = 0;
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t len = row_ptr[x + 1] - row_ptr[x];
     const uint32_t np = pair_ptr[x + 1] - pair_ptr[x];
@@ -810,6 +811,7 @@ __global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ r
       lg = lg > kLgTask ? kLgTask : lg;
       b = (uint8_t)(lg * kTaskClasses + cls);
       atomicAdd(&s_cnt[b], cls <= kHubBits ? owner_parts(w, whole) : 1u);
+      hubs += cls <= kHubBits ? 1u : 0u;
       if (cls == kHubHash) hash = max(hash, len);
       if (cls == kHubBits) {
         blen = max(blen, len);
@@ -824,6 +826,7 @@ __global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ r
   atomicMax(&s_hash, hash);
   atomicMax(&s_len, blen);
   atomicMax(&s_bits, bits);
+  if (hubs) atomicAdd(&s_hubs, hubs);
   __syncthreads();
   for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x)
     if (s_cnt[i]) atomicAdd(&stats[kStatBuckets + i], (unsigned long long)s_cnt[i]);
@@ -833,6 +836,7 @@ __global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ r
     atomicMax(&stats[3], (unsigned long long)s_hash);
     atomicMax(&stats[4], (unsigned long long)s_len);
     atomicMax(&stats[5], (unsigned long long)s_bits);
+    if (s_hubs) atomicAdd(&stats[7], (unsigned long long)s_hubs);
   }
 }
 
@@ -1564,6 +1568,7 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
   g->max_bits = (int64_t)stats[5];
   g->warp_bits = T.warp_bits;
   g->merge_first = merge_from < n ? (int64_t)stats[6] : m;
+  g->hub_vertices = (int64_t)stats[7];
   g->hub_threshold = hub_thr;
   g->giant_threshold = giant_thr;
   g->block_work = block_work;
@@ -1585,7 +1590,7 @@ extern "C" ubt_status ubt_graph_get_info(const ubt_graph* g, ubt_graph_info* h_i
   h_info->n = g->n;
   h_info->m = g->m;
   h_info->max_out_degree = g->max_out;
-  h_info->hub_vertices = g->n_tasks[kGiant] + g->n_tasks[kHubHash] + g->n_tasks[kHubBits];
+  h_info->hub_vertices = g->hub_vertices;
   h_info->wedges = g->wedges;
   h_info->kind = g->kind;
   h_info->probes = g->probes;

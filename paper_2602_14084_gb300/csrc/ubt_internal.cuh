@@ -205,6 +205,7 @@ struct ubt_graph {
   int64_t max_hash_len = 0;                 // longest list of a kHubHash task
   int64_t max_bits_len = 0, max_bits = 0;   // longest list and largest bit range of a kHubBits task
   int64_t warp_bits = 0;                    // bit range of the kMedBits tasks
+  int64_t hub_vertices = 0;                 // owners whose tasks are block tasks
   int64_t merge_first = 0;                  // pairs from here on are merged lane by lane (ubt_traverse.cuh)
   int64_t hub_threshold = 0, giant_threshold = 0, block_work = 0, pull = 1;
   double kept[66] = {0};  // FIXED: share of the edges with |q| >= 512 b (of a sample; [65] = 0)
