@@ -504,8 +504,12 @@ ubt_status ubt_topk(ubt_graph* g, int64_t K, int32_t which, ubt_tri_rec* d_out, 
  *                     written); queries do not depend on it
  *   "hub_threshold"   owners with longer lists than this are whole-block
  *                     tasks (default 128)
- *   "block_work"      owners whose pairs stream more entries than this are
- *                     whole-block tasks too (default 16384)
+ *   "block_work"      owners whose pairs stream more entries than this (a
+ *                     pair's own loads count as 16) are whole-block tasks too.
+ *                     The default, 16384, is lowered on a small graph to
+ *                     1/4096 of the whole work, at the least 2048; any other
+ *                     value is the limit as it is (an owner of more than
+ *                     65,536 pairs is a whole-block task under any)
  *   "block_threads"   threads per block of the kernel of the block tasks with
  *                     hash tables (64..512, /32, default 512)
  *   "warp_threads"    threads per block of the kernel of all other tasks

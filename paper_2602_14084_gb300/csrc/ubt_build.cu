@@ -790,9 +790,9 @@ __global__ void k_row_stats(int64_t n, int64_t m, const uint32_t* __restrict__ r
   for (int i = threadIdx.x; i < kTaskBuckets; i += blockDim.x) s_cnt[i] = 0;
   if (threadIdx.x == 0) { s_wedges = 0; s_max = 0; s_hash = 0; s_len = 0; s_bits = 0; s_hubs = 0; }
   __syncthreads();
-  // small graphs: smaller block tasks, so that one warp's work is not the whole query's length
   const unsigned long long whole = whole_work(stats[2], m);
-  block_work = min(block_work, max(2048ull, whole / 4096));
+  // the default limit on small graphs: smaller, so that one warp's work is not the whole query's length
+  if (block_work == kBlockWork) block_work = min(block_work, max(2048ull, whole / 4096));
   unsigned long long wedges = 0;
   uint32_t mx = 0, hash = 0, blen = 0, bits = 0, hubs = 0;
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {

@@ -216,10 +216,11 @@ namespace ubt {
 
 // ---------------------------------------------------------------- tuning
 
+constexpr int64_t kBlockWork = 1 << 14;
 struct Tuning {
   int64_t pull = 1;               // ubt_graph_export_pairs: 1 the longer list's endpoint owns, 0 the earlier one
   int64_t count_visitor = 0;      // threshold counts: 0 binned in the finding lane, 1 queued per warp
-  int64_t block_work = 1 << 14;   // owners streaming more entries are whole-block tasks
+  int64_t block_work = kBlockWork;  // owners streaming more entries are whole-block tasks (the default: fewer on small graphs)
   int64_t hub_threshold = 128;    // owners with longer lists are whole-block tasks
   int64_t block_threads = 512;    // threads of the block-task kernel
   int64_t warp_threads = 128;     // threads of the warp-task kernel (at most 128)

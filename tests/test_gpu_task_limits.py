@@ -44,3 +44,23 @@ def test_hub_vertices_counts_vertices(ubt):
     with knobs(ubt, block_work=1):
         G = ubt.Graph(400, s, d, k=synth.k_uniform(s.size, 1))
     assert G.info()["hub_vertices"] == 398
+
+
+@pytest.mark.parametrize("block_work", [1 << 16, 1 << 20, 1 << 30])
+def test_block_work_is_a_plain_limit(ubt, block_work):
+    """A limit that no owner of a 120-clique reaches leaves no block tasks."""
+    s, d = clique(120)
+    k = synth.k_uniform(s.size, 2)
+    with knobs(ubt, block_work=block_work):
+        G = ubt.Graph(120, s, d, k=k)
+    assert G.info()["hub_vertices"] == 0
+    want = oracle.count_threshold(120, s, d, k, [0.6, 0.9])
+    got = G.count_threshold([0.6, 0.9])
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+
+
+def test_default_block_work_spreads_small_graphs(ubt):
+    """The default limit is lowered for a small graph, so that no warp task is
+    the whole query."""
+    s, d = clique(120)
+    assert ubt.Graph(120, s, d, k=synth.k_uniform(s.size, 2)).info()["hub_vertices"] > 0
