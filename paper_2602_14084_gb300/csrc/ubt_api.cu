@@ -18,7 +18,10 @@ Tuning& tuning() {
 
 static char g_last_error[512];
 
+// Also takes the error off the runtime's own record: left there, the next call's
+// cudaGetLastError() after its launches would report it as its own.
 void set_last_cuda_error(cudaError_t e, const char* what, const char* file, int line) {
+  cudaGetLastError();
   snprintf(g_last_error, sizeof(g_last_error), "%s: %s (%s:%d)", cudaGetErrorString(e), what, file, line);
 }
 

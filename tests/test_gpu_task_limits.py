@@ -64,3 +64,17 @@ def test_default_block_work_spreads_small_graphs(ubt):
     the whole query."""
     s, d = clique(120)
     assert ubt.Graph(120, s, d, k=synth.k_uniform(s.size, 2)).info()["hub_vertices"] > 0
+
+
+def test_a_refused_launch_leaves_no_error_behind(ubt):
+    """A tuning whose tables no block has the shared memory for is refused; the
+    calls after it are not."""
+    n = 9000
+    s, d = core_graph(n, 300000, 4200, 3)
+    k = synth.k_uniform(s.size, 4)
+    with knobs(ubt, hub_threshold=4096, warp_bits=0, block_work=1 << 40):
+        G = ubt.Graph(n, s, d, k=k)
+        with pytest.raises(ubt.UbtError):
+            G.sample_worlds(seed=5, W=64)
+    w, total = ubt.Graph(n, s, d, k=k).sample_worlds(seed=5, W=64)
+    assert total == int(w.sum())
