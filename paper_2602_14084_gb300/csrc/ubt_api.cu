@@ -65,8 +65,10 @@ extern "C" const char* ubt_status_str(ubt_status s) {
 namespace ubt {
 
 // A fixed table of launch shapes, by a hash of the kernel and its shape; a
-// shape that meets another one's place replaces it.  Shared memory is allowed
-// up to the device's limit at once, so no later call lowers it.
+// shape that meets another one's place replaces it.  A kernel is allowed all
+// the shared memory of the device's limit that its own arrays leave, every
+// time, so no later shape lowers what a kept one needs; a shape above that is
+// cudaErrorInvalidValue.
 cudaError_t resident_blocks(const void* kernel, int device, int threads, size_t smem, int* per_sm) {
   struct Shape {
     const void* kernel;
@@ -81,8 +83,14 @@ cudaError_t resident_blocks(const void* kernel, int device, int threads, size_t 
   std::lock_guard<std::mutex> lock(mu);
   Shape& x = shapes[at];
   if (x.kernel != kernel || x.device != device || x.threads != threads || x.smem != smem) {
-    const size_t most = std::max(smem, (size_t)226 * 1024);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    int limit = 0;
+    cudaFuncAttributes own;
+    cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&own, kernel);
+    if (e != cudaSuccess) return e;
+    const size_t most = (size_t)limit - own.sharedSizeBytes;
+    if (smem > most) return cudaErrorInvalidValue;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     int n = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem);
     if (e != cudaSuccess) return e;

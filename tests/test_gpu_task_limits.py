@@ -78,3 +78,22 @@ def test_a_refused_launch_leaves_no_error_behind(ubt):
             G.sample_worlds(seed=5, W=64)
     w, total = ubt.Graph(n, s, d, k=k).sample_worlds(seed=5, W=64)
     assert total == int(w.sum())
+
+
+def test_a_shape_near_the_limit_stays_allowed(ubt):
+    """A launch with 226.4 KB of dynamic shared memory (a bitmap range of 65,536
+    and a list of 3,850 entries a warp, eight warps) runs again after a smaller
+    launch of the same kernel."""
+    core, n = 3900, 70000
+    s, d = clique(core)
+    T = math.comb(core, 3)
+    with knobs(ubt, hub_threshold=3850, warp_bits=65536, block_work=1 << 40, count_visitor=1):
+        G = ubt.Graph(n, s, d, k=synth.k_uniform(s.size, 6))
+        small_s, small_d = clique(80)
+        S = ubt.Graph(80, small_s, small_d, k=synth.k_uniform(small_s.size, 7))
+        first = G.count_threshold([0.5], prune=False)
+        b, u = S.count_threshold([0.5], prune=False)
+        assert b[0] + u[0] == math.comb(80, 3)
+        again = G.count_threshold([0.5], prune=False)
+    assert first[0][0] + first[1][0] == T
+    assert again[0][0] == first[0][0] and again[1][0] == first[1][0]
