@@ -1069,10 +1069,18 @@ ubt_status launch_kernel(const ubt_graph* g, const TravArgs& a, const typename V
   if (kKernel == kMainKernel && 2 * threads <= Bounds<V, kKernel>::kThreads &&
       8 * resident_warps<V, kKernel>(a, p, threads) < 7 * resident_warps<V, kKernel>(a, p, 2 * threads))
     threads *= 2;
-  const size_t smem = visitor_bytes<V>(p, threads) + traverse_table_bytes<V>(a, kKernel, threads);
+  // Smaller blocks where that many warps' tables do not fit at all (a large
+  // hub_threshold with a visitor that prefers large blocks).
+  size_t smem = 0;
   int per_sm = 0;
-  UBT_CUDA(resident_blocks((const void*)k_traverse<V, kKernel>, g->device, threads, smem, &per_sm));
-  if (per_sm < 1) return UBT_ERR_INVALID_ARG;
+  for (;; threads -= 32) {
+    smem = visitor_bytes<V>(p, threads) + traverse_table_bytes<V>(a, kKernel, threads);
+    const cudaError_t e = resident_blocks((const void*)k_traverse<V, kKernel>, g->device, threads, smem, &per_sm);
+    if (e == cudaSuccess && per_sm > 0) break;
+    if (threads > 64 && (e == cudaSuccess || e == cudaErrorInvalidValue)) continue;
+    UBT_CUDA(e);
+    return UBT_ERR_INVALID_ARG;
+  }
   per_sm = (int)std::min<int64_t>(per_sm, std::max<int64_t>(1, T.blocks_per_sm));
   int64_t blocks = (int64_t)g->sm_count * per_sm;
   if (kKernel == kMainKernel) {  // no more blocks than there is work for: each sets up its visitor's tables

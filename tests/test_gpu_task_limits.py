@@ -97,3 +97,17 @@ def test_a_shape_near_the_limit_stays_allowed(ubt):
         again = G.count_threshold([0.5], prune=False)
     assert first[0][0] + first[1][0] == T
     assert again[0][0] == first[0][0] and again[1][0] == first[1][0]
+
+
+@pytest.mark.parametrize("hub_threshold,warp_threads", [(1024, 64), (1024, 96), (1024, 128), (2048, 64)])
+def test_worlds_with_large_warp_tables(ubt, hub_threshold, warp_threads):
+    """Warp tables that leave no room for the block size the sign worlds prefer:
+    smaller blocks, not a refusal."""
+    n = 40000
+    s, d = core_graph(n, 1200000, 600, 3)
+    k = synth.k_uniform(s.size, 4)
+    want, total = ubt.Graph(n, s, d, k=k).sample_worlds(seed=5, W=128)
+    with knobs(ubt, hub_threshold=hub_threshold, warp_threads=warp_threads, warp_bits=0):
+        G = ubt.Graph(n, s, d, k=k)
+        got, t = G.sample_worlds(seed=5, W=128)
+    assert np.array_equal(got, want) and t == total and G.guard() == 0
