@@ -361,10 +361,10 @@ ubt_status ubt_traversal_stats(ubt_graph* g, const double* h_tau, int32_t n_tau,
 ubt_status ubt_query_guard(ubt_graph* g, int64_t* h_word, void* stream);
 
 /*
- * ubt_graph_export -- SYNC.  Copies the built graph to host memory for
- * inspection (any pointer may be NULL):
- * The host rearranges the device's arrays (kept in reverse Node Order) to the
- * caller's ids; this takes host memory for several copies of the graph.
+ * ubt_graph_export -- SYNC.  A view of the built graph by the caller's ids, in
+ * host memory (any pointer may be NULL).  The host rearranges the device's
+ * arrays, which ubt_graph_export_traversal shows as they are; this takes host
+ * memory for several copies of the graph.
  *   h_row_ptr  uint32[n + 1] forward-list offsets; FIXED lists by |1 - 2 P+|
  *              descending (ties by neighbour id), REAL lists by neighbour id
  *   h_adj      uint64[m] entries (low 32 bits neighbour id, high 32 bits the
@@ -392,6 +392,36 @@ ubt_status ubt_graph_export(const ubt_graph* g, uint32_t* h_row_ptr, uint64_t* h
  *              the edge (high 32 bits); order within an owner is unspecified
  */
 ubt_status ubt_graph_export_pairs(const ubt_graph* g, uint32_t* h_pair_ptr, uint64_t* h_pairs, void* stream);
+
+/*
+ * ubt_graph_export_traversal -- SYNC.  Copies the arrays that the queries read
+ * to host memory as the device holds them (any pointer may be NULL).  Here a
+ * vertex is its number: its position in reverse Node Order (the last vertex,
+ * of the highest degree, is 0; the graphs of a batch one after another, each
+ * ordered by itself).
+ *   h_vid      uint32[n] the caller's id of every number
+ *   h_row_ptr  uint32[n + 1] forward-list offsets; every list ascending by
+ *              number
+ *   h_adj      uint64[m] entries (low 32 bits the neighbour's number, high 32
+ *              bits the value, as in ubt_graph_export)
+ *   h_eid      uint32[m] input edge index of every entry
+ *   h_rowid    uint32[m] row of every entry (FIXED graphs; UBT_ERR_UNSUPPORTED
+ *              for a REAL one if not NULL)
+ *   h_pair_ptr uint32[n + 1] pairs of owner x are [h_pair_ptr[x], h_pair_ptr[x + 1])
+ *   h_pairs    uint64[m] one word per forward edge u -> v, at its owner v: bits
+ *              0..31 the start of row u, bits 32..48 the edge's position in
+ *              it (so many entries are streamed), bits 49..63 |q| >> 1 (FIXED);
+ *              order within an owner is unspecified
+ *   h_tasks    uint64[tasks] owner | part << 32 | (parts - 1) << 48, by class
+ *              and in a class the heavier (by the log2 of their work) first
+ *   h_sizes    int64[6] tasks of the five classes -- giant lists; block tasks
+ *              with a hash table, with a bitmap; warp tasks with a hash table,
+ *              with a bitmap -- and the first of the pairs that are merged
+ *              lane by lane (their owners are no tasks)
+ */
+ubt_status ubt_graph_export_traversal(const ubt_graph* g, uint32_t* h_vid, uint32_t* h_row_ptr, uint64_t* h_adj,
+                                      uint32_t* h_eid, uint32_t* h_rowid, uint32_t* h_pair_ptr, uint64_t* h_pairs,
+                                      uint64_t* h_tasks, int64_t* h_sizes, void* stream);
 
 /*
  * ubt_count_aeo -- ASYNC.  The counting problem (Def. 8) answered by the

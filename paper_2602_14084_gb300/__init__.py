@@ -84,6 +84,7 @@ def lib():
             "ubt_query_guard": (I32, [P, ctypes.POINTER(I64), P]),
             "ubt_graph_export": (I32, [P, P, P, P, P, P, P]),
             "ubt_graph_export_pairs": (I32, [P, P, P, P]),
+            "ubt_graph_export_traversal": (I32, [P] * 11),
             "ubt_graph_export_undirected": (I32, [P, P, P, P, P, P, P, P]),
             "ubt_count_aeo": (I32, [P, P, I32, P, P]),
             "ubt_topk_workspace_size": (I32, [I64, ctypes.POINTER(SZ)]),
@@ -261,6 +262,26 @@ class Graph:
                 "lists": lists[: int(sizes.sum())], "list_sizes": sizes, "pair_ptr": pp,
                 "pair_streamed": (pw[: self.m] & 0xFFFFFFFF).astype(np.uint32),
                 "pair_pos": (pw[: self.m] >> 32).astype(np.uint32)}
+
+    def export_traversal(self, stream=None) -> dict:
+        """The arrays the queries read, as the device holds them: vertices by
+        number, pair words, task lists (ubt_graph_export_traversal)."""
+        n, m = self.n, self.m
+        sizes = np.zeros(6, dtype=np.int64)
+        fn = lib().ubt_graph_export_traversal
+        c = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+        _check(fn(self._h, *[None] * 8, c(sizes), _stream(stream)), "ubt_graph_export_traversal")
+        ex = {"vid": np.zeros(max(n, 1), np.uint32), "row_ptr": np.zeros(n + 1, np.uint32),
+              "adj": np.zeros(max(m, 1), np.uint64), "eid": np.zeros(max(m, 1), np.uint32),
+              "rowid": np.zeros(max(m, 1), np.uint32) if self.kind == FIXED else None,
+              "pair_ptr": np.zeros(n + 1, np.uint32), "pairs": np.zeros(max(m, 1), np.uint64),
+              "tasks": np.zeros(max(int(sizes[:5].sum()), 1), np.uint64)}
+        _check(fn(self._h, *[None if a is None else c(a) for a in ex.values()], None, _stream(stream)),
+               "ubt_graph_export_traversal")
+        cut = {"vid": n, "adj": m, "eid": m, "rowid": m, "pairs": m, "tasks": int(sizes[:5].sum())}
+        ex = {k: a if a is None or k not in cut else a[: cut[k]] for k, a in ex.items()}
+        ex.update(task_sizes=sizes[:5], merge_first=int(sizes[5]))
+        return ex
 
     # ---------------------------------------------------------------- queries
 

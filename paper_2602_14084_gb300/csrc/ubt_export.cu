@@ -1,8 +1,8 @@
 // ubt_export.cu -- the built graph copied to the host for inspection.
 //
 // The library numbers vertices by reverse Node Order and sorts rows for the
-// traversal (ubt_internal.cuh).  The exports show the graph by the caller's
-// ids: forward lists in id order of their owners, FIXED lists by |q|
+// traversal (ubt_internal.cuh).  ubt_graph_export_traversal copies those arrays;
+// the other exports show the graph by the caller's ids: forward lists in id order of their owners, FIXED lists by |q|
 // descending (then id) and REAL ones by id, the pairs grouped by the owner
 // the "pull" tuning names, and the owners split into task classes by their
 // lists and streamed work.  The host rearranges copies of the device arrays.
@@ -152,4 +152,32 @@ extern "C" ubt_status ubt_graph_export_pairs(const ubt_graph* g, uint32_t* h_pai
   } catch (const std::exception&) {
     return UBT_ERR_INVALID_ARG;
   }
+}
+
+extern "C" ubt_status ubt_graph_export_traversal(const ubt_graph* g, uint32_t* h_vid, uint32_t* h_row_ptr,
+                                                 uint64_t* h_adj, uint32_t* h_eid, uint32_t* h_rowid,
+                                                 uint32_t* h_pair_ptr, uint64_t* h_pairs, uint64_t* h_tasks,
+                                                 int64_t* h_sizes, void* stream) {
+  if (!g) return UBT_ERR_INVALID_ARG;
+  if (h_rowid && !g->rowid) return UBT_ERR_UNSUPPORTED;
+  cudaStream_t s = (cudaStream_t)stream;
+  auto copy = [&](void* to, const void* from, size_t bytes) {
+    return to && bytes ? cudaMemcpyAsync(to, from, bytes, cudaMemcpyDeviceToHost, s) : cudaSuccess;
+  };
+  const size_t n = (size_t)g->n, m = (size_t)g->m;
+  UBT_CUDA(copy(h_vid, g->vid, 4 * n));
+  UBT_CUDA(copy(h_row_ptr, g->row_ptr, 4 * (n + 1)));
+  UBT_CUDA(copy(h_adj, g->adj, 8 * m));
+  UBT_CUDA(copy(h_eid, g->eid, 4 * m));
+  UBT_CUDA(copy(h_rowid, g->rowid, 4 * m));
+  UBT_CUDA(copy(h_pair_ptr, g->pair_ptr, 4 * (n + 1)));
+  UBT_CUDA(copy(h_pairs, g->pairs, 8 * m));
+  for (int c = 0; c < kTaskClasses; c++) {
+    UBT_CUDA(copy(h_tasks, g->lists[c], 8 * (size_t)g->n_tasks[c]));
+    if (h_tasks) h_tasks += g->n_tasks[c];
+    if (h_sizes) h_sizes[c] = g->n_tasks[c];
+  }
+  if (h_sizes) h_sizes[kTaskClasses] = g->merge_first;
+  UBT_CUDA(cudaStreamSynchronize(s));
+  return UBT_OK;
 }
