@@ -148,10 +148,8 @@ struct CountReg : ProductItem {
   __device__ void block_end() { flush(); }
 };
 
-__global__ void k_finish_reg(const unsigned long long* __restrict__ acc, int nt, int NT, const int* perm_unused,
-                             int64_t* __restrict__ out) {
+__global__ void k_finish_reg(const unsigned long long* __restrict__ acc, int nt, int NT, int64_t* __restrict__ out) {
   const int i = threadIdx.x;
-  (void)perm_unused;
   if (i < nt) {
     out[i] = (int64_t)acc[i];
     out[nt + i] = (int64_t)acc[NT + i];
@@ -769,7 +767,7 @@ ubt_status count_reg_at(const ubt_graph* g, const double* h_tau, int n_tau, int 
     default: st = launch_traversal<CountReg<8>>(g, a, p, s); break;
   }
   if (st != UBT_OK) return st;
-  k_finish_reg<<<1, kRegTau, 0, s>>>(acc, n_tau, NT, nullptr, d_counts);
+  k_finish_reg<<<1, kRegTau, 0, s>>>(acc, n_tau, NT, d_counts);
   UBT_CUDA(cudaGetLastError());
   return UBT_OK;
 }
@@ -854,7 +852,7 @@ ubt_status count_impl(ubt_graph* g, const double* h_tau, int32_t n_tau, int32_t 
       default: st = launch_count<CountReg<8>>(g, p, L, aeo, s); break;
     }
     if (st != UBT_OK) return st;
-    k_finish_reg<<<1, kRegTau, 0, s>>>(acc, n_tau, NT, nullptr, d_counts);
+    k_finish_reg<<<1, kRegTau, 0, s>>>(acc, n_tau, NT, d_counts);
     UBT_CUDA(cudaGetLastError());
     return UBT_OK;
   }

@@ -463,12 +463,6 @@ __device__ __forceinline__ void entry(const Table& t, uint32_t slot, uint32_t& v
   w = t.key[slot];
 }
 
-// entries a lane probes at a time in a long list, at most
-template <class T>
-struct ProbeWidth {
-  static constexpr int value = 4;
-};
-
 // ------------------------------------------------------------ the queue of hits
 
 // A warp's queue of items (V::Item, 8 or 16 bytes, the table slot in x) and, if
@@ -596,7 +590,7 @@ __device__ __forceinline__ void probe_pairs(const TravArgs& a, V& vis, Queue<V>&
     const uint32_t pj = __shfl_sync(kFull, pr.pe, j);
     uint32_t left = dvj, pos = vsj + lane;
     const uint64_t* __restrict__ row = adj + vsj + lane;
-    constexpr int kU = V::kU < ProbeWidth<T>::value ? V::kU : ProbeWidth<T>::value;
+    constexpr int kU = V::kU;
     while (left >= 32 * kU) {
       long_steps<V, T, kU, true>(row, pos, left, sc, vis, queue, t, lane, pr.x, sj, qj, pj);
       row += 32 * kU;
