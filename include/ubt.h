@@ -53,7 +53,7 @@ typedef int32_t ubt_status;
 #define UBT_ERR_PROB_OOB (-5)             /* k > 65536, or p outside [0,1] / NaN */
 #define UBT_ERR_TAU_OOB (-6)              /* t outside [0.5, 1] or NaN */
 #define UBT_ERR_CAPACITY (-7)             /* enumeration output too small */
-#define UBT_ERR_WORKSPACE_TOO_SMALL (-8)  /* workspace below the queried size */
+#define UBT_ERR_WORKSPACE_TOO_SMALL (-8)  /* workspace smaller than the call needs */
 #define UBT_ERR_TIMEOUT (-9)              /* reserved: a bounded device wait gave up */
 #define UBT_ERR_CUDA (-10)                /* a CUDA runtime call failed */
 #define UBT_ERR_UNSUPPORTED (-11)         /* operation not defined for this graph kind */
@@ -272,13 +272,12 @@ ubt_status ubt_expected_counts_backward(ubt_graph* g, const double* d_gout, floa
  * with d_p (device float[m], input edge order, each in [0, 1]) without
  * rebuilding it: every stored s = 1 - 2p is recomputed from the new p, in the
  * arithmetic of ubt_create_graph.  Structure, orientation and work lists are
- * unchanged (REAL rows are ordered by neighbour id, which p does not affect),
- * so expected counts and their adjoint then answer for the new p (Sec. 3's
+ * unchanged (no order of a REAL graph depends on p), so expected counts and their adjoint then answer for the new p (Sec. 3's
  * P_bal equation, with the new P+).  This is what a gradient step on p needs.
  * An entry outside [0, 1] or NaN keeps its old value, and the first such
  * input index is recorded in the self-check word (ubt_query_guard, code 6).
- * Graph kind: REAL only (UBT_ERR_UNSUPPORTED for FIXED: their rows are
- * ordered by |q|, which a new k would change).
+ * Graph kind: REAL only (UBT_ERR_UNSUPPORTED for FIXED: their pair words hold
+ * |q|, and their undirected rows are ordered by it).
  * Errors: UBT_ERR_INVALID_ARG, UBT_ERR_UNSUPPORTED, UBT_ERR_CUDA.
  */
 ubt_status ubt_set_edge_values(ubt_graph* g, const float* d_p, void* stream);
@@ -523,11 +522,10 @@ ubt_status ubt_topk(ubt_graph* g, int64_t K, int32_t which, ubt_tri_rec* d_out, 
  * ubt_set_tuning / ubt_get_tuning -- process-wide launch parameters that the
  * autotuner picks (they change speed, never results).  Unknown names return
  * UBT_ERR_INVALID_ARG.  Names:
- *   "count_visitor"   threshold counts: 0 (default) classify each triangle
- *                     in the lane that finds it (binned by a slice table);
- *                     1 queue products per warp and classify 32 at a time
- *                     (by binary search over the levels, or compared with
- *                     every threshold for at most 8)
+ *   "count_visitor"   threshold counts, classified 32 triangles of a warp at
+ *                     a time: 0 (default) placed among the levels by a slice
+ *                     table; 1 compared with every threshold for at most 8,
+ *                     by binary search over the levels for more
  *   "pull"            how ubt_graph_export_pairs groups the pairs of graphs
  *                     created afterwards: 1 (default) by the endpoint whose
  *                     list is longer, 0 by the earlier vertex (Alg. 1 as

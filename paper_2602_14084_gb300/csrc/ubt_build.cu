@@ -1601,7 +1601,7 @@ namespace ubt {
 namespace {
 
 // New edge values of a REAL graph: CSR position pos holds input edge eid[pos],
-// so its value becomes s(p[eid[pos]]); the rows stay sorted (by neighbour id).
+// so its value becomes s(p[eid[pos]]); the rows stay sorted (by vertex number).
 // A p outside [0, 1] (or NaN) leaves the entry as it was and records the
 // first such input index in the self-check word (code 6).
 __global__ void k_set_edge_values(int64_t m, const float* __restrict__ p, const uint32_t* __restrict__ eid,

@@ -219,11 +219,11 @@ namespace ubt {
 constexpr int64_t kBlockWork = 1 << 14;
 struct Tuning {
   int64_t pull = 1;               // ubt_graph_export_pairs: 1 the longer list's endpoint owns, 0 the earlier one
-  int64_t count_visitor = 0;      // threshold counts: 0 binned in the finding lane, 1 queued per warp
+  int64_t count_visitor = 0;      // threshold counts: 0 binned by a slice table, 1 compared or searched
   int64_t block_work = kBlockWork;  // owners streaming more entries are whole-block tasks (the default: fewer on small graphs)
   int64_t hub_threshold = 128;    // owners with longer lists are whole-block tasks
-  int64_t block_threads = 512;    // threads of the block-task kernel
-  int64_t warp_threads = 128;     // threads of the warp-task kernel (at most 128)
+  int64_t block_threads = 512;    // threads of the kernel of the block tasks with hash tables
+  int64_t warp_threads = 128;     // threads of the main kernel (bitmap block tasks, warp tasks, merges)
   int64_t blocks_per_sm = 32;     // cap on resident blocks (occupancy decides below it)
   int64_t smem_table_max = 8192;  // hash slots of a shared-memory table
   int64_t block_bits = 1 << 18;   // block tasks: largest vertex range of a bitmap table
