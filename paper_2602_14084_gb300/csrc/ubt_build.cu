@@ -1021,52 +1021,60 @@ __global__ void k_edge_index(int64_t m, const uint32_t* __restrict__ src, const 
 __device__ inline bool aeo_owns(uint32_t x, uint32_t y, uint32_t dx, uint32_t dy) {
   return dx > dy || (dx == dy && x > y);
 }
-__global__ void k_apair_count(int64_t m2, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
-                              const uint32_t* __restrict__ urow, uint32_t* __restrict__ pcount) {
+// The pairs keep the order of the rows -- an owner's strongest edges first -- so
+// that the edges a warp takes together pass or fail the cutoffs together: placed
+// by atomics, in the order that warps came, they cost k_aeo up to a fifth
+// (Chung-Lu of 1e6 vertices, t = 0.8: 9.3-10.0 ms, in order 8.5).  own[c]: which of the
+// entries [32 c, 32 c + 32) belong to their row's vertex, cnt[c] how many; the
+// scan of cnt then places every pair and every owner's first one.
+// work[x]: the entries that x's edges stream.
+__global__ void k_apair_own(int64_t m2, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
+                            const uint32_t* __restrict__ urow, uint32_t* __restrict__ own_bits,
+                            uint32_t* __restrict__ cnt, unsigned long long* __restrict__ work) {
   const uint32_t lane = lane_id();
   UBT_FOR_EDGE_WARPS(base, m2) {
     const int64_t p = base + lane;
+    uint32_t x = kEmpty, dy = 0;
     bool own = false;
-    uint32_t x = 0;
     if (p < m2) {
       x = urow[p];
       const uint32_t y = adj_col(uadj[p]);
-      own = aeo_owns(x, y, uptr[x + 1] - uptr[x], uptr[y + 1] - uptr[y]);
-    }
-    add_by_runs(pcount, x, own);
-  }
-}
-// pair words by owner: streamed endpoint | position of the edge in x's row << 32.
-// next[x] as in k_pair_fill (from apair_ptr[x], streamed entries in units); the
-// entries of a row are neighbours, so a warp adds once per row it holds.
-__global__ void k_apair_fill(int64_t m2, const uint32_t* __restrict__ uptr, const uint64_t* __restrict__ uadj,
-                             const uint32_t* __restrict__ urow, unsigned long long* __restrict__ next,
-                             uint64_t* __restrict__ apairs) {
-  const uint32_t lane = lane_id();
-  UBT_FOR_EDGE_WARPS(base, m2) {
-    const int64_t p = base + lane;
-    uint32_t x = kEmpty, y = 0, dy = 0;
-    bool own = false;
-    if (p < m2) {
-      x = urow[p];
-      y = adj_col(uadj[p]);
       dy = uptr[y + 1] - uptr[y];
       own = aeo_owns(x, y, uptr[x + 1] - uptr[x], dy);
     }
-    const unsigned row = __match_any_sync(kFull, x);  // the lanes of this lane's row
-    unsigned long long add = own ? ((unsigned long long)((dy + kWorkUnit - 1) / kWorkUnit) << 32) | 1ull : 0ull, incl = add;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {  // sums over the row's lanes up to this one (they are consecutive)
-      const unsigned long long o = __shfl_up_sync(kFull, incl, d);
-      if (lane >= (uint32_t)d && ((row >> (lane - d)) & 1u)) incl += o;
+    const unsigned bits = __ballot_sync(kFull, own);
+    if (lane == 0) {
+      own_bits[base >> 5] = bits;
+      cnt[base >> 5] = __popc(bits);
     }
-    const int last = 31 - __clz((int)row), head = __ffs(row) - 1;
-    const unsigned long long all = __shfl_sync(kFull, incl, last);
-    unsigned long long at = 0;
-    if ((int)lane == head && all) at = atomicAdd(&next[x], all);
-    at = __shfl_sync(kFull, at, head);
-    if (own) apairs[(uint32_t)at + (uint32_t)(incl - add)] = ((uint64_t)p << 32) | y;
+    // the entries of a row are neighbours: one add per row that the warp holds
+    const unsigned row = __match_any_sync(kFull, x);
+    unsigned long long sum = own ? dy : 0ull;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const unsigned long long o = __shfl_up_sync(kFull, sum, d);
+      if (lane >= (uint32_t)d && ((row >> (lane - d)) & 1u)) sum += o;
+    }
+    if ((int)lane == 31 - __clz((int)row) && sum) atomicAdd(&work[x], sum);
   }
+}
+// pairs before entry p (m2: all)
+__device__ __forceinline__ uint32_t apairs_before(uint32_t p, const uint32_t* __restrict__ own_bits,
+                                                  const uint32_t* __restrict__ before) {
+  const uint32_t in = p & 31u;
+  return before[p >> 5] + (in ? __popc(own_bits[p >> 5] & ((1u << in) - 1u)) : 0u);
+}
+__global__ void k_apair_ptr(int64_t n, const uint32_t* __restrict__ uptr, const uint32_t* __restrict__ own_bits,
+                            const uint32_t* __restrict__ before, uint32_t* __restrict__ apair_ptr) {
+  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x)
+    apair_ptr[x] = apairs_before(uptr[x], own_bits, before);
+}
+// pair words by owner: streamed endpoint | position of the edge in x's row << 32
+__global__ void k_apair_fill(int64_t m2, const uint64_t* __restrict__ uadj, const uint32_t* __restrict__ own_bits,
+                             const uint32_t* __restrict__ before, uint64_t* __restrict__ apairs) {
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m2; p += (int64_t)gridDim.x * blockDim.x)
+    if ((own_bits[p >> 5] >> (p & 31)) & 1u)
+      apairs[apairs_before((uint32_t)p, own_bits, before)] = ((uint64_t)p << 32) | adj_col(uadj[p]);
 }
 // owners by decreasing log2 of their streamed work, those with rows longer
 // than kAeoWarpRow (whole-block tasks) first: bucket = lg * 2 + (1 if block)
@@ -1085,7 +1093,7 @@ __global__ void k_afill_lists(int64_t n, const uint32_t* __restrict__ uptr, cons
     int b = 0;
     uint32_t rank = 0;
     if (on) {
-      const unsigned long long w = (work[x] >> 32) * kWorkUnit;
+      const unsigned long long w = work[x];
       b = (w ? 63 - __clzll(w) : 0) * 2 + (uptr[x + 1] - uptr[x] > kAeoWarpRow ? 1 : 0);
       rank = atomicAdd(&s_cnt[b], 1u);
     }
@@ -1176,7 +1184,7 @@ BuildLayout layout(void* ws, size_t cap, int64_t n, int64_t m, int32_t kind, con
   L.adj = c.take<uint64_t>(std::max<int64_t>(m, 1));
   L.eid = c.take<uint32_t>(std::max<int64_t>(m, 1));
   L.rowid = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(std::max<int64_t>(m, 1)) : nullptr;
-  L.keep = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(m + 1) : nullptr;
+  L.keep = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(m + 2) : nullptr;
   L.keep_tmp = kind == UBT_GRAPH_FIXED ? c.take<uint32_t>(scan_tmp_words(m)) : nullptr;
   L.ekey = has_key ? c.take<uint32_t>(std::max<int64_t>(m, 1)) : nullptr;
   L.pair_ptr = c.take<uint32_t>(n + 1);
@@ -1469,10 +1477,16 @@ extern "C" ubt_status ubt_create_graph(int64_t n, int64_t m, const uint32_t* d_s
       k_uepos<<<grid_2, thr, 0, s>>>(m2, urow, L.uadj, L.ueid, L.uepos);
       k_umirror<<<grid_e, thr, 0, s>>>(m, L.uepos, L.umir);
     }
-    UBT_CUDA(cudaMemsetAsync(L.fill, 0, sizeof(uint32_t) * (n + 1), s));
-    if (m > 0) k_apair_count<<<grid_2, thr, 0, s>>>(m2, L.uptr, L.uadj, urow, L.fill);
-    UBT_CUDA(exclusive_scan_u32(L.fill, L.apair_ptr, n, L.scan_tmp, s, nullptr, L.awork));
-    if (m > 0) k_apair_fill<<<grid_2, thr, 0, s>>>(m2, L.uptr, L.uadj, urow, L.awork, L.apairs);
+    // which entries are pairs, and how many before each 32 of them, in the (not
+    // yet used) words of the kept counts: 2 ceil(2m / 32) + 1 <= m + 2
+    const int64_t chunks = (m2 + 31) / 32;
+    uint32_t* const own_bits = L.keep;
+    uint32_t* const before = L.keep + chunks;
+    UBT_CUDA(cudaMemsetAsync(L.awork, 0, sizeof(unsigned long long) * n, s));
+    if (m > 0) k_apair_own<<<grid_2, thr, 0, s>>>(m2, L.uptr, L.uadj, urow, own_bits, before, L.awork);
+    UBT_CUDA(exclusive_scan_u32(before, before, chunks, L.keep_tmp, s));
+    k_apair_ptr<<<grid_v, thr, 0, s>>>(n, L.uptr, own_bits, before, L.apair_ptr);
+    if (m > 0) k_apair_fill<<<grid_2, thr, 0, s>>>(m2, L.uadj, own_bits, before, L.apairs);
     unsigned long long* acur = L.stats;  // 2 (kLgMax + 1) cursors
     constexpr int kAB = 2 * (kLgMax + 1);
     UBT_CUDA(cudaMemsetAsync(acur, 0, sizeof(unsigned long long) * kAB, s));

@@ -181,3 +181,24 @@ def test_the_check_sees_a_planted_mistake(ubt):
     plant("tasks", lambda a: a.__setitem__(split, a[split + 1]))
     plant("tasks", lambda a: a.__setitem__(split, a[split] - np.uint64(1 << 48)))
     plant("task_sizes", lambda a: a.__iadd__(np.array([0, 1, -1, 0, 0])))
+
+
+@pytest.mark.parametrize("name", ["empty", "one", "core", "rmat15", "star"])
+def test_edges_of_alg_2_keep_the_order_of_their_rows(ubt, name):
+    """Every edge once, at the endpoint with the longer row (ties: the larger
+    id), and an owner's edges in the order of its row."""
+    n, (s, d) = {"empty": (7, (np.zeros(0, np.uint32), np.zeros(0, np.uint32))),
+                 "one": (40, (np.array([3], np.uint32), np.array([39], np.uint32))),
+                 "core": (3000, core_graph(3000, 20000, 600, 15)),
+                 "rmat15": (1 << 15, synth.rmat(15, 16, 0.57, 0.19, 0.19, 3)),
+                 "star": (70001, (np.zeros(70000, np.uint32), np.arange(1, 70001, dtype=np.uint32)))}[name]
+    G = ubt.Graph(n, s, d, k=synth.k_uniform(s.size, 5), undirected=True)
+    ex = G.export_undirected()
+    up = ex["uptr"].astype(np.int64)
+    deg = np.diff(up)
+    row, col = np.repeat(np.arange(n), deg), ex["col"].astype(np.int64)
+    own = (deg[row] > deg[col]) | ((deg[row] == deg[col]) & (row > col))
+    pos = np.nonzero(own)[0]
+    assert pos.size == s.size
+    assert np.array_equal(ex["apair_ptr"], np.concatenate([[0], np.cumsum(np.bincount(row[pos], minlength=n))]))
+    assert np.array_equal(ex["apair_pos"], pos) and np.array_equal(ex["apair_other"], col[pos])
