@@ -681,6 +681,9 @@ __global__ void k_row_ids(int64_t n, const uint32_t* __restrict__ row_ptr, const
 // returning atomic from most rows, one after another in L2: a block ranks the
 // pairs of the first kHotOwners vertices among its kFillTile entries in shared
 // memory and reserves one range per vertex (Chung-Lu of 1e6 vertices: 656 -> 185 us).
+// Counts and work are 32-bit words there: a returning 64-bit shared-memory add
+// goes round a loop once per lane of the same address, and where one vertex is
+// in every row (a star of 2e6 leaves) that was the kernel (329 us, now 25).
 // What remains is bound by the atomics' and the pair words' random sectors.
 constexpr uint32_t kWorkUnit = 8;
 constexpr int kFillThreads = 256, kFillItems = 16;
@@ -691,11 +694,11 @@ k_pair_fill(int64_t m, const uint32_t* __restrict__ row_ptr, const uint64_t* __r
             const uint32_t* __restrict__ rowid, unsigned long long* __restrict__ next, uint64_t* __restrict__ pairs,
             unsigned long long* __restrict__ absq, unsigned long long* __restrict__ streamed) {
   __shared__ uint32_t s_q[65];
-  __shared__ unsigned long long s_hot[kHotOwners];  // count | work << 32, then the reserved base
+  __shared__ uint32_t s_hot[kHotOwners], s_work[kHotOwners];  // count, then the reserved base; work
   for (int i = threadIdx.x; i < 65; i += kFillThreads) s_q[i] = 0;
   unsigned long long sum = 0;
   for (int64_t base = blockIdx.x * kFillTile; base < m; base += (int64_t)gridDim.x * kFillTile) {
-    for (uint32_t i = threadIdx.x; i < kHotOwners; i += kFillThreads) s_hot[i] = 0;
+    for (uint32_t i = threadIdx.x; i < kHotOwners; i += kFillThreads) s_hot[i] = s_work[i] = 0;
     __syncthreads();
     uint32_t v[kFillItems], at[kFillItems];
     unsigned long long word[kFillItems];
@@ -715,18 +718,23 @@ k_pair_fill(int64_t m, const uint32_t* __restrict__ row_ptr, const uint64_t* __r
       }
       word[j] = pair_pack(start, len, aq >> 1);
       sum += len;
-      const unsigned long long add = ((unsigned long long)((len + kWorkUnit - 1) / kWorkUnit) << 32) | 1ull;
-      at[j] = v[j] < kHotOwners ? (uint32_t)atomicAdd(&s_hot[v[j]], add) : (uint32_t)atomicAdd(&next[v[j]], add);
+      const uint32_t units = (len + kWorkUnit - 1) / kWorkUnit;
+      if (v[j] < kHotOwners) {
+        at[j] = atomicAdd(&s_hot[v[j]], 1u);
+        if (units) atomicAdd(&s_work[v[j]], units);
+      } else {
+        at[j] = (uint32_t)atomicAdd(&next[v[j]], ((unsigned long long)units << 32) | 1ull);
+      }
     }
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < kHotOwners; i += kFillThreads) {
-      const unsigned long long c = s_hot[i];
-      if (c) s_hot[i] = atomicAdd(&next[i], c);
+      const uint32_t c = s_hot[i];
+      if (c) s_hot[i] = (uint32_t)atomicAdd(&next[i], ((unsigned long long)s_work[i] << 32) | c);
     }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kFillItems; j++)
-      if (v[j] != kEmpty) pairs[v[j] < kHotOwners ? (uint32_t)s_hot[v[j]] + at[j] : at[j]] = word[j];
+      if (v[j] != kEmpty) pairs[v[j] < kHotOwners ? s_hot[v[j]] + at[j] : at[j]] = word[j];
     __syncthreads();
   }
 #pragma unroll
