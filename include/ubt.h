@@ -570,7 +570,7 @@ ubt_status ubt_topk(ubt_graph* g, int64_t K, int32_t which, ubt_tri_rec* d_out, 
  *                     spread over the warps of all blocks by a second launch
  *                     (at most 3,072 per call, and 1,024 with rows of more
  *                     than 1,024 entries; of the rest those with more than
- *                     256 entries are counted by one block each, the others
+ *                     1,024 entries are counted by one block each, the others
  *                     by one warp each)
  *   "world_words_per_pass"  most 64-world words per traversal of
  *                     ubt_sample_worlds (1, 2, 4, 8, 16, 32 or 64, default

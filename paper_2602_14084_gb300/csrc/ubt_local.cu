@@ -187,10 +187,12 @@ EdgeIndex edge_index_of(const ubt_graph* g) {
 // one is marked (kLeftOver as its first balanced count) and counted by a whole
 // block of the split launch, whose 16 warps share its entries: a hub left to
 // one warp was the length of the call (the 2,400-clique's vertex behind a full
-// queue: 148.6 ms, now 13.5).
+// queue: 148.6 ms, now 14.0).  Shorter ones are some milliseconds of a warp at
+// the most, and a call with many of them keeps every warp busy without the
+// blocks' barriers (20,000 samples of rows of 900: 73 ms in place, 82 by blocks).
 constexpr int kLongCap = kLongQueue;
 constexpr int kLongFirst = kLongCap - kLongest;
-constexpr uint32_t kLeftVertex = 256, kLeftEdge = kLongestRow;
+constexpr uint32_t kLeftVertex = kLongestRow, kLeftEdge = 32768;
 constexpr int64_t kLeftOver = -1;
 
 struct LocalArgs {
@@ -605,7 +607,9 @@ __global__ void __launch_bounds__(512, 2) k_local_split(LocalArgs a, LocalP p) {
   }
   if (cur != 0xFFFFFFFFu) flush_bins(a, p, wb, cur_item, lane);
   if (a.lq[3] == 0) return;
-  // the samples left over, 32 looked at a time: the whole block counts each
+  // the samples left over, at most 32 looked at a time (fewer in a small call,
+  // or a few blocks had them all): the whole block counts each
+  const uint32_t grab = min(32u, a.n_items / (8 * gridDim.x) + 1);
   __shared__ unsigned long long s_first;
   __shared__ unsigned s_left;
   const uint32_t nw = blockDim.x >> 5;
@@ -613,9 +617,9 @@ __global__ void __launch_bounds__(512, 2) k_local_split(LocalArgs a, LocalP p) {
     __syncthreads();
     if (wid == 0) {
       unsigned long long first = 0;
-      if (lane == 0) first = atomicAdd(&a.lq[4], 32ull);
+      if (lane == 0) first = atomicAdd(&a.lq[4], (unsigned long long)grab);
       first = __shfl_sync(kFull, first, 0);
-      const unsigned m = __ballot_sync(kFull, first + lane < a.n_items && a.bal[(first + lane) * p.nt] == kLeftOver);
+      const unsigned m = __ballot_sync(kFull, (uint32_t)lane < grab && first + lane < a.n_items && a.bal[(first + lane) * p.nt] == kLeftOver);
       if (lane == 0) {
         s_first = first;
         s_left = m;

@@ -63,7 +63,7 @@ def test_a_hub_behind_a_full_queue_is_not_left_to_one_warp(ubt):
 
 
 @pytest.mark.parametrize("taus", [[0.5], [0.8, 0.6, 0.95]])
-@pytest.mark.parametrize("split", [32, 300, 1100])
+@pytest.mark.parametrize("split", [32, 300, 1050])
 def test_more_long_samples_than_the_queue_holds(ubt, split, taus):
     """Every sample's counts, with both parts of the queue full, the rest above
     and below the length that whole blocks take."""
