@@ -14,7 +14,11 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture(scope="module")
 def ubt():
-    return require_gpu()
+    ubt = require_gpu()
+    old = ubt.get_tuning("world_words_per_pass")
+    ubt.set_tuning("world_words_per_pass", 64)  # the default, whatever ran before
+    yield ubt
+    ubt.set_tuning("world_words_per_pass", old)
 
 
 def run_in(ubt, G, W, nbytes):
