@@ -235,6 +235,9 @@ struct Worlds {
   static constexpr bool kMore = false;
   static constexpr int kU = 2;
   static constexpr bool kPos = true;
+  // the main kernel's form of Worlds<2> spills at this cap (964 bytes of stores,
+  // 1,784 of loads a thread by the compiler's account): 24 planes and 16 words of
+  // 64 bits are live beside the flush
   static constexpr int kRegCap = 128;
   // a block's counters are 32 KB that L1, where the owner's sign rows stay, loses
   // (R-MAT scale 20, 4,096 worlds: 94.7 ms in blocks of 128 threads, 76.7 of 256)
@@ -387,7 +390,9 @@ struct Batch {
   static constexpr bool kMore = false;
   static constexpr int kU = 2;
   // 24 warps an SM instead of 16: the triangles' sign words and list entries are
-  // waited on (batch of 1,000 graphs: 9.9 ms with up to 128 registers, 8.7 with 85, 9.0 with 64)
+  // waited on (batch of 1,000 graphs: 9.9 ms with up to 128 registers, 8.7 with
+  // 85, 9.0 with 64; at 85 the compiler takes 80 and spills 568 bytes of stores,
+  // 836 of loads a thread)
   static constexpr int kRegCap = 85;
   static __host__ __device__ int smem_bytes(const P&, int) { return 0; }
   static constexpr int K = 8;                        // planes: fewer than 256 words between two flushes
