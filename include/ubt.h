@@ -494,7 +494,8 @@ ubt_status ubt_vertex_topk(ubt_graph* g, const uint32_t* d_vertices, int64_t k, 
  *   h_umir uint32[2m] position of the same edge in the other endpoint's row;
  *   h_apair_ptr uint32[n+1], h_apairs uint64[m]: the edges ubt_count_aeo
  *   handles from x (the endpoint with the longer row, ties to the larger id):
- *   the other endpoint (low 32 bits), the edge's position in x's row (high).
+ *   the other endpoint (low 32 bits), the edge's position in x's row (high),
+ *   in the order of x's row.
  */
 ubt_status ubt_graph_export_undirected(const ubt_graph* g, uint32_t* h_uptr, uint64_t* h_uadj, uint32_t* h_ueid,
                                        uint32_t* h_umir, uint32_t* h_apair_ptr, uint64_t* h_apairs, void* stream);
